@@ -540,7 +540,8 @@ def main():
     scatter_region = max(4096, (n // p + 7) // 8)
     scatter_peak = bfs.measure_scatter_reads(scatter_region) / 1e9
     nb_range = -(-n // p)
-    window = 8 * -(-nb_range // 32) + 4096 <= 227 * 1024      # the library's row-window rule
+    # the library's row-window rule: a range's visited bits fit beside the warps' scratch
+    window = n >= 1 << 21 and 4 * -(-nb_range // 32) <= 227 * 1024 - 32 * 896 - 2048
     roofline = None
     if ex:
         ex_ms = ex["avg_launch_ms"] * ex["launches"]
@@ -705,11 +706,10 @@ def main():
 
     valid = invariant_ok == len(roots) and oracle_exact in (None, 1)
     # kernels of the timed steps, per level: the encoder's three passes (not PLAIN), the
-    # expansion and the piece kernel (two variants each off the row window), the
-    # row encoder's three passes and the fold (row exchange), the reduction and the
-    # level step; per search the init, root and first-level kernels
-    variants = 1 if window else 2
-    launches_per_level = (0 if args.mode == 0 else 3) + 2 * variants + 2 + (4 if value_rowx else 0)
+    # expansion and the piece kernel, the row encoder's three passes and the fold (row
+    # exchange), the reduction and the level step; per search the init, root and
+    # first-level kernels
+    launches_per_level = (0 if args.mode == 0 else 3) + 2 + 2 + (4 if value_rowx else 0)
     if args.direction != "top_down":     # bottom-up expansion (+ clear and decode of the streams)
         launches_per_level += 1 if args.mode == 0 else (4 if args.format == "adaptive" else 3)
     gpu_launches = args.steps * sum(3 + launches_per_level * st.n_levels for st in main_arm["stats"])

@@ -55,13 +55,17 @@ namespace {
 constexpr int kNT = 256;            // threads of the small kernels
 constexpr int kXT = 1024;           // threads of the expansion CTAs
 constexpr int kXW = kXT / 32;       // warps of the expansion CTAs
-constexpr uint32_t kCoop = 64;      // columns of at least this many entries take the whole warp
-constexpr uint32_t kHub = 2048;     // columns longer than this are cut into pieces
-constexpr uint32_t kPiece = 2048;   // entries per piece
+#ifndef BFS_COOP
+#define BFS_COOP 64
+#endif
+constexpr uint32_t kCoop = BFS_COOP;      // columns of at least this many entries take the whole warp
+constexpr uint32_t kHub = 2048;     // columns longer than this are cut into pieces of this size
+constexpr uint32_t kHubSparse = 512;  // the same on levels with fewer units than warps
 #ifndef BFS_GUIDE
 #define BFS_GUIDE 1
 #endif
 constexpr int64_t kGuide = BFS_GUIDE;  // a grab takes 1/(kGuide * warps) of the units left in the row
+constexpr int64_t kWindowMinVertices = 1 << 21;   // below, all visited bits fit in L1: no row window
 constexpr int64_t kSmemLimit = 227 * 1024;
 
 // Per-level values that the device keeps from level to level, so that one
@@ -70,7 +74,8 @@ struct LevelCtl {
     int64_t frontier;      // vertices of the current frontier
     int64_t visited;       // vertices visited so far
     int32_t level;         // current level k
-    int32_t plain_batch;   // PLAIN units per hand-out
+    int32_t window;        // the expansion loads the row window (dense levels)
+    int32_t win_ratio;     // entries of the frontier per vertex of the graph from which on it does
     int32_t dedup;         // read the parent before updating it
     int32_t go;            // 1 while another level follows
     int64_t m_f;           // degree sum of the frontier
@@ -95,6 +100,7 @@ struct LevelArgs {
     const uint32_t* f;
     const uint32_t* pi;
     uint32_t* t;
+    const uint8_t* fsum;                // frontier summary: 1 per 1024 bits of f with a set bit
     int32_t* parent;
     // exchange
     const void* xbuf;
@@ -127,7 +133,6 @@ struct LevelArgs {
     const int64_t* col_first;           // the same for the column slots (bottom-up levels)
     int64_t row_cps;                    // encoder chunks per slot
     int64_t row_bcps;                   // fold chunks per range
-    int sweep;                          // all CTAs start at row 0 (rows in turn)
     const LevelCtl* ctl;                // this level's values
     // bottom-up levels
     uint32_t* gbits;                    // decoded streams (n bits, OR over the block-rows)
@@ -145,45 +150,49 @@ __device__ __forceinline__ int64_t range_begin(const LevelArgs& a, int64_t b) {
 // -------------------------------------------------------------- visiting --
 // Visit entry u -> v: if v was not visited before this level, lower parent[v]
 // to u and set v's next bit.  The parent update is a reduction whose result
-// is not used (fire-and-forget at L2).  With a row window, the visited test
-// and the next bit live in shared memory; without, the visited word is read
-// through the read-only path (pi does not change during the expansion) and
-// the next bit is a reduction at L2.
-template <bool WIN, bool DEDUP, bool ROWX>
+// is not used (fire-and-forget at L2).  WIN says what the CTA's row window in
+// shared memory holds:
+//   kWinNone  nothing: the visited word is read through the read-only path (pi
+//             does not change during the expansion) and the next bit is a
+//             reduction at L2;
+//   kWinPi    the visited bits pi_i of the row; the next bit goes to L2 (or,
+//             with the row exchange, to the visiting block's partial);
+//   kWinBoth  pi_i and the CTA's partial next bits t_i.
+enum Window : int { kWinNone = 0, kWinPi = 1, kWinBoth = 2 };
+constexpr uint32_t kNoVertex = 0xffffffffu;
+
+template <int WIN, bool DEDUP, bool ROWX>
 struct Visitor {
     const uint32_t* s_pi;
     uint32_t* s_t;
-    int64_t rb;     // first vertex of the row
+    uint32_t rb;    // first vertex of the row
     uint32_t* tb;   // row exchange: the partial bitmap of the visiting block (i,j), or nullptr
     uint32_t jb;    // row exchange: first vertex of the block's source range j
     // The visited word of v (loads of several entries are issued before
     // their visits, so that their latencies overlap).
-    __device__ __forceinline__ uint32_t probe(const LevelArgs& a, int32_t v) const {
-        if (WIN) return s_pi[(uint32_t)(v - rb) >> 5];
-        return __ldg(a.pi + ((uint32_t)v >> 5));
+    __device__ __forceinline__ uint32_t probe(const LevelArgs& a, uint32_t v) const {
+        if (WIN != kWinNone) return s_pi[(v - rb) >> 5];
+        return __ldg(a.pi + (v >> 5));
     }
-    __device__ __forceinline__ bool fresh(int32_t v, uint32_t piw) const {
-        const uint32_t b = WIN ? (uint32_t)(v - rb) : (uint32_t)v;
-        return !(piw & (1u << (b & 31u)));
+    __device__ __forceinline__ bool fresh(uint32_t v, uint32_t piw) const {
+        const uint32_t b = WIN != kWinNone ? v - rb : v;
+        return !((piw >> (b & 31u)) & 1u);
     }
     // The parent recorded so far for a fresh v (possibly an older value: the
     // parent only decreases during a level, from -1 = the largest unsigned).
-    __device__ __forceinline__ uint32_t seen(const LevelArgs& a, int32_t v) const {
+    __device__ __forceinline__ uint32_t seen(const LevelArgs& a, uint32_t v) const {
         return __ldcg(reinterpret_cast<const unsigned int*>(a.parent) + v);
     }
     // The word of v's bit in the visiting block's partial t_{i,j} (row exchange).
-    __device__ __forceinline__ uint32_t seen_t(int32_t v) const {
-        const uint32_t vl = (uint32_t)(v - rb);
-        return __ldcg(tb + (vl >> 5));
-    }
-    // After the visited word piw of v was probed: v <- -1 if v was visited
-    // before the level (nothing to do), else pv <- the parent read first
-    // (DEDUP) or -1, and tw <- the partial's word read first (DEDUP with the
-    // row exchange) or 0.
-    __device__ __forceinline__ void stage(const LevelArgs& a, int32_t& v, uint32_t& piw, uint32_t& tw) const {
+    __device__ __forceinline__ uint32_t seen_t(uint32_t v) const { return __ldcg(tb + ((v - rb) >> 5)); }
+    // After the visited word piw of v was probed: v <- kNoVertex if v was
+    // visited before the level (nothing to do), else piw <- the parent read
+    // first (DEDUP) or -1, and tw <- the partial's word read first (DEDUP with
+    // the row exchange) or 0.
+    __device__ __forceinline__ void stage(const LevelArgs& a, uint32_t& v, uint32_t& piw, uint32_t& tw) const {
         tw = 0u;
-        if (v < 0 || !fresh(v, piw)) {
-            v = -1;
+        if (v == kNoVertex || !fresh(v, piw)) {
+            v = kNoVertex;
             return;
         }
         piw = DEDUP ? seen(a, v) : 0xffffffffu;
@@ -194,27 +203,27 @@ struct Visitor {
     // visitor in this level, which set the next bit); otherwise lower the
     // parent, and the visitor that read -1 sets the next bit.  The visitor of
     // the first update read -1, so the bit is always set.
-    __device__ __forceinline__ void mark(const LevelArgs& a, int32_t v, int32_t u, uint32_t pv, uint32_t tw) const {
+    __device__ __forceinline__ void mark(const LevelArgs& a, uint32_t v, uint32_t u, uint32_t pv, uint32_t tw) const {
         if (ROWX) {
             // Row exchange: every block that reaches v records it in its own
             // partial t_{i,j}.  The bit is already there when the word read
             // first has it, or when the parent read first lies in [jb, u]: a
             // visitor of the same source range lowered it and records v in
             // the same partial.  The parent is lowered when pv > u.
-            const uint32_t vl = (uint32_t)(v - rb);
-            const bool have = ((tw >> (vl & 31u)) & 1u) || (pv <= (uint32_t)u && pv >= jb);
-            if (pv > (uint32_t)u) atomicMin(reinterpret_cast<unsigned int*>(a.parent) + v, (unsigned int)u);
+            const uint32_t vl = v - rb;
+            const bool have = ((tw >> (vl & 31u)) & 1u) || (pv <= u && pv >= jb);
+            if (pv > u) atomicMin(reinterpret_cast<unsigned int*>(a.parent) + v, u);
             if (!have) atomicOr(tb + (vl >> 5), 1u << (vl & 31u));
             return;
         }
-        if (pv <= (uint32_t)u) return;
-        atomicMin(reinterpret_cast<unsigned int*>(a.parent) + v, (unsigned int)u);
+        if (pv <= u) return;
+        atomicMin(reinterpret_cast<unsigned int*>(a.parent) + v, u);
         if (pv != 0xffffffffu) return;
-        if (WIN) {
-            const uint32_t vl = (uint32_t)(v - rb);
+        if (WIN == kWinBoth) {
+            const uint32_t vl = v - rb;
             atomicOr(s_t + (vl >> 5), 1u << (vl & 31u));
         } else {
-            atomicOr(a.t + ((uint32_t)v >> 5), 1u << ((uint32_t)v & 31u));
+            atomicOr(a.t + (v >> 5), 1u << (v & 31u));
         }
     }
 };
@@ -229,93 +238,140 @@ constexpr int kIlp = 4;
 #endif
 constexpr int kPieceIlp = BFS_PIECE_ILP;   // the piece kernel: long columns only, more entries in flight
 
+// Scratch of one warp in shared memory: the nonempty words of its unit and the
+// short columns of its batch, packed to the front, so that the owner of an
+// item or entry is found by counting heads (below) and read in one access.
+struct WarpScratch {
+    uint4 word[32];        // bits, directory bits at the same vertices, first column, first vertex (local)
+    uint32_t wexcl[32];    // items before the word
+    uint32_t off[32];      // column offset minus the entries before it
+    uint32_t u[32];        // column's source
+};
+
+__device__ __forceinline__ uint32_t lanes_below() { return (1u << lane_id()) - 1u; }
+
 // All 32 lanes expand one column: ILP x 32 consecutive entries per step.
-template <bool WIN, bool DEDUP, bool ROWX, int ILP = kIlp>
-__device__ __forceinline__ void warp_column(const LevelArgs& a, const Visitor<WIN, DEDUP, ROWX>& vis, int32_t u, int64_t beg,
-                                            uint32_t len) {
-    const int32_t* col = a.ir + beg;
+template <int WIN, bool DEDUP, bool ROWX, int ILP = kIlp>
+__device__ __forceinline__ void warp_column(const LevelArgs& a, const Visitor<WIN, DEDUP, ROWX>& vis, uint32_t u,
+                                            const int32_t* col, uint32_t len) {
     for (uint32_t e = lane_id(); e < len; e += 32 * ILP) {
-        int32_t v[ILP];
-        uint32_t w[ILP], t[ILP];
+        uint32_t v[ILP], w[ILP], t[ILP];
 #pragma unroll
-        for (int k = 0; k < ILP; ++k) v[k] = (e + 32 * k < len) ? __ldcs(col + e + 32 * k) : -1;
+        for (int k = 0; k < ILP; ++k) v[k] = (e + 32 * k < len) ? (uint32_t)__ldcs(col + e + 32 * k) : kNoVertex;
 #pragma unroll
-        for (int k = 0; k < ILP; ++k) w[k] = (v[k] >= 0) ? vis.probe(a, v[k]) : 0u;
+        for (int k = 0; k < ILP; ++k) w[k] = (v[k] != kNoVertex) ? vis.probe(a, v[k]) : 0u;
 #pragma unroll
         for (int k = 0; k < ILP; ++k) vis.stage(a, v[k], w[k], t[k]);
 #pragma unroll
         for (int k = 0; k < ILP; ++k)
-            if (v[k] >= 0) vis.mark(a, v[k], u, w[k], t[k]);
+            if (v[k] != kNoVertex) vis.mark(a, v[k], u, w[k], t[k]);
     }
 }
 
-// Expand one item per lane (u, offset of its column in ir, length; length 0 =
-// none).  Columns longer than kHub go to the row's piece list; columns of at
-// least kCoop entries are expanded by the whole warp one after the other; the
-// short ones share the warp through a load-balanced search over their entry
-// counts, 32 consecutive entries of the concatenated columns per step.
-template <bool WIN, bool DEDUP, bool ROWX>
-__device__ __forceinline__ void warp_expand(const LevelArgs& a, const Visitor<WIN, DEDUP, ROWX>& vis, int row, int32_t u,
-                                            int64_t beg, uint32_t len, unsigned long long& edges,
-                                            unsigned long long& hits) {
+// How a level's units are shared out, from its number of units, frontier
+// vertices and entries (the same for every CTA).  A unit is 32 words of one
+// stream (or of one raw slice), which hold up to 992 vertices with columns of
+// any length: a level with fewer units than warps would leave most of the chip
+// idle, so its units are cut into `parts`, each taking every parts-th group of
+// `bw` of the unit's items, and its long columns into shorter pieces.
+struct Split {
+    uint32_t parts;        // power of two
+    uint32_t bw;           // items per batch of a part (1..32)
+    uint32_t hub;          // columns longer than this go to the piece list, in pieces of this size
+};
+
+__device__ __forceinline__ Split split_level(int64_t units, int64_t items, int64_t entries) {
+    Split s{1u, 32u, kHub};
+    const int64_t warps = (int64_t)gridDim.x * kXW;
+    // pieces of about a quarter of a warp's share of the entries
+    while (s.hub > kHubSparse && (int64_t)s.hub * 4 * warps > entries) s.hub /= 2;
+    if (units <= 0 || units >= warps) return s;
+    const int64_t avg = items / units > 1 ? items / units : 1;        // items per unit (at most: before the sieve)
+    while ((int64_t)s.parts * units < 2 * warps && s.parts < 256u && (int64_t)s.parts < avg) s.parts *= 2u;
+    const int64_t bw = (avg + s.parts - 1) / s.parts;
+    s.bw = bw < 32 ? (uint32_t)bw : 32u;
+    return s;
+}
+
+// Expand one column per lane (source u, offset c0 of its column in the block's
+// entries irb, length; length 0 = none).  Columns longer than the level's hub
+// size go to the row's piece list; columns of at least kCoop entries are
+// expanded by the whole warp one after the other; the short ones share the warp, 32
+// consecutive entries of the concatenated columns per step: every column's
+// first entry sets its bit in the step's head mask (one warp-wide OR), and the
+// owner of an entry is the number of heads up to it.
+template <int WIN, bool DEDUP, bool ROWX>
+__device__ __forceinline__ void warp_expand(const LevelArgs& a, const Visitor<WIN, DEDUP, ROWX>& vis, int row,
+                                            const Split& sp, const int32_t* irb, uint32_t u, uint32_t c0, uint32_t len,
+                                            WarpScratch& ws, unsigned long long& edges, uint32_t& hits) {
     const uint32_t lane = lane_id();
     hits += (len > 0);
     edges += len;
-    if (__any_sync(0xffffffffu, len > kHub)) {
-        if (len > kHub) {
-            const uint32_t np = (len + kPiece - 1) / kPiece;
-            const unsigned long long base = atomicAdd(a.row_piece_count + row, (unsigned long long)np);
-            if (base + np <= (unsigned long long)a.row_piece_cap[row]) {
-                Item* dst = a.pieces + a.row_piece_base[row] + base;
-                for (uint32_t k = 0; k < np; ++k) {
-                    Item it;
-                    it.u = u;
-                    it.len = (len - k * kPiece < kPiece) ? len - k * kPiece : kPiece;
-                    it.begin = beg + (int64_t)k * kPiece;
-                    dst[k] = it;
-                }
-            } else {
-                atomicOr(a.ctr + C_ERROR, 8ull);        // piece list overflow (cannot happen by the bound)
+    uint32_t hm = __ballot_sync(0xffffffffu, len > sp.hub);
+    while (hm) {                            // the warp queues the column's pieces
+        const int src = __ffs(hm) - 1;
+        hm &= hm - 1;
+        const uint32_t hl = __shfl_sync(0xffffffffu, len, src), hc = __shfl_sync(0xffffffffu, c0, src);
+        const uint32_t hu = __shfl_sync(0xffffffffu, u, src);
+        const uint32_t np = (hl + sp.hub - 1) / sp.hub;
+        unsigned long long base = 0;
+        if (lane == 0) base = atomicAdd(a.row_piece_count + row, (unsigned long long)np);
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (base + np <= (unsigned long long)a.row_piece_cap[row]) {
+            Item* dst = a.pieces + a.row_piece_base[row] + base;
+            for (uint32_t k = lane; k < np; k += 32) {
+                Item it;
+                it.u = (int32_t)hu;
+                it.len = ((hl - k * sp.hub < sp.hub) ? hl - k * sp.hub : sp.hub);
+                it.begin = (irb - a.ir) + (int64_t)hc + (int64_t)k * sp.hub;
+                dst[k] = it;
             }
-            len = 0;
+        } else if (lane == 0) {
+            atomicOr(a.ctr + C_ERROR, 8ull);        // piece list overflow (cannot happen by the bound)
         }
+        if (lane == (uint32_t)src) len = 0;
     }
     uint32_t coop = __ballot_sync(0xffffffffu, len >= kCoop);
     while (coop) {
         const int src = __ffs(coop) - 1;
         coop &= coop - 1;
-        warp_column<WIN, DEDUP, ROWX>(a, vis, __shfl_sync(0xffffffffu, u, src), __shfl_sync(0xffffffffu, beg, src),
-                         __shfl_sync(0xffffffffu, len, src));
+        warp_column<WIN, DEDUP, ROWX>(a, vis, __shfl_sync(0xffffffffu, u, src),
+                                      irb + __shfl_sync(0xffffffffu, c0, src), __shfl_sync(0xffffffffu, len, src));
     }
     if (len >= kCoop) len = 0;
+    const uint32_t nz = __ballot_sync(0xffffffffu, len > 0);
+    if (!nz) return;
     const uint32_t incl = warp_incl_sum(len);
     const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
     const uint32_t excl = incl - len;
+    __syncwarp();                           // the previous batch's readers are done
+    if (len > 0) {
+        const int r = __popc(nz & lanes_below());
+        ws.off[r] = c0 - excl;
+        ws.u[r] = u;
+    }
+    __syncwarp();
+    const uint32_t upto = lanes_below() | (1u << lane);
+    int before = -1;                        // the last head before the step
     for (uint32_t e0 = 0; e0 < total; e0 += 32 * kIlp) {
-        int32_t v[kIlp], ou[kIlp];
-        uint32_t w[kIlp], t[kIlp];
+        uint32_t v[kIlp], w[kIlp], t[kIlp];
+        int ow[kIlp];
 #pragma unroll
         for (int k = 0; k < kIlp; ++k) {
+            const uint32_t rel = excl - (e0 + 32 * k);
+            const uint32_t heads = __reduce_or_sync(0xffffffffu, (len > 0 && rel < 32u) ? 1u << rel : 0u);
             const uint32_t e = e0 + 32 * k + lane;
-            int lo = 0, hi = 31;                   // owner: first lane whose inclusive count exceeds e
-#pragma unroll
-            for (int step = 0; step < 5; ++step) {
-                const int mid = (lo + hi) >> 1;
-                const uint32_t im = __shfl_sync(0xffffffffu, incl, mid);
-                if (im > e) hi = mid; else lo = mid + 1;
-            }
-            const int64_t ob = __shfl_sync(0xffffffffu, beg, lo);
-            const uint32_t oe = __shfl_sync(0xffffffffu, excl, lo);
-            ou[k] = __shfl_sync(0xffffffffu, u, lo);
-            v[k] = (e < total) ? __ldcs(a.ir + ob + (int64_t)(e - oe)) : -1;
+            ow[k] = before + __popc(heads & upto);
+            before += __popc(heads);
+            v[k] = (e < total) ? (uint32_t)__ldcs(irb + (uint32_t)(ws.off[ow[k]] + e)) : kNoVertex;
         }
 #pragma unroll
-        for (int k = 0; k < kIlp; ++k) w[k] = (v[k] >= 0) ? vis.probe(a, v[k]) : 0u;
+        for (int k = 0; k < kIlp; ++k) w[k] = (v[k] != kNoVertex) ? vis.probe(a, v[k]) : 0u;
 #pragma unroll
         for (int k = 0; k < kIlp; ++k) vis.stage(a, v[k], w[k], t[k]);
 #pragma unroll
         for (int k = 0; k < kIlp; ++k)
-            if (v[k] >= 0) vis.mark(a, v[k], ou[k], w[k], t[k]);
+            if (v[k] != kNoVertex) vis.mark(a, v[k], ws.u[ow[k]], w[k], t[k]);
     }
 }
 
@@ -336,15 +392,15 @@ __device__ __forceinline__ BlockView block_view(const LevelArgs& a, int64_t b) {
     return bv;
 }
 
-__device__ __forceinline__ void column_of(const LevelArgs& a, const BlockView& bv, int64_t ul, bool test_dir,
-                                          int64_t* begin, uint32_t* len) {
+__device__ __forceinline__ void column_of(const LevelArgs& a, const BlockView& bv, int64_t ul, int64_t* begin,
+                                          uint32_t* len) {
     const uint32_t dw = __ldg(bv.dir + (ul >> 5));
     const uint32_t rk = __ldg(bv.rank + (ul >> 5));
     const uint32_t bit = 1u << (ul & 31);
-    if (!(dw & bit)) {                  // empty column: nothing to expand
+    if (!(dw & bit)) {                  // a vertex of the directory's frontier must have a column
         *begin = 0;
         *len = 0;
-        if (!test_dir) atomicOr(a.ctr + C_ERROR, 4ull);   // a sieved vertex must have a column
+        atomicOr(a.ctr + C_ERROR, 4ull);
         return;
     }
     const uint32_t c = rk + __popc(dw & (bit - 1u));
@@ -355,24 +411,91 @@ __device__ __forceinline__ void column_of(const LevelArgs& a, const BlockView& b
 
 // Bring the L2 lines of a short column's entries on chip ahead of their use
 // (long columns are read by the whole warp, coalesced).
-__device__ __forceinline__ void prefetch_column(const LevelArgs& a, int64_t begin, uint32_t len) {
+__device__ __forceinline__ void prefetch_column(const int32_t* p0, uint32_t len) {
     if (len == 0 || len >= kCoop) return;
-    const int32_t* p0 = a.ir + begin;
     asm volatile("prefetch.global.L2 [%0];" ::"l"(p0));
     const int32_t* p1 = p0 + (len - 1);
     if ((reinterpret_cast<uintptr_t>(p0) >> 7) != (reinterpret_cast<uintptr_t>(p1) >> 7))
         asm volatile("prefetch.global.L2 [%0];" ::"l"(p1));
 }
 
-__device__ __forceinline__ void flush_counts(const LevelArgs& a, unsigned long long edges, unsigned long long hits,
-                                             unsigned long long items) {
+// Expand the vertices of one unit: lane l holds the bits x of 32 vertices of
+// the source range from local vertex wb on (any alignment), `sieved` says that
+// every one has a column (else the directory decides).  The directory bits and
+// the first column's number are read once per word, and an item's column is a
+// popcount away; the packed nonempty words number the unit's items, which the
+// warp takes bw at a time (the part's share of them), the next batch's column
+// lookups and prefetches issued before a batch is expanded.
+template <int WIN, bool DEDUP, bool ROWX>
+__device__ __forceinline__ void warp_words(const LevelArgs& a, const Visitor<WIN, DEDUP, ROWX>& vis, int row,
+                                           const BlockView& bv, const Split& sp, uint32_t part, uint32_t jb, uint32_t x,
+                                           uint32_t wb, bool sieved, WarpScratch& ws, unsigned long long& edges,
+                                           uint32_t& hits) {
+    uint32_t g = 0, cb = 0;
+    if (x) {
+        const uint32_t w = wb >> 5, sh = wb & 31u;
+        const uint32_t d0 = __ldg(bv.dir + w), d1 = __ldg(bv.dir + w + 1);   // rows are padded
+        g = __funnelshift_r(d0, d1, sh);
+        cb = __ldg(bv.rank + w) + __popc(d0 & ((1u << sh) - 1u));
+        if (sieved && (x & ~g)) atomicOr(a.ctr + C_ERROR, 4ull);            // a sieved vertex must have a column
+        x &= g;
+    }
+    const uint32_t nz = __ballot_sync(0xffffffffu, x != 0u);
+    if (!nz) return;
+    const uint32_t cnt = __popc(x);
+    const uint32_t incl = warp_incl_sum(cnt);
+    const uint32_t items = __shfl_sync(0xffffffffu, incl, 31);
+    const uint32_t excl = incl - cnt;
+    __syncwarp();
+    if (x) {
+        const int r = __popc(nz & lanes_below());
+        ws.word[r] = make_uint4(x, g, cb, wb);
+        ws.wexcl[r] = excl;
+    }
+    __syncwarp();
+    const int32_t* irb = a.ir + bv.ir0;
+    const uint32_t upto = lanes_below() | (1u << lane_id());
+    const uint32_t step = sp.parts * sp.bw;
+    auto batch = [&](uint32_t q0, uint32_t& u, uint32_t& c0, uint32_t& len) {
+        // heads before the batch, and in it
+        const uint32_t rel = excl - q0;
+        const uint32_t heads = __reduce_or_sync(0xffffffffu, (x && rel < 32u) ? 1u << rel : 0u);
+        const int before = __popc(__ballot_sync(0xffffffffu, x && excl < q0)) - 1;
+        const uint32_t q = q0 + lane_id();
+        u = 0;
+        c0 = 0;
+        len = 0;
+        if (q < items && lane_id() < sp.bw) {
+            const int o = before + __popc(heads & upto);
+            const uint4 wd = ws.word[o];
+            const uint32_t b = (uint32_t)select32(wd.x, (int)(q - ws.wexcl[o]));
+            const uint32_t c = wd.z + __popc(wd.y & ((1u << b) - 1u));
+            c0 = __ldg(bv.cp + c);
+            len = __ldg(bv.cp + c + 1) - c0;
+            u = jb + wd.w + b;
+            prefetch_column(irb + c0, len);
+        }
+    };
+    uint32_t q0 = part * sp.bw;
+    if (q0 >= items) return;
+    uint32_t u, c0, len;
+    batch(q0, u, c0, len);
+    for (; q0 < items; q0 += step) {
+        uint32_t un = 0, cn = 0, ln = 0;
+        if (q0 + step < items) batch(q0 + step, un, cn, ln);
+        warp_expand<WIN, DEDUP, ROWX>(a, vis, row, sp, irb, u, c0, len, ws, edges, hits);
+        u = un;
+        c0 = cn;
+        len = ln;
+    }
+}
+
+__device__ __forceinline__ void flush_counts(const LevelArgs& a, unsigned long long edges, unsigned long long hits) {
     edges = warp_sum(edges);
     hits = warp_sum(hits);
-    items = warp_sum(items);
     if (lane_id() == 0) {
         if (edges) atomicAdd(a.ctr + C_EDGES, edges);
         if (hits) atomicAdd(a.ctr + C_HITS, hits);
-        if (items) atomicAdd(a.ctr + C_ITEMS, items);
     }
 }
 
@@ -391,10 +514,8 @@ __device__ __forceinline__ int owner_lane(uint32_t excl, uint64_t q) {
 
 // ------------------------------------------------------------ row window --
 // Leave the current row: fold the CTA's partial next bits into t (OR through
-// L2).  With the row exchange the visits record their blocks' partials in HBM
-// instead and the window holds no next bits.
+// L2).
 __device__ void window_leave(const LevelArgs& a, uint32_t* s_t, int row) {
-    if (a.row_exchange) return;
     const int64_t rb = range_begin(a, row);
     for (int64_t w = threadIdx.x; w < a.win_words; w += kXT) {
         const uint32_t x = s_t[w];
@@ -407,53 +528,114 @@ __device__ void window_leave(const LevelArgs& a, uint32_t* s_t, int row) {
     }
 }
 
-// Enter a row: load pi_i into the window and clear the partial next bits.
+// Enter a row: load pi_i into the window and, with kWinBoth, clear the partial
+// next bits.
+template <int WIN>
 __device__ void window_enter(const LevelArgs& a, uint32_t* s_pi, uint32_t* s_t, int row) {
     const int64_t rb = range_begin(a, row);
-    for (int64_t w = threadIdx.x; w < a.win_words; w += kXT) {
-        const int64_t pos = rb + 32 * w;
-        s_pi[w] = (pos < a.n) ? bits32_at_cg(a.pi, (uint64_t)pos) : 0xffffffffu;
-        s_t[w] = 0u;
+    if ((rb & 127) == 0) {                  // 16-byte aligned words: copied four at a time (pi is padded past n)
+        const uint4* src = reinterpret_cast<const uint4*>(a.pi + (rb >> 5));
+        const int quads = (int)((a.win_words + 3) / 4);
+        const int left = (int)((((a.n + 31) >> 5) - (rb >> 5) + 3) / 4);      // quads of pi from rb on
+        uint4* dst = reinterpret_cast<uint4*>(s_pi);
+        for (int q = threadIdx.x; q < quads; q += kXT)
+            dst[q] = q < left ? __ldcg(src + q) : make_uint4(~0u, ~0u, ~0u, ~0u);
+    } else {
+        for (int64_t w = threadIdx.x; w < a.win_words; w += kXT) {
+            const int64_t pos = rb + 32 * w;
+            s_pi[w] = (pos < a.n) ? bits32_at_cg(a.pi, (uint64_t)pos) : 0xffffffffu;
+        }
+    }
+    if (WIN == kWinBoth)
+        for (int64_t w = threadIdx.x; w < a.win_words; w += kXT) s_t[w] = 0u;
+}
+
+// Hand out the units [0, total) of a level without a row window: a warp takes
+// `batch` consecutive units at a time.  Few units are dealt out in turn (no
+// counter to wait for), many by a counter: a guided hand-out of a share of
+// what is left (at least `batch`), so that early grabs are large and the last
+// ones small.  The units come in the order of the block-rows; the share is one
+// of a row's units, so that all warps work on about one row at a time (its
+// visited, next and parent lines stay on chip).
+template <typename Work>
+__device__ __forceinline__ void flat_units(unsigned long long* counter, int64_t total, int64_t batch, int rows,
+                                           Work do_units) {
+    const int64_t warps = (int64_t)gridDim.x * kXW;
+    if (total <= 4 * warps * batch) {
+        const int64_t stride = warps * batch;
+        for (int64_t x = ((int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * batch; x < total; x += stride)
+            do_units(x, (x + batch < total) ? x + batch : total);
+        return;
+    }
+    for (;;) {
+        int64_t x = 0, b = batch;
+        if (lane_id() == 0) {
+            const int64_t cur = (int64_t)*reinterpret_cast<volatile unsigned long long*>(counter);
+            if (cur < total) {
+                const int64_t g = (total - cur) / (kGuide * warps * rows);
+                b = g > batch ? g : batch;
+                x = (int64_t)atomicAdd(counter, (unsigned long long)b);
+            } else {
+                x = total;
+            }
+        }
+        x = __shfl_sync(0xffffffffu, x, 0);
+        b = __shfl_sync(0xffffffffu, b, 0);
+        if (x >= total) break;
+        do_units(x, (x + b < total) ? x + b : total);
     }
 }
 
-// Row-affine persistent loop.  The CTA settles on a block-row with units
-// left; its warps take the row's units one at a time (warp-granular, no block
-// barrier per unit; `batch` units per hand-out) until the row is drained, then
-// the CTA folds its partial next bits into t, picks the next row with units
-// left and loads that row's visited bits.  Every row is tried at most once
-// per CTA.
-template <bool WIN, typename Units, typename Work>
+// Row-affine persistent loop of a level with a row window.  The CTA settles on
+// a block-row with units left; its warps take the row's units one at a time
+// (warp-granular, no block barrier per unit; the same guided hand-out) until
+// the row is drained, then the CTA folds its partial next bits into t, picks
+// the next row with units left and loads that row's visited bits.  Every row
+// is tried at most once per CTA.  row_begin(r) is the first unit of row r
+// among all units of the level.
+template <int WIN, typename Begin, typename Units, typename Work>
 __device__ __forceinline__ void row_affine(const LevelArgs& a, unsigned long long* counters, int64_t batch,
-                                           Units units_in_row, Work do_unit, uint32_t* s_pi, uint32_t* s_t,
-                                           int* s_row) {
+                                           Begin row_begin, Units units_in_row, Work do_units, uint32_t* s_pi,
+                                           uint32_t* s_t, int* s_row) {
     const int p = a.p;
     int tried = 0;
-    int start = a.sweep ? 0 : blockIdx.x % p;
-    auto pick = [&](int from) -> int {          // thread 0: next row with units, or -1
-        while (tried < p) {
-            const int r = from;
-            from = (from + 1 == p) ? 0 : from + 1;
-            ++tried;
-            if ((int64_t)*reinterpret_cast<volatile unsigned long long*>(counters + r) < units_in_row(r)) return r;
+    int from = blockIdx.x % p;
+    // warp 0: the next row with units left, 32 rows tested together, or -1
+    auto pick = [&]() {
+        if (threadIdx.x >= 32) return;
+        int row = -1;
+        while (tried < p && row < 0) {
+            const int q = tried + (int)lane_id();
+            int r = from + (int)lane_id();
+            while (r >= p) r -= p;
+            bool has = false;
+            if (q < p)
+                has = (int64_t)*reinterpret_cast<volatile unsigned long long*>(counters + r) < units_in_row(r);
+            const uint32_t m = __ballot_sync(0xffffffffu, has);
+            if (m) {
+                row = from + __ffs(m) - 1;
+                while (row >= p) row -= p;
+            }
+            const int skip = m ? __ffs(m) : 32;                      // rows this round leaves behind
+            tried += skip;
+            from += skip;
+            while (from >= p) from -= p;
         }
-        return -1;
+        if (lane_id() == 0) s_row[0] = row;
     };
-    if (threadIdx.x == 0) s_row[0] = pick(start);
+    pick();
     __syncthreads();
     int row = s_row[0];
-    if (WIN && row >= 0) window_enter(a, s_pi, s_t, row);
+    if (row >= 0) window_enter<WIN>(a, s_pi, s_t, row);
     __syncthreads();
     while (row >= 0) {
-        const int64_t nu = units_in_row(row);
+        const int64_t nu = units_in_row(row), u0 = row_begin(row);
         for (;;) {
-            // guided hand-out: a share of what is left (at least `batch`), so
-            // that early grabs are large and the last ones small
             int64_t x = 0, b = batch;
             if (lane_id() == 0) {
                 const int64_t cur = (int64_t)*reinterpret_cast<volatile unsigned long long*>(counters + row);
                 if (cur < nu) {
-                    const int64_t g = (uint32_t)(nu - cur) / (uint32_t)(kGuide * gridDim.x * kXW);   // units of a row < 2^31
+                    const int64_t g = (uint32_t)(nu - cur) / (uint32_t)(kGuide * gridDim.x * kXW);   // below 2^31 units
                     b = g > batch ? g : batch;
                     x = (int64_t)atomicAdd(counters + row, (unsigned long long)b);
                 } else {
@@ -463,15 +645,14 @@ __device__ __forceinline__ void row_affine(const LevelArgs& a, unsigned long lon
             x = __shfl_sync(0xffffffffu, x, 0);
             b = __shfl_sync(0xffffffffu, b, 0);
             if (x >= nu) break;
-            const int64_t xe = (x + b < nu) ? x + b : nu;
-            for (; x < xe; ++x) do_unit(row, x);
+            do_units(u0 + x, u0 + ((x + b < nu) ? x + b : nu));
         }
         __syncthreads();
-        if (WIN) window_leave(a, s_t, row);
-        if (threadIdx.x == 0) s_row[0] = pick(row + 1 == p ? 0 : row + 1);
+        if (WIN == kWinBoth) window_leave(a, s_t, row);
+        pick();
         __syncthreads();
         row = s_row[0];
-        if (WIN && row >= 0) window_enter(a, s_pi, s_t, row);
+        if (row >= 0) window_enter<WIN>(a, s_pi, s_t, row);
         __syncthreads();
     }
 }
@@ -479,221 +660,301 @@ __device__ __forceinline__ void row_affine(const LevelArgs& a, unsigned long lon
 // ---------------------------------------------------------------- kernels --
 // Expansion of the WAH units (COMPRESS, COMPRESS_SIEVE).  Unit = 32 words of
 // one stream, decoded by one warp: a warp scan of run lengths from the
-// chunk's group base places every word, a scan of item counts numbers the
-// decoded vertices, and the warp expands them 32 at a time.
-template <typename W, bool WIN, bool DEDUP, bool ROWX>
-__global__ void __launch_bounds__(kXT, 1) expand_wah(LevelArgs a) {
-    if (a.ctl->dedup != (DEDUP ? 1 : 0) || a.ctl->bu) return;   // another variant expands this level
+// chunk's group base places every word, and warp_words expands the words'
+// vertices (the two halves of a 64-bit word's group, and the words of a
+// 1-fill, one after the other).
+template <typename W, int WIN, bool DEDUP, bool ROWX>
+__device__ __forceinline__ void expand_wah_level(const LevelArgs& a, uint32_t* s_pi, uint32_t* s_t, WarpScratch& ws,
+                                                 int* s_row) {
     using T = Wah<W>;
     constexpr int GB = T::GB;
-    extern __shared__ uint32_t s_win[];                   // s_pi | s_t (WIN only)
-    __shared__ int s_row[2];
-    uint32_t* s_pi = s_win;
-    uint32_t* s_t = s_win + a.win_words;
     const int p = a.p;
-    unsigned long long edges = 0, hits = 0, nitems = 0;
-    auto units_in_row = [&](int r) -> int64_t {
-        return a.slot_unit_base[(int64_t)(r + 1) * p] - a.slot_unit_base[(int64_t)r * p];
-    };
+    unsigned long long edges = 0;
+    uint32_t hits = 0;
+    const bool sieved = a.mode == BFS_MODE_COMPRESS_SIEVE;
+    const int64_t units = a.slot_unit_base[(int64_t)p * p];
+    const Split sp = split_level(units, a.ctl->frontier * p, a.ctl->m_f);
+    const int shift = __ffs((int)sp.parts) - 1;
     // the slot of the previous unit: a grab hands out consecutive units, so the
     // next one is mostly in the same slot or a few slots on
     int last_slot = -1;
-    auto do_unit = [&](int row, int64_t x) {
-        // unit -> (slot, chunk): the slot s of the row with base[s] <= g < base[s+1]
-        const int r0 = row * p;
-        const int64_t g = a.slot_unit_base[r0] + x;
-        int sl;
-        if (last_slot >= r0 && last_slot < r0 + p && a.slot_unit_base[last_slot] <= g) {
-            sl = last_slot;
-            while (sl + 1 < r0 + p && a.slot_unit_base[sl + 1] <= g) ++sl;
-        } else {
-            int lo = r0, hi = r0 + p - 1;
+    auto do_unit = [&](int64_t g, uint32_t part) {
+        // unit -> (slot, chunk): the slot s with base[s] <= g < base[s+1]; the warp
+        // searches 32-ary
+        int sl = last_slot;
+        if (sl >= 0 && a.slot_unit_base[sl + 1] <= g && sl + 2 <= p * p) ++sl;
+        if (sl < 0 || a.slot_unit_base[sl] > g || a.slot_unit_base[sl + 1] <= g) {
+            int lo = 0, hi = p * p - 1;
             while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (a.slot_unit_base[mid] <= g) lo = mid; else hi = mid - 1;
+                const int step = (hi - lo + 32) / 32;
+                const int at = lo + step * (int)lane_id();
+                const uint32_t m = __ballot_sync(0xffffffffu, at <= hi && a.slot_unit_base[at] <= g);
+                lo += step * (31 - __clz(m));              // lane 0 always holds
+                hi = lo + step - 1 < hi ? lo + step - 1 : hi;
             }
             sl = lo;
         }
         last_slot = sl;
+        const int row = (int)((uint32_t)sl / (uint32_t)p);
         const int64_t s = sl, k = g - a.slot_unit_base[sl];
-        const int64_t j = sl - r0;
-        const int64_t stream = (a.mode == BFS_MODE_COMPRESS_SIEVE) ? s : j;
-        const int64_t jb = range_begin(a, j), jl = range_begin(a, j + 1) - jb;
-        const int64_t G = (uint32_t)jl / (uint32_t)GB;                 // a range is below 2^31 vertices
-        const int r = (int)((uint32_t)jl - (uint32_t)G * (uint32_t)GB);
+        const int64_t j = sl - row * p;
+        const int64_t stream = sieved ? s : j;
+        const uint32_t jb = (uint32_t)range_begin(a, j), jl = (uint32_t)range_begin(a, j + 1) - jb;
+        const uint32_t G = jl / (uint32_t)GB;                          // a range is below 2^31 vertices
+        const int r = (int)(jl - G * (uint32_t)GB);
         const W* in = static_cast<const W*>(a.xbuf) + stream * a.slot_cap;
         const int64_t count = a.xcount[stream];
         const int64_t xw = k * 32 + lane_id();
-        const W y = (xw < count) ? in[xw] : W(0);
-        // per lane: its element's vertices as (first vertex, bits in group
-        // order; a 1-fill is a run, marked by an empty bit pattern)
-        uint32_t c = 0;
+        const bool valid = xw < count;
+        const W y = valid ? in[xw] : W(0);
+        // per lane: the bits of its element's vertices from local vertex wbase
+        // on; a 1-fill is a run of `run` vertices instead
         W wbits = W(0);
-        int64_t wbase = 0;
+        uint32_t wbase = 0, run = 0;
         const int fm = a.fmt ? (int)a.fmt[stream] : FMT_WAH;
         if (fm == FMT_WAH) {
-            // groups of a slot fit in 32 bits (n < 2^31)
-            const uint32_t glen = (xw < count) ? (uint32_t)word_groups<W>(y) : 0u;
+            const uint32_t glen = valid ? (uint32_t)word_groups<W>(y) : 0u;   // groups of a slot fit in 32 bits
             const uint32_t gincl = warp_incl_sum(glen);
-            const int64_t gs = a.chunk_base[stream * a.chunks_per_slot + k] + (int64_t)(gincl - glen);
-            if (xw < count) {
+            const uint32_t gs = (uint32_t)a.chunk_base[stream * a.chunks_per_slot + k] + (gincl - glen);
+            if (valid) {
                 if (gs < G) {
                     wbase = gs * GB;
-                    if (is_fill<W>(y)) c = (y & T::VAL) ? (uint32_t)(glen * GB) : 0u;
-                    else { wbits = T::from_payload(y); c = (uint32_t)T::popc(wbits); }
+                    if (is_fill<W>(y)) run = (y & T::VAL) ? glen * GB : 0u;
+                    else wbits = T::from_payload(y);
                 } else if (r > 0) {
                     wbase = G * GB;
                     wbits = T::from_active(y, r);                     // the active word
-                    c = (uint32_t)T::popc(wbits);
                 }
             }
-        } else if (xw < count) {
+        } else if (valid) {
             const uint32_t e = (uint32_t)y;
             if (fm == FMT_LIST) {                                     // one vertex offset
                 wbase = e;
-                c = 1;
+                wbits = W(1);
             } else {                                                  // 32 bits of the raw slice
-                wbase = xw * 32;
+                wbase = (uint32_t)xw * 32u;
                 wbits = (W)e;
-                c = (uint32_t)__popc(e);
             }
         }
-        const uint32_t cincl = warp_incl_sum(c);
-        const uint32_t cexcl = cincl - c;
-        const uint32_t items = __shfl_sync(0xffffffffu, cincl, 31);
-        nitems += c;
         const BlockView bv = block_view(a, s);
-        const Visitor<WIN, DEDUP, ROWX> vis{s_pi, s_t, range_begin(a, row), ROWX ? a.tblk + s * a.dir_stride : nullptr,
-                                            (uint32_t)jb};
-        // items q0 .. q0+31, one per lane: decode, look up the column and
-        // prefetch its entries; the next batch's lookups and prefetches are
-        // issued before this batch is expanded
-        auto item = [&](uint32_t q0, int32_t& u, int64_t& begin, uint32_t& len) {
-            const uint32_t q = q0 + lane_id();
-            const int o = owner_lane(cexcl, q < items ? q : items - 1);
-            const W ob = __shfl_sync(0xffffffffu, wbits, o);
-            const int64_t obase = __shfl_sync(0xffffffffu, wbase, o);
-            const uint32_t oex = __shfl_sync(0xffffffffu, cexcl, o);
-            u = 0;
-            begin = 0;
-            len = 0;
-            if (q < items) {
-                const int kk = (int)(q - oex);
-                const int64_t ul = obase + (ob ? T::select(ob, kk) : kk);   // empty pattern: a 1-fill
-                column_of(a, bv, ul, a.mode != BFS_MODE_COMPRESS_SIEVE, &begin, &len);
-                u = (int32_t)(jb + ul);
-                prefetch_column(a, begin, len);
+        const Visitor<WIN, DEDUP, ROWX> vis{s_pi, s_t, (uint32_t)range_begin(a, row),
+                                            ROWX ? a.tblk + s * a.dir_stride : nullptr, jb};
+        // one pass per 32 bits of the words, then the words of the 1-fills:
+        // lane l takes the vertices 32 l .. 32 l + 31 of every 1024 of a run
+        uint32_t fills = __ballot_sync(0xffffffffu, run > 0);
+        uint32_t left = 0, at = 0;
+        for (int h = 0;; ++h) {
+            uint32_t xb, wb;
+            if (h < (int)(sizeof(W) / 4)) {
+                xb = (uint32_t)(wbits >> (sizeof(W) == 8 && h == 1 ? 32 : 0));
+                wb = wbase + 32u * (uint32_t)h;
+            } else {
+                if (left == 0) {
+                    if (!fills) break;
+                    const int o = __ffs(fills) - 1;
+                    fills &= fills - 1;
+                    left = __shfl_sync(0xffffffffu, run, o);
+                    at = __shfl_sync(0xffffffffu, wbase, o);
+                }
+                const uint32_t f0 = 32u * lane_id();
+                const uint32_t n1 = left > f0 ? left - f0 : 0u;
+                xb = n1 >= 32u ? 0xffffffffu : (1u << n1) - 1u;
+                wb = at + f0;
+                const uint32_t took = left < 1024u ? left : 1024u;
+                left -= took;
+                at += took;
             }
-        };
-        int32_t u;
-        int64_t begin;
-        uint32_t len;
-        item(0, u, begin, len);
-        for (uint32_t q0 = 0; q0 < items; q0 += 32) {
-            int32_t un = 0;
-            int64_t bn = 0;
-            uint32_t ln = 0;
-            if (q0 + 32 < items) item(q0 + 32, un, bn, ln);
-            warp_expand<WIN, DEDUP, ROWX>(a, vis, row, u, begin, len, edges, hits);
-            u = un;
-            begin = bn;
-            len = ln;
+            warp_words<WIN, DEDUP, ROWX>(a, vis, row, bv, sp, part, jb, xb, wb, sieved, ws, edges, hits);
         }
     };
-    row_affine<WIN>(a, a.row_next, 2, units_in_row, do_unit, s_pi, s_t, s_row);
-    flush_counts(a, edges, hits, nitems);
+    auto do_units = [&](int64_t x, int64_t xe) {
+        for (; x < xe; ++x) do_unit(x >> shift, (uint32_t)x & (sp.parts - 1u));
+    };
+    if (WIN == kWinNone) {
+        const int64_t each = (units << shift) / (2 * (int64_t)gridDim.x * kXW);   // few hand-outs per warp
+        flat_units(a.row_next, units << shift, each < 1 ? 1 : (each < 8 ? each : 8), p, do_units);
+    } else {
+        auto row_begin = [&](int r) -> int64_t { return a.slot_unit_base[(int64_t)r * p] << shift; };
+        auto units_in_row = [&](int r) -> int64_t {
+            return (a.slot_unit_base[(int64_t)(r + 1) * p] - a.slot_unit_base[(int64_t)r * p]) << shift;
+        };
+        row_affine<WIN>(a, a.row_next, sp.parts > 1 ? 1 : 2, row_begin, units_in_row, do_units, s_pi, s_t, s_row);
+    }
+    flush_counts(a, edges, (unsigned long long)hits);
 }
 
 // Expansion of the PLAIN units.  Unit = (block (row, j), 32 raw frontier words
-// of range j), one warp: lane l keeps word l's bits whose column is nonempty
-// (word-wise AND with V_{i,j}, the block's column index) and the warp expands
-// them 32 at a time.
-template <bool WIN, bool DEDUP>
-__global__ void __launch_bounds__(kXT, 1) expand_plain(LevelArgs a) {
-    if (a.ctl->dedup != (DEDUP ? 1 : 0) || a.ctl->bu) return;   // another variant expands this level
-    extern __shared__ uint32_t s_win[];
-    __shared__ int s_row[2];
-    uint32_t* s_pi = s_win;
-    uint32_t* s_t = s_win + a.win_words;
+// of range j), one warp.  A hand-out tests up to 32 units against the frontier
+// summary at once and expands those with a frontier bit.
+template <int WIN, bool DEDUP>
+__device__ __forceinline__ void expand_plain_level(const LevelArgs& a, uint32_t* s_pi, uint32_t* s_t, WarpScratch& ws,
+                                                   int* s_row) {
     const int p = a.p;
-    unsigned long long edges = 0, hits = 0, nitems = 0;
+    unsigned long long edges = 0;
+    uint32_t hits = 0;
     const int64_t per_row = (int64_t)p * a.plain_upb;
-    auto units_in_row = [&](int) -> int64_t { return per_row; };
-    auto do_unit = [&](int row, int64_t x) {
-        const uint32_t xu = (uint32_t)x, upb = (uint32_t)a.plain_upb;   // p * upb units per row fit in 32 bits
-        const int64_t j = xu / upb, c = xu - (uint32_t)j * upb;
-        const int64_t b = (int64_t)row * p + j;
-        const int64_t jb = range_begin(a, j), jl = range_begin(a, j + 1) - jb;
-        const int64_t w = c * 32 + lane_id();
-        uint32_t bits = 0;
-        if (w * 32 < jl) {
-            bits = bits32_at_cg(a.f, (uint64_t)(jb + w * 32));
-            const int64_t left = jl - w * 32;
-            if (left < 32) bits &= (1u << left) - 1u;
-            if (bits) bits &= __ldg(a.dir + b * a.dir_stride + w);
-        }
-        const uint32_t cnt = __popc(bits);
-        const uint32_t cincl = warp_incl_sum(cnt);
-        const uint32_t cexcl = cincl - cnt;
-        const uint32_t items = __shfl_sync(0xffffffffu, cincl, 31);
-        if (items == 0) return;
-        nitems += cnt;
-        const BlockView bv = block_view(a, b);
-        const Visitor<WIN, DEDUP, false> vis{s_pi, s_t, range_begin(a, row), nullptr, (uint32_t)jb};
-        auto item = [&](uint32_t q0, int32_t& u, int64_t& begin, uint32_t& len) {
-            const uint32_t q = q0 + lane_id();
-            const int o = owner_lane(cexcl, q < items ? q : items - 1);
-            const uint32_t ob = __shfl_sync(0xffffffffu, bits, o);
-            const uint32_t oex = __shfl_sync(0xffffffffu, cexcl, o);
-            u = 0;
-            begin = 0;
-            len = 0;
-            if (q < items) {
-                const int64_t ul = (c * 32 + o) * 32 + select32(ob, (int)(q - oex));
-                column_of(a, bv, ul, false, &begin, &len);
-                u = (int32_t)(jb + ul);
-                prefetch_column(a, begin, len);
+    // the units that hold a frontier bit are at most the frontier's vertices, per block-row
+    const int64_t live = min(per_row, a.ctl->frontier) * p;
+    const Split sp = split_level(live, a.ctl->frontier * p, a.ctl->m_f);
+    const int shift = __ffs((int)sp.parts) - 1;
+    auto do_units = [&](int64_t x0, int64_t xe) {
+        for (int64_t xb = x0; xb < xe; xb += 32) {
+            const int64_t xl = xb + lane_id();
+            bool has = false;
+            if (xl < xe) {
+                const uint32_t xu = (uint32_t)(xl >> shift), upb = (uint32_t)a.plain_upb;   // fits in 32 bits
+                const uint32_t b = xu / upb;
+                const int64_t c = xu - b * upb, j = b % (uint32_t)p;
+                const int64_t g0 = range_begin(a, j) + c * 1024, g1 = min(g0 + 1024, range_begin(a, j + 1));
+                has = g0 < g1 && (__ldcg(a.fsum + (g0 >> 10)) | __ldcg(a.fsum + ((g1 - 1) >> 10)));
             }
-        };
-        int32_t u;
-        int64_t begin;
-        uint32_t len;
-        item(0, u, begin, len);
-        for (uint32_t q0 = 0; q0 < items; q0 += 32) {
-            int32_t un = 0;
-            int64_t bn = 0;
-            uint32_t ln = 0;
-            if (q0 + 32 < items) item(q0 + 32, un, bn, ln);
-            warp_expand<WIN, DEDUP, false>(a, vis, row, u, begin, len, edges, hits);
-            u = un;
-            begin = bn;
-            len = ln;
+            uint32_t m = __ballot_sync(0xffffffffu, has);
+            while (m) {
+                const int64_t x = xb + __ffs(m) - 1;
+                m &= m - 1;
+                const uint32_t xu = (uint32_t)(x >> shift), upb = (uint32_t)a.plain_upb;
+                const int64_t b = xu / upb, c = xu - (uint32_t)b * upb;
+                const int row = (int)((uint32_t)b / (uint32_t)p);
+                const int64_t j = b - (int64_t)row * p;
+                const int64_t jb = range_begin(a, j), jl = range_begin(a, j + 1) - jb;
+                const int64_t w = c * 32 + lane_id();
+                uint32_t bits = 0;
+                if (w * 32 < jl) {
+                    bits = bits32_at_cg(a.f, (uint64_t)(jb + w * 32));
+                    const int64_t left = jl - w * 32;
+                    if (left < 32) bits &= (1u << left) - 1u;
+                }
+                const Visitor<WIN, DEDUP, false> vis{s_pi, s_t, (uint32_t)range_begin(a, row), nullptr, (uint32_t)jb};
+                warp_words<WIN, DEDUP, false>(a, vis, row, block_view(a, b), sp, (uint32_t)x & (sp.parts - 1u),
+                                              (uint32_t)jb, bits, (uint32_t)(32 * w), false, ws, edges, hits);
+            }
         }
     };
-    row_affine<WIN>(a, a.row_next, a.ctl->plain_batch, units_in_row, do_unit, s_pi, s_t, s_row);
-    flush_counts(a, edges, hits, nitems);
+    // sparse levels: many units per hand-out (few hold a vertex), as long as every warp
+    // gets some; dense ones: few (balance)
+    const int64_t total = (per_row << shift) * p;
+    const int64_t each = (total + 4 * (int64_t)gridDim.x * kXW - 1) / (4 * (int64_t)gridDim.x * kXW);
+    const bool dense = a.ctl->frontier * 64 >= a.n;
+    const int64_t batch = dense ? (sp.parts > 1 ? 1 : 2) : (each < 32 ? each : 32);
+    if (WIN == kWinNone) {
+        flat_units(a.row_next, total, dense ? (each < 8 ? each : 8) : batch, p, do_units);
+    } else {
+        auto row_begin = [&](int r) -> int64_t { return (per_row << shift) * r; };
+        auto units_in_row = [&](int) -> int64_t { return per_row << shift; };
+        row_affine<WIN>(a, a.row_next, batch, row_begin, units_in_row, do_units, s_pi, s_t, s_row);
+    }
+    flush_counts(a, edges, (unsigned long long)hits);
 }
 
 // Pieces of long columns, row by row: one warp per piece.
-template <bool WIN, bool DEDUP, bool ROWX>
-__global__ void __launch_bounds__(kXT, 1) expand_pieces(LevelArgs a) {
-    if (a.ctl->dedup != (DEDUP ? 1 : 0) || a.ctl->bu) return;   // another variant expands this level
-    extern __shared__ uint32_t s_win[];
-    __shared__ int s_row[2];
-    uint32_t* s_pi = s_win;
-    uint32_t* s_t = s_win + a.win_words;
-    auto units_in_row = [&](int r) -> int64_t {
-        return (int64_t)min(a.row_piece_count[r], (unsigned long long)a.row_piece_cap[r]);
-    };
-    auto do_unit = [&](int row, int64_t x) {
-        const Item it = a.pieces[a.row_piece_base[row] + x];
+template <int WIN, bool DEDUP, bool ROWX>
+__device__ __forceinline__ void expand_pieces_level(const LevelArgs& a, uint32_t* s_pi, uint32_t* s_t, int* s_row) {
+    int row = 0;
+    auto piece = [&](int64_t at) {
+        const Item it = a.pieces[at];
         const uint32_t j = (uint32_t)it.u / (uint32_t)a.nb;               // the piece's source range
-        const Visitor<WIN, DEDUP, ROWX> vis{s_pi, s_t, range_begin(a, row),
+        const Visitor<WIN, DEDUP, ROWX> vis{s_pi, s_t, (uint32_t)range_begin(a, row),
                                             ROWX ? a.tblk + ((int64_t)row * a.p + j) * a.dir_stride : nullptr,
                                             (uint32_t)range_begin(a, j)};
-        warp_column<WIN, DEDUP, ROWX, kPieceIlp>(a, vis, it.u, it.begin, it.len);
+        warp_column<WIN, DEDUP, ROWX, kPieceIlp>(a, vis, (uint32_t)it.u, a.ir + it.begin, it.len);
     };
-    row_affine<WIN>(a, a.row_piece_next, 1, units_in_row, do_unit, s_pi, s_t, s_row);
+    auto pieces_of = [&](int r) -> int64_t {
+        return (int64_t)min(a.row_piece_count[r], (unsigned long long)a.row_piece_cap[r]);
+    };
+    if (WIN == kWinNone) {
+        // the rows in turn: few pieces are dealt out over all warps, the pieces of
+        // a long row handed out one by one
+        const int64_t warps = (int64_t)gridDim.x * kXW;
+        int64_t next = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;   // this warp's next piece among all
+        int64_t begin = 0;                                                    // pieces of the rows before
+        for (int r0 = 0; r0 < a.p; r0 += 32) {
+            const int64_t mine = r0 + (int)lane_id() < a.p ? pieces_of(r0 + (int)lane_id()) : 0;
+            uint32_t some = __ballot_sync(0xffffffffu, mine > 0);
+            while (some) {
+                const int l = __ffs(some) - 1;
+                some &= some - 1;
+                row = r0 + l;
+                const int64_t n = __shfl_sync(0xffffffffu, mine, l), base = a.row_piece_base[row];
+                if (n <= 4 * warps) {
+                    for (; next < begin + n; next += warps) piece(base + next - begin);
+                } else {
+                    flat_units(a.row_piece_next + row, n, 1, 1, [&](int64_t x, int64_t xe) {
+                        for (; x < xe; ++x) piece(base + x);
+                    });
+                    next += n;
+                }
+                begin += n;
+            }
+        }
+    } else {
+        auto row_begin = [&](int r) -> int64_t {
+            row = r;
+            return a.row_piece_base[r];
+        };
+        auto do_units = [&](int64_t x, int64_t xe) {
+            for (; x < xe; ++x) piece(x);
+        };
+        row_affine<WIN>(a, a.row_piece_next, 1, row_begin, pieces_of, do_units, s_pi, s_t, s_row);
+    }
+}
+
+// One launch expands a level: WIN is the window the graph's ranges allow, and
+// the level's own values pick the body -- with the window on dense levels,
+// without it on sparse ones (their visits are too few to pay for loading it),
+// where DEDUP says whether the parent is read first.
+template <typename W, int WIN, bool ROWX>
+__global__ void __launch_bounds__(kXT, 1) expand_wah(LevelArgs a) {
+    if (a.ctl->bu) return;                                // a bottom-up level
+    extern __shared__ __align__(16) uint32_t s_win[];     // s_pi | s_t
+    __shared__ WarpScratch s_ws[kXW];
+    __shared__ int s_row[2];
+    uint32_t* s_t = s_win + (a.win_words + 3) / 4 * 4;
+    WarpScratch& ws = s_ws[threadIdx.x >> 5];
+    if (WIN == kWinPi && a.ctl->window && a.ctl->dedup) {
+        expand_wah_level<W, WIN, true, ROWX>(a, s_win, s_t, ws, s_row);
+    } else if (WIN != kWinNone && a.ctl->window) {
+        expand_wah_level<W, WIN, false, ROWX>(a, s_win, s_t, ws, s_row);
+    } else if (a.ctl->dedup) {
+        expand_wah_level<W, kWinNone, true, ROWX>(a, s_win, s_t, ws, s_row);
+    } else {
+        expand_wah_level<W, kWinNone, false, ROWX>(a, s_win, s_t, ws, s_row);
+    }
+}
+
+template <int WIN>
+__global__ void __launch_bounds__(kXT, 1) expand_plain(LevelArgs a) {
+    if (a.ctl->bu) return;
+    extern __shared__ __align__(16) uint32_t s_win[];
+    __shared__ WarpScratch s_ws[kXW];
+    __shared__ int s_row[2];
+    uint32_t* s_t = s_win + (a.win_words + 3) / 4 * 4;
+    WarpScratch& ws = s_ws[threadIdx.x >> 5];
+    if (WIN == kWinPi && a.ctl->window && a.ctl->dedup) {
+        expand_plain_level<WIN, true>(a, s_win, s_t, ws, s_row);
+    } else if (WIN != kWinNone && a.ctl->window) {
+        expand_plain_level<WIN, false>(a, s_win, s_t, ws, s_row);
+    } else if (a.ctl->dedup) {
+        expand_plain_level<kWinNone, true>(a, s_win, s_t, ws, s_row);
+    } else {
+        expand_plain_level<kWinNone, false>(a, s_win, s_t, ws, s_row);
+    }
+}
+
+template <int WIN, bool ROWX>
+__global__ void __launch_bounds__(kXT, 1) expand_pieces(LevelArgs a) {
+    if (a.ctl->bu) return;
+    extern __shared__ __align__(16) uint32_t s_win[];
+    __shared__ int s_row[2];
+    uint32_t* s_t = s_win + (a.win_words + 3) / 4 * 4;
+    if (WIN == kWinPi && a.ctl->window && a.ctl->dedup) {
+        expand_pieces_level<WIN, true, ROWX>(a, s_win, s_t, s_row);
+    } else if (WIN != kWinNone && a.ctl->window) {
+        expand_pieces_level<WIN, false, ROWX>(a, s_win, s_t, s_row);
+    } else if (a.ctl->dedup) {
+        expand_pieces_level<kWinNone, true, ROWX>(a, s_win, s_t, s_row);
+    } else {
+        expand_pieces_level<kWinNone, false, ROWX>(a, s_win, s_t, s_row);
+    }
 }
 
 // ------------------------------------------------------------------ fold --
@@ -945,8 +1206,8 @@ __global__ void __launch_bounds__(kNT) dyn_sieve(LevelArgs a, uint32_t* __restri
             len = 0;
             if (q < items) {
                 ul = (c * 32 + o) * 32 + select32(ob, (int)(q - oex));
-                column_of(a, bv, ul, false, &begin, &len);
-                prefetch_column(a, begin, len);
+                column_of(a, bv, ul, &begin, &len);
+                prefetch_column(a.ir + begin, len);
             }
         };
         int64_t ul, begin;
@@ -1241,7 +1502,7 @@ __global__ void __launch_bounds__(kNT) expand_bottom_up(LevelArgs a) {
         const uint32_t m = __ballot_sync(0xffffffffu, found);
         if (lane_id() == 0 && m) a.t[w] = m;
     }
-    flush_counts(a, edges, cols, 0ull);
+    flush_counts(a, edges, cols);
     if (blockIdx.x == 0 && threadIdx.x == 0) a.ctr[C_BOTTOM_UP] = 1ull;
 }
 
@@ -1272,17 +1533,21 @@ __global__ void __launch_bounds__(kNT) reduce_level(uint32_t* __restrict__ t, ui
         // the levels (and degrees) of the fresh vertices, one word at a time
         // by the whole warp: lane l takes bit l (coalesced stores and loads)
         for (uint32_t m = any; m;) {
-            const int k = __ffs(m) - 1;
-            m &= m - 1;
-            const uint32_t xk = __shfl_sync(0xffffffffu, x, k);
-            const int64_t v = (gw * 32 + k) * 32 + lane_id();
-            if (((xk >> lane_id()) & 1u) && v < n) {
-                level[v] = next_level;
-                if (deg) dsum += __ldg(deg + v);
+            uint32_t d[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {               // four words' degree loads in flight
+                const int k = m ? __ffs(m) - 1 : 0;
+                const uint32_t xk = m ? __shfl_sync(0xffffffffu, x, k) : 0u;
+                m &= m - 1;
+                const int64_t v = (gw * 32 + k) * 32 + lane_id();
+                const bool fresh = ((xk >> lane_id()) & 1u) && v < n;
+                if (fresh) level[v] = next_level;
+                d[q] = fresh ? __ldg(deg + v) : 0u;
             }
+            dsum += (unsigned long long)d[0] + d[1] + d[2] + d[3];
         }
         const int cnt = warp_sum(__popc(x));
-        if (deg) dsum = warp_sum(dsum);
+        dsum = warp_sum(dsum);
         if (lane_id() == 0) {
             fsum[gw] = any ? 1 : 0;
             if (cnt) atomicAdd(ctr + C_NEXT_COUNT, (unsigned long long)cnt);
@@ -1298,7 +1563,7 @@ __global__ void __launch_bounds__(kNT) reduce_level(uint32_t* __restrict__ t, ui
 // counters and the row hand-out counters (lvl, nlvl of them) for the next
 // level, in place of memset nodes; the stepwise loop reads them first and
 // clears them itself.
-__global__ void level_next(LevelCtl* c, unsigned long long* ctr, int64_t n, int win, int32_t max_levels,
+__global__ void level_next(LevelCtl* c, unsigned long long* ctr, int64_t n, int32_t max_levels,
                            cudaGraphConditionalHandle handle, int use_handle, unsigned long long* lvl, int nlvl) {
     const int64_t f = (int64_t)ctr[C_NEXT_COUNT];
     const int64_t prev = c->frontier;
@@ -1319,14 +1584,13 @@ __global__ void level_next(LevelCtl* c, unsigned long long* ctr, int64_t n, int 
     c->frontier = f;
     c->visited += f;
     c->level += 1;
-    // PLAIN scans every raw word of every block: many units per hand-out on
-    // sparse levels (few items each), few on dense ones (balance)
-    c->plain_batch = (f * 64 < n) ? 32 : 2;
+    // the row window pays once a level visits every row's vertices several times
+    c->window = (n >= kWindowMinVertices && mf >= (int64_t)c->win_ratio * n) ? 1 : 0;
     // While few vertices are visited, most entries lead to fresh vertices,
     // each reached from many frontier vertices: reading the parent first turns
-    // most of those visits into one L2 read instead of two atomics.  With a
-    // window the next bit is a shared-memory atomic: not worth it.
-    c->dedup = (!win && c->visited * 16 < n) ? 1 : 0;
+    // most of those visits into one L2 read instead of two atomics.  With the
+    // next bits in the window the bit is a shared-memory atomic: not worth it.
+    c->dedup = (c->visited * 16 < n) ? 1 : 0;
     const int go = (f > 0 && ctr[C_ERROR] == 0 && c->level < max_levels) ? 1 : 0;
     c->go = go;
     if (use_handle) {
@@ -1337,19 +1601,20 @@ __global__ void level_next(LevelCtl* c, unsigned long long* ctr, int64_t n, int 
     }
 }
 
-__global__ void level_first(LevelCtl* c, int64_t n, int win, int policy, int alpha, int beta,
+__global__ void level_first(LevelCtl* c, int64_t n, int win_ratio, int policy, int alpha, int beta,
                             const uint32_t* deg, int32_t root, int64_t entries) {
     c->frontier = 1;
     c->visited = 1;
     c->level = 0;
-    c->plain_batch = (64 < n) ? 32 : 2;
-    c->dedup = (!win && 16 < n) ? 1 : 0;
+    c->window = 0;
+    c->win_ratio = win_ratio;
+    c->dedup = (16 < n) ? 1 : 0;
     c->go = 1;
     c->policy = policy;
     c->alpha = alpha;
     c->beta = beta;
     c->bu = (policy == BFS_DIRECTION_BOTTOM_UP) ? 1 : 0;
-    c->m_f = deg ? (int64_t)deg[root] : 0;
+    c->m_f = (int64_t)deg[root];
     c->m_u = entries - c->m_f;
 }
 
@@ -1471,48 +1736,43 @@ int sm_count() {
     return cached;
 }
 
-int64_t l2_bytes() {
-    static int64_t cached = 0;
-    if (!cached) {
-        int dev = 0, v = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&v, cudaDevAttrL2CacheSize, dev);
-        cached = v > 0 ? v : (64ll << 20);
-    }
-    return cached;
+// Dynamic shared memory of the expansion kernels: the row window.  Its kind
+// is the largest that fits beside the warps' scratch: pi_i and the partial t_i,
+// else pi_i alone (all the row exchange needs), else none.
+size_t window_bytes(int64_t win_words, int kind) {
+    return (size_t)((win_words + 3) / 4 * 16) * (kind == kWinBoth ? 2 : (kind == kWinPi ? 1 : 0));
 }
 
-// Dynamic shared memory of the expansion kernels: the row window (pi_i and
-// the partial t_i), when it fits next to the static arrays.
-size_t window_bytes(int64_t win_words) { return (size_t)(2 * win_words * sizeof(uint32_t)); }
+constexpr size_t kWindowRoom = (size_t)kSmemLimit - sizeof(WarpScratch) * kXW - 2048;
 
+int window_kind(int64_t win_words, bool rowx) {
+    if (!rowx && window_bytes(win_words, kWinBoth) <= kWindowRoom) return kWinBoth;
+    return window_bytes(win_words, kWinPi) <= kWindowRoom ? kWinPi : kWinNone;
+}
+
+// The limit is the function's, shared by every graph: always the whole room.
 template <typename K>
-bfs_status allow_smem(K kernel, size_t dyn) {
-    BFS_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+bfs_status allow_smem(K kernel) {
+    BFS_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWindowRoom));
     return BFS_OK;
 }
 
-// The expansion of a level: with the row window one kernel; without, the two
-// variants (with and without reading the parent first), of which the level's
-// device-side choice runs and the other returns at once.
-template <typename W, bool ROWX>
-void launch_expand_wah(const LevelArgs& a, bool win, int grid, size_t dyn, cudaStream_t s) {
-    if (win) {
-        expand_wah<W, true, false, ROWX><<<grid, kXT, dyn, s>>>(a);
-    } else {
-        expand_wah<W, false, true, ROWX><<<grid, kXT, 0, s>>>(a);
-        expand_wah<W, false, false, ROWX><<<grid, kXT, 0, s>>>(a);
-    }
+template <int WIN, bool ROWX>
+bfs_status allow_window() {
+    BFS_TRY(allow_smem(expand_wah<uint32_t, WIN, ROWX>));
+    BFS_TRY(allow_smem(expand_wah<unsigned long long, WIN, ROWX>));
+    BFS_TRY(allow_smem(expand_pieces<WIN, ROWX>));
+    if (!ROWX) BFS_TRY(allow_smem(expand_plain<WIN>));
+    return BFS_OK;
 }
 
-template <bool ROWX>
-void launch_expand_pieces(const LevelArgs& a, bool win, int grid, size_t dyn, cudaStream_t s) {
-    if (win) {
-        expand_pieces<true, false, ROWX><<<grid, kXT, dyn, s>>>(a);
-    } else {
-        expand_pieces<false, true, ROWX><<<grid, kXT, 0, s>>>(a);
-        expand_pieces<false, false, ROWX><<<grid, kXT, 0, s>>>(a);
-    }
+// The expansion of a level's units, then of its long columns' pieces.
+template <int WIN, bool ROWX>
+void launch_expand(const LevelArgs& a, int wbits, int grid, size_t dyn, cudaStream_t s) {
+    if (a.mode == BFS_MODE_PLAIN) expand_plain<WIN><<<grid, kXT, dyn, s>>>(a);
+    else if (wbits == 32) expand_wah<uint32_t, WIN, ROWX><<<grid, kXT, dyn, s>>>(a);
+    else expand_wah<unsigned long long, WIN, ROWX><<<grid, kXT, dyn, s>>>(a);
+    expand_pieces<WIN, ROWX><<<grid, kXT, dyn, s>>>(a);
 }
 
 }  // namespace
@@ -1558,13 +1818,13 @@ bfs_status ensure_workspace_once(bfs_graph* g) {
     BFS_TRY(W.ctl.alloc(sizeof(LevelCtl)));
     BFS_CUDA_TRY(cudaMemset(W.enc_done.ptr, 0, sizeof(unsigned int)));
     BFS_TRY(W.counters.alloc(sizeof(unsigned long long) * C_NUM));
-    // pieces: per row, sum over long columns of ceil(len/kPiece) <= nnz_row/kPiece + nnz_row/kHub
+    // pieces: per row, sum over the columns longer than h of ceil(len/h) <= 2 nnz_row/h, most for the smallest h
     std::vector<int64_t> meta(2 * (size_t)p);
     int64_t total = 0;
     for (int i = 0; i < p; ++i) {
         int64_t nnz_row = 0;
         for (int j = 0; j < p; ++j) nnz_row += L.nnz_b[(int64_t)i * p + j];
-        const int64_t cap = nnz_row / kPiece + nnz_row / kHub + 4;
+        const int64_t cap = 2 * (nnz_row / kHubSparse) + 4;
         meta[i] = total;
         meta[p + i] = cap;
         total += cap;
@@ -1584,20 +1844,12 @@ bfs_status ensure_workspace_once(bfs_graph* g) {
         for (auto& e : W.ev) BFS_CUDA_TRY(cudaEventCreate(&e));
         W.events = true;
     }
-    // the row window of the expansion: pi_i and t_i of one range, if they fit
-    const int64_t win = (L.nb + 31) / 32;
-    const size_t static_bytes = 4096;
-    W.win_words = (window_bytes(win) + static_bytes <= (size_t)kSmemLimit) ? win : 0;
-    if (W.win_words) {
-        const size_t dyn = window_bytes(W.win_words);
-        BFS_TRY(allow_smem(expand_wah<uint32_t, true, false, false>, dyn));
-        BFS_TRY(allow_smem(expand_wah<unsigned long long, true, false, false>, dyn));
-        BFS_TRY(allow_smem(expand_wah<uint32_t, true, false, true>, dyn));
-        BFS_TRY(allow_smem(expand_wah<unsigned long long, true, false, true>, dyn));
-        BFS_TRY(allow_smem(expand_pieces<true, false, true>, dyn));
-        BFS_TRY(allow_smem(expand_plain<true, false>, dyn));
-        BFS_TRY(allow_smem(expand_pieces<true, false, false>, dyn));
-    }
+    // the row window of the expansion
+    W.win_words = (L.nb + 31) / 32;
+    const int both = window_kind(W.win_words, false), rows = window_kind(W.win_words, true);
+    if (both == kWinBoth) BFS_TRY((allow_window<kWinBoth, false>()));
+    if (both == kWinPi) BFS_TRY((allow_window<kWinPi, false>()));
+    if (rows == kWinPi) BFS_TRY((allow_window<kWinPi, true>()));
     return BFS_OK;
 }
 
@@ -1681,7 +1933,6 @@ bfs_status run_search(bfs_graph* g, int32_t root, int32_t* parent, int32_t* leve
     const bool timing = stats && stats->timing;
     const bool tracing = stats && stats->trace_words && stats->trace_counts && nslots > 0;
     unsigned long long* ctr = W.counters.as<unsigned long long>();
-    const bool win = W.win_words > 0;
     const int xgrid = sm_count();                  // persistent: one 1024-thread CTA per SM
     // the compressed row exchange of the fold belongs to DIR-WAH (COMPRESS_SIEVE)
     const bool rowx = g->row_exchange && mode == BFS_MODE_COMPRESS_SIEVE;
@@ -1716,10 +1967,11 @@ bfs_status run_search(bfs_graph* g, int32_t root, int32_t* parent, int32_t* leve
         // allocated once: captured level loops keep the address
         BFS_TRY(W.ddir.alloc(sizeof(uint32_t) * (size_t)(p2 * L.dir_stride)));
     }
-    const size_t dyn = win ? window_bytes(W.win_words) : 0;
+    const int win = window_kind(W.win_words, rowx);
+    const size_t dyn = window_bytes(W.win_words, win);
     // bottom-up levels: degrees (direction choice) and the decoded streams
     const bool bu_kernels = g->direction != BFS_DIRECTION_TOP_DOWN;
-    if (bu_kernels) BFS_TRY(ensure_degrees(g, st));
+    if (bu_kernels) BFS_TRY(ensure_bottom_up(g, st));
     const int64_t g_words = (W.bm_words + 3) / 4 * 4;
     if (bu_kernels && (!W.gbits.ptr || !W.colfirst.ptr)) {
         // allocated once (both or neither): captured level loops keep the addresses
@@ -1772,11 +2024,6 @@ bfs_status run_search(bfs_graph* g, int32_t root, int32_t* parent, int32_t* leve
     a.plain_upb = (L.nb + 1023) / 1024;               // 32 raw words per PLAIN unit
     a.win_words = W.win_words;
     a.row_exchange = rowx ? 1 : 0;
-    // Without a window the visited test, the next bit and the parent update
-    // go through L2.  When the parent array does not fit in half of L2, all
-    // CTAs take the block-rows in turn, so that only one row's slice of it
-    // (and of pi and t) is being updated at a time.
-    a.sweep = (!win && 4 * L.n > l2_bytes() / 2) ? 1 : 0;
     a.tblk = W.tblk.as<uint32_t>();
     a.rowbuf = W.rowbuf.ptr;
     a.row_cap = row_cap;
@@ -1846,15 +2093,16 @@ bfs_status run_search(bfs_graph* g, int32_t root, int32_t* parent, int32_t* leve
     LevelCtl* ctl = W.ctl.as<LevelCtl>();
     a.f = f;
     a.t = t;
+    a.fsum = W.fsum.as<uint8_t>();
     a.ctl = ctl;
     ea.frontier = f;
     ra.skip = &ctl->bu;                      // bottom-up levels have no row exchange
     const int32_t max_levels = (int32_t)std::min<int64_t>(L.n + 1, INT32_MAX);
-    const uint32_t* deg = bu_kernels ? L.deg.as<uint32_t>() : nullptr;
+    const uint32_t* deg = L.deg.as<uint32_t>();
 
     if (dynamic)                     // the search's directories start as V
         BFS_CUDA_TRY(cudaMemcpyAsync(W.ddir.ptr, L.dir.ptr, W.ddir.bytes, cudaMemcpyDeviceToDevice, st));
-    level_first<<<1, 1, 0, st>>>(ctl, L.n, win ? 1 : 0, g->direction, g->alpha, g->beta, deg, root, L.nnz);
+    level_first<<<1, 1, 0, st>>>(ctl, L.n, rowx ? 4 : 2, g->direction, g->alpha, g->beta, deg, root, L.nnz);
     BFS_CUDA_TRY(cudaGetLastError());
 
     // One level: the same launch sequence every time.  `host` adds the
@@ -1876,13 +2124,6 @@ bfs_status run_search(bfs_graph* g, int32_t root, int32_t* parent, int32_t* leve
         if (host && timing) cudaEventRecord(W.ev[0], s);
         if (mode == BFS_MODE_PLAIN) {
             if (host && timing) { cudaEventRecord(W.ev[1], s); cudaEventRecord(W.ev[2], s); }
-            if (win) {
-                expand_plain<true, false><<<xgrid, kXT, dyn, s>>>(a);
-            } else {
-                expand_plain<false, true><<<xgrid, kXT, 0, s>>>(a);
-                expand_plain<false, false><<<xgrid, kXT, 0, s>>>(a);
-            }
-            BFS_CUDA_TRY(cudaGetLastError());
         } else {
             // the exchanged-vertex and chunk counts are statistics: only the stepwise loop asks for them
             EncodeArgs eh = ea;
@@ -1912,17 +2153,15 @@ bfs_status run_search(bfs_graph* g, int32_t root, int32_t* parent, int32_t* leve
                 BFS_CUDA_TRY(cudaGetLastError());
             }
             if (host && timing) cudaEventRecord(W.ev[2], s);
-            if (wbits == 32) {
-                if (rowx) launch_expand_wah<uint32_t, true>(a, win, xgrid, dyn, s);
-                else launch_expand_wah<uint32_t, false>(a, win, xgrid, dyn, s);
-            } else {
-                if (rowx) launch_expand_wah<unsigned long long, true>(a, win, xgrid, dyn, s);
-                else launch_expand_wah<unsigned long long, false>(a, win, xgrid, dyn, s);
-            }
-            BFS_CUDA_TRY(cudaGetLastError());
         }
-        if (rowx) launch_expand_pieces<true>(a, win, xgrid, dyn, s);
-        else launch_expand_pieces<false>(a, win, xgrid, dyn, s);
+        if (rowx) {
+            if (win == kWinPi) launch_expand<kWinPi, true>(a, wbits, xgrid, dyn, s);
+            else launch_expand<kWinNone, true>(a, wbits, xgrid, 0, s);
+        } else {
+            if (win == kWinBoth) launch_expand<kWinBoth, false>(a, wbits, xgrid, dyn, s);
+            else if (win == kWinPi) launch_expand<kWinPi, false>(a, wbits, xgrid, dyn, s);
+            else launch_expand<kWinNone, false>(a, wbits, xgrid, 0, s);
+        }
         BFS_CUDA_TRY(cudaGetLastError());
         if (bu_kernels) {
             expand_bottom_up<<<sm_count() * 8, kNT, 0, s>>>(a);
@@ -1962,7 +2201,7 @@ bfs_status run_search(bfs_graph* g, int32_t root, int32_t* parent, int32_t* leve
             t, W.pi.as<uint32_t>(), f, W.fsum.as<uint8_t>(), W.bm_words, L.n, level, ctl, ctr, deg);
         BFS_CUDA_TRY(cudaGetLastError());
         if (host && timing) cudaEventRecord(W.ev[4], s);
-        level_next<<<1, 1, 0, s>>>(ctl, ctr, L.n, win ? 1 : 0, max_levels, handle, host ? 0 : 1, lvl, 3 * p + 1);
+        level_next<<<1, 1, 0, s>>>(ctl, ctr, L.n, max_levels, handle, host ? 0 : 1, lvl, 3 * p + 1);
         BFS_CUDA_TRY(cudaGetLastError());
         return BFS_OK;
     };

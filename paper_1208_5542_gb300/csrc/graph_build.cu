@@ -229,23 +229,13 @@ __global__ void scatter_entries(const int32_t* __restrict__ src, const int32_t* 
     }
 }
 
-// Degree of every vertex u (range j): the lengths of its columns in blocks
-// (i, j), i = 0 .. p-1, saturated at 2^32 - 1.
-__global__ void vertex_degrees(const uint32_t* __restrict__ dir, const uint32_t* __restrict__ rank,
-                               int64_t dir_stride, const uint32_t* __restrict__ cp,
-                               const int64_t* __restrict__ cp_base, int p, int64_t nb, int64_t n,
+// Degree of every vertex u: its entries in blocks (i, j(u)), i = 0 .. p-1,
+// saturated at 2^32 - 1 (the rows of the counts, read in order).
+__global__ void vertex_degrees(const uint32_t* __restrict__ cnt, int p, int64_t row_stride, int64_t n,
                                uint32_t* __restrict__ deg) {
     for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < n; u += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t j = u / nb, ul = u - j * nb;
-        const uint32_t bit = 1u << (ul & 31);
         uint64_t d = 0;
-        for (int i = 0; i < p; ++i) {
-            const int64_t b = (int64_t)i * p + j;
-            const uint32_t dw = dir[b * dir_stride + (ul >> 5)];
-            if (!(dw & bit)) continue;
-            const int64_t c = cp_base[b] + rank[b * dir_stride + (ul >> 5)] + __popc(dw & (bit - 1u));
-            d += cp[c + 1] - cp[c];
-        }
+        for (int i = 0; i < p; ++i) d += cnt[i * row_stride + u];
         deg[u] = d > 0xffffffffull ? 0xffffffffu : (uint32_t)d;
     }
 }
@@ -404,6 +394,10 @@ bfs_status build_layout(bfs_graph* g, int64_t n, int64_t m, const int32_t* d_src
     BFS_CUDA_TRY(cudaStreamSynchronize(st));
     if (h_err) return set_error(BFS_ERR_INVALID_ARG, "an edge names a vertex outside [0, %lld)", (long long)n);
 
+    BFS_TRY(L.deg.alloc(sizeof(uint32_t) * n));
+    vertex_degrees<<<grid_for(n, 256), 256, 0, st>>>(cnt.as<uint32_t>(), p, row_stride, n, L.deg.as<uint32_t>());
+    BFS_CUDA_TRY(cudaGetLastError());
+
     // directory + popcounts
     BFS_TRY(L.dir.alloc(sizeof(uint32_t) * nblocks * L.dir_stride));
     BFS_TRY(L.rank.alloc(sizeof(uint32_t) * nblocks * L.dir_stride));
@@ -459,15 +453,11 @@ bfs_status build_layout(bfs_graph* g, int64_t n, int64_t m, const int32_t* d_src
     return BFS_OK;
 }
 
-bfs_status ensure_degrees(bfs_graph* g, cudaStream_t st) {
+bfs_status ensure_bottom_up(bfs_graph* g, cudaStream_t st) {
     Layout& L = g->L;
-    if (L.deg.ptr) return BFS_OK;
-    DevBuf deg, iso;
-    BFS_TRY(deg.alloc(sizeof(uint32_t) * L.n));
-    vertex_degrees<<<grid_for(L.n, 256), 256, 0, st>>>(L.dir.as<uint32_t>(), L.rank.as<uint32_t>(), L.dir_stride,
-                                                       L.cp.as<uint32_t>(), L.cp_base_d.as<int64_t>(), L.p, L.nb,
-                                                       L.n, deg.as<uint32_t>());
-    BFS_CUDA_TRY(cudaGetLastError());
+    if (L.bu_ptr.ptr) return BFS_OK;
+    const DevBuf& deg = L.deg;
+    DevBuf iso;
     const int64_t iso_words = ((L.n + 31) / 32 + 4 + 3) / 4 * 4;        // the search bitmaps' padded size
     BFS_TRY(iso.alloc(sizeof(uint32_t) * iso_words));
     isolated_bits<<<grid_for(iso_words, 256), 256, 0, st>>>(deg.as<uint32_t>(), L.n, iso_words, iso.as<uint32_t>());
@@ -501,8 +491,6 @@ bfs_status ensure_degrees(bfs_graph* g, cudaStream_t st) {
                                                        L.n, ptr.as<int64_t>(), adj.as<int32_t>());
     BFS_CUDA_TRY(cudaGetLastError());
     BFS_CUDA_TRY(cudaStreamSynchronize(st));
-    std::swap(L.deg.ptr, deg.ptr);
-    std::swap(L.deg.bytes, deg.bytes);
     std::swap(L.iso.ptr, iso.ptr);
     std::swap(L.iso.bytes, iso.bytes);
     std::swap(L.bu_ptr.ptr, ptr.ptr);
@@ -772,7 +760,7 @@ bfs_status bfs_graph_set_direction(bfs_graph_t g, int32_t policy, int32_t alpha,
         int cur = 0;
         cudaGetDevice(&cur);
         cudaSetDevice(g->device);
-        const bfs_status rc = ensure_degrees(g, nullptr);
+        const bfs_status rc = ensure_bottom_up(g, nullptr);
         cudaSetDevice(cur);
         BFS_TRY(rc);
     }

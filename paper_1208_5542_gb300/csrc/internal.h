@@ -64,7 +64,7 @@ struct Layout {
     int64_t dir_stride = 0; // uint32 words per block directory (padded)
     int64_t nnzc_total = 0; // nonempty columns over all blocks
     DevBuf dir, rank, cp, ir, cp_base_d, ir_base_d;
-    DevBuf deg;             // entries per source vertex (uint32, saturated), computed for bottom-up levels
+    DevBuf deg;             // entries per source vertex (uint32, saturated)
     DevBuf iso;             // bitmap of the vertices without entries (bottom-up levels mark them visited)
     DevBuf bu_ptr, bu_adj;  // bottom-up levels: the columns of v in blocks (0,i) .. (p-1,i) back to back
                             // (int64 offsets n+1, int32 ids), grouped by range in ascending order
@@ -179,7 +179,7 @@ namespace bfsgb {
 bfs_status build_layout(bfs_graph* g, int64_t n, int64_t m, const int32_t* d_src,
                         const int32_t* d_dst, int symmetrize, cudaStream_t st);
 bfs_status ensure_workspace(bfs_graph* g, cudaStream_t st);
-bfs_status ensure_degrees(bfs_graph* g, cudaStream_t st);
+bfs_status ensure_bottom_up(bfs_graph* g, cudaStream_t st);
 void free_workspace(bfs_graph* g);
 
 // wah.cu
