@@ -484,8 +484,7 @@ BFS_API bfs_status bfs_debug_fail_allocation(int64_t k);
 /*
  * WAH-encode one bitmap (Sec. IV, Table 3) on the device.
  *   bits: device, bit b of the bitmap = bit b%32 of bits[b/32], nbits >= 0
- *         bits; the array must hold ceil(nbits/32) + 2 words (the encoder
- *         reads up to two words past the end and ignores them).
+ *         bits in ceil(nbits/32) words.
  *   word_bits: 32 or 64.  Words are (word_bits-1)-bit groups, first bit of a
  *         group most significant; literal top bit 0; fill top bit 1, next bit
  *         the fill value, the rest the run length in groups; an all-0 or all-1
@@ -494,7 +493,7 @@ BFS_API bfs_status bfs_debug_fail_allocation(int64_t k);
  *   words: device output, capacity_words words of word_bits bits; at most
  *         floor(nbits/(word_bits-1)) + 1 are written.
  *   nwords: device int64, receives the word count.
- * Uses scratch memory allocated on `cuda_stream` (stream-ordered allocator).
+ * Uses no scratch memory and does not synchronise.
  * Errors: BFS_ERR_INVALID_ARG (bad width, capacity below the bound above).
  */
 BFS_API bfs_status bfs_wah_encode(const uint32_t *bits, int64_t nbits, int32_t word_bits, void *words,
@@ -547,12 +546,13 @@ BFS_API bfs_status bfs_wah_decode_static(const void *words, int64_t nwords, int6
  * bit is carried by the run's position and not written.  The exchange of the
  * search keeps WAH; this code is offered beside it, for callers that ship
  * bitmaps themselves and for comparing the two codes on the same frontiers.
- *   bits: device, as for bfs_wah_encode (ceil(nbits/32) + 2 words readable).
+ *   bits: device, as for bfs_wah_encode.
  *   nbits: 0 .. 1,040,187,361 (31 x (2^25 - 1): every run fits the 25-bit
  *         length); larger requests return BFS_ERR_INVALID_ARG.
  *   words: device output, capacity_words >= floor(nbits/31) + 1.
  *   nwords: device int64, receives the word count.
- * Allocates scratch (cudaMalloc) and synchronises `cuda_stream`.
+ * Takes stream-ordered scratch from the library's pool (which keeps at most
+ * 64 MiB per device between calls) and synchronises `cuda_stream`.
  */
 BFS_API bfs_status bfs_plwah_encode(const uint32_t *bits, int64_t nbits, uint32_t *words, int64_t capacity_words,
                                    int64_t *nwords, void *cuda_stream);
@@ -599,7 +599,8 @@ BFS_API bfs_status bfs_plwah_decode(const uint32_t *words, int64_t nwords, int64
  *   nbits: 0 .. 2^31 - 1.
  *   bytes: device output, capacity_bytes >= n + n/15 + 11 for n = ceil(nbits/8).
  *   nbytes: device int64, receives the stream's length.
- * Allocates scratch (cudaMalloc) and synchronises `cuda_stream`.
+ * Takes stream-ordered scratch from the library's pool (which keeps at most
+ * 64 MiB per device between calls) and synchronises `cuda_stream`.
  */
 BFS_API bfs_status bfs_bbc_encode(const uint32_t *bits, int64_t nbits, uint8_t *bytes, int64_t capacity_bytes,
                                   int64_t *nbytes, void *cuda_stream);

@@ -248,18 +248,28 @@ class Graph:
         return int(t.value), int(c.value)
 
 
+def _bitmap_words(bits, words_in: int) -> torch.Tensor:
+    """The bitmap's words as the library reads them: ``bits`` itself when it is a whole
+    int32 CUDA vector, else a copy of its first ``words_in`` words."""
+    if (words_in and isinstance(bits, torch.Tensor) and bits.is_cuda and bits.dtype == torch.int32 and bits.dim() == 1
+            and bits.is_contiguous() and bits.numel() >= words_in
+            and bits.device.index == torch.cuda.current_device()):
+        return bits
+    src = torch.zeros(words_in + 2, dtype=torch.int32, device="cuda")
+    if words_in:
+        src[:words_in] = bits[:words_in]
+    return src
+
+
 def wah_encode(bits: torch.Tensor, nbits: int, word_bits: int = 32, stream=None) -> torch.Tensor:
     """Encode the first ``nbits`` bits of ``bits`` (int32 CUDA words, bit b = bit b%32 of word b//32).
 
     Returns the words as an int32 tensor (32-bit words) or int64 tensor (64-bit words).
     """
-    words_in = (nbits + 31) // 32
-    src = torch.zeros(words_in + 2, dtype=torch.int32, device="cuda")
-    if words_in:
-        src[:words_in] = bits[:words_in]
+    src = _bitmap_words(bits, (nbits + 31) // 32)
     cap = nbits // (word_bits - 1) + 1
-    out = torch.zeros(max(1, cap), dtype=torch.int32 if word_bits == 32 else torch.int64, device="cuda")
-    cnt = torch.zeros(1, dtype=torch.int64, device="cuda")
+    out = torch.empty(max(1, cap), dtype=torch.int32 if word_bits == 32 else torch.int64, device="cuda")
+    cnt = torch.empty(1, dtype=torch.int64, device="cuda")
     check(native.lib().bfs_wah_encode(_ptr(src), int(nbits), int(word_bits), _ptr(out), int(cap), _ptr(cnt),
                                       _stream_ptr(stream)))
     return out[: int(cnt.item())]
@@ -267,7 +277,7 @@ def wah_encode(bits: torch.Tensor, nbits: int, word_bits: int = 32, stream=None)
 
 def wah_decode(words: torch.Tensor, nbits: int, word_bits: int = 32, stream=None) -> torch.Tensor:
     """Decode a stream (int32 / int64 CUDA tensor) into int32 bitmap words; raises on a malformed stream."""
-    out = torch.zeros(max(1, (nbits + 31) // 32), dtype=torch.int32, device="cuda")
+    out = torch.empty(max(1, (nbits + 31) // 32), dtype=torch.int32, device="cuda")
     check(native.lib().bfs_wah_decode(_ptr(words) if words.numel() else None, int(words.numel()), int(nbits),
                                       int(word_bits), _ptr(out), _stream_ptr(stream)))
     return out[: (nbits + 31) // 32]
@@ -275,20 +285,17 @@ def wah_decode(words: torch.Tensor, nbits: int, word_bits: int = 32, stream=None
 
 def plwah_encode(bits: torch.Tensor, nbits: int, stream=None) -> torch.Tensor:
     """PLWAH words (int32 CUDA tensor) of the first ``nbits`` bits of ``bits`` (int32 CUDA words)."""
-    words_in = (nbits + 31) // 32
-    src = torch.zeros(words_in + 2, dtype=torch.int32, device="cuda")
-    if words_in:
-        src[:words_in] = bits[:words_in]
+    src = _bitmap_words(bits, (nbits + 31) // 32)
     cap = nbits // 31 + 1
-    out = torch.zeros(max(1, cap), dtype=torch.int32, device="cuda")
-    cnt = torch.zeros(1, dtype=torch.int64, device="cuda")
+    out = torch.empty(max(1, cap), dtype=torch.int32, device="cuda")
+    cnt = torch.empty(1, dtype=torch.int64, device="cuda")
     check(native.lib().bfs_plwah_encode(_ptr(src), int(nbits), _ptr(out), int(cap), _ptr(cnt), _stream_ptr(stream)))
     return out[: int(cnt.item())]
 
 
 def plwah_decode(words: torch.Tensor, nbits: int, stream=None) -> torch.Tensor:
     """Decode a PLWAH stream (int32 CUDA tensor) into int32 bitmap words; raises on a malformed stream."""
-    out = torch.zeros(max(1, (nbits + 31) // 32), dtype=torch.int32, device="cuda")
+    out = torch.empty(max(1, (nbits + 31) // 32), dtype=torch.int32, device="cuda")
     check(native.lib().bfs_plwah_decode(_ptr(words) if words.numel() else None, int(words.numel()), int(nbits),
                                         _ptr(out), _stream_ptr(stream)))
     return out[: (nbits + 31) // 32]
@@ -296,21 +303,18 @@ def plwah_decode(words: torch.Tensor, nbits: int, stream=None) -> torch.Tensor:
 
 def bbc_encode(bits: torch.Tensor, nbits: int, stream=None) -> torch.Tensor:
     """BBC bytes (uint8 CUDA tensor) of the first ``nbits`` bits of ``bits`` (int32 CUDA words)."""
-    words_in = (nbits + 31) // 32
-    src = torch.zeros(max(1, words_in), dtype=torch.int32, device="cuda")
-    if words_in:
-        src[:words_in] = bits[:words_in]
+    src = _bitmap_words(bits, (nbits + 31) // 32)
     n = (nbits + 7) // 8
     cap = n + n // 15 + 11
-    out = torch.zeros(cap, dtype=torch.uint8, device="cuda")
-    cnt = torch.zeros(1, dtype=torch.int64, device="cuda")
+    out = torch.empty(cap, dtype=torch.uint8, device="cuda")
+    cnt = torch.empty(1, dtype=torch.int64, device="cuda")
     check(native.lib().bfs_bbc_encode(_ptr(src), int(nbits), _ptr(out), int(cap), _ptr(cnt), _stream_ptr(stream)))
     return out[: int(cnt.item())]
 
 
 def bbc_decode(data: torch.Tensor, nbits: int, stream=None) -> torch.Tensor:
     """Decode a BBC stream (uint8 CUDA tensor) into int32 bitmap words; raises on a malformed stream."""
-    out = torch.zeros(max(1, (nbits + 31) // 32), dtype=torch.int32, device="cuda")
+    out = torch.empty(max(1, (nbits + 31) // 32), dtype=torch.int32, device="cuda")
     check(native.lib().bfs_bbc_decode(_ptr(data) if data.numel() else None, int(data.numel()), int(nbits),
                                       _ptr(out), _stream_ptr(stream)))
     return out[: (nbits + 31) // 32]

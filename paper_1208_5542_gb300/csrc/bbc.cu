@@ -20,13 +20,18 @@
 // the first header of each unit, one the map bytes and the later headers.
 // Decoding splits the stream into chunks: a record is at most 25 bytes, so a
 // chunk's first header lies within its first 25 bytes.  Every chunk is parsed
-// from each of the 25 possible entries (where it leaves the chunk, the records
-// and bytes it produced); one thread chains the entries from the stream's
-// start; then every chunk is parsed again from its real entry, one warp per
-// chunk writing the one-fills and the tails into the zeroed output.
+// from each of the 25 possible entries (where it leaves the chunk and the
+// bytes it produced); every group of 64 chunks is chased from its 25 entries
+// through the chunks' tables, one thread chains the groups from the stream's
+// start and every group its chunks; then every chunk is parsed again from its
+// real entry, one warp per chunk writing the one-fills and the tails into the
+// zeroed output.  Parsing is a chain of dependent byte loads, so its time is
+// the chunk's length: chunks of 128 bytes (1024 before the two-level chain)
+// take a 4M-bit slice of density 0.02 from 453 to 129 us a call.
 #include <algorithm>
 #include <cstring>
 
+#include "cluster.cuh"
 #include "common.cuh"
 #include "internal.h"
 
@@ -37,7 +42,8 @@ constexpr int kBT = 256;                    // threads per CTA
 constexpr int kBPerThread = 16;             // bytes per thread in the flag passes
 constexpr int64_t kBTile = kBT * kBPerThread;
 constexpr int kMaxRecord = 25;              // header + 9 counter bytes + 15 tail bytes
-constexpr int64_t kChunk = 1024;            // stream bytes per decoding chunk
+constexpr int64_t kChunk = 128;             // stream bytes per decoding chunk
+constexpr int kGroup = 64;                  // chunks chased together
 constexpr int64_t kBbcMaxBits = (int64_t)1 << 31;
 
 // Multiprocessors of the current device (grid sizes).
@@ -132,28 +138,36 @@ __global__ void __launch_bounds__(kBT) bbc_flags(const uint32_t* __restrict__ bi
     }
 }
 
-// Exclusive scan of n values in one CTA (in place); *total gets their sum.
-__global__ void __launch_bounds__(1024) scan_one_cta(uint32_t* __restrict__ v, int64_t n, uint32_t* __restrict__ total) {
-    __shared__ uint32_t s_w[33];
+// Exclusive scan of `in` into `out` (may be the same array) by one cluster;
+// the length is *n_dev, or n without it; the sum goes to *total and *total64
+// (either may be nullptr).
+__global__ void __launch_bounds__(kCT) scan_cluster(const uint32_t* in, const uint32_t* n_dev, int64_t n, uint32_t* out,
+                                                    uint32_t* total, int64_t* total64) {
+    __shared__ ClusterScan<uint32_t> s_scan;
+    if (n_dev) n = *n_dev;
     uint32_t carry = 0;
-    for (int64_t b = 0; b < n; b += blockDim.x) {
-        const int64_t i = b + threadIdx.x;
-        const uint32_t x = i < n ? v[i] : 0u;
-        const uint32_t incl = warp_incl_sum(x);
-        if (lane_id() == 31) s_w[threadIdx.x >> 5] = incl;
-        __syncthreads();
-        if (threadIdx.x < 32) {
-            const uint32_t t = threadIdx.x < (blockDim.x >> 5) ? s_w[threadIdx.x] : 0u;
-            const uint32_t ti = warp_incl_sum(t);
-            s_w[threadIdx.x] = ti - t;
-            if (threadIdx.x == 31) s_w[32] = ti;
+    int turn = 0;
+    for (int64_t b = 0; b < n; b += kClusterRound, ++turn) {
+        const int64_t i0 = b + cluster_thread() * kCK;
+        uint32_t x[kCK], sum = 0, all;
+#pragma unroll
+        for (int i = 0; i < kCK; ++i) {
+            x[i] = i0 + i < n ? in[i0 + i] : 0u;
+            sum += x[i];
         }
-        __syncthreads();
-        if (i < n) v[i] = carry + s_w[threadIdx.x >> 5] + incl - x;
-        carry += s_w[32];
-        __syncthreads();
+        uint32_t at = carry + cluster_excl_scan(sum, 0u, OpSum(), s_scan, turn, &all);
+#pragma unroll
+        for (int i = 0; i < kCK; ++i) {
+            if (i0 + i < n) out[i0 + i] = at;
+            at += x[i];
+        }
+        carry += all;
     }
-    if (threadIdx.x == 0) *total = carry;
+    if (cluster_thread() == 0) {
+        if (total) *total = carry;
+        if (total64) *total64 = carry;
+    }
+    cluster_done();
 }
 
 // Unit numbers: every unit's first byte and first map byte.
@@ -284,11 +298,6 @@ __global__ void __launch_bounds__(kBT) bbc_tails(const uint32_t* __restrict__ bi
     }
 }
 
-__global__ void bbc_total(const uint32_t* offs, const uint32_t* sizes, const uint32_t* nunits, int64_t* nout) {
-    const uint32_t U = *nunits;
-    *nout = U ? (int64_t)offs[U - 1] + sizes[U - 1] : 0;
-}
-
 // ---------------------------------------------------------------- decode --
 // One record from position at: fills F bytes of value b, then T tail bytes
 // from tail_at, or one odd byte.  Returns the position after it, or -1 if
@@ -335,7 +344,7 @@ __device__ __forceinline__ int64_t rec_bytes(const Rec& r) { return r.f + (r.odd
 // the position reaches the chunk's end; exit = position - end (0 .. 24), or
 // 255 when a record is malformed; bytes = output bytes of the records.
 __global__ void __launch_bounds__(kBT) bbc_entries(const uint8_t* __restrict__ in, int64_t nin,
-                                                   uint8_t* __restrict__ exits, int64_t* __restrict__ outb) {
+                                                   uint8_t* __restrict__ exits, uint32_t* __restrict__ outb) {
     const int64_t nch = (nin + kChunk - 1) / kChunk;
     const int64_t total = nch * kMaxRecord;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -355,51 +364,103 @@ __global__ void __launch_bounds__(kBT) bbc_entries(const uint8_t* __restrict__ i
             if (at >= c1) ex = (uint8_t)(at - c1);
         }
         exits[x] = ex;
-        outb[x] = bytes;
+        outb[x] = (uint32_t)(bytes < kBbcMaxBits ? bytes : kBbcMaxBits);   // more than any bitmap holds
     }
 }
 
-// The real entry of every chunk, chained from the stream's start by one
-// thread through shared-memory copies of the exit tables (kChainChunks chunks
-// at a time); then the output bytes of every chunk from its real entry.  The
-// last chunk must end exactly at the stream's end.
-constexpr int kChainChunks = 1536;
+// Where every group of chunks is left, per entry into its first chunk (one
+// warp per group, a lane per entry, through a shared copy of the chunks'
+// tables).
+__global__ void __launch_bounds__(kBT) bbc_groups(const uint8_t* __restrict__ exits, int64_t nch,
+                                                  uint8_t* __restrict__ gexits) {
+    __shared__ uint8_t s_ex[kBT / 32][kGroup * kMaxRecord];
+    const int64_t ng = (nch + kGroup - 1) / kGroup;
+    uint8_t* ex = s_ex[threadIdx.x >> 5];
+    const int lane = (int)lane_id();
+    const int64_t ws = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; g < ng; g += ws) {
+        const int cn = (int)(nch - g * kGroup < kGroup ? nch - g * kGroup : kGroup);
+        for (int x = lane; x < cn * kMaxRecord; x += 32) ex[x] = exits[g * kGroup * kMaxRecord + x];
+        __syncwarp();
+        if (lane < kMaxRecord) {
+            uint32_t e = (uint32_t)lane;
+            for (int c = 0; c < cn && e != 255; ++c) e = ex[c * kMaxRecord + e];
+            gexits[g * kMaxRecord + lane] = (uint8_t)e;
+        }
+        __syncwarp();
+    }
+}
 
-__global__ void __launch_bounds__(1024) bbc_chain(const uint8_t* __restrict__ exits, const int64_t* __restrict__ outb,
-                                                  int64_t nin, uint8_t* __restrict__ entry, uint32_t* __restrict__ sel,
-                                                  unsigned long long* err) {
-    __shared__ uint8_t s_ex[kChainChunks * kMaxRecord];
+// The real entry of every group, chained from the stream's start by one thread
+// through shared-memory copies of the groups' tables (kChainGroups at a time).
+// The last group must end exactly at the stream's end; after a malformed
+// record the later groups keep entry 0.
+constexpr int kChainGroups = 1536;
+
+__global__ void __launch_bounds__(1024) bbc_chain(const uint8_t* __restrict__ gexits, int64_t ng,
+                                                  uint8_t* __restrict__ gentry, unsigned long long* err) {
+    __shared__ uint8_t s_ex[kChainGroups * kMaxRecord];
     __shared__ int s_e;
-    const int64_t nch = (nin + kChunk - 1) / kChunk;
     if (threadIdx.x == 0) s_e = 0;
-    for (int64_t c0 = 0; c0 < nch; c0 += kChainChunks) {
-        const int64_t cn = (nch - c0 < kChainChunks) ? nch - c0 : kChainChunks;
+    for (int64_t g0 = 0; g0 < ng; g0 += kChainGroups) {
+        const int64_t gn = (ng - g0 < kChainGroups) ? ng - g0 : kChainGroups;
         __syncthreads();
-        for (int64_t x = threadIdx.x; x < cn * kMaxRecord; x += blockDim.x) s_ex[x] = exits[c0 * kMaxRecord + x];
+        for (int64_t x = threadIdx.x; x < gn * kMaxRecord; x += blockDim.x) s_ex[x] = gexits[g0 * kMaxRecord + x];
         __syncthreads();
         if (threadIdx.x == 0) {
             int e = s_e;
-            for (int64_t c = 0; c < cn; ++c) {
-                entry[c0 + c] = (uint8_t)e;
-                const uint8_t ex = s_ex[c * kMaxRecord + e];
+            for (int64_t g = 0; g < gn; ++g) {
+                gentry[g0 + g] = (uint8_t)e;
+                const uint8_t ex = s_ex[g * kMaxRecord + e];
                 if (ex == 255) { *err = 1; e = 0; break; }
                 e = ex;
             }
             s_e = e;
         }
     }
-    __syncthreads();
     if (threadIdx.x == 0 && s_e != 0) *err = 1;
-    __syncthreads();
-    for (int64_t c = threadIdx.x; c < nch; c += blockDim.x)
-        sel[c] = (uint32_t)outb[c * kMaxRecord + entry[c]];
+}
+
+// The real entry and output bytes of every chunk (one warp per group; after
+// its malformed record a group's chunks get entry 0).
+__global__ void __launch_bounds__(kBT) bbc_fill(const uint8_t* __restrict__ exits, const uint32_t* __restrict__ outb,
+                                                int64_t nch, const uint8_t* __restrict__ gentry,
+                                                uint8_t* __restrict__ entry, uint32_t* __restrict__ sel) {
+    __shared__ uint8_t s_ex[kBT / 32][kGroup * kMaxRecord];
+    __shared__ uint8_t s_en[kBT / 32][kGroup];
+    const int64_t ng = (nch + kGroup - 1) / kGroup;
+    const int w = threadIdx.x >> 5, lane = (int)lane_id();
+    const int64_t ws = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; g < ng; g += ws) {
+        const int cn = (int)(nch - g * kGroup < kGroup ? nch - g * kGroup : kGroup);
+        for (int x = lane; x < cn * kMaxRecord; x += 32) s_ex[w][x] = exits[g * kGroup * kMaxRecord + x];
+        __syncwarp();
+        if (lane == 0) {
+            uint32_t e = gentry[g];
+            for (int c = 0; c < cn; ++c) {
+                s_en[w][c] = (uint8_t)e;
+                const uint32_t ex = s_ex[w][c * kMaxRecord + e];
+                e = ex == 255 ? 0 : ex;
+            }
+        }
+        __syncwarp();
+        for (int c = lane; c < cn; c += 32) {
+            const int64_t k = g * kGroup + c;
+            entry[k] = s_en[w][c];
+            sel[k] = outb[k * kMaxRecord + s_en[w][c]];
+        }
+        __syncwarp();
+    }
 }
 
 // One warp per chunk: parse from its real entry; write the one-fill bytes and
-// the tails (bytes past nbytes are an error; the output was zeroed).
+// the tails (bytes past nbytes are an error; the output was zeroed).  Nothing
+// is written when the chunks do not chain or hold another number of bytes.
 __global__ void __launch_bounds__(kBT) bbc_expand(const uint8_t* __restrict__ in, int64_t nin, int64_t nbytes,
                                                   const uint8_t* __restrict__ entry, const uint32_t* __restrict__ out_base,
-                                                  uint8_t* __restrict__ out8, unsigned long long* err) {
+                                                  const uint32_t* __restrict__ held, uint8_t* __restrict__ out8,
+                                                  unsigned long long* err) {
+    if (*static_cast<volatile unsigned long long*>(err) || (int64_t)*held != nbytes) return;
     const int64_t nch = (nin + kChunk - 1) / kChunk;
     const int lane = (int)lane_id();
     const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
@@ -428,12 +489,25 @@ __global__ void __launch_bounds__(kBT) bbc_expand(const uint8_t* __restrict__ in
     }
 }
 
-// Bits past nbits in the last decoded byte must be 0.
-__global__ void bbc_padding(const uint8_t* out8, int64_t nbits, unsigned long long* err) {
+// The decode's outcome: no error, the stream's bytes those of the bitmap, and
+// bits past nbits in the last decoded byte 0.
+__global__ void bbc_outcome(const uint8_t* out8, int64_t nbits, const uint32_t* held, const unsigned long long* err,
+                            volatile unsigned long long* bad) {
     const int64_t nbytes = (nbits + 7) / 8;
     const int r = (int)(nbits & 7);
-    if (r && (out8[nbytes - 1] >> r)) *err = 1;        // stored LSB-first: bit j of the byte = bit 8k+j
+    // stored LSB-first: bit j of the byte = bit 8k+j
+    if (*err || (int64_t)*held != nbytes || (r && (out8[nbytes - 1] >> r))) *bad = 1;
 }
+
+// Parts of one scratch block, each from a 16-byte boundary.
+struct Parts {
+    size_t bytes = 0;
+    size_t add(size_t n) {
+        const size_t at = bytes;
+        bytes = (bytes + n + 15) / 16 * 16;
+        return at;
+    }
+};
 
 }  // namespace
 }  // namespace bfsgb
@@ -459,36 +533,32 @@ bfs_status bfs_bbc_encode(const uint32_t* bits, int64_t nbits, uint8_t* bytes, i
     }
     const int64_t ntiles = (nbytes + kBTile - 1) / kBTile;
     const int sms = bbc_sms();
-    DevBuf flags, tiles, cnt, upos, mpos, sizes, offs;
-    BFS_TRY(flags.alloc((size_t)nbytes));
-    BFS_TRY(tiles.alloc(sizeof(uint32_t) * (size_t)ntiles));
-    BFS_TRY(cnt.alloc(sizeof(uint32_t) * 2));
-    BFS_TRY(upos.alloc(sizeof(int32_t) * (size_t)nbytes));
-    BFS_TRY(mpos.alloc(sizeof(int32_t) * (size_t)nbytes));
-    BFS_TRY(sizes.alloc(sizeof(uint32_t) * (size_t)nbytes));
-    BFS_TRY(offs.alloc(sizeof(uint32_t) * (size_t)nbytes));
+    Parts parts;
+    const size_t p_flags = parts.add((size_t)nbytes), p_tiles = parts.add(4 * (size_t)ntiles), p_cnt = parts.add(8),
+                 p_upos = parts.add(4 * (size_t)nbytes), p_mpos = parts.add(4 * (size_t)nbytes),
+                 p_sizes = parts.add(4 * (size_t)nbytes), p_offs = parts.add(4 * (size_t)nbytes);
+    Scratch tmp;
+    BFS_TRY(tmp.alloc(parts.bytes, st));
+    char* t = tmp.as<char>();
+    uint8_t* flags = reinterpret_cast<uint8_t*>(t + p_flags);
+    uint32_t* tiles = reinterpret_cast<uint32_t*>(t + p_tiles);
+    uint32_t* nunits = reinterpret_cast<uint32_t*>(t + p_cnt);
+    int32_t* upos = reinterpret_cast<int32_t*>(t + p_upos);
+    int32_t* mpos = reinterpret_cast<int32_t*>(t + p_mpos);
+    uint32_t* sizes = reinterpret_cast<uint32_t*>(t + p_sizes);
+    uint32_t* offs = reinterpret_cast<uint32_t*>(t + p_offs);
     const int grid = (int)std::min<int64_t>(std::max<int64_t>(ntiles, 1), (int64_t)sms * 8);
     const int egrid = (int)std::min<int64_t>((nbytes + kBT - 1) / kBT, (int64_t)sms * 16);
-    BFS_CUDA_TRY(cudaMemsetAsync(mpos.ptr, 0xFF, mpos.bytes, st));
-    uint32_t* nunits = cnt.as<uint32_t>();
-    bbc_flags<<<grid, kBT, 0, st>>>(bits, nbits, nbytes, flags.as<uint8_t>(), tiles.as<uint32_t>());
-    scan_one_cta<<<1, 1024, 0, st>>>(tiles.as<uint32_t>(), ntiles, nunits);
-    bbc_number<<<grid, kBT, 0, st>>>(flags.as<uint8_t>(), nbytes, tiles.as<uint32_t>(), upos.as<int32_t>(),
-                                     mpos.as<int32_t>());
-    bbc_sizes<<<egrid, kBT, 0, st>>>(bits, nbits, nbytes, upos.as<int32_t>(), mpos.as<int32_t>(), nunits,
-                                     sizes.as<uint32_t>());
-    BFS_CUDA_TRY(cudaMemcpyAsync(offs.ptr, sizes.ptr, sizes.bytes, cudaMemcpyDeviceToDevice, st));
-    uint32_t h_units = 0;
-    BFS_CUDA_TRY(cudaMemcpyAsync(&h_units, nunits, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
-    BFS_CUDA_TRY(cudaStreamSynchronize(st));
-    scan_one_cta<<<1, 1024, 0, st>>>(offs.as<uint32_t>(), (int64_t)h_units, nunits + 1);
-    bbc_heads<<<egrid, kBT, 0, st>>>(bits, nbits, nbytes, upos.as<int32_t>(), mpos.as<int32_t>(), nunits,
-                                     offs.as<uint32_t>(), bytes);
-    bbc_tails<<<egrid, kBT, 0, st>>>(bits, nbits, nbytes, upos.as<int32_t>(), mpos.as<int32_t>(), nunits,
-                                     offs.as<uint32_t>(), bytes);
-    bbc_total<<<1, 1, 0, st>>>(offs.as<uint32_t>(), sizes.as<uint32_t>(), nunits, nbytes_out);
+    BFS_CUDA_TRY(cudaMemsetAsync(mpos, 0xFF, 4 * (size_t)nbytes, st));
+    bbc_flags<<<grid, kBT, 0, st>>>(bits, nbits, nbytes, flags, tiles);
+    BFS_CUDA_TRY(launch_cluster(scan_cluster, st, tiles, nullptr, ntiles, tiles, nunits, nullptr));
+    bbc_number<<<grid, kBT, 0, st>>>(flags, nbytes, tiles, upos, mpos);
+    bbc_sizes<<<egrid, kBT, 0, st>>>(bits, nbits, nbytes, upos, mpos, nunits, sizes);
+    BFS_CUDA_TRY(launch_cluster(scan_cluster, st, sizes, nunits, int64_t(0), offs, nullptr, nbytes_out));
+    bbc_heads<<<egrid, kBT, 0, st>>>(bits, nbits, nbytes, upos, mpos, nunits, offs, bytes);
+    bbc_tails<<<egrid, kBT, 0, st>>>(bits, nbits, nbytes, upos, mpos, nunits, offs, bytes);
     BFS_CUDA_TRY(cudaGetLastError());
-    BFS_CUDA_TRY(cudaStreamSynchronize(st));          // the scratch is released on return
+    BFS_CUDA_TRY(cudaStreamSynchronize(st));
     return BFS_OK;
 }
 
@@ -506,33 +576,38 @@ bfs_status bfs_bbc_decode(const uint8_t* bytes, int64_t nbytes_in, int64_t nbits
     }
     const int64_t nch = (nbytes_in + kChunk - 1) / kChunk;
     const int sms = bbc_sms();
-    DevBuf exits, outb, entry, obase, err, tot;
-    BFS_TRY(exits.alloc((size_t)(nch * kMaxRecord)));
-    BFS_TRY(outb.alloc(sizeof(int64_t) * (size_t)(nch * kMaxRecord)));
-    BFS_TRY(entry.alloc((size_t)nch));
-    BFS_TRY(obase.alloc(sizeof(uint32_t) * (size_t)nch));
-    BFS_TRY(err.alloc(sizeof(unsigned long long)));
-    BFS_TRY(tot.alloc(sizeof(uint32_t)));
-    BFS_CUDA_TRY(cudaMemsetAsync(err.ptr, 0, sizeof(unsigned long long), st));
+    Parts parts;
+    const int64_t ng = (nch + kGroup - 1) / kGroup;
+    const size_t p_outb = parts.add(4 * (size_t)(nch * kMaxRecord)), p_exits = parts.add((size_t)(nch * kMaxRecord)),
+                 p_gexits = parts.add((size_t)(ng * kMaxRecord)), p_obase = parts.add(4 * (size_t)nch),
+                 p_entry = parts.add((size_t)nch), p_gentry = parts.add((size_t)ng), p_err = parts.add(16);
+    Scratch tmp;
+    BFS_TRY(tmp.alloc(parts.bytes, st));
+    HostFlag bad;
+    BFS_TRY(bad.take());
+    char* t = tmp.as<char>();
+    uint32_t* outb = reinterpret_cast<uint32_t*>(t + p_outb);
+    uint8_t* exits = reinterpret_cast<uint8_t*>(t + p_exits);
+    uint8_t* gexits = reinterpret_cast<uint8_t*>(t + p_gexits);
+    uint32_t* obase = reinterpret_cast<uint32_t*>(t + p_obase);
+    uint8_t* entry = reinterpret_cast<uint8_t*>(t + p_entry);
+    uint8_t* gentry = reinterpret_cast<uint8_t*>(t + p_gentry);
+    unsigned long long* err = reinterpret_cast<unsigned long long*>(t + p_err);
+    uint32_t* held = reinterpret_cast<uint32_t*>(err + 1);
+    BFS_CUDA_TRY(cudaMemsetAsync(gentry, 0, parts.bytes - p_gentry, st));   // groups past a broken chain, the error
     const int grid = (int)std::min<int64_t>((nch * kMaxRecord + kBT - 1) / kBT, (int64_t)sms * 16);
-    bbc_entries<<<grid, kBT, 0, st>>>(bytes, nbytes_in, exits.as<uint8_t>(), outb.as<int64_t>());
-    bbc_chain<<<1, 1024, 0, st>>>(exits.as<uint8_t>(), outb.as<int64_t>(), nbytes_in, entry.as<uint8_t>(),
-                                  obase.as<uint32_t>(), err.as<unsigned long long>());
-    scan_one_cta<<<1, 1024, 0, st>>>(obase.as<uint32_t>(), nch, tot.as<uint32_t>());
-    unsigned long long h_err = 0;
-    uint32_t h_tot = 0;
-    BFS_CUDA_TRY(cudaMemcpyAsync(&h_err, err.ptr, sizeof(h_err), cudaMemcpyDeviceToHost, st));
-    BFS_CUDA_TRY(cudaMemcpyAsync(&h_tot, tot.ptr, sizeof(h_tot), cudaMemcpyDeviceToHost, st));
-    BFS_CUDA_TRY(cudaStreamSynchronize(st));
-    if (h_err || (int64_t)h_tot != nbytes) return set_error(BFS_ERR_CORRUPT, "malformed BBC stream");
+    const int ggrid = (int)std::min<int64_t>((ng * 32 + kBT - 1) / kBT, (int64_t)sms * 4);
+    bbc_entries<<<grid, kBT, 0, st>>>(bytes, nbytes_in, exits, outb);
+    bbc_groups<<<ggrid, kBT, 0, st>>>(exits, nch, gexits);
+    bbc_chain<<<1, 1024, 0, st>>>(gexits, ng, gentry, err);
+    bbc_fill<<<ggrid, kBT, 0, st>>>(exits, outb, nch, gentry, entry, obase);
+    BFS_CUDA_TRY(launch_cluster(scan_cluster, st, obase, nullptr, nch, obase, held, nullptr));
     const int xgrid = (int)std::min<int64_t>((nch * 32 + kBT - 1) / kBT, (int64_t)sms * 16);
-    bbc_expand<<<xgrid, kBT, 0, st>>>(bytes, nbytes_in, nbytes, entry.as<uint8_t>(), obase.as<uint32_t>(),
-                                      reinterpret_cast<uint8_t*>(bits), err.as<unsigned long long>());
-    bbc_padding<<<1, 1, 0, st>>>(reinterpret_cast<const uint8_t*>(bits), nbits, err.as<unsigned long long>());
+    bbc_expand<<<xgrid, kBT, 0, st>>>(bytes, nbytes_in, nbytes, entry, obase, held, reinterpret_cast<uint8_t*>(bits), err);
+    bbc_outcome<<<1, 1, 0, st>>>(reinterpret_cast<const uint8_t*>(bits), nbits, held, err, bad.device());
     BFS_CUDA_TRY(cudaGetLastError());
-    BFS_CUDA_TRY(cudaMemcpyAsync(&h_err, err.ptr, sizeof(h_err), cudaMemcpyDeviceToHost, st));
     BFS_CUDA_TRY(cudaStreamSynchronize(st));
-    if (h_err) return set_error(BFS_ERR_CORRUPT, "malformed BBC stream");
+    if (bad.value()) return set_error(BFS_ERR_CORRUPT, "malformed BBC stream");
     return BFS_OK;
 }
 

@@ -8,6 +8,7 @@
 // directory V_{i,j} (Eq. 4); a scan of directory popcounts gives the rank of
 // every nonempty column; the entries are then scattered column by column.
 #include <atomic>
+#include <condition_variable>
 #include <cstdarg>
 #include <cstring>
 #include <new>
@@ -74,6 +75,84 @@ void DevBuf::release() {
     if (ptr) cudaFree(ptr);
     ptr = nullptr;
     bytes = 0;
+}
+
+// ---------------------------------------------------------- call scratch --
+namespace {
+constexpr int kMaxDevices = 64;
+std::mutex t_pool_mu;
+cudaMemPool_t t_pool[kMaxDevices] = {};
+
+std::mutex t_flag_mu;
+std::condition_variable t_flag_free;
+unsigned long long* t_flags = nullptr;             // kHostFlags pairs, mapped and portable
+uint64_t t_flag_used[kHostFlags / 64] = {};
+}
+
+bfs_status Scratch::alloc(size_t nbytes, cudaStream_t st) {
+    int64_t k = g_fail_countdown.load();
+    while (k > 0 && !g_fail_countdown.compare_exchange_weak(k, k - 1)) {
+    }
+    if (k == 1) return set_error(BFS_ERR_OUT_OF_MEMORY, "scratch of %zu bytes: injected failure", nbytes);
+    int dev = 0;
+    BFS_CUDA_TRY(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= kMaxDevices) return set_error(BFS_ERR_INVALID_ARG, "device ordinal %d out of range", dev);
+    {
+        std::lock_guard<std::mutex> lk(t_pool_mu);
+        if (!t_pool[dev]) {
+            cudaMemPoolProps props = {};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.handleTypes = cudaMemHandleTypeNone;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            cudaMemPool_t pool = nullptr;
+            BFS_CUDA_TRY(cudaMemPoolCreate(&pool, &props));
+            uint64_t keep = kScratchKept;
+            cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+            t_pool[dev] = pool;
+        }
+    }
+    stream = st;
+    cudaError_t e = cudaMallocFromPoolAsync(&ptr, nbytes ? nbytes : 16, t_pool[dev], st);
+    if (e != cudaSuccess) {
+        ptr = nullptr;
+        cudaGetLastError();
+        return set_error(BFS_ERR_OUT_OF_MEMORY, "scratch of %zu bytes: %s", nbytes, cudaGetErrorString(e));
+    }
+    return BFS_OK;
+}
+
+bfs_status HostFlag::take() {
+    std::unique_lock<std::mutex> lk(t_flag_mu);
+    if (!t_flags) {
+        void* p = nullptr;
+        BFS_CUDA_TRY(cudaHostAlloc(&p, sizeof(unsigned long long) * 2 * kHostFlags,
+                                   cudaHostAllocMapped | cudaHostAllocPortable));
+        t_flags = static_cast<unsigned long long*>(p);
+    }
+    for (;;) {
+        for (int w = 0; w < kHostFlags / 64; ++w)
+            if (~t_flag_used[w]) {
+                const int b = __builtin_ctzll(~t_flag_used[w]);
+                t_flag_used[w] |= 1ull << b;
+                slot = 64 * w + b;
+                t_flags[2 * slot] = t_flags[2 * slot + 1] = 0ull;
+                return BFS_OK;
+            }
+        t_flag_free.wait(lk);
+    }
+}
+
+HostFlag::~HostFlag() {
+    if (slot < 0) return;
+    std::lock_guard<std::mutex> lk(t_flag_mu);
+    t_flag_used[slot / 64] &= ~(1ull << (slot % 64));
+    t_flag_free.notify_one();
+}
+
+volatile unsigned long long* HostFlag::device(int word) const { return t_flags + 2 * slot + word; }   // unified addressing
+unsigned long long HostFlag::value(int word) const {
+    return *static_cast<volatile unsigned long long*>(t_flags + 2 * slot + word);
 }
 
 // ------------------------------------------------------------ build kernels --

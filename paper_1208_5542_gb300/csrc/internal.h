@@ -50,6 +50,41 @@ struct DevBuf {
     template <typename T> T* as() const { return static_cast<T*>(ptr); }
 };
 
+// Scratch of one codec call: stream-ordered memory of the library's own pool
+// of the device, which keeps at most kScratchKept bytes between calls (the
+// rest goes back to the device at the next synchronisation).  The pool's
+// allocations are ordered on the call's stream, so calls on several streams
+// and threads do not meet.
+constexpr uint64_t kScratchKept = 64ull << 20;
+
+struct Scratch {
+    void* ptr = nullptr;
+    cudaStream_t stream = nullptr;
+    Scratch() = default;
+    Scratch(const Scratch&) = delete;
+    Scratch& operator=(const Scratch&) = delete;
+    ~Scratch() { if (ptr) cudaFreeAsync(ptr, stream); }
+    bfs_status alloc(size_t nbytes, cudaStream_t st);
+    template <typename T> T* as() const { return static_cast<T*>(ptr); }
+};
+
+// Two 8-byte words of mapped pinned memory for a call's kernels to report in
+// (an error, a count): read by the host after the stream has been
+// synchronised, with no copy.  kHostFlags pairs live in one page for the life
+// of the process; a call (which takes one) that finds none free waits for one.
+constexpr int kHostFlags = 256;
+
+struct HostFlag {
+    int slot = -1;
+    HostFlag() = default;
+    HostFlag(const HostFlag&) = delete;
+    HostFlag& operator=(const HostFlag&) = delete;
+    ~HostFlag();
+    bfs_status take();                              // cleared
+    volatile unsigned long long* device(int word = 0) const;
+    unsigned long long value(int word = 0) const;
+};
+
 // ------------------------------------------------------------ the layout --
 // Blocks b = i*p + j: block-row i = destinations in range i, block column j =
 // sources in range j.  Per block: directory V_{i,j} (range_len(j) bits, padded
@@ -219,15 +254,11 @@ struct EncodeArgs {
     uint8_t* slot_bits;         // or nullptr: the scan writes 1 for a slot whose stream carries a set bit
     const uint8_t* slot_live;   // or nullptr: a slot with slot_live[s] == 0 is all zero (not read)
 };
-bfs_status launch_wah_encode(const EncodeArgs& a, int wah_bits, cudaStream_t st);
 
-struct DecodeArgs {             // standalone decode into a bitmap
-    const void* words;
-    int64_t nwords;
-    int64_t nbits;
-    uint32_t* bits;
-    unsigned long long* err;
-};
-bfs_status launch_wah_decode_bitmap(const DecodeArgs& a, int wah_bits, cudaStream_t st);
+// One bitmap, standalone (one cluster, no scratch; ordered on st).
+bfs_status launch_wah_encode(const uint32_t* bits, int64_t nbits, int wah_bits, void* words, int64_t* count,
+                             cudaStream_t st);
+bfs_status launch_wah_decode_bitmap(const void* words, int64_t nwords, int64_t nbits, int wah_bits, uint32_t* bits,
+                                    volatile unsigned long long* err, cudaStream_t st);
 
 }  // namespace bfsgb

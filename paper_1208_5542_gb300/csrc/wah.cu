@@ -2,19 +2,14 @@
 // fused with the cross-directory sieve (Alg. 3, Sec. V-A), and the standalone
 // codec entry points of the C ABI.
 //
-// Encoder: one CTA per exchange slot walks the slot's groups in tiles of
-// kTile groups.  Inside a tile every thread classifies kK consecutive groups
-// (all-zero / all-one / literal); a block scan of "head" flags (a literal, or
-// a group whose type differs from its predecessor) gives every word its index,
-// and a block max-scan of head positions gives every group the start of its
-// run, so the group that ends a fill run writes the merged fill word.  The open
-// run, the word count and the previous type carry from tile to tile.  Tiles
-// whose frontier bits are all zero (frontier summary: one byte per 1024 bits)
-// are skipped without loading a word.
+// The search's encoder works on all slots of an exchange at once in three
+// data-parallel passes (enc_chunk_*); the codec entry points encode or decode
+// one bitmap with one cluster of CTAs (wah_encode_bitmap, wah_decode_bitmap).
 #include <algorithm>
 #include <cstring>
 #include <mutex>
 
+#include "cluster.cuh"
 #include "common.cuh"
 #include "internal.h"
 #include "wah.cuh"
@@ -22,10 +17,8 @@
 namespace bfsgb {
 namespace {
 
-constexpr int kNT = 256;          // threads per encoder CTA
-constexpr int kK = 4;             // groups per thread per tile
-constexpr int kTile = kNT * kK;   // groups per tile
-static_assert(kTile == kEncChunkGroups, "the encoder's chunk is the unit of its chunk index");
+constexpr int kNT = 256;          // threads of the raw writer's CTAs
+constexpr int kTile = kEncChunkGroups;   // groups per chunk of the parallel encoder
 
 struct SlotGeom {
     int64_t src0;      // first bitmap bit of the slot's source range
@@ -46,170 +39,88 @@ __device__ __forceinline__ SlotGeom slot_geom(const EncodeArgs& a, int s) {
     return g;
 }
 
-// True if the frontier-summary bytes q0..q1 (inclusive) are all zero; the
-// summary is padded to whole 32-bit words.
-__device__ __forceinline__ bool fsum_zero(const uint8_t* fsum, int64_t q0, int64_t q1) {
-    const uint32_t* w = reinterpret_cast<const uint32_t*>(fsum);
-    const int64_t a = q0 >> 2, b = q1 >> 2;
-    for (int64_t i = a; i <= b; ++i) {
-        uint32_t x = __ldcg(w + i);
-        if (i == a) x &= 0xffffffffu << (8 * (q0 & 3));
-        if (i == b) x &= 0xffffffffu >> (8 * (3 - (q1 & 3)));
-        if (x) return false;
+// ------------------------------------------------------ standalone encode --
+// One bitmap as a WAH stream, by one cluster: per round every thread classifies
+// kCK consecutive groups (all-zero / all-one / literal) and the group before
+// and after them, which gives it its "heads" (a literal, or a group whose type
+// differs from its predecessor); a scan of the head counts gives every word
+// its index and a max-scan of the head positions the start of every run, so
+// the group that ends a fill run writes the merged fill word.  The open run
+// and the word count carry from round to round.  Only the words that hold bits
+// are read.
+template <typename W>
+__device__ __forceinline__ W bitmap_bits(const uint32_t* __restrict__ bits, int64_t words, int64_t pos) {
+    const int64_t w = pos >> 5;
+    const uint32_t sh = (uint32_t)(pos & 31);
+    const uint32_t a = w < words ? __ldg(bits + w) : 0u, b = w + 1 < words ? __ldg(bits + w + 1) : 0u;
+    const uint32_t lo = __funnelshift_r(a, b, sh);
+    if constexpr (sizeof(W) == 4) {
+        return lo;
+    } else {
+        const uint32_t c = w + 2 < words ? __ldg(bits + w + 2) : 0u;
+        return ((unsigned long long)__funnelshift_r(b, c, sh) << 32) | lo;
     }
-    return true;
 }
 
 template <typename W>
-__device__ __forceinline__ W load_group(const EncodeArgs& a, const SlotGeom& sg, int64_t g) {
-    W x = Wah<W>::group(a.frontier, (uint64_t)(sg.src0 + g * Wah<W>::GB));
-    if (sg.dirb && x) x &= Wah<W>::group(sg.dirb, (uint64_t)(g * Wah<W>::GB));
-    return x;
-}
-
-template <typename W>
-__global__ void __launch_bounds__(kNT) wah_encode_kernel(EncodeArgs a, unsigned long long* setbits) {
+__global__ void __launch_bounds__(kCT) wah_encode_bitmap(const uint32_t* bits, int64_t nbits, W* out, int64_t* count) {
     using T = Wah<W>;
     constexpr int GB = T::GB;
-    const int s = blockIdx.x;
-    const SlotGeom sg = slot_geom(a, s);
-    const int64_t G = sg.nbits / GB;
-    const int r = (int)(sg.nbits % GB);
-    W* out = static_cast<W*>(a.out) + (int64_t)s * a.slot_cap;
-
-    __shared__ int64_t sm64[kNT / 32 + 1];
-    __shared__ unsigned long long smu[kNT / 32 + 1];
-    __shared__ uint8_t sm_first[kNT], sm_last[kNT];
-    __shared__ int sm_flag;
-    __shared__ int sm_next_type;
-    __shared__ int sm_carry_type;
-    __shared__ int64_t sm_carry_start;
-
+    __shared__ ClusterScan<int64_t> s_heads, s_last;
+    const int64_t G = nbits / GB, words = (nbits + 31) >> 5;
+    const int r = (int)(nbits % GB);
     int64_t nw = 0;            // words assigned so far (the open run's word included)
-    int prev_type = -1;        // type of the group before the tile (-1: none)
-    int64_t run_start = 0;     // start group of the run holding the group before the tile
-    unsigned long long ones = 0;
-
-    for (int64_t tb = 0; tb < G;) {
-        int64_t tend = (tb + kTile < G) ? tb + kTile : G;
-        // ---- zero skip from the frontier summary: lane l of warp 0 tests tile
-        // tb + l*kTile; a run of leading all-zero tiles extends the zero fill ----
-        if (a.fsum) {
-            if (threadIdx.x < 32) {
-                const int64_t t0 = tb + (int64_t)lane_id() * kTile;
-                bool zero = false;
-                if (t0 < G) {
-                    const int64_t t1 = (t0 + kTile < G) ? t0 + kTile : G;
-                    zero = fsum_zero(a.fsum, (sg.src0 + t0 * GB) >> 10, (sg.src0 + t1 * GB - 1) >> 10);
-                }
-                const uint32_t zmask = __ballot_sync(0xffffffffu, zero);
-                if (threadIdx.x == 0) sm_flag = __ffs(~zmask) - 1;      // leading zero tiles (0..31)
-                if (threadIdx.x == 0 && zmask == 0xffffffffu) sm_flag = 32;
-            }
-            __syncthreads();
-            const int nz = sm_flag;
-            __syncthreads();
-            if (nz > 0) {
-                const int64_t skip_end = (tb + (int64_t)nz * kTile < G) ? tb + (int64_t)nz * kTile : G;
-                if (prev_type != G_ZERO) { nw += 1; run_start = tb; prev_type = G_ZERO; }
-                if (skip_end == G && threadIdx.x == 0) out[nw - 1] = fill_word<W>(G_ZERO, (uint64_t)(G - run_start));
-                tb = skip_end;
-                continue;
-            }
-        }
-        // ---- classify this thread's groups ----
-        const int64_t g0 = tb + (int64_t)threadIdx.x * kK;
-        W x[kK];
-        int ty[kK];
+    int64_t run_start = 0;     // start group of the run holding the group before the round
+    auto group = [&](int64_t g) { return bitmap_bits<W>(bits, words, g * GB) & T::ONES; };
+    int turn = 0;
+    for (int64_t tb = 0; tb < G; tb += kClusterRound, ++turn) {
+        const int64_t g0 = tb + cluster_thread() * kCK;
+        W x[kCK];
+        int ty[kCK + 1];
 #pragma unroll
-        for (int k = 0; k < kK; ++k) {
-            const int64_t g = g0 + k;
-            if (g < tend) {
-                x[k] = load_group<W>(a, sg, g);
-                ty[k] = group_type<W>(x[k]);
-                ones += (unsigned long long)T::popc(x[k]);
-            } else {
-                x[k] = W(0);
-                ty[k] = G_NONE;
-            }
+        for (int k = 0; k < kCK; ++k) {
+            x[k] = g0 + k < G ? group(g0 + k) : W(0);
+            ty[k] = g0 + k < G ? group_type<W>(x[k]) : G_NONE;
         }
-        // a zero run carried into this tile (possibly across skipped tiles) ends
-        // here if the tile opens with another type: write its fill word (when the
-        // run ended in a processed tile the same word was already written there)
-        if (threadIdx.x == 0 && prev_type == G_ZERO && ty[0] != G_ZERO)
-            out[nw - 1] = fill_word<W>(G_ZERO, (uint64_t)(tb - run_start));
-        sm_first[threadIdx.x] = (uint8_t)ty[0];
-        sm_last[threadIdx.x] = (uint8_t)ty[kK - 1];
-        if (threadIdx.x == 0) sm_next_type = (tend < G) ? group_type<W>(load_group<W>(a, sg, tend)) : G_NONE;
-        __syncthreads();
-        const int prev0 = (threadIdx.x == 0) ? prev_type : (int)sm_last[threadIdx.x - 1];
-        // heads and last head position of this thread
-        bool h[kK];
-        int hc = 0;
-        int64_t lastpos = -1;
-        int pt = prev0;
+        ty[kCK] = g0 + kCK < G ? group_type<W>(group(g0 + kCK)) : G_NONE;
+        int pt = (g0 > 0 && g0 < G) ? group_type<W>(group(g0 - 1)) : -1;
+        uint32_t h = 0;
+        int64_t last = -1;
 #pragma unroll
-        for (int k = 0; k < kK; ++k) {
-            h[k] = (ty[k] != G_NONE) && (ty[k] == G_LIT || ty[k] != pt);
-            if (h[k]) { ++hc; lastpos = g0 + k; }
+        for (int k = 0; k < kCK; ++k) {
+            if (ty[k] != G_NONE && (ty[k] == G_LIT || ty[k] != pt)) {
+                h |= 1u << k;
+                last = g0 + k;
+            }
             pt = ty[k];
         }
-        int64_t tot_h;
-        const int64_t excl_h = block_excl_scan<kNT>((int64_t)hc, (int64_t)0, OpSum(), sm64, &tot_h);
-        int64_t dummy;
-        const int64_t excl_pos = block_excl_scan<kNT>(lastpos, (int64_t)-1, OpMax(), sm64, &dummy);
-        // ---- write literals and the fill words of runs that end here ----
-        int64_t cur_start = excl_pos > run_start ? excl_pos : run_start;
-        int64_t widx = nw + excl_h - 1;
+        int64_t heads, latest;
+        int64_t widx = nw - 1 + cluster_excl_scan((int64_t)__popc(h), (int64_t)0, OpSum(), s_heads, turn, &heads);
+        const int64_t start = cluster_excl_scan(last, (int64_t)-1, OpMax(), s_last, turn, &latest);
+        int64_t cur = start > run_start ? start : run_start;
 #pragma unroll
-        for (int k = 0; k < kK; ++k) {
-            const int64_t g = g0 + k;
+        for (int k = 0; k < kCK; ++k) {
             if (ty[k] == G_NONE) break;
-            if (h[k]) { cur_start = g; ++widx; }
-            int nt;
-            if (k + 1 < kK) nt = ty[k + 1];
-            else nt = (threadIdx.x + 1 < kNT) ? (int)sm_first[threadIdx.x + 1] : G_NONE;
-            if (g + 1 == tend) nt = sm_next_type;
-            if (ty[k] == G_LIT) {
-                out[widx] = T::to_payload(x[k]);
-            } else if (nt != ty[k]) {
-                out[widx] = fill_word<W>(ty[k], (uint64_t)(g - cur_start + 1));
+            if ((h >> k) & 1u) {
+                cur = g0 + k;
+                ++widx;
             }
-            if (g + 1 == tend) { sm_carry_type = ty[k]; sm_carry_start = cur_start; }
+            if (ty[k] == G_LIT) out[widx] = T::to_payload(x[k]);
+            else if (ty[k + 1] != ty[k]) out[widx] = fill_word<W>(ty[k], (uint64_t)(g0 + k - cur + 1));
         }
-        __syncthreads();
-        nw += tot_h;
-        prev_type = sm_carry_type;
-        run_start = sm_carry_start;
-        __syncthreads();
-        tb = tend;
+        nw += heads;
+        run_start = latest > run_start ? latest : run_start;
     }
-    if (setbits) {
-        unsigned long long tot;
-        block_excl_scan<kNT>(ones, 0ull, OpSum(), smu, &tot);
-        if (threadIdx.x == 0 && tot) atomicAdd(setbits, tot);
+    if (cluster_thread() == 0) {
+        if (r > 0) out[nw++] = T::to_active(bitmap_bits<W>(bits, words, G * GB) & (W)((W(1) << r) - W(1)), r);
+        *count = nw;
     }
-    if (threadIdx.x == 0) {
-        int64_t total = nw;
-        if (r > 0) {
-            const uint64_t pos = (uint64_t)(sg.src0 + G * GB);
-            W y = T::tail(a.frontier, pos, r);
-            if (a.invert_frontier) y = ~y & (W)((W(1) << r) - W(1));
-            if (sg.dirb && y) y &= T::tail(sg.dirb, (uint64_t)(G * GB), r);
-            if (a.dir_clear) {              // the tail words no chunk of the write pass owns
-                uint32_t* d = a.dir_clear + (int64_t)s * a.dir_stride;
-                for (int64_t w = (G * GB + 31) >> 5; w < (sg.nbits + 31) >> 5; ++w) d[w] = 0u;
-            }
-            if (setbits && y) atomicAdd(setbits, (unsigned long long)T::popc(y));
-            out[total++] = T::to_active(y, r);
-        }
-        a.counts[s] = total;
-    }
+    cluster_done();
 }
 
 // ------------------------------------------------- parallel slot encoder --
-// The same stream as wah_encode_kernel, built in three data-parallel passes
-// over (slot, chunk of kTile groups):
+// All slots' streams, built in three data-parallel passes over (slot, chunk of
+// kTile groups):
 //   1. enc_chunk_sums32 / enc_chunk_sums64: one warp per chunk tests the
 //      frontier summary (a chunk without frontier bits is flagged all-zero and
 //      not read) and, for the others, stages the chunk in shared memory and
@@ -1036,23 +947,108 @@ __global__ void __launch_bounds__(kNT) enc_raw32(EncodeArgs a) {
 }
 
 // ------------------------------------------------------- standalone decode --
-// One CTA decodes the stream into the zeroed output (cta_wah_decode_or);
-// malformed streams set *err.
+// One stream into a zeroed bitmap of ceil(nbits/32) words, by one cluster: per
+// round every thread takes kCK consecutive words, a scan of their run lengths
+// places them, and it ORs their bits in; the words of a long 1-fill are set by
+// the whole warp.  Malformed streams (a fill of length 0, groups past nbits, a
+// missing or oversized active word, trailing words) set *err; nothing past the
+// bitmap is written.
+constexpr int64_t kLongFill = 1024;      // bits of a 1-fill from which on the warp sets it
+
+__device__ __forceinline__ void set_bits(uint32_t* bits, int64_t b0, int64_t b1, int first, int step) {
+    const int64_t w0 = b0 >> 5, w1 = (b1 - 1) >> 5;
+    for (int64_t w = w0 + first; w <= w1; w += step) {
+        uint32_t mask = 0xffffffffu;
+        if (w == w0) mask &= 0xffffffffu << (b0 & 31);
+        if (w == w1) mask &= 0xffffffffu >> (31 - ((b1 - 1) & 31));
+        if (mask == 0xffffffffu) bits[w] = mask;
+        else atomicOr(bits + w, mask);
+    }
+}
+
 template <typename W>
-__global__ void __launch_bounds__(kNT) wah_decode_bitmap_kernel(DecodeArgs a) {
-    __shared__ unsigned long long smu[kNT / 32 + 1];
-    cta_wah_decode_or<W, kNT>(static_cast<const W*>(a.words), a.nwords, a.nbits, a.bits, 0ull, a.err, smu);
+__global__ void __launch_bounds__(kCT) wah_decode_bitmap(const W* in, int64_t nwords, int64_t nbits, uint32_t* bits,
+                                                         volatile unsigned long long* err) {
+    using T = Wah<W>;
+    constexpr int GB = T::GB;
+    __shared__ ClusterScan<long long> s_len;
+    const long long G = nbits / GB;
+    const int r = (int)(nbits % GB);
+    const int64_t words = (nbits + 31) >> 5;
+    bool bad = false;
+    long long gpos = 0;        // groups consumed before the round
+    auto or_group = [&](int64_t b, W v) {
+        if (!v) return;
+        const int64_t w = b >> 5;
+        const uint32_t sh = (uint32_t)(b & 31);
+        const unsigned long long lo = (unsigned long long)v << sh;
+        if ((uint32_t)lo) atomicOr(bits + w, (uint32_t)lo);
+        if ((uint32_t)(lo >> 32) && w + 1 < words) atomicOr(bits + w + 1, (uint32_t)(lo >> 32));
+        if (sizeof(W) == 8 && sh && (v >> (sizeof(W) * 8 - sh)) && w + 2 < words)
+            atomicOr(bits + w + 2, (uint32_t)(v >> (sizeof(W) * 8 - sh)));
+    };
+    int turn = 0;
+    for (int64_t wb = 0; wb < nwords; wb += kClusterRound, ++turn) {
+        const int64_t x0 = wb + cluster_thread() * kCK;
+        W y[kCK];
+        long long len[kCK], sum = 0, tot;
+#pragma unroll
+        for (int k = 0; k < kCK; ++k) {
+            y[k] = x0 + k < nwords ? in[x0 + k] : W(0);
+            // a longer run than the bitmap is malformed whatever its length: capped, the sums fit
+            const unsigned long long l = x0 + k < nwords ? word_groups<W>(y[k]) : 0ull;
+            len[k] = l <= (unsigned long long)G + 1 ? (long long)l : G + 1;
+            sum += len[k];
+        }
+        long long gs = gpos + cluster_excl_scan(sum, 0ll, OpSum(), s_len, turn, &tot);
+#pragma unroll
+        for (int k = 0; k < kCK; ++k) {
+            int64_t f0 = 0, f1 = 0;                  // bits of a long 1-fill
+            if (x0 + k < nwords) {
+                if (gs < G) {
+                    if (!is_fill<W>(y[k])) {
+                        or_group(gs * GB, T::from_payload(y[k]));
+                    } else if (len[k] == 0 || gs + len[k] > G) {
+                        bad = true;
+                    } else if (y[k] & T::VAL) {
+                        f0 = gs * GB;
+                        f1 = (gs + len[k]) * GB;
+                        if (f1 - f0 < kLongFill) {
+                            set_bits(bits, f0, f1, 0, 1);
+                            f0 = f1 = 0;
+                        }
+                    }
+                } else if (gs == G && r > 0 && x0 + k == nwords - 1) {
+                    if ((y[k] >> r) != W(0)) bad = true;
+                    else or_group(G * GB, T::from_active(y[k], r));
+                } else {
+                    bad = true;                      // word past the groups, or misplaced active word
+                }
+            }
+            gs += len[k];
+            uint32_t m = __ballot_sync(0xffffffffu, f1 > f0);
+            while (m) {
+                const int o = __ffs(m) - 1;
+                m &= m - 1;
+                set_bits(bits, __shfl_sync(0xffffffffu, f0, o), __shfl_sync(0xffffffffu, f1, o), (int)lane_id(), 32);
+            }
+        }
+        gpos += tot;
+    }
+    if (cluster_thread() == 0 && gpos != G + (r > 0 ? 1 : 0)) bad = true;
+    if (bad) *err = 1ull;
+    cluster_done();
 }
 
 }  // namespace
 
-bfs_status launch_wah_encode(const EncodeArgs& a, int wah_bits, cudaStream_t st) {
-    if (a.nslots <= 0) return BFS_OK;
+bfs_status launch_wah_encode(const uint32_t* bits, int64_t nbits, int wah_bits, void* words, int64_t* count,
+                             cudaStream_t st) {
     if (wah_bits == 32)
-        wah_encode_kernel<uint32_t><<<a.nslots, kNT, 0, st>>>(a, nullptr);
+        BFS_CUDA_TRY(launch_cluster(wah_encode_bitmap<uint32_t>, st, bits, nbits, static_cast<uint32_t*>(words), count));
     else
-        wah_encode_kernel<unsigned long long><<<a.nslots, kNT, 0, st>>>(a, nullptr);
-    BFS_CUDA_TRY(cudaGetLastError());
+        BFS_CUDA_TRY(launch_cluster(wah_encode_bitmap<unsigned long long>, st, bits, nbits,
+                                    static_cast<unsigned long long*>(words), count));
     return BFS_OK;
 }
 
@@ -1088,12 +1084,18 @@ bfs_status launch_wah_encode_parallel(const EncodeArgs& a, int wah_bits, void* s
 size_t parallel_encode_sum_bytes() { return sizeof(ChunkSum); }
 size_t parallel_encode_base_bytes() { return sizeof(ChunkBase); }
 
-bfs_status launch_wah_decode_bitmap(const DecodeArgs& a, int wah_bits, cudaStream_t st) {
+// `bits` (ceil(nbits/32) words) is cleared first; *err (device memory or a
+// mapped host word) is set to 1 for a malformed stream.
+bfs_status launch_wah_decode_bitmap(const void* words, int64_t nwords, int64_t nbits, int wah_bits, uint32_t* bits,
+                                    volatile unsigned long long* err, cudaStream_t st) {
+    const int64_t out_words = (nbits + 31) / 32;
+    if (out_words > 0) BFS_CUDA_TRY(cudaMemsetAsync(bits, 0, sizeof(uint32_t) * (size_t)out_words, st));
     if (wah_bits == 32)
-        wah_decode_bitmap_kernel<uint32_t><<<1, kNT, 0, st>>>(a);
+        BFS_CUDA_TRY(launch_cluster(wah_decode_bitmap<uint32_t>, st, static_cast<const uint32_t*>(words), nwords, nbits,
+                                    bits, err));
     else
-        wah_decode_bitmap_kernel<unsigned long long><<<1, kNT, 0, st>>>(a);
-    BFS_CUDA_TRY(cudaGetLastError());
+        BFS_CUDA_TRY(launch_cluster(wah_decode_bitmap<unsigned long long>, st,
+                                    static_cast<const unsigned long long*>(words), nwords, nbits, bits, err));
     return BFS_OK;
 }
 
@@ -1142,22 +1144,11 @@ bfs_status bfs_wah_encode(const uint32_t* bits, int64_t nbits, int32_t word_bits
     if (capacity_words < bound)
         return set_error(BFS_ERR_INVALID_ARG, "capacity %lld below the bound %lld", (long long)capacity_words, (long long)bound);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    EncodeArgs a;
-    memset(&a, 0, sizeof(a));
-    a.frontier = bits;
-    a.p = 1;
-    a.nb = nbits;
-    a.n = nbits;
-    a.sieve = 0;
-    a.nslots = 1;
-    a.out = words;
-    a.slot_cap = capacity_words;
-    a.counts = nwords;
     if (nbits == 0) {
         BFS_CUDA_TRY(cudaMemsetAsync(nwords, 0, sizeof(int64_t), st));
         return BFS_OK;
     }
-    return launch_wah_encode(a, word_bits, st);
+    return launch_wah_encode(bits, nbits, word_bits, words, nwords, st);
 }
 
 bfs_status bfs_wah_decode(const void* words, int64_t nwords, int64_t nbits, int32_t word_bits, uint32_t* bits,
@@ -1166,26 +1157,21 @@ bfs_status bfs_wah_decode(const void* words, int64_t nwords, int64_t nbits, int3
     if (nbits < 0 || nwords < 0 || (nwords > 0 && !words) || (nbits > 0 && !bits))
         return set_error(BFS_ERR_INVALID_ARG, "bad decode arguments");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int64_t out_words = (nbits + 31) / 32;
-    DevBuf err, pad;
-    BFS_TRY(err.alloc(sizeof(unsigned long long)));
-    BFS_CUDA_TRY(cudaMemsetAsync(err.ptr, 0, sizeof(unsigned long long), st));
-    // the kernel may OR into the word after the last one: decode into a padded copy
-    BFS_TRY(pad.alloc(sizeof(uint32_t) * (out_words + 2)));
-    BFS_CUDA_TRY(cudaMemsetAsync(pad.ptr, 0, pad.bytes, st));
-    DecodeArgs a;
-    a.words = words;
-    a.nwords = nwords;
-    a.nbits = nbits;
-    a.bits = pad.as<uint32_t>();
-    a.err = err.as<unsigned long long>();
-    BFS_TRY(launch_wah_decode_bitmap(a, word_bits, st));
-    unsigned long long h_err = 0;
-    BFS_CUDA_TRY(cudaMemcpyAsync(&h_err, err.ptr, sizeof(h_err), cudaMemcpyDeviceToHost, st));
-    if (out_words > 0)
-        BFS_CUDA_TRY(cudaMemcpyAsync(bits, pad.ptr, sizeof(uint32_t) * out_words, cudaMemcpyDeviceToDevice, st));
+    HostFlag err;
+    BFS_TRY(err.take());
+    // a stream inside the output would be overwritten while it is read: decoded aside
+    const size_t out_bytes = sizeof(uint32_t) * (size_t)((nbits + 31) / 32);
+    const char *w0 = static_cast<const char*>(words), *b0 = reinterpret_cast<const char*>(bits);
+    Scratch aside;
+    uint32_t* dst = bits;
+    if (nwords > 0 && out_bytes > 0 && w0 < b0 + out_bytes && b0 < w0 + nwords * (word_bits / 8)) {
+        BFS_TRY(aside.alloc(out_bytes, st));
+        dst = aside.as<uint32_t>();
+    }
+    BFS_TRY(launch_wah_decode_bitmap(words, nwords, nbits, word_bits, dst, err.device(), st));
+    if (dst != bits) BFS_CUDA_TRY(cudaMemcpyAsync(bits, dst, out_bytes, cudaMemcpyDeviceToDevice, st));
     BFS_CUDA_TRY(cudaStreamSynchronize(st));
-    if (h_err) return set_error(BFS_ERR_CORRUPT, "malformed WAH stream");
+    if (err.value()) return set_error(BFS_ERR_CORRUPT, "malformed WAH stream");
     return BFS_OK;
 }
 
@@ -1203,16 +1189,9 @@ bfs_status bfs_wah_decode_static(const void* words, int64_t nwords, int64_t nbit
     unsigned long long* err = static_cast<unsigned long long*>(scratch);
     uint32_t* staging = reinterpret_cast<uint32_t*>(err + 1);
     const int64_t out_words = (nbits + 31) / 32;
-    // the array keeps the previous call's contents: clear the error word and the staging words used
+    // the array keeps the previous call's contents: the error word is cleared here, the staging words by the decode
     BFS_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(unsigned long long), st));
-    BFS_CUDA_TRY(cudaMemsetAsync(staging, 0, sizeof(uint32_t) * (out_words + 2), st));
-    DecodeArgs a;
-    a.words = words;
-    a.nwords = nwords;
-    a.nbits = nbits;
-    a.bits = staging;
-    a.err = err;
-    BFS_TRY(launch_wah_decode_bitmap(a, word_bits, st));
+    BFS_TRY(launch_wah_decode_bitmap(words, nwords, nbits, word_bits, staging, err, st));
     unsigned long long h_err = 0;
     BFS_CUDA_TRY(cudaMemcpyAsync(&h_err, err, sizeof(h_err), cudaMemcpyDeviceToHost, st));
     if (out_words > 0)
