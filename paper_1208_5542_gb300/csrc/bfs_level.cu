@@ -1801,23 +1801,7 @@ bfs_status ensure_workspace_once(bfs_graph* g) {
     W.chunk_words = 32;
     W.chunks_per_slot = (cap32 + 31) / 32;
     const int64_t xbytes = p2 * std::max<int64_t>(4 * cap32, 8 * cap64);
-    BFS_TRY(W.pi.alloc(4 * W.bm_words));
-    BFS_TRY(W.fa.alloc(4 * W.bm_words));
-    BFS_TRY(W.fb.alloc(4 * W.bm_words));
-    BFS_TRY(W.fsum.alloc(W.fsum_len));
-    BFS_TRY(W.xbuf.alloc(xbytes));
-    BFS_TRY(W.xcount.alloc(sizeof(int64_t) * p2));
-    BFS_TRY(W.chunk_base.alloc(sizeof(int64_t) * p2 * W.chunks_per_slot));
-    BFS_TRY(W.units.alloc(sizeof(int64_t) * (p2 + 1)));              // slot unit bases
-    BFS_TRY(W.xfmt.alloc((size_t)p2));
     W.enc_cps = parallel_encode_chunks(L.nb, 32);                       // 31-bit groups: the most chunks
-    BFS_TRY(W.enc_sums.alloc(parallel_encode_sum_bytes() * p2 * W.enc_cps));
-    BFS_TRY(W.enc_bases.alloc(parallel_encode_base_bytes() * p2 * W.enc_cps));
-    BFS_TRY(W.enc_flags.alloc(p2 * W.enc_cps));
-    BFS_TRY(W.enc_done.alloc(sizeof(unsigned int)));
-    BFS_TRY(W.ctl.alloc(sizeof(LevelCtl)));
-    BFS_CUDA_TRY(cudaMemset(W.enc_done.ptr, 0, sizeof(unsigned int)));
-    BFS_TRY(W.counters.alloc(sizeof(unsigned long long) * C_NUM));
     // pieces: per row, sum over the columns longer than h of ceil(len/h) <= 2 nnz_row/h, most for the smallest h
     std::vector<int64_t> meta(2 * (size_t)p);
     int64_t total = 0;
@@ -1830,10 +1814,27 @@ bfs_status ensure_workspace_once(bfs_graph* g) {
         total += cap;
     }
     W.piece_cap = total;
-    BFS_TRY(W.pieces.alloc(sizeof(Item) * (total > 0 ? total : 1)));
-    // per-level scratch: row_next[p], row_piece_count[p], row_piece_next[p]; row piece bases and caps
-    BFS_TRY(W.level_scratch.alloc(sizeof(unsigned long long) * (3 * p + 1)));
-    BFS_TRY(W.row_meta.alloc(sizeof(int64_t) * 2 * p));
+    const size_t chunks = (size_t)(p2 * W.enc_cps);
+    BFS_TRY(alloc_parts(W.whole, {{&W.pi, (size_t)(4 * W.bm_words)},
+                                  {&W.fa, (size_t)(4 * W.bm_words)},
+                                  {&W.fb, (size_t)(4 * W.bm_words)},
+                                  {&W.fsum, (size_t)W.fsum_len},
+                                  {&W.xbuf, (size_t)xbytes},
+                                  {&W.xcount, sizeof(int64_t) * p2},
+                                  {&W.chunk_base, sizeof(int64_t) * p2 * W.chunks_per_slot},
+                                  {&W.units, sizeof(int64_t) * (p2 + 1)},      // slot unit bases
+                                  {&W.xfmt, (size_t)p2},
+                                  {&W.enc_sums, parallel_encode_sum_bytes() * chunks},
+                                  {&W.enc_bases, parallel_encode_base_bytes() * chunks},
+                                  {&W.enc_flags, chunks},
+                                  {&W.enc_done, sizeof(unsigned int)},
+                                  {&W.ctl, sizeof(LevelCtl)},
+                                  {&W.counters, sizeof(unsigned long long) * C_NUM},
+                                  {&W.pieces, sizeof(Item) * total},
+                                  // per-level scratch: row_next[p], row_piece_count[p], row_piece_next[p]
+                                  {&W.level_scratch, sizeof(unsigned long long) * (3 * p + 1)},
+                                  {&W.row_meta, sizeof(int64_t) * 2 * p}}));   // row piece bases and caps
+    BFS_CUDA_TRY(cudaMemset(W.enc_done.ptr, 0, sizeof(unsigned int)));
     BFS_CUDA_TRY(cudaMemcpy(W.row_meta.ptr, meta.data(), sizeof(int64_t) * 2 * p, cudaMemcpyHostToDevice));
     if (!W.h_counters) {
         void* h = nullptr;
@@ -1876,6 +1877,7 @@ void free_workspace(bfs_graph* g) {
     W.h_counters = nullptr;
     if (W.events) for (auto& e : W.ev) cudaEventDestroy(e);
     W.events = false;
+    W.whole.release();
     W.bm_words = 0;
 }
 

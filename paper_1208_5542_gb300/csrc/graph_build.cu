@@ -7,6 +7,7 @@
 // of those counts gives the block-local column offsets; set counts give the
 // directory V_{i,j} (Eq. 4); a scan of directory popcounts gives the rank of
 // every nonempty column; the entries are then scattered column by column.
+#include <algorithm>
 #include <atomic>
 #include <condition_variable>
 #include <cstdarg>
@@ -72,9 +73,26 @@ bfs_status DevBuf::alloc(size_t nbytes) {
 }
 
 void DevBuf::release() {
-    if (ptr) cudaFree(ptr);
+    if (ptr && !part) cudaFree(ptr);
     ptr = nullptr;
     bytes = 0;
+    part = false;
+}
+
+bfs_status alloc_parts(DevBuf& whole, std::initializer_list<PartSize> parts) {
+    auto padded = [](size_t n) { return (n + 255) / 256 * 256 + 256; };     // parts start 256-byte aligned
+    size_t total = 0;
+    for (const PartSize& p : parts) total += padded(p.bytes);
+    BFS_TRY(whole.alloc(total));
+    char* at = whole.as<char>();
+    for (const PartSize& p : parts) {
+        p.buf->release();
+        p.buf->ptr = at;
+        p.buf->bytes = p.bytes;
+        p.buf->part = true;
+        at += padded(p.bytes);
+    }
+    return BFS_OK;
 }
 
 // ---------------------------------------------------------- call scratch --
@@ -161,6 +179,11 @@ namespace {
 constexpr int kScanThreads = 256;
 constexpr int kScanItems = 16;
 constexpr int64_t kScanTile = (int64_t)kScanThreads * kScanItems;
+// Graphs whose column counts take at most this are built in tuple order: the
+// counts stay in L2 (scale 20 on 8 x 8, 32 MiB of counts: 1.66 ms against 1.95
+// partitioned; scale 21, 64 MiB: 3.37 against 2.87; scale 22 on one block, 16
+// MiB: 4.1 against 4.6; scale 22 on 8 x 8, 128 MiB: 8.3 against 4.6).
+constexpr int64_t kDirectBytes = 48ll << 20;
 
 // Count entries per (block-row of the destination, source) and flag bad ids.
 __global__ void count_entries(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, int64_t m,
@@ -308,13 +331,201 @@ __global__ void scatter_entries(const int32_t* __restrict__ src, const int32_t* 
     }
 }
 
-// Degree of every vertex u: its entries in blocks (i, j(u)), i = 0 .. p-1,
-// saturated at 2^32 - 1 (the rows of the counts, read in order).
-__global__ void vertex_degrees(const uint32_t* __restrict__ cnt, int p, int64_t row_stride, int64_t n,
+// ------------------------------------------------------ partitioned build --
+// Counting and scattering the entries in tuple order costs an L2 reduction and
+// an atomic with its result per entry on random counts, and a random 4-byte
+// store: at 134M entries 1.3 + 5.6 ms, most of it 32-byte sectors moved to and
+// from DRAM for 4 bytes each (with the counts in L2 still 1.1 + 2.2 ms: the
+// rate of L2 atomics).  Larger graphs therefore partition the entries by their
+// block and a part of its source range first (0.7 ms); a bucket's columns are
+// then counted, and its entries placed, by one CTA through counts in shared
+// memory, and the bucket's stores fall into one stretch of the entries.  A
+// partitioned entry is its column's count index, relative to the first
+// block-row of its group, and its destination.
+constexpr int kPartThreads = 512;
+constexpr int kPartTuples = 8;                                  // per thread and tile
+constexpr int kPartTile = kPartThreads * kPartTuples;           // tuples per tile: up to twice the entries
+constexpr int kGroupBuckets = 1024;                             // buckets of one partition pass
+constexpr int kAllBuckets = 16384;                              // buckets of all passes
+constexpr int kColThreads = 1024;
+constexpr int kColWindow = 32768;                               // columns counted together in shared memory
+constexpr int kMaxPartGrid = 32;                                // grids up to 32 x 32 (1024 blocks) are partitioned
+
+struct PartArgs {
+    const int32_t* src;
+    const int32_t* dst;
+    int64_t m;
+    int symmetrize, p;
+    int parts, shift;        // parts of a block's source range, 2^shift sources each
+    uint32_t n, nb;
+};
+
+// Bucket of the entry u -> v, u in range ru, v in range rv.
+__device__ __forceinline__ uint32_t bucket_of(const PartArgs& a, uint32_t u, uint32_t ru, uint32_t rv) {
+    return (rv * (uint32_t)a.p + ru) * (uint32_t)a.parts + ((u - ru * a.nb) >> a.shift);
+}
+
+// Entries per bucket; flags ids outside [0, n).
+__global__ void __launch_bounds__(kPartThreads) bucket_counts(PartArgs a, int buckets, unsigned long long* counts,
+                                                              unsigned long long* err) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    uint32_t* s_cnt = reinterpret_cast<uint32_t*>(smem);
+    for (int b = threadIdx.x; b < buckets; b += kPartThreads) s_cnt[b] = 0;
+    __syncthreads();
+    bool bad = false;
+    // a CTA's tuples are below 2^31 for any grid of a CTA or more per SM
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < a.m; e += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t u = (uint32_t)a.src[e], v = (uint32_t)a.dst[e];
+        if (u >= a.n || v >= a.n) {
+            bad = true;
+            continue;
+        }
+        const uint32_t ru = u / a.nb, rv = v / a.nb;
+        atomicAdd(s_cnt + bucket_of(a, u, ru, rv), 1u);
+        if (a.symmetrize) atomicAdd(s_cnt + bucket_of(a, v, rv, ru), 1u);
+    }
+    if (bad) atomicOr(err, 1ull);
+    __syncthreads();
+    for (int b = threadIdx.x; b < buckets; b += kPartThreads)
+        if (s_cnt[b]) atomicAdd(counts + b, (unsigned long long)s_cnt[b]);
+}
+
+// The entries of block-rows [r0, r1) into their buckets (b0: the first of
+// them): a tile's entries are ranked per bucket in shared memory, every bucket
+// takes its space with one atomic, and the tile is written out bucket by
+// bucket from a sorted copy.
+__global__ void __launch_bounds__(kPartThreads) partition_entries(PartArgs a, int r0, int r1, uint32_t b0,
+                                                                  unsigned long long* __restrict__ cursor,
+                                                                  uint2* __restrict__ out) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    uint2* s_pair = reinterpret_cast<uint2*>(smem);                                   // 2 * kPartTile
+    unsigned long long* s_base = reinterpret_cast<unsigned long long*>(s_pair + 2 * kPartTile);
+    uint32_t* s_off = reinterpret_cast<uint32_t*>(s_base + kGroupBuckets);            // counts, then offsets
+    uint16_t* s_bkt = reinterpret_cast<uint16_t*>(s_off + kGroupBuckets);             // 2 * kPartTile
+    __shared__ uint32_t s_scan[kPartThreads / 32 + 1];
+    const uint32_t stride = (uint32_t)a.p * a.nb;
+    const int64_t ntiles = (a.m + kPartTile - 1) / kPartTile;
+    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+        s_off[2 * threadIdx.x] = 0;
+        s_off[2 * threadIdx.x + 1] = 0;
+        __syncthreads();
+        uint32_t u[kPartTuples], v[kPartTuples], bk[2 * kPartTuples], rk[2 * kPartTuples];
+#pragma unroll
+        for (int k = 0; k < kPartTuples; ++k) {
+            const int64_t e = t * kPartTile + k * kPartThreads + threadIdx.x;
+            u[k] = e < a.m ? (uint32_t)a.src[e] : 0u;
+            v[k] = e < a.m ? (uint32_t)a.dst[e] : 0u;
+        }
+#pragma unroll
+        for (int k = 0; k < kPartTuples; ++k) {
+            const bool in = t * kPartTile + k * kPartThreads + threadIdx.x < a.m;
+            const uint32_t ru = u[k] / a.nb, rv = v[k] / a.nb;
+            bk[2 * k] = (in && (int)rv >= r0 && (int)rv < r1) ? bucket_of(a, u[k], ru, rv) - b0 : ~0u;
+            bk[2 * k + 1] = (in && a.symmetrize && (int)ru >= r0 && (int)ru < r1) ? bucket_of(a, v[k], rv, ru) - b0 : ~0u;
+            rk[2 * k] = bk[2 * k] != ~0u ? atomicAdd(s_off + bk[2 * k], 1u) : 0u;
+            rk[2 * k + 1] = bk[2 * k + 1] != ~0u ? atomicAdd(s_off + bk[2 * k + 1], 1u) : 0u;
+        }
+        __syncthreads();
+        // space for every bucket's entries, and their places in the sorted copy
+        const uint32_t c0 = s_off[2 * threadIdx.x], c1 = s_off[2 * threadIdx.x + 1];
+        uint32_t total;
+        const uint32_t excl = block_excl_scan<kPartThreads>(c0 + c1, 0u, OpSum(), s_scan, &total);
+        s_off[2 * threadIdx.x] = excl;
+        s_off[2 * threadIdx.x + 1] = excl + c0;
+        if (c0) s_base[2 * threadIdx.x] = atomicAdd(cursor + 2 * threadIdx.x, (unsigned long long)c0) - excl;
+        if (c1) s_base[2 * threadIdx.x + 1] = atomicAdd(cursor + 2 * threadIdx.x + 1, (unsigned long long)c1) - (excl + c0);
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < kPartTuples; ++k) {
+            // the column's count index: block-row (relative to the group's first) x p*nb + source
+            if (bk[2 * k] != ~0u) {
+                const uint32_t at = s_off[bk[2 * k]] + rk[2 * k];
+                s_pair[at] = make_uint2((v[k] / a.nb - (uint32_t)r0) * stride + u[k], v[k]);
+                s_bkt[at] = (uint16_t)bk[2 * k];
+            }
+            if (bk[2 * k + 1] != ~0u) {
+                const uint32_t at = s_off[bk[2 * k + 1]] + rk[2 * k + 1];
+                s_pair[at] = make_uint2((u[k] / a.nb - (uint32_t)r0) * stride + v[k], u[k]);
+                s_bkt[at] = (uint16_t)bk[2 * k + 1];
+            }
+        }
+        __syncthreads();
+        for (uint32_t q = threadIdx.x; q < total; q += kPartThreads) out[s_base[s_bkt[q]] + q] = s_pair[q];
+        __syncthreads();
+    }
+}
+
+constexpr size_t kPartSmem = sizeof(uint2) * 2 * kPartTile + (sizeof(uint32_t) + sizeof(unsigned long long)) * kGroupBuckets +
+                             sizeof(uint16_t) * 2 * kPartTile;
+static_assert(kGroupBuckets == 2 * kPartThreads, "a thread scans two buckets");
+
+// One CTA per bucket of a group, kColWindow of its columns at a time (a bucket
+// with more columns reads its entries again, from L2).
+//   COUNT: the entries of every column, written to cnt (the group's counts).
+//   else:  every entry into its column (order inside a column is arbitrary);
+//          off holds the columns' offsets in their blocks, ir_base the blocks'.
+template <bool COUNT>
+__global__ void __launch_bounds__(kColThreads) bucket_columns(PartArgs a, const uint2* __restrict__ pairs,
+                                                              const int64_t* __restrict__ starts, int buckets,
+                                                              uint32_t* __restrict__ cnt,
+                                                              const int64_t* __restrict__ ir_base,
+                                                              int32_t* __restrict__ ir) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    uint32_t* s_col = reinterpret_cast<uint32_t*>(smem);
+    constexpr int K = 4;
+    for (int bkt = blockIdx.x; bkt < buckets; bkt += gridDim.x) {
+        const uint32_t block = (uint32_t)bkt / (uint32_t)a.parts, part = (uint32_t)bkt % (uint32_t)a.parts;
+        const uint32_t first = part << a.shift;
+        const uint32_t cols = first < a.nb ? min(1u << a.shift, a.nb - first) : 0u;
+        const int64_t e0 = starts[bkt], e1 = starts[bkt + 1];
+        for (uint32_t w0 = 0; w0 < cols; w0 += kColWindow) {
+            const uint32_t wn = min((uint32_t)kColWindow, cols - w0);
+            const uint32_t c0 = block * a.nb + first + w0;         // count index of the window's first column
+            uint32_t* g = cnt + c0;
+            for (uint32_t c = threadIdx.x; c < wn; c += kColThreads) s_col[c] = COUNT ? 0u : g[c];
+            __syncthreads();
+            int32_t* out = COUNT ? nullptr : ir + ir_base[block];
+            for (int64_t e = e0 + threadIdx.x; e < e1; e += K * kColThreads) {
+                uint2 x[K];
+#pragma unroll
+                for (int k = 0; k < K; ++k) x[k] = e + k * kColThreads < e1 ? pairs[e + k * kColThreads] : make_uint2(~0u, 0u);
+#pragma unroll
+                for (int k = 0; k < K; ++k) {
+                    if (e + k * kColThreads >= e1 || x[k].x - c0 >= wn) continue;
+                    const uint32_t pos = atomicAdd(s_col + (x[k].x - c0), 1u);
+                    if (!COUNT) out[pos] = (int32_t)x[k].y;
+                }
+            }
+            __syncthreads();
+            if (COUNT)
+                for (uint32_t c = threadIdx.x; c < wn; c += kColThreads) g[c] = s_col[c];
+            __syncthreads();
+        }
+    }
+}
+
+// The parts of a block's source range: as many as give kColWindow columns
+// each, on all blocks at most kAllBuckets and in a block-row at most kGroupBuckets.
+void choose_parts(PartArgs& a) {
+    const int64_t nblocks = (int64_t)a.p * a.p;
+    a.shift = 31;
+    while (a.shift > 0 && (1ll << (a.shift - 1)) >= (int64_t)a.nb) --a.shift;
+    a.parts = 1;
+    while (a.shift > 0 && (1ll << a.shift) > kColWindow) {
+        const int64_t more = ((int64_t)a.nb + (1ll << (a.shift - 1)) - 1) >> (a.shift - 1);
+        if (nblocks * more > kAllBuckets || a.p * more > kGroupBuckets) break;
+        a.parts = (int)more;
+        --a.shift;
+    }
+}
+
+// Degree of every vertex u: its entries in the blocks of `rows` block-rows (the
+// rows of the counts, read in order), added to deg, saturated at 2^32 - 1.
+__global__ void vertex_degrees(const uint32_t* __restrict__ cnt, int rows, int64_t row_stride, int64_t n,
                                uint32_t* __restrict__ deg) {
     for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < n; u += (int64_t)gridDim.x * blockDim.x) {
-        uint64_t d = 0;
-        for (int i = 0; i < p; ++i) d += cnt[i * row_stride + u];
+        uint64_t d = deg[u];
+        for (int i = 0; i < rows; ++i) d += cnt[i * row_stride + u];
         deg[u] = d > 0xffffffffull ? 0xffffffffu : (uint32_t)d;
     }
 }
@@ -421,9 +632,9 @@ int grid_for(int64_t work, int threads) {
 bfs_status segmented_scan(uint32_t* a, int64_t nseg, int64_t seg_len, int64_t seg_stride,
                           std::vector<uint64_t>& totals, cudaStream_t st) {
     const int64_t tiles_per_seg = seg_len > 0 ? (seg_len + kScanTile - 1) / kScanTile : 1;
-    DevBuf tile_sum, seg_total;
-    BFS_TRY(tile_sum.alloc(sizeof(unsigned long long) * nseg * tiles_per_seg));
-    BFS_TRY(seg_total.alloc(sizeof(unsigned long long) * nseg));
+    Scratch tile_sum, seg_total;
+    BFS_TRY(tile_sum.alloc(sizeof(unsigned long long) * nseg * tiles_per_seg, st));
+    BFS_TRY(seg_total.alloc(sizeof(unsigned long long) * nseg, st));
     const int64_t ntiles = nseg * tiles_per_seg;
     if (ntiles > 0x7fffffffLL) return set_error(BFS_ERR_INVALID_ARG, "graph too large for the layout scan");
     scan_tile_sums<<<(unsigned)ntiles, kScanThreads, 0, st>>>(a, nseg, seg_len, seg_stride, tiles_per_seg,
@@ -460,37 +671,121 @@ bfs_status build_layout(bfs_graph* g, int64_t n, int64_t m, const int32_t* d_src
     const int64_t words_per_block = (nb + 31) / 32;
     L.dir_stride = ((words_per_block + 3 + 3) / 4) * 4;   // >= 3 words of padding, 16-byte rows
 
-    DevBuf cnt, err;
+    const bool partitioned = p <= kMaxPartGrid && 4 * nblocks * nb > kDirectBytes;
+    PartArgs pa{d_src, d_dst, m, symmetrize, p, 1, 31, (uint32_t)n, (uint32_t)nb};
+    if (partitioned) choose_parts(pa);
+    const int buckets = (int)nblocks * pa.parts, per_row = p * pa.parts;
+    DevBuf cnt, pairs;
+    Scratch err, cursor, starts;
     BFS_TRY(cnt.alloc(sizeof(uint32_t) * nblocks * nb));
-    BFS_TRY(err.alloc(sizeof(unsigned long long)));
-    BFS_CUDA_TRY(cudaMemsetAsync(cnt.ptr, 0, cnt.bytes, st));
-    BFS_CUDA_TRY(cudaMemsetAsync(err.ptr, 0, err.bytes, st));
-    count_entries<<<grid_for(m, 256), 256, 0, st>>>(d_src, d_dst, m, symmetrize, n, nb, row_stride,
-                                                    cnt.as<uint32_t>(), err.as<unsigned long long>());
+    BFS_TRY(err.alloc(sizeof(unsigned long long), st));
+    BFS_CUDA_TRY(cudaMemsetAsync(err.ptr, 0, sizeof(unsigned long long), st));
+    std::vector<uint64_t> held(partitioned ? buckets : 0);             // entries per bucket
+    if (partitioned) {
+        const size_t cursor_bytes = sizeof(unsigned long long) * std::max(buckets, kGroupBuckets);
+        BFS_TRY(cursor.alloc(cursor_bytes, st));
+        BFS_CUDA_TRY(cudaMemsetAsync(cursor.ptr, 0, cursor_bytes, st));
+        const size_t smem = sizeof(uint32_t) * (size_t)buckets;
+        BFS_CUDA_TRY(cudaFuncSetAttribute(bucket_counts, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)(sizeof(uint32_t) * kAllBuckets)));
+        bucket_counts<<<152 * 3, kPartThreads, smem, st>>>(pa, buckets, cursor.as<unsigned long long>(),
+                                                           err.as<unsigned long long>());
+    } else {
+        BFS_CUDA_TRY(cudaMemsetAsync(cnt.ptr, 0, cnt.bytes, st));
+        count_entries<<<grid_for(m, 256), 256, 0, st>>>(d_src, d_dst, m, symmetrize, n, nb, row_stride,
+                                                        cnt.as<uint32_t>(), err.as<unsigned long long>());
+    }
     BFS_CUDA_TRY(cudaGetLastError());
     unsigned long long h_err = 0;
     BFS_CUDA_TRY(cudaMemcpyAsync(&h_err, err.ptr, sizeof(h_err), cudaMemcpyDeviceToHost, st));
+    if (partitioned)
+        BFS_CUDA_TRY(cudaMemcpyAsync(held.data(), cursor.ptr, sizeof(uint64_t) * buckets, cudaMemcpyDeviceToHost, st));
     BFS_CUDA_TRY(cudaStreamSynchronize(st));
     if (h_err) return set_error(BFS_ERR_INVALID_ARG, "an edge names a vertex outside [0, %lld)", (long long)n);
 
-    BFS_TRY(L.deg.alloc(sizeof(uint32_t) * n));
-    vertex_degrees<<<grid_for(n, 256), 256, 0, st>>>(cnt.as<uint32_t>(), p, row_stride, n, L.deg.as<uint32_t>());
-    BFS_CUDA_TRY(cudaGetLastError());
-
-    // directory + popcounts
-    BFS_TRY(L.dir.alloc(sizeof(uint32_t) * nblocks * L.dir_stride));
-    BFS_TRY(L.rank.alloc(sizeof(uint32_t) * nblocks * L.dir_stride));
+    BFS_TRY(alloc_parts(L.small, {{&L.dir, sizeof(uint32_t) * nblocks * L.dir_stride},
+                                  {&L.rank, sizeof(uint32_t) * nblocks * L.dir_stride},
+                                  {&L.deg, sizeof(uint32_t) * n},
+                                  {&L.cp_base_d, sizeof(int64_t) * nblocks},
+                                  {&L.ir_base_d, sizeof(int64_t) * nblocks}}));
+    BFS_TRY(L.ir.alloc(sizeof(int32_t) * (L.nnz > 0 ? L.nnz : 1)));
     BFS_CUDA_TRY(cudaMemsetAsync(L.dir.ptr, 0, L.dir.bytes, st));
     BFS_CUDA_TRY(cudaMemsetAsync(L.rank.ptr, 0, L.rank.bytes, st));
-    directory_words<<<grid_for(nblocks * words_per_block * 32, 256), 256, 0, st>>>(
-        cnt.as<uint32_t>(), nblocks, nb, words_per_block, L.dir_stride, L.dir.as<uint32_t>(), L.rank.as<uint32_t>());
-    BFS_CUDA_TRY(cudaGetLastError());
+    BFS_CUDA_TRY(cudaMemsetAsync(L.deg.ptr, 0, L.deg.bytes, st));
+
+    // block-rows [r0, r1) counted: their degrees, directory and popcounts; then
+    // the counts become block-local column offsets (an exclusive scan per block)
+    std::vector<uint64_t> nnzc_b, nnz_b;
+    auto counted = [&](int r0, int r1) -> bfs_status {
+        uint32_t* c = cnt.as<uint32_t>() + r0 * row_stride;
+        const int64_t blocks = (int64_t)(r1 - r0) * p, b0 = (int64_t)r0 * p;
+        vertex_degrees<<<grid_for(n, 256), 256, 0, st>>>(c, r1 - r0, row_stride, n, L.deg.as<uint32_t>());
+        directory_words<<<grid_for(blocks * words_per_block * 32, 256), 256, 0, st>>>(
+            c, blocks, nb, words_per_block, L.dir_stride, L.dir.as<uint32_t>() + b0 * L.dir_stride,
+            L.rank.as<uint32_t>() + b0 * L.dir_stride);
+        BFS_CUDA_TRY(cudaGetLastError());
+        std::vector<uint64_t> totals;
+        BFS_TRY(segmented_scan(c, blocks, nb, nb, totals, st));
+        nnz_b.insert(nnz_b.end(), totals.begin(), totals.end());
+        return BFS_OK;
+    };
+
+    if (!partitioned) {
+        BFS_TRY(counted(0, p));
+    } else {
+        // groups of block-rows: at most kGroupBuckets buckets, and entries that fit the
+        // partition buffer (an eighth of all entries, at least 1 GiB); every group
+        // reads all tuples once
+        struct Group { int r0, r1; int64_t entries; };
+        std::vector<Group> groups;
+        const int64_t room = std::max<int64_t>(L.nnz / 8, (1ll << 30) / (int64_t)sizeof(uint2));
+        int64_t most = 1;
+        for (int r = 0; r < p; ++r) {
+            int64_t row = 0;
+            for (int k = 0; k < per_row; ++k) row += (int64_t)held[(size_t)r * per_row + k];
+            if (groups.empty() || groups.back().entries + row > room ||
+                (r + 1 - groups.back().r0) * per_row > kGroupBuckets ||
+                (int64_t)(r + 1 - groups.back().r0) * row_stride > 0xffffffffll)
+                groups.push_back({r, r + 1, row});
+            else
+                groups.back() = {groups.back().r0, r + 1, groups.back().entries + row};
+            most = std::max(most, groups.back().entries);
+        }
+        BFS_TRY(pairs.alloc(sizeof(uint2) * (size_t)most));
+        BFS_TRY(starts.alloc(sizeof(int64_t) * (kGroupBuckets + 1 + (size_t)nblocks), st));
+        std::vector<int64_t> base((size_t)nblocks, 0);                  // first entry of every block
+        for (int64_t b = 0, at = 0; b < nblocks; ++b) {
+            base[b] = at;
+            for (int k = 0; k < pa.parts; ++k) at += (int64_t)held[(size_t)b * pa.parts + k];
+        }
+        int64_t* d_base = starts.as<int64_t>() + kGroupBuckets + 1;
+        BFS_CUDA_TRY(cudaMemcpyAsync(d_base, base.data(), sizeof(int64_t) * nblocks, cudaMemcpyHostToDevice, st));
+        const int col_smem = (int)sizeof(uint32_t) * (int)std::min<int64_t>(kColWindow, nb);
+        BFS_CUDA_TRY(cudaFuncSetAttribute(partition_entries, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPartSmem));
+        for (auto k : {bucket_columns<true>, bucket_columns<false>})
+            BFS_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)sizeof(uint32_t) * kColWindow));
+        for (const Group& g : groups) {
+            const int b0 = g.r0 * per_row, nbk = (g.r1 - g.r0) * per_row;
+            std::vector<int64_t> at((size_t)nbk + 1, 0);
+            for (int k = 0; k < nbk; ++k) at[k + 1] = at[k] + (int64_t)held[(size_t)b0 + k];
+            BFS_CUDA_TRY(cudaMemcpyAsync(starts.ptr, at.data(), sizeof(int64_t) * (nbk + 1), cudaMemcpyHostToDevice, st));
+            BFS_CUDA_TRY(cudaMemcpyAsync(cursor.ptr, starts.ptr, sizeof(int64_t) * nbk, cudaMemcpyDeviceToDevice, st));
+            partition_entries<<<152 * 2, kPartThreads, kPartSmem, st>>>(pa, g.r0, g.r1, (uint32_t)b0,
+                                                                        cursor.as<unsigned long long>(), pairs.as<uint2>());
+            uint32_t* c = cnt.as<uint32_t>() + g.r0 * row_stride;
+            bucket_columns<true><<<152, kColThreads, col_smem, st>>>(pa, pairs.as<uint2>(), starts.as<int64_t>(), nbk, c,
+                                                                     nullptr, nullptr);
+            BFS_CUDA_TRY(cudaGetLastError());
+            BFS_TRY(counted(g.r0, g.r1));                                // synchronises: `at` is free to go
+            bucket_columns<false><<<152, kColThreads, col_smem, st>>>(pa, pairs.as<uint2>(), starts.as<int64_t>(), nbk, c,
+                                                                      d_base + (int64_t)g.r0 * p, L.ir.as<int32_t>());
+            BFS_CUDA_TRY(cudaGetLastError());
+        }
+    }
 
     // rank = exclusive scan of popcounts per block; nnzc_b = totals
-    std::vector<uint64_t> nnzc_b, nnz_b;
     BFS_TRY(segmented_scan(L.rank.as<uint32_t>(), nblocks, L.dir_stride, L.dir_stride, nnzc_b, st));
-    // block-local column offsets = exclusive scan of counts per block; nnz_b = totals
-    BFS_TRY(segmented_scan(cnt.as<uint32_t>(), nblocks, nb, nb, nnz_b, st));
 
     L.cp_base.assign(nblocks, 0);
     L.ir_base.assign(nblocks, 0);
@@ -509,12 +804,9 @@ bfs_status build_layout(bfs_graph* g, int64_t n, int64_t m, const int32_t* d_src
     if (irt != L.nnz) return set_error(BFS_ERR_CUDA, "layout build lost entries (%lld of %lld)", (long long)irt, (long long)L.nnz);
 
     BFS_TRY(L.cp.alloc(sizeof(uint32_t) * (cpt > 0 ? cpt : 1)));
-    BFS_TRY(L.ir.alloc(sizeof(int32_t) * (L.nnz > 0 ? L.nnz : 1)));
-    BFS_TRY(L.cp_base_d.alloc(sizeof(int64_t) * nblocks));
-    BFS_TRY(L.ir_base_d.alloc(sizeof(int64_t) * nblocks));
-    DevBuf d_nnz_b, d_nnzc_b;
-    BFS_TRY(d_nnz_b.alloc(sizeof(uint64_t) * nblocks));
-    BFS_TRY(d_nnzc_b.alloc(sizeof(uint64_t) * nblocks));
+    Scratch d_nnz_b, d_nnzc_b;
+    BFS_TRY(d_nnz_b.alloc(sizeof(uint64_t) * nblocks, st));
+    BFS_TRY(d_nnzc_b.alloc(sizeof(uint64_t) * nblocks, st));
     BFS_CUDA_TRY(cudaMemcpyAsync(L.cp_base_d.ptr, L.cp_base.data(), sizeof(int64_t) * nblocks, cudaMemcpyHostToDevice, st));
     BFS_CUDA_TRY(cudaMemcpyAsync(L.ir_base_d.ptr, L.ir_base.data(), sizeof(int64_t) * nblocks, cudaMemcpyHostToDevice, st));
     BFS_CUDA_TRY(cudaMemcpyAsync(d_nnz_b.ptr, nnz_b.data(), sizeof(uint64_t) * nblocks, cudaMemcpyHostToDevice, st));
@@ -525,8 +817,9 @@ bfs_status build_layout(bfs_graph* g, int64_t n, int64_t m, const int32_t* d_src
         L.cp_base_d.as<int64_t>(), d_nnz_b.as<unsigned long long>(), d_nnzc_b.as<unsigned long long>(),
         L.cp.as<uint32_t>());
     BFS_CUDA_TRY(cudaGetLastError());
-    scatter_entries<<<grid_for(m, 256), 256, 0, st>>>(d_src, d_dst, m, symmetrize, nb, p, row_stride,
-                                                      cnt.as<uint32_t>(), L.ir_base_d.as<int64_t>(), L.ir.as<int32_t>());
+    if (!partitioned)
+        scatter_entries<<<grid_for(m, 256), 256, 0, st>>>(d_src, d_dst, m, symmetrize, nb, p, row_stride,
+                                                          cnt.as<uint32_t>(), L.ir_base_d.as<int64_t>(), L.ir.as<int32_t>());
     BFS_CUDA_TRY(cudaGetLastError());
     BFS_CUDA_TRY(cudaStreamSynchronize(st));
     return BFS_OK;

@@ -5,6 +5,7 @@
 #include <atomic>
 #include <cstdint>
 #include <cstdio>
+#include <initializer_list>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -37,10 +38,12 @@ bfs_status cuda_error(cudaError_t e, const char* what, const char* file, int lin
 bool is_device_pointer(const void* p);
 
 // ---------------------------------------------------------- device arrays --
-// Owning device buffer (cudaMalloc / cudaFree).
+// Owning device buffer (cudaMalloc / cudaFree), or a part of another one
+// (alloc_parts), which release() only forgets.
 struct DevBuf {
     void* ptr = nullptr;
     size_t bytes = 0;
+    bool part = false;
     DevBuf() = default;
     DevBuf(const DevBuf&) = delete;
     DevBuf& operator=(const DevBuf&) = delete;
@@ -50,7 +53,16 @@ struct DevBuf {
     template <typename T> T* as() const { return static_cast<T*>(ptr); }
 };
 
-// Scratch of one codec call: stream-ordered memory of the library's own pool
+// Buffers that live and die together as parts of one allocation, `whole` (a
+// call to the device's allocator costs 30-40 us each way, and a graph has
+// some thirty small buffers).
+struct PartSize {
+    DevBuf* buf;
+    size_t bytes;
+};
+bfs_status alloc_parts(DevBuf& whole, std::initializer_list<PartSize> parts);
+
+// Scratch of one call: stream-ordered memory of the library's own pool
 // of the device, which keeps at most kScratchKept bytes between calls (the
 // rest goes back to the device at the next synchronisation).  The pool's
 // allocations are ordered on the call's stream, so calls on several streams
@@ -98,6 +110,7 @@ struct Layout {
     int64_t nnz = 0;        // directed entries
     int64_t dir_stride = 0; // uint32 words per block directory (padded)
     int64_t nnzc_total = 0; // nonempty columns over all blocks
+    DevBuf small;           // the allocation that holds dir, rank, deg, cp_base_d and ir_base_d
     DevBuf dir, rank, cp, ir, cp_base_d, ir_base_d;
     DevBuf deg;             // entries per source vertex (uint32, saturated)
     DevBuf iso;             // bitmap of the vertices without entries (bottom-up levels mark them visited)
@@ -156,6 +169,7 @@ struct Workspace {
     int slots = 0;              // exchange slots of the current mode
     int wah_bits = 0;
     int mode = -1;
+    DevBuf whole;               // the allocation that holds what every search needs
     DevBuf pi, fa, fb, fsum, xbuf, xcount, chunk_base, units, counters, pieces;
     DevBuf level_scratch;       // per-level work counters (3 per row)
     DevBuf row_meta;            // per-row piece bases and capacities
