@@ -83,6 +83,7 @@ struct LevelCtl {
     int32_t bu;            // 1: this level runs bottom-up
     int32_t policy;        // BFS_DIRECTION_*
     int32_t alpha, beta;   // thresholds of the hybrid
+    unsigned int done;     // CTAs of reduce_level that have finished
 };
 
 struct LevelArgs {
@@ -1507,67 +1508,24 @@ __global__ void __launch_bounds__(kNT) expand_bottom_up(LevelArgs a) {
 }
 
 // ---------------------------------------------------------------- reduce --
-// x = t & ~pi; pi |= x; level of the new vertices; |x|; the next frontier f = x
-// and t cleared for the next level; frontier summary of x.
-__global__ void __launch_bounds__(kNT) reduce_level(uint32_t* __restrict__ t, uint32_t* __restrict__ pi,
-                                                    uint32_t* __restrict__ f, uint8_t* __restrict__ fsum,
-                                                    int64_t words, int64_t n, int32_t* __restrict__ level,
-                                                    const LevelCtl* __restrict__ ctl, unsigned long long* ctr,
-                                                    const uint32_t* __restrict__ deg) {
-    const int32_t next_level = ctl->level + 1;
-    const int64_t nwarps = (words + 31) / 32;
-    const int64_t gw0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t gstride = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t gw = gw0; gw < nwarps; gw += gstride) {
-        const int64_t w = gw * 32 + lane_id();
-        uint32_t x = 0;
-        unsigned long long dsum = 0;
-        if (w < words) {
-            const uint32_t pw = pi[w];
-            x = t[w] & ~pw;
-            if (x) pi[w] = pw | x;
-            f[w] = x;
-            t[w] = 0u;
-        }
-        const uint32_t any = __ballot_sync(0xffffffffu, x != 0u);
-        // the levels (and degrees) of the fresh vertices, one word at a time
-        // by the whole warp: lane l takes bit l (coalesced stores and loads)
-        for (uint32_t m = any; m;) {
-            uint32_t d[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {               // four words' degree loads in flight
-                const int k = m ? __ffs(m) - 1 : 0;
-                const uint32_t xk = m ? __shfl_sync(0xffffffffu, x, k) : 0u;
-                m &= m - 1;
-                const int64_t v = (gw * 32 + k) * 32 + lane_id();
-                const bool fresh = ((xk >> lane_id()) & 1u) && v < n;
-                if (fresh) level[v] = next_level;
-                d[q] = fresh ? __ldg(deg + v) : 0u;
-            }
-            dsum += (unsigned long long)d[0] + d[1] + d[2] + d[3];
-        }
-        const int cnt = warp_sum(__popc(x));
-        dsum = warp_sum(dsum);
-        if (lane_id() == 0) {
-            fsum[gw] = any ? 1 : 0;
-            if (cnt) atomicAdd(ctr + C_NEXT_COUNT, (unsigned long long)cnt);
-            if (dsum) atomicAdd(ctr + C_NEXT_DEGREE, dsum);
-        }
-    }
-}
+// The values of the next level, and whether it runs (the frontier is not
+// empty, no invariant failed, fewer than max_levels levels).  In a CUDA graph
+// the decision drives the conditional WHILE node.
+struct NextArgs {
+    int64_t n;
+    int32_t max_levels;
+    cudaGraphConditionalHandle handle;
+    int use_handle;                 // the graph-launched loop: also clear the counters for the next level
+    unsigned long long* lvl;        // row hand-out counters, nlvl of them
+    int nlvl;
+};
 
-// One thread: the values of the next level, and whether it runs (the
-// frontier is not empty, no invariant failed, fewer than max_levels levels).
-// In a CUDA graph the decision drives the conditional WHILE node.
-// In the graph-launched loop (use_handle) it also clears the per-level
-// counters and the row hand-out counters (lvl, nlvl of them) for the next
-// level, in place of memset nodes; the stepwise loop reads them first and
-// clears them itself.
-__global__ void level_next(LevelCtl* c, unsigned long long* ctr, int64_t n, int32_t max_levels,
-                           cudaGraphConditionalHandle handle, int use_handle, unsigned long long* lvl, int nlvl) {
-    const int64_t f = (int64_t)ctr[C_NEXT_COUNT];
+// One thread; the counters of the level are complete.
+__device__ void level_next(LevelCtl* c, unsigned long long* ctr, const NextArgs& nx) {
+    const int64_t n = nx.n;
+    const int64_t f = (int64_t)__ldcg(ctr + C_NEXT_COUNT);
     const int64_t prev = c->frontier;
-    const int64_t mf = (int64_t)ctr[C_NEXT_DEGREE];
+    const int64_t mf = (int64_t)__ldcg(ctr + C_NEXT_DEGREE);
     c->m_u -= mf;
     c->m_f = mf;
     // direction of the next level (Beamer et al.): bottom-up once the growing
@@ -1591,14 +1549,99 @@ __global__ void level_next(LevelCtl* c, unsigned long long* ctr, int64_t n, int3
     // most of those visits into one L2 read instead of two atomics.  With the
     // next bits in the window the bit is a shared-memory atomic: not worth it.
     c->dedup = (c->visited * 16 < n) ? 1 : 0;
-    const int go = (f > 0 && ctr[C_ERROR] == 0 && c->level < max_levels) ? 1 : 0;
+    const int go = (f > 0 && __ldcg(ctr + C_ERROR) == 0 && c->level < nx.max_levels) ? 1 : 0;
     c->go = go;
-    if (use_handle) {
-        for (int k = 0; k < C_ERROR; ++k) ctr[k] = 0ull;          // the error flag and trace cursors stay
-        for (int k = C_WAH_WORDS; k < C_NUM; ++k) ctr[k] = 0ull;
-        for (int k = 0; k < nlvl; ++k) lvl[k] = 0ull;
-        cudaGraphSetConditional(handle, go ? 1u : 0u);
+    if (nx.use_handle) cudaGraphSetConditional(nx.handle, go ? 1u : 0u);
+}
+
+// x = t & ~pi; pi |= x; level of the new vertices; |x| and its degree sum; the
+// next frontier f = x and t cleared for the next level; frontier summary of x.
+// A warp takes WPW words: 32, so that the bitmaps are read and written in whole
+// lines, or 4 on small graphs (below kSmallReduce vertices), where the chain of
+// a word's level stores and degree loads, one word after the other, is the
+// kernel's time (4,096 vertices: 128 words on 4 warps took 9 us).
+// The last CTA to finish (a counter, no waiting) sets up the next level.
+// In the graph-launched loop it also clears the per-level counters and the
+// row hand-out counters, in place of memset nodes; the stepwise loop reads them
+// first and clears them itself.
+constexpr int64_t kSmallReduce = 1 << 20;
+
+template <int WPW>
+__global__ void __launch_bounds__(kNT) reduce_level(uint32_t* __restrict__ t, uint32_t* __restrict__ pi,
+                                                    uint32_t* __restrict__ f, uint8_t* __restrict__ fsum,
+                                                    int64_t words, int64_t n, int32_t* __restrict__ level,
+                                                    LevelCtl* ctl, unsigned long long* ctr,
+                                                    const uint32_t* __restrict__ deg, NextArgs nx) {
+    constexpr int W = kNT / 32;                         // warps
+    __shared__ unsigned long long s_sum[2][W];
+    __shared__ int s_last;
+    const int32_t next_level = ctl->level + 1;
+    const int lane = (int)lane_id(), warp = (int)(threadIdx.x >> 5);
+    const int64_t per_cta = (int64_t)W * WPW;
+    unsigned long long cnt = 0, dsum = 0;
+    for (int64_t w0 = blockIdx.x * per_cta; w0 < words; w0 += gridDim.x * per_cta) {
+        const int64_t wb = w0 + (int64_t)warp * WPW, w = wb + lane;
+        uint32_t x = 0;
+        if (lane < WPW && w < words) {
+            const uint32_t pw = pi[w];
+            x = t[w] & ~pw;
+            if (x) pi[w] = pw | x;
+            f[w] = x;
+            t[w] = 0u;
+            cnt += __popc(x);
+        }
+        const uint32_t any = __ballot_sync(0xffffffffu, x != 0u);
+        // the levels (and degrees) of the fresh vertices, one word at a time
+        // by the whole warp: lane l takes bit l (coalesced stores and loads)
+        for (uint32_t m = any; m;) {
+            uint32_t d[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {               // four words' degree loads in flight
+                const int k = m ? __ffs(m) - 1 : 0;
+                const uint32_t xk = m ? __shfl_sync(0xffffffffu, x, k) : 0u;
+                m &= m - 1;
+                const int64_t v = (wb + k) * 32 + lane;
+                const bool fresh = ((xk >> lane) & 1u) && v < n;
+                if (fresh) level[v] = next_level;
+                d[q] = fresh ? __ldg(deg + v) : 0u;
+            }
+            dsum += (unsigned long long)d[0] + d[1] + d[2] + d[3];
+        }
+        if (WPW == 32) {
+            if (lane == 0) fsum[wb >> 5] = any ? 1 : 0;
+        } else {                                        // the CTA's words are one byte of the summary
+            const int some = __syncthreads_or(any != 0u);
+            if (threadIdx.x == 0) fsum[w0 >> 5] = some ? 1 : 0;
+        }
     }
+    static_assert(WPW == 32 || W * WPW == 32, "a warp or a CTA covers one byte of the frontier summary");
+    cnt = warp_sum(cnt);
+    dsum = warp_sum(dsum);
+    if (lane == 0) {
+        s_sum[0][warp] = cnt;
+        s_sum[1][warp] = dsum;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int k = 1; k < W; ++k) {
+            cnt += s_sum[0][k];
+            dsum += s_sum[1][k];
+        }
+        if (cnt) atomicAdd(ctr + C_NEXT_COUNT, cnt);
+        if (dsum) atomicAdd(ctr + C_NEXT_DEGREE, dsum);
+        __threadfence();
+        s_last = atomicAdd(&ctl->done, 1u) == gridDim.x - 1;
+        if (s_last) {
+            __threadfence();
+            ctl->done = 0u;
+            level_next(ctl, ctr, nx);
+        }
+    }
+    __syncthreads();
+    if (!s_last || !nx.use_handle) return;
+    for (int k = threadIdx.x; k < C_NUM; k += kNT)
+        if (k < C_ERROR || k >= C_WAH_WORDS) ctr[k] = 0ull;          // the error flag and trace cursors stay
+    for (int k = threadIdx.x; k < nx.nlvl; k += kNT) nx.lvl[k] = 0ull;
 }
 
 __global__ void level_first(LevelCtl* c, int64_t n, int win_ratio, int policy, int alpha, int beta,
@@ -1606,6 +1649,7 @@ __global__ void level_first(LevelCtl* c, int64_t n, int win_ratio, int policy, i
     c->frontier = 1;
     c->visited = 1;
     c->level = 0;
+    c->done = 0u;
     c->window = 0;
     c->win_ratio = win_ratio;
     c->dedup = (16 < n) ? 1 : 0;
@@ -2199,12 +2243,15 @@ bfs_status run_search(bfs_graph* g, int32_t root, int32_t* parent, int32_t* leve
             cudaEventRecord(W.ev[5], s);
             cudaEventRecord(W.ev[6], s);
         }
-        reduce_level<<<std::min<int64_t>((W.bm_words + 255) / 256 + 1, sm_count() * 16), kNT, 0, s>>>(
-            t, W.pi.as<uint32_t>(), f, W.fsum.as<uint8_t>(), W.bm_words, L.n, level, ctl, ctr, deg);
+        const NextArgs nx{L.n, max_levels, handle, host ? 0 : 1, lvl, 3 * p + 1};
+        if (L.n < kSmallReduce)
+            reduce_level<4><<<(unsigned)((W.bm_words + 31) / 32), kNT, 0, s>>>(
+                t, W.pi.as<uint32_t>(), f, W.fsum.as<uint8_t>(), W.bm_words, L.n, level, ctl, ctr, deg, nx);
+        else
+            reduce_level<32><<<std::min<int64_t>((W.bm_words + 255) / 256, sm_count() * 16), kNT, 0, s>>>(
+                t, W.pi.as<uint32_t>(), f, W.fsum.as<uint8_t>(), W.bm_words, L.n, level, ctl, ctr, deg, nx);
         BFS_CUDA_TRY(cudaGetLastError());
         if (host && timing) cudaEventRecord(W.ev[4], s);
-        level_next<<<1, 1, 0, s>>>(ctl, ctr, L.n, max_levels, handle, host ? 0 : 1, lvl, 3 * p + 1);
-        BFS_CUDA_TRY(cudaGetLastError());
         return BFS_OK;
     };
 

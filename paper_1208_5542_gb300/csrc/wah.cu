@@ -118,6 +118,250 @@ __global__ void __launch_bounds__(kCT) wah_encode_bitmap(const uint32_t* bits, i
     cluster_done();
 }
 
+// The last slot to finish (a counter, no waiting; one warp per slot calls this)
+// lays out the decoder's units: block (i,j) of the p x p grid (row-major)
+// decodes stream s = i*p+j (sieved) or j, in chunks of 32 words; plan_base is
+// the exclusive scan of the chunk counts.
+__device__ __forceinline__ void lay_out_units(const EncodeArgs& a) {
+    if (!a.plan_base) return;
+    const int lane = (int)lane_id();
+    unsigned int last = 0;
+    if (lane == 0) {
+        __threadfence();
+        last = atomicAdd(a.plan_done, 1u) == (unsigned)(a.nslots - 1);
+    }
+    if (!__shfl_sync(0xffffffffu, last, 0)) return;
+    __threadfence();
+    const int64_t nblocks = (int64_t)a.p * a.p;
+    unsigned long long sum = 0;
+    for (int64_t b0 = 0; b0 < nblocks; b0 += 128) {          // four blocks a lane, their loads in flight together
+        unsigned long long n[4], mine = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int64_t b = b0 + 4 * lane + k;
+            n[k] = 0;
+            if (b < nblocks) n[k] = (unsigned long long)((__ldcg(a.counts + (a.sieve ? b : b % a.p)) + 31) / 32);
+            mine += n[k];
+        }
+        const unsigned long long incl = warp_incl_sum(mine);
+        unsigned long long at = sum + incl - mine;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int64_t b = b0 + 4 * lane + k;
+            if (b < nblocks) a.plan_base[b] = (int64_t)at;
+            at += n[k];
+        }
+        sum += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    if (lane == 0) {
+        a.plan_base[nblocks] = (int64_t)sum;
+        *a.plan_units = sum;
+        *a.plan_done = 0u;                       // ready for the next level
+    }
+}
+
+// -------------------------------------------- slot encoder, short slots --
+// The same streams in one launch, one CTA per slot, for slots of up to
+// kSmallChunks chunks: a round takes kSK consecutive groups per thread straight
+// from the operands, one scan of (heads, last head) over the CTA places the
+// words, and the threads write them.  Its time is one chain of dependent steps
+// (about 5 us for a one-round slot), where the three launches below, built for
+// throughput, take 16-25 us however little there is to encode; above the limit
+// their warps, which need not wait for one another, are the faster ones.
+constexpr int kSK = 4;              // groups per thread and round
+constexpr int kSmallChunks = 8;     // two rounds (five rounds, 17 chunks of scale 22 on 8 x 8: 38 us against 26)
+
+// (count, position + 1) packed: counts add, positions take the larger.
+struct OpHeads {
+    __device__ __forceinline__ unsigned long long operator()(unsigned long long a, unsigned long long b) const {
+        const uint32_t x = (uint32_t)a, y = (uint32_t)b;
+        return ((a >> 32) + (b >> 32)) << 32 | (x > y ? x : y);
+    }
+};
+
+// Group g of the slot, both operands read together.
+template <typename W>
+__device__ __forceinline__ W slot_group(const EncodeArgs& a, const SlotGeom& sg, int64_t g) {
+    W x = Wah<W>::group_cg(a.frontier, (uint64_t)(sg.src0 + g * Wah<W>::GB));
+    const W d = sg.dirb ? Wah<W>::group_cg(sg.dirb, (uint64_t)(g * Wah<W>::GB)) : Wah<W>::ONES;
+    if (a.invert_frontier) x = ~x & Wah<W>::ONES;
+    return x & d;
+}
+
+template <typename W, int NT>
+__global__ void __launch_bounds__(NT) enc_small(EncodeArgs a, int64_t cps, unsigned long long* setbits) {
+    using T = Wah<W>;
+    constexpr int GB = T::GB;
+    constexpr int RG = NT * kSK;                            // groups per round
+    __shared__ unsigned long long s_scan[NT / 32 + 1];
+    const int s = blockIdx.x;
+    if (a.skip && *a.skip) {                // a level without this exchange: empty streams
+        if (threadIdx.x == 0) a.counts[s] = 0;
+        return;
+    }
+    const SlotGeom sg = slot_geom(a, s);
+    const int64_t G = sg.nbits / GB;
+    const int r = (int)(sg.nbits % GB);
+    W* out = static_cast<W*>(a.out) + (int64_t)s * a.slot_cap;
+    int64_t* ub = a.unit_base ? a.unit_base + (int64_t)s * a.unit_stride : nullptr;
+    const bool dead = a.slot_live && !a.slot_live[s];
+    W tail = W(0);                          // the trailing r bits of the slot
+    if (r > 0 && !dead) {
+        const uint64_t pos = (uint64_t)(sg.src0 + G * GB);
+        tail = T::tail(a.frontier, pos, r);
+        const W td = sg.dirb ? T::tail(sg.dirb, (uint64_t)(G * GB), r) : T::ONES;
+        if (a.invert_frontier) tail = ~tail & (W)((W(1) << r) - W(1));
+        tail &= td;
+    }
+    int fm = FMT_WAH;
+    int64_t nw = 0, total_ones = 0;         // words (the open run's included) and set bits so far
+    bool bits = false;                      // a group holds a set bit
+    unsigned long long counted = 0;
+    uint32_t live_chunks = 0;
+    const int rounds = (int)((G + RG - 1) / RG);
+    for (int pass = (a.adaptive && rounds > 1) ? 0 : 1; pass < 2; ++pass) {
+        nw = 0;
+        total_ones = 0;
+        int64_t run_start = 0;
+        for (int64_t tb = 0; tb < G; tb += RG) {
+            const int64_t tend = (tb + RG < G) ? tb + RG : G;
+            // of several rounds one without frontier bits is not read (the frontier summary: 1
+            // byte per 1024 bits); the statistics want the test for a single one, too
+            bool nz = !dead;
+            if (a.fsum && !dead && (rounds > 1 || a.live_chunks)) {
+                const int64_t q0 = (sg.src0 + tb * GB) >> 10, q1 = (sg.src0 + tend * GB - 1) >> 10;
+                nz = false;
+                for (int64_t q = q0 + threadIdx.x; q <= q1; q += NT) nz |= __ldcg(a.fsum + q) != 0;
+            }
+            const bool live = __syncthreads_or(nz);
+            const int64_t g0 = tb + (int64_t)threadIdx.x * kSK;
+            W x[kSK];
+            int ty[kSK + 1], pt = -1;
+            uint32_t ones = 0;
+            if (live) {
+#pragma unroll
+                for (int k = 0; k < kSK; ++k) x[k] = g0 + k < G ? slot_group<W>(a, sg, g0 + k) : W(0);
+                ty[kSK] = g0 + kSK < G ? group_type<W>(slot_group<W>(a, sg, g0 + kSK)) : G_NONE;
+                if (g0 > 0 && g0 < G) pt = group_type<W>(slot_group<W>(a, sg, g0 - 1));
+            } else {
+#pragma unroll
+                for (int k = 0; k < kSK; ++k) x[k] = W(0);
+                // only the groups around the round can differ from a zero run
+                ty[kSK] = g0 + kSK >= G ? G_NONE
+                          : (g0 + kSK < tend || dead ? (int)G_ZERO : group_type<W>(slot_group<W>(a, sg, g0 + kSK)));
+                if (g0 > 0 && g0 < G) pt = g0 > tb || dead ? (int)G_ZERO : group_type<W>(slot_group<W>(a, sg, g0 - 1));
+            }
+            uint32_t h = 0, last = 0;
+#pragma unroll
+            for (int k = 0; k < kSK; ++k) {
+                ty[k] = g0 + k < G ? group_type<W>(x[k]) : G_NONE;
+                if (g0 + k < G) {
+                    ones += (uint32_t)T::popc(x[k]);
+                    if (ty[k] == G_LIT || ty[k] != pt) {
+                        h |= 1u << k;
+                        last = (uint32_t)(g0 + k) + 1u;
+                    }
+                }
+                pt = ty[k];
+            }
+            unsigned long long all;
+            const unsigned long long ex = block_excl_scan<NT>((unsigned long long)__popc(h) << 32 | last, 0ull, OpHeads(),
+                                                              s_scan, &all);
+            int64_t ones_at = 0;
+            if (a.adaptive) {
+                unsigned long long sum;
+                ones_at = total_ones + (int64_t)block_excl_scan<NT>((unsigned long long)ones, 0ull, OpSum(), s_scan, &sum);
+                total_ones += (int64_t)sum;
+            }
+            const int64_t before = nw;
+            nw += (int64_t)(all >> 32);
+            const int64_t opened = (int64_t)(uint32_t)ex - 1;
+            int64_t cur = opened >= 0 ? opened : run_start;
+            if ((uint32_t)all) run_start = (int64_t)(uint32_t)all - 1;
+            if (pass == 0) continue;
+            if (rounds == 1 && a.adaptive) {
+                // the smallest in bytes, the lower format on a tie (every element is 4 bytes)
+                const int64_t wah = nw + (r > 0 ? 1 : 0), list = total_ones + T::popc(tail), raw = (sg.nbits + 31) >> 5;
+                fm = (wah <= list && wah <= raw) ? FMT_WAH : (list <= raw ? FMT_LIST : FMT_RAW);
+                if (fm != FMT_WAH) ub = nullptr;            // no WAH units in this slot
+            }
+            counted += ones;
+            bits |= ones != 0;
+            if (live) live_chunks += (uint32_t)((tend - tb + kTile - 1) / kTile);
+            if (fm == FMT_RAW) continue;
+            int64_t widx = before - 1 + (int64_t)(ex >> 32);
+#pragma unroll
+            for (int k = 0; k < kSK; ++k) {
+                const int64_t g = g0 + k;
+                if (g >= G) break;
+                if (fm == FMT_LIST) {       // the sparse vector: every set bit's offset in the slice, in order
+                    for (W y = x[k]; y; y &= y - W(1)) out[ones_at++] = (W)(g * GB + T::select(y, 0));
+                    continue;
+                }
+                if ((h >> k) & 1u) {
+                    cur = g;
+                    ++widx;
+                    if (ub && (widx & 31) == 0) ub[widx >> 5] = g;
+                }
+                if (a.chunk_first && g % kTile == 0) {       // where a decoder of this chunk alone starts
+                    a.chunk_first[2 * ((int64_t)s * cps + g / kTile)] = widx;
+                    a.chunk_first[2 * ((int64_t)s * cps + g / kTile) + 1] = cur;
+                }
+                if (ty[k] == G_LIT) out[widx] = T::to_payload(x[k]);
+                else if (ty[k + 1] != ty[k]) out[widx] = fill_word<W>(ty[k], (uint64_t)(g - cur + 1));
+            }
+        }
+        if (a.adaptive && (pass == 0 || rounds == 0)) {
+            const int64_t wah = nw + (r > 0 ? 1 : 0), list = total_ones + T::popc(tail), raw = (sg.nbits + 31) >> 5;
+            fm = (wah <= list && wah <= raw) ? FMT_WAH : (list <= raw ? FMT_LIST : FMT_RAW);
+            if (fm != FMT_WAH) ub = nullptr;
+        }
+    }
+    if (fm == FMT_RAW) {                    // the raw bitmap, bits past the slice cleared
+        for (int64_t w = threadIdx.x; w < (sg.nbits + 31) >> 5; w += NT) {
+            uint32_t x = bits32_at_cg(a.frontier, (uint64_t)(sg.src0 + 32 * w));
+            if (sg.dirb) x &= __ldcg(sg.dirb + w);
+            const int64_t left = sg.nbits - 32 * w;
+            if (left < 32) x &= (1u << left) - 1u;
+            out[w] = (W)x;
+        }
+    }
+    if (setbits) {
+        counted = warp_sum(counted);
+        if (lane_id() == 0 && counted) atomicAdd(setbits, counted);
+    }
+    bits = __syncthreads_or(bits);          // and every read of the operands is done
+    if (a.dir_clear && !dead) {             // the operand is clear for its next use
+        uint32_t* d = a.dir_clear + (int64_t)s * a.dir_stride;
+        for (int64_t w = threadIdx.x; w < (sg.nbits + 31) >> 5; w += NT)
+            if (__ldcg(d + w)) d[w] = 0u;
+    }
+    if (threadIdx.x >= 32) return;
+    if (threadIdx.x == 0) {
+        int64_t count = nw;
+        if (r > 0) {
+            if (setbits && tail) atomicAdd(setbits, (unsigned long long)T::popc(tail));
+            if (fm == FMT_WAH) {
+                if (ub && (count & 31) == 0) ub[count >> 5] = G;
+                out[count++] = T::to_active(tail, r);
+            }
+            bits |= tail != W(0);
+        }
+        if (fm == FMT_LIST) {               // the offsets of the trailing bits close the vector
+            count = total_ones;
+            for (W y = tail; y; y &= y - W(1)) out[count++] = (W)(G * GB + T::select(y, 0));
+        } else if (fm == FMT_RAW) {
+            count = (sg.nbits + 31) >> 5;
+        }
+        a.counts[s] = count;
+        if (a.fmt) a.fmt[s] = (uint8_t)fm;
+        if (a.slot_bits) a.slot_bits[s] = bits ? 1 : 0;
+        if (a.wah_words) atomicAdd(a.wah_words, (unsigned long long)count);
+        if (a.live_chunks && live_chunks) atomicAdd(a.live_chunks, (unsigned long long)live_chunks);
+    }
+    lay_out_units(a);
+}
+
 // ------------------------------------------------- parallel slot encoder --
 // All slots' streams, built in three data-parallel passes over (slot, chunk of
 // kTile groups):
@@ -370,41 +614,7 @@ __global__ void enc_chunk_scan(EncodeArgs a, const ChunkSum* sums, const uint8_t
         if (a.slot_bits) a.slot_bits[s] = bits ? 1 : 0;
         if (a.wah_words) atomicAdd(a.wah_words, (unsigned long long)total);
     }
-    if (!a.plan_base) return;
-    // The last slot to finish lays out the decoder's units: block (i,j) of the
-    // p x p grid (row-major) decodes stream s = i*p+j (sieved) or j, in chunks
-    // of 32 words; plan_base is the exclusive scan of the chunk counts.
-    __shared__ bool s_last;
-    if (lane == 0) {
-        __threadfence();
-        s_last = atomicAdd(a.plan_done, 1u) == (unsigned)(a.nslots - 1);
-    }
-    __syncwarp();
-    if (!s_last) return;
-    __threadfence();
-    const int64_t nblocks = (int64_t)a.p * a.p;
-    unsigned long long carry = 0;
-    for (int64_t b0 = 0; b0 < nblocks; b0 += 32) {
-        const int64_t b = b0 + lane;
-        unsigned long long nch = 0;
-        if (b < nblocks) {
-            const int64_t stream = a.sieve ? b : b % a.p;
-            nch = (unsigned long long)((__ldcg(a.counts + stream) + 31) / 32);
-        }
-        unsigned long long incl = nch;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, d);
-            if (lane >= d) incl += y;
-        }
-        if (b < nblocks) a.plan_base[b] = (int64_t)(carry + incl - nch);
-        carry += __shfl_sync(0xffffffffu, incl, 31);
-    }
-    if (lane == 0) {
-        a.plan_base[nblocks] = (int64_t)carry;
-        *a.plan_units = carry;
-        *a.plan_done = 0u;                       // ready for the next level
-    }
+    lay_out_units(a);
 }
 
 
@@ -1064,7 +1274,16 @@ bfs_status launch_wah_encode_parallel(const EncodeArgs& a, int wah_bits, void* s
     ChunkBase* cb = static_cast<ChunkBase*>(bases);
     uint8_t* fl = static_cast<uint8_t*>(flags);
     if (a.adaptive && (wah_bits != 32 || !a.fmt)) return set_error(BFS_ERR_INVALID_ARG, "adaptive format needs 32-bit words");
-    if (wah_bits == 32) {
+    const int64_t groups = a.nb / (wah_bits - 1);
+    if (groups <= (int64_t)kSmallChunks * kTile) {
+        if (wah_bits == 32) {
+            if (groups <= 256 * kSK) enc_small<uint32_t, 256><<<a.nslots, 256, 0, st>>>(a, cps, setbits);
+            else enc_small<uint32_t, 1024><<<a.nslots, 1024, 0, st>>>(a, cps, setbits);
+        } else {
+            if (groups <= 256 * kSK) enc_small<unsigned long long, 256><<<a.nslots, 256, 0, st>>>(a, cps, setbits);
+            else enc_small<unsigned long long, 1024><<<a.nslots, 1024, 0, st>>>(a, cps, setbits);
+        }
+    } else if (wah_bits == 32) {
         enc_chunk_sums32<<<grid, kEW, 0, st>>>(a, cs, fl, cps, setbits);
         enc_chunk_scan<uint32_t><<<a.nslots, 32, 0, st>>>(a, cs, fl, cb, cps, setbits);
         enc_chunk_write32<<<grid, kEW, 0, st>>>(a, cb, fl, cps);
