@@ -272,8 +272,8 @@ enum {
  * (1, i), ... back to back (4 + 8 bytes per vertex and 4 bytes per entry, kept
  * with the graph and counted by bfs_graph_footprint; ordered on the legacy
  * default stream and synchronised).  Applies to bfs_run; the batched and
- * served searches (bfs_run_batch, bfs_server_*) stay top-down.  Not safe
- * while a search on `g` is running.
+ * served searches (bfs_run_batch, bfs_server_*) choose the side of each level
+ * by a rule of their own.  Not safe while a search on `g` is running.
  */
 BFS_API bfs_status bfs_graph_set_direction(bfs_graph_t g, int32_t policy, int32_t alpha, int32_t beta);
 
@@ -377,7 +377,8 @@ BFS_API bfs_status bfs_check_search(bfs_graph_t g, int32_t root, const int32_t *
 typedef struct {
     int32_t n_levels;            /* levels performed (the deepest search's depth + 1) */
     int32_t reserved;
-    int64_t edges_scanned;       /* adjacency entries read, all levels */
+    int64_t edges_scanned;       /* adjacency entries of the active vertices, all levels: what a
+                                    level read from its sources reads */
 } bfs_batch_stats;
 
 /*
@@ -392,8 +393,7 @@ typedef struct {
  *     roots[r], or -1.
  *   parents: device [n_roots][n] or NULL; parents[r][v] = the smallest
  *     neighbour u of v with levels[r][u] = levels[r][v] - 1 (roots[r] for the
- *     root, -1 if unreached).  Computing parents adds one reduction per newly
- *     reached (vertex, search) pair per candidate edge and is markedly slower.
+ *     root, -1 if unreached).  Computing parents is markedly slower.
  *   stats: NULL or filled after the batch.
  * Synchronises `cuda_stream` before returning.  The first call on a graph
  * builds and instantiates the CUDA graph.

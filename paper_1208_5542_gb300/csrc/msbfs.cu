@@ -1,11 +1,17 @@
 // msbfs.cu -- batched multi-source BFS: up to 64 searches at once, bit-parallel.
 //
-// Every vertex holds three 64-bit lane words (bit r = search r): vis (visited),
-// f (frontier) and nxt (next).  One level is the boolean SpMV of Sec. III-A
-// applied to all 64 lane vectors at once:
+// Every vertex holds three 64-bit lane words (bit r = search r): vis (visited)
+// and nxt (next), side by side, and f (frontier).  One level is the boolean
+// SpMV of Sec. III-A applied to all 64 lane vectors at once:
 //   nxt[v] |= f[u] & ~vis[v]     for every entry u -> v of a nonempty column
 // of a block whose source u is active (f[u] != 0); the directory V_{i,j}
 // (Eq. 4) sieves the (vertex, block) pairs, exactly as in the single search.
+// On an undirected graph the same product can be taken from v's side, v's own
+// columns holding its neighbours: a level whose active vertices hold much of
+// the graph's entries lets every vertex that some running lane has not visited
+// OR its neighbours' frontier words, without an atomic, until no lane is
+// missing.  The block-rows are scanned in order, so the first that holds a
+// frontier neighbour of a lane holds its smallest: its parent there.
 // Then new = nxt & ~vis; vis |= new; f = new; level[r][v] = k + 1 for every new
 // bit r; and the next level's active list is the set of v with new != 0.
 // Optional parents: parent[r][v] = the smallest u of lane r's previous level
@@ -30,8 +36,8 @@ namespace {
 
 constexpr int kMT = 256;            // threads of the small kernels
 constexpr uint32_t kMsCoop = 32;    // columns of at least this many entries take the whole warp
-constexpr uint32_t kMsHub = 1024;   // longer columns are cut into pieces
-constexpr uint32_t kMsPiece = 1024;
+constexpr uint32_t kMsHub = 512;    // longer columns are cut into pieces
+constexpr uint32_t kMsPiece = 512;
 
 // Device-resident arguments and counters of a batch (one per graph).
 struct MsState {
@@ -46,9 +52,10 @@ struct MsState {
     int p;
     int64_t nb, n;
     // lane words and active lists (constant buffers)
-    unsigned long long* vis;
+    ulonglong2* vn;             // x: vis, y: nxt
     unsigned long long* f[2];
-    unsigned long long* nxt;
+    const uint32_t* deg;        // entries per source vertex
+    int symmetric;              // undirected: levels may run from the destinations' side
     int32_t* act[2];
     Item* pieces;
     int64_t piece_cap;
@@ -66,7 +73,12 @@ struct MsState {
     unsigned long long act_next;     // hand-out cursor over the current active list
     unsigned long long piece_count;
     unsigned long long piece_next;
-    unsigned long long edges;        // entries scanned (all levels)
+    unsigned long long edges;        // entries of the active vertices (all levels)
+    unsigned long long act_edges;    // the same of the next level
+    unsigned long long miss_edges;   // entries of the vertices that a running lane has not visited
+    unsigned long long lanes;        // lanes with a frontier vertex at the current level
+    int32_t pull;                    // 1: this level runs from the destinations' side
+    unsigned int done;               // CTAs of the reduction that have finished
     unsigned long long levels_done;  // levels performed
     // continuous batching (server): lane r's level of v is (iteration + 1) - lane_start[r]
     int32_t lane_start[64];
@@ -97,6 +109,11 @@ __global__ void ms_reset(MsState* S) {
     S->piece_count = 0;
     S->piece_next = 0;
     S->edges = 0;
+    S->act_edges = 0;
+    S->miss_edges = 0;
+    S->lanes = 0;
+    S->pull = 0;
+    S->done = 0;
     S->levels_done = 0;
     S->err = 0;
     S->err_a = 0;
@@ -108,10 +125,9 @@ __global__ void ms_clear(MsState* S) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     for (int64_t v = tid; v < s.n; v += stride) {
-        s.vis[v] = 0ull;
+        s.vn[v] = make_ulonglong2(0ull, 0ull);
         s.f[0][v] = 0ull;
         s.f[1][v] = 0ull;
-        s.nxt[v] = 0ull;
     }
     const int64_t total = (int64_t)s.n_roots * s.n;
     for (int64_t x = tid; x < total; x += stride) {
@@ -126,24 +142,33 @@ __global__ void ms_roots(MsState* S) {
     if (r >= s.n_roots) return;
     const int32_t v = s.roots[r];
     const unsigned long long bit = 1ull << r;
-    const unsigned long long old = atomicOr(s.vis + v, bit);
+    const unsigned long long old = atomicOr(&s.vn[v].x, bit);
     atomicOr(s.f[0] + v, bit);
     s.levels[(int64_t)r * s.n + v] = 0;
     if (s.parents) s.parents[(int64_t)r * s.n + v] = v;
     if (old == 0ull) {                       // first lane at this vertex: make it active
         const unsigned long long pos = atomicAdd(&s.act_count[0], 1ull);
         s.act[0][pos] = v;
+        atomicAdd(&s.edges, (unsigned long long)s.deg[v]);
     }
+    atomicOr(&s.lanes, bit);
 }
 
 // ----------------------------------------------------------------- level --
+// Visit u -> v given v's words read before (several entries' reads are in
+// flight together; a stale nxt only costs an atomic that changes nothing).
 struct MsVisit {
     const MsState* s;
-    __device__ __forceinline__ void operator()(int32_t v, int32_t u, unsigned long long fu) const {
-        if ((uint64_t)(uint32_t)v >= (uint64_t)s->n) { ms_fault(const_cast<MsState*>(s), 2, (uint32_t)v, (uint32_t)u); return; }
-        const unsigned long long nb = fu & ~__ldg(s->vis + v);     // vis does not change during the expansion
+    __device__ __forceinline__ bool valid(int32_t v, int32_t u) const {
+        if ((uint64_t)(uint32_t)v < (uint64_t)s->n) return true;
+        ms_fault(const_cast<MsState*>(s), 2, (uint32_t)v, (uint32_t)u);
+        return false;
+    }
+    __device__ __forceinline__ ulonglong2 probe(int32_t v) const { return __ldcg(s->vn + v); }
+    __device__ __forceinline__ void mark(int32_t v, int32_t u, unsigned long long fu, const ulonglong2& w) const {
+        const unsigned long long nb = fu & ~w.x;               // vis does not change during the expansion
         if (!nb) return;
-        atomicOr(s->nxt + v, nb);
+        if (nb & ~w.y) atomicOr(&s->vn[v].y, nb);
         if (s->parents) {
             unsigned long long m = nb & s->parent_mask;
             while (m) {
@@ -155,18 +180,42 @@ struct MsVisit {
     }
 };
 
+constexpr int kMsIlp = 4;           // entries per lane in flight
+
 __device__ __forceinline__ void ms_column(const MsVisit& vis, const int32_t* ir, int32_t u, unsigned long long fu,
                                           int64_t beg, uint32_t len) {
     const int32_t* col = ir + beg;
-    for (uint32_t e = lane_id(); e < len; e += 32) vis(__ldg(col + e), u, fu);
+    for (uint32_t e = lane_id(); e < len; e += 32 * kMsIlp) {
+        int32_t v[kMsIlp];
+        ulonglong2 w[kMsIlp];
+#pragma unroll
+        for (int k = 0; k < kMsIlp; ++k) v[k] = e + 32 * k < len ? __ldg(col + e + 32 * k) : -1;
+#pragma unroll
+        for (int k = 0; k < kMsIlp; ++k)
+            if (e + 32 * k < len && !vis.valid(v[k], u)) v[k] = -1;
+#pragma unroll
+        for (int k = 0; k < kMsIlp; ++k)
+            if (v[k] >= 0) w[k] = vis.probe(v[k]);
+#pragma unroll
+        for (int k = 0; k < kMsIlp; ++k)
+            if (v[k] >= 0) vis.mark(v[k], u, fu, w[k]);
+    }
 }
 
 // One item per lane (u, f[u], column); long columns go to the piece list,
 // columns of at least kMsCoop entries take the whole warp, the rest share the
-// warp through a load-balanced search over their entry counts.
+// warp, 32 consecutive entries of the concatenated columns per step: every
+// column's first entry sets its bit in the step's head mask, and the owner of
+// an entry is the number of heads up to it (the columns are packed in the
+// warp's scratch).
+struct MsScratch {
+    unsigned long long fu[32];
+    int64_t off[32];            // column offset minus the entries before it
+    int32_t u[32];
+};
+
 __device__ __forceinline__ void ms_warp_expand(MsState& s, const MsVisit& vis, int32_t u, unsigned long long fu,
-                                               int64_t beg, uint32_t len, unsigned long long& edges) {
-    edges += len;
+                                               int64_t beg, uint32_t len, MsScratch& ws) {
     if (__any_sync(0xffffffffu, len > kMsHub)) {
         if (len > kMsHub) {
             const uint32_t np = (len + kMsPiece - 1) / kMsPiece;
@@ -189,78 +238,132 @@ __device__ __forceinline__ void ms_warp_expand(MsState& s, const MsVisit& vis, i
                   __shfl_sync(0xffffffffu, beg, src), __shfl_sync(0xffffffffu, len, src));
     }
     if (len >= kMsCoop) len = 0;
+    const uint32_t nz = __ballot_sync(0xffffffffu, len > 0);
+    if (!nz) return;
     const uint32_t incl = warp_incl_sum(len);
     const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
     const uint32_t excl = incl - len;
-    for (uint32_t e0 = 0; e0 < total; e0 += 32) {
-        const uint32_t e = e0 + lane_id();
-        int lo = 0, hi = 31;
+    const uint32_t below = (1u << lane_id()) - 1u, upto = below | (1u << lane_id());
+    __syncwarp();                           // the previous batch's readers are done
+    if (len > 0) {
+        const int r = __popc(nz & below);
+        ws.fu[r] = fu;
+        ws.off[r] = beg - (int64_t)excl;
+        ws.u[r] = u;
+    }
+    __syncwarp();
+    int before = -1;
+    for (uint32_t e0 = 0; e0 < total; e0 += 32 * kMsIlp) {
+        int32_t v[kMsIlp];
+        int ow[kMsIlp];
+        ulonglong2 w[kMsIlp];
 #pragma unroll
-        for (int step = 0; step < 5; ++step) {
-            const int mid = (lo + hi) >> 1;
-            const uint32_t im = __shfl_sync(0xffffffffu, incl, mid);
-            if (im > e) hi = mid; else lo = mid + 1;
+        for (int k = 0; k < kMsIlp; ++k) {
+            const uint32_t rel = excl - (e0 + 32 * k);
+            const uint32_t heads = __reduce_or_sync(0xffffffffu, (len > 0 && rel < 32u) ? 1u << rel : 0u);
+            const uint32_t e = e0 + 32 * k + lane_id();
+            ow[k] = before + __popc(heads & upto);
+            before += __popc(heads);
+            v[k] = e < total ? __ldg(s.ir + ws.off[ow[k]] + (int64_t)e) : -1;
+            if (e < total && !vis.valid(v[k], ws.u[ow[k]])) v[k] = -1;
         }
-        const int64_t ob = __shfl_sync(0xffffffffu, beg, lo);
-        const uint32_t oe = __shfl_sync(0xffffffffu, excl, lo);
-        const int32_t ou = __shfl_sync(0xffffffffu, u, lo);
-        const unsigned long long of = __shfl_sync(0xffffffffu, fu, lo);
-        if (e < total) vis(__ldg(s.ir + ob + (int64_t)(e - oe)), ou, of);
+#pragma unroll
+        for (int k = 0; k < kMsIlp; ++k)
+            if (v[k] >= 0) w[k] = vis.probe(v[k]);
+#pragma unroll
+        for (int k = 0; k < kMsIlp; ++k)
+            if (v[k] >= 0) vis.mark(v[k], ws.u[ow[k]], ws.fu[ow[k]], w[k]);
     }
 }
 
-// Expansion: warps take 32 active vertices at a time; for every block-row i,
-// the vertices whose column of block (i, j(u)) is nonempty (directory test)
-// are expanded.
-__global__ void ms_expand(MsState* S) {
+// Column of local source ul in block b: offset into ir and length (0: empty).
+__device__ __forceinline__ void ms_lookup(const MsState& s, int64_t b, int64_t ul, int64_t& beg, uint32_t& len) {
+    const uint32_t dw = __ldg(s.dir + b * s.dir_stride + (ul >> 5));
+    const uint32_t rk = __ldg(s.rank + b * s.dir_stride + (ul >> 5));
+    const uint32_t bit = 1u << (ul & 31);
+    beg = 0;
+    len = 0;
+    if (!(dw & bit)) return;
+    const uint32_t* cpb = s.cp + __ldg(s.cp_base + b);
+    const uint32_t c = rk + __popc(dw & (bit - 1u));
+    const uint32_t c0 = __ldg(cpb + c), c1 = __ldg(cpb + c + 1);
+    beg = __ldg(s.ir_base + b) + c0;
+    len = c1 - c0;
+}
+
+// Expansion.  Unit = (32 active vertices, one block-row i): the vertices whose
+// column of block (i, j(u)) is nonempty (directory test) are expanded by one
+// warp, the next unit's columns looked up before.  With fewer units than warps
+// a unit holds fewer vertices (down to one), so that a short active list, which
+// holds the hubs of the early levels, still fills the chip.  Few units are
+// dealt out in turn, many handed out by a counter, several at a time.
+__global__ void __launch_bounds__(1024) ms_expand(MsState* S) {
     MsState& s = *S;
+    if (s.pull) return;
+    extern __shared__ MsScratch s_ws[];
+    MsScratch& ws = s_ws[threadIdx.x >> 5];
     const MsVisit vis{S};
-    const int cur = s.cur;
+    const int cur = s.cur, p = s.p;
     const int32_t* act = s.act[cur];
-    const unsigned long long nact = s.act_count[cur];
+    const int64_t nact = (int64_t)s.act_count[cur];
     const unsigned long long* f = s.f[cur];
-    unsigned long long edges = 0;
+    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    int64_t bw = nact * p / (2 * warps);                       // vertices per unit
+    bw = bw < 1 ? 1 : (bw < 32 ? bw : 32);
+    const int64_t groups = (nact + bw - 1) / bw, units = groups * p;
+    int64_t each = units / (4 * warps);                        // units per hand-out
+    each = each < 1 ? 1 : (each < 16 ? each : 16);
+    // the column of this lane's vertex in unit x (none past the units or the group)
+    auto lookup = [&](int64_t x, int32_t& u, unsigned long long& fu, int64_t& beg, uint32_t& len) {
+        fu = 0;
+        len = 0;
+        beg = 0;
+        u = 0;
+        if (x >= units) return;
+        const int64_t i = x / groups, q = (x - i * groups) * bw + lane_id();   // block-row by block-row
+        if ((int64_t)lane_id() >= bw || q >= nact) return;
+        u = act[q];
+        if ((uint64_t)(uint32_t)u >= (uint64_t)s.n) {
+            ms_fault(S, 1, (uint64_t)q, (uint32_t)u);
+            u = 0;
+            return;
+        }
+        fu = f[u];
+        const int64_t j = (uint32_t)u / (uint32_t)s.nb;        // ids and ranges are below 2^31
+        ms_lookup(s, i * p + j, u - j * s.nb, beg, len);
+    };
+    auto run = [&](int64_t x0, int64_t x1) {
+        int32_t u, un;
+        unsigned long long fu, fn;
+        int64_t beg, bn;
+        uint32_t len, ln;
+        lookup(x0, u, fu, beg, len);
+        for (int64_t x = x0; x < x1; ++x) {
+            lookup(x + 1 < x1 ? x + 1 : units, un, fn, bn, ln);
+            if (__any_sync(0xffffffffu, len > 0)) ms_warp_expand(s, vis, u, fu, beg, len, ws);
+            u = un;
+            fu = fn;
+            beg = bn;
+            len = ln;
+        }
+    };
+    if (units <= 4 * warps) {
+        const int64_t w0 = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+        for (int64_t x = w0; x < units; x += warps) run(x, x + 1);
+        return;
+    }
     for (;;) {
         unsigned long long base = 0;
-        if (lane_id() == 0) base = atomicAdd(&s.act_next, 32ull);
+        if (lane_id() == 0) base = atomicAdd(&s.act_next, (unsigned long long)each);
         base = __shfl_sync(0xffffffffu, base, 0);
-        if (base >= nact) break;
-        const unsigned long long q = base + lane_id();
-        int32_t u = 0;
-        unsigned long long fu = 0;
-        int64_t j = 0, ul = 0;
-        if (q < nact) {
-            u = act[q];
-            if ((uint64_t)(uint32_t)u >= (uint64_t)s.n) { ms_fault(S, 1, q, (uint32_t)u); u = 0; }
-            else fu = f[u];
-            j = (uint32_t)u / (uint32_t)s.nb;                 // ids and ranges are below 2^31
-            ul = u - j * s.nb;
-        }
-        for (int i = 0; i < s.p; ++i) {
-            int64_t beg = 0;
-            uint32_t len = 0;
-            if (fu) {
-                const int64_t b = (int64_t)i * s.p + j;
-                const uint32_t* dirb = s.dir + b * s.dir_stride;
-                const uint32_t dw = __ldg(dirb + (ul >> 5));
-                const uint32_t bit = 1u << (ul & 31);
-                if (dw & bit) {
-                    const uint32_t c = __ldg(s.rank + b * s.dir_stride + (ul >> 5)) + __popc(dw & (bit - 1u));
-                    const uint32_t* cpb = s.cp + __ldg(s.cp_base + b);
-                    const uint32_t c0 = __ldg(cpb + c), c1 = __ldg(cpb + c + 1);
-                    beg = __ldg(s.ir_base + b) + c0;
-                    len = c1 - c0;
-                }
-            }
-            if (__any_sync(0xffffffffu, len > 0)) ms_warp_expand(s, vis, u, fu, beg, len, edges);
-        }
+        if ((int64_t)base >= units) break;
+        run((int64_t)base, (int64_t)base + each < units ? (int64_t)base + each : units);
     }
-    edges = warp_sum(edges);
-    if (lane_id() == 0 && edges) atomicAdd(&s.edges, edges);
 }
 
-__global__ void ms_pieces(MsState* S) {
+__global__ void __launch_bounds__(kMT) ms_pieces(MsState* S) {
     MsState& s = *S;
+    if (s.pull) return;
     const MsVisit vis{S};
     const unsigned long long* f = s.f[s.cur];
     const unsigned long long np = min(s.piece_count, (unsigned long long)s.piece_cap);
@@ -278,80 +381,220 @@ __global__ void ms_pieces(MsState* S) {
     }
 }
 
-// new = nxt & ~vis; vis |= new; f' = new; level of every new lane; next active list.
-__global__ void __launch_bounds__(kMT) ms_reduce(MsState* S) {
+// A level from the destinations' side (undirected graphs): every vertex v that
+// a running lane has not visited ORs the frontier words of its neighbours --
+// its own columns, block-row by block-row -- and stops once no lane is
+// missing.  A lane that wants parents takes the smallest neighbour with its
+// bit of the first block-row that has one (a column is in any order: it is
+// read to its end for such a lane).  A lane of the warp scans its column kMsIlp
+// entries at a time; the rest of a column beyond kMsPullLane entries is read
+// by the whole warp.
+constexpr uint32_t kMsPullLane = 32;
+
+// Lower the parents of v in the lanes `bits` to u; v belongs to one thread.
+__device__ __forceinline__ void ms_parents(const MsState& s, int64_t v, int32_t u, unsigned long long bits) {
+    for (; bits; bits &= bits - 1ull) {
+        unsigned int* q = reinterpret_cast<unsigned int*>(s.parents + (int64_t)(__ffsll((long long)bits) - 1) * s.n + v);
+        if ((unsigned int)u < *q) *q = (unsigned int)u;
+    }
+}
+
+__global__ void __launch_bounds__(kMT) ms_pull(MsState* S) {
+    MsState& s = *S;
+    if (!s.pull) return;
+    const unsigned long long* f = s.f[s.cur];
+    const unsigned long long lanes = s.lanes, pmask = s.parents ? s.parent_mask : 0ull;
+    const int p = s.p;
+    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; 32 * g < s.n; g += warps) {
+        const int64_t v = 32 * g + lane_id();
+        unsigned long long need = v < s.n ? lanes & ~s.vn[v].x : 0ull;
+        if (need && s.deg[v] == 0) need = 0;
+        if (!__any_sync(0xffffffffu, need != 0ull)) continue;
+        const int64_t j = (uint32_t)v / (uint32_t)s.nb, vl = v - j * s.nb;
+        unsigned long long got = 0;
+        int64_t beg = 0, beg_n = 0;
+        uint32_t len = 0, len_n = 0;
+        if (need) ms_lookup(s, j, vl, beg, len);
+        for (int i = 0; i < p; ++i) {
+            len_n = 0;
+            if (need && i + 1 < p) ms_lookup(s, (int64_t)(i + 1) * p + j, vl, beg_n, len_n);
+            const unsigned long long need0 = need;          // missing before this block-row
+            uint32_t e = 0;
+            const uint32_t own = len < kMsPullLane ? len : kMsPullLane;
+            while (e < own && (need | (need0 & pmask))) {
+                int32_t u[kMsIlp];
+                unsigned long long w[kMsIlp];
+#pragma unroll
+                for (int k = 0; k < kMsIlp; ++k) u[k] = e + k < own ? __ldg(s.ir + beg + e + k) : -1;
+#pragma unroll
+                for (int k = 0; k < kMsIlp; ++k) {
+                    w[k] = 0ull;
+                    if (u[k] < 0) continue;
+                    if ((uint64_t)(uint32_t)u[k] < (uint64_t)s.n) w[k] = __ldg(f + u[k]) & need0;
+                    else ms_fault(S, 2, (uint32_t)u[k], (uint64_t)v);
+                }
+#pragma unroll
+                for (int k = 0; k < kMsIlp; ++k) {
+                    need &= ~w[k];
+                    if (w[k] & pmask) ms_parents(s, v, u[k], w[k] & pmask);
+                }
+                e += kMsIlp;
+            }
+            uint32_t more = __ballot_sync(0xffffffffu, len > kMsPullLane && (need | (need0 & pmask)));
+            while (more) {                  // the rest of the long columns, one after the other
+                const int src = __ffs(more) - 1;
+                more &= more - 1;
+                const int64_t cb = __shfl_sync(0xffffffffu, beg, src), cv = __shfl_sync(0xffffffffu, v, src);
+                const uint32_t cl = __shfl_sync(0xffffffffu, len, src);
+                const unsigned long long c0 = __shfl_sync(0xffffffffu, need0, src);
+                unsigned long long cn = __shfl_sync(0xffffffffu, need, src);
+                __syncwarp();               // the parents lowered by lane src are seen below
+                for (uint32_t e0 = kMsPullLane; e0 < cl && (cn | (c0 & pmask)); e0 += 32 * kMsIlp) {
+                    unsigned long long w = 0;
+#pragma unroll
+                    for (int k = 0; k < kMsIlp; ++k) {
+                        const uint32_t x = e0 + 32 * k + lane_id();
+                        if (x >= cl) continue;
+                        const int32_t u = __ldg(s.ir + cb + x);
+                        if ((uint64_t)(uint32_t)u >= (uint64_t)s.n) {
+                            ms_fault(S, 2, (uint32_t)u, (uint64_t)cv);
+                            continue;
+                        }
+                        const unsigned long long h = __ldg(f + u) & c0;
+                        w |= h;
+                        for (unsigned long long m = h & pmask; m; m &= m - 1ull)
+                            atomicMin(reinterpret_cast<unsigned int*>(s.parents) +
+                                          (int64_t)(__ffsll((long long)m) - 1) * s.n + cv, (unsigned int)u);
+                    }
+                    const uint32_t lo = __reduce_or_sync(0xffffffffu, (uint32_t)w);
+                    const uint32_t hi = __reduce_or_sync(0xffffffffu, (uint32_t)(w >> 32));
+                    cn &= ~(((unsigned long long)hi << 32) | lo);
+                }
+                if ((int)lane_id() == src) need = cn;
+            }
+            got |= need0 & ~need;
+            if (!__any_sync(0xffffffffu, need != 0ull)) break;
+            beg = beg_n;
+            len = len_n;
+        }
+        if (got) s.vn[v].y = got;
+    }
+}
+
+// The next level runs from the destinations' side when the vertices that miss
+// a lane hold no more entries than the active ones -- a visit there is a read,
+// from the sources' side a read and often an atomic, and a miss in any of 64
+// lanes means that the whole column is read -- or, when a lane wants parents
+// (an atomic per entry and lane on the sources' side), up to kMsPullParents
+// times as many.  A level with few entries stays on the sources' side.
+// Scale 20, 64 lanes: 1.28 ms (never: 1.82; always on dense levels: 1.85), with
+// parents 4.7 (never: 7.2).
+constexpr unsigned long long kMsPullParents = 8;
+constexpr unsigned long long kMsPullShare = 64;
+
+// One level ends: switch to the next one's buffers (one thread, the level's
+// counts complete).
+__device__ void ms_advance(MsState& s, unsigned long long alive) {
+    const int nxt_i = s.cur ^ 1;
+    s.act_count[s.cur] = 0;
+    s.cur = nxt_i;
+    s.level += 1;
+    s.levels_done += 1;
+    s.act_next = 0;
+    s.piece_count = 0;
+    s.piece_next = 0;
+    const unsigned long long e = __ldcg(&s.act_edges), miss = __ldcg(&s.miss_edges);
+    s.edges += e;
+    s.act_edges = 0;
+    s.miss_edges = 0;
+    s.lanes = alive;
+    const unsigned long long worth = s.parents && (s.parent_mask & alive) ? kMsPullParents : 1ull;
+    s.pull = (s.symmetric && worth * e * kMsPullShare > (unsigned long long)s.nnz && miss <= worth * e) ? 1 : 0;
+}
+
+// new = nxt & ~vis; vis |= new; f' = new; level of every new lane, lane by lane
+// over the warp's vertices (coalesced stores); next active list, one hand-out
+// of places per CTA.  The last CTA to finish (a counter, no waiting) switches
+// to the next level; in the batch's loop (use_handle) it decides whether to
+// iterate again, in the server's step it leaves `alive` for the host.
+__global__ void __launch_bounds__(kMT) ms_reduce(MsState* S, cudaGraphConditionalHandle handle, int use_handle) {
+    constexpr int NW = kMT / 32;
+    __shared__ uint32_t s_cnt[NW];
+    __shared__ unsigned long long s_base, s_any[NW], s_deg[NW], s_miss[NW];
     MsState& s = *S;
     const int cur = s.cur, nxt_i = cur ^ 1;
     unsigned long long* fn = s.f[nxt_i];
     int32_t* actn = s.act[nxt_i];
     const int32_t lv = s.level + 1;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int64_t nwarp_iters = (s.n + stride - 1) / stride;
-    const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    for (int64_t it = 0; it < nwarp_iters; ++it) {
-        const int64_t v = it * stride + tid;
+    const int lane = (int)lane_id(), warp = (int)(threadIdx.x >> 5);
+    const unsigned long long lanes = s.lanes;
+    unsigned long long alive = 0, edges = 0, miss = 0;
+    for (int64_t v0 = blockIdx.x * (int64_t)kMT; v0 < s.n; v0 += (int64_t)gridDim.x * kMT) {
+        const int64_t v = v0 + threadIdx.x;
         unsigned long long nv = 0;
         if (v < s.n) {
-            const unsigned long long x = s.nxt[v];
-            if (x) {
-                s.nxt[v] = 0ull;
-                nv = x & ~s.vis[v];
-                if (nv) {
-                    s.vis[v] |= nv;
-                    unsigned long long m = nv;
-                    while (m) {
-                        const int r = __ffsll((long long)m) - 1;
-                        m &= m - 1;
-                        s.levels[(int64_t)r * s.n + v] = lv - s.lane_start[r];
-                    }
-                }
-            }
+            const ulonglong2 x = s.vn[v];
+            nv = x.y & ~x.x;
+            if (x.y) s.vn[v] = make_ulonglong2(x.x | nv, 0ull);
             fn[v] = nv;
+            const bool missed = (lanes & ~(x.x | nv)) != 0ull;
+            const uint32_t d = nv || missed ? s.deg[v] : 0u;
+            if (nv) edges += d;
+            if (missed) miss += d;
+        }
+        const uint32_t lo = __reduce_or_sync(0xffffffffu, (uint32_t)nv);
+        const uint32_t hi = __reduce_or_sync(0xffffffffu, (uint32_t)(nv >> 32));
+        unsigned long long any = ((unsigned long long)hi << 32) | lo;
+        alive |= any;
+        for (; any; any &= any - 1ull) {
+            const int r = __ffsll((long long)any) - 1;
+            if ((nv >> r) & 1ull) s.levels[(int64_t)r * s.n + v] = lv - s.lane_start[r];
         }
         const uint32_t ball = __ballot_sync(0xffffffffu, nv != 0ull);
-        unsigned long long any = nv;
+        if (lane == 0) s_cnt[warp] = __popc(ball);
+        __syncthreads();
+        uint32_t before = 0, total = 0;
 #pragma unroll
-        for (int d = 16; d > 0; d >>= 1) any |= __shfl_xor_sync(0xffffffffu, any, d);
-        if (any && lane_id() == 0) atomicOr(&s.alive, any);
-        if (ball) {
-            unsigned long long base = 0;
-            if (lane_id() == 0) base = atomicAdd(&s.act_count[nxt_i], (unsigned long long)__popc(ball));
-            base = __shfl_sync(0xffffffffu, base, 0);
-            const unsigned long long at = base + __popc(ball & ((1u << lane_id()) - 1u));
-            if (nv) {
-                if (at < (unsigned long long)s.n) actn[at] = (int32_t)v;
-                else ms_fault(S, 3, at, (uint64_t)v);
-            }
+        for (int k = 0; k < NW; ++k) {
+            if (k < warp) before += s_cnt[k];
+            total += s_cnt[k];
+        }
+        if (threadIdx.x == 0) s_base = total ? atomicAdd(&s.act_count[nxt_i], (unsigned long long)total) : 0ull;
+        __syncthreads();
+        if (nv) {
+            const unsigned long long at = s_base + before + __popc(ball & ((1u << lane) - 1u));
+            if (at < (unsigned long long)s.n) actn[at] = (int32_t)v;
+            else ms_fault(S, 3, at, (uint64_t)v);
         }
     }
-}
-
-// One thread: switch to the next level and decide whether to iterate again.
-__global__ void ms_finalize(MsState* S, cudaGraphConditionalHandle handle) {
-    MsState& s = *S;
-    const int nxt_i = s.cur ^ 1;
-    const unsigned long long cnt = s.act_count[nxt_i];
-    s.act_count[s.cur] = 0;
-    s.cur = nxt_i;
-    s.level += 1;
-    s.levels_done += 1;
-    s.act_next = 0;
-    s.piece_count = 0;
-    s.piece_next = 0;
-    cudaGraphSetConditional(handle, (cnt > 0 && s.level < s.max_levels) ? 1u : 0u);
-}
-
-// One server iteration ends: switch buffers, advance the iteration.
-__global__ void ms_step_end(MsState* S) {
-    MsState& s = *S;
-    const int nxt_i = s.cur ^ 1;
-    s.act_count[s.cur] = 0;
-    s.cur = nxt_i;
-    s.level += 1;
-    s.levels_done += 1;
-    s.act_next = 0;
-    s.piece_count = 0;
-    s.piece_next = 0;
+    edges = warp_sum(edges);
+    miss = warp_sum(miss);
+    if (lane == 0) {
+        s_any[warp] = alive;
+        s_deg[warp] = edges;
+        s_miss[warp] = miss;
+    }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    for (int k = 1; k < NW; ++k) {
+        alive |= s_any[k];
+        edges += s_deg[k];
+        miss += s_miss[k];
+    }
+    if (alive) atomicOr(&s.alive, alive);
+    if (edges) atomicAdd(&s.act_edges, edges);
+    if (miss) atomicAdd(&s.miss_edges, miss);
+    __threadfence();
+    if (atomicAdd(&s.done, 1u) != gridDim.x - 1) return;
+    __threadfence();
+    s.done = 0;
+    const unsigned long long cnt = __ldcg(&s.act_count[nxt_i]);
+    ms_advance(s, __ldcg(&s.alive));
+    if (use_handle) {
+        s.alive = 0;
+        cudaGraphSetConditional(handle, (cnt > 0 && s.level < s.max_levels) ? 1u : 0u);
+    }
 }
 
 // Admission, phase A: lanes in `mask` start over -- clear their bits in every
@@ -362,9 +605,9 @@ __global__ void ms_admit_clear(MsState* S, unsigned long long mask, const int32_
     const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const unsigned long long keep = ~mask;
     for (int64_t v = tid; v < s.n; v += stride) {
-        if (s.vis[v] & mask) s.vis[v] &= keep;
+        if (s.vn[v].x & mask) s.vn[v].x &= keep;
         if (s.f[s.cur][v] & mask) s.f[s.cur][v] &= keep;
-        if (s.nxt[v] & mask) s.nxt[v] &= keep;
+        if (s.vn[v].y & mask) s.vn[v].y &= keep;
     }
     const int64_t total = (int64_t)nlanes * s.n;
     for (int64_t x = tid; x < total; x += stride) {
@@ -390,7 +633,9 @@ __global__ void ms_admit_roots(MsState* S, const int32_t* lanes, const int32_t* 
     const unsigned long long bit = 1ull << r;
     if (want_parents[q]) atomicOr(&s.parent_mask, bit);
     else atomicAnd(&s.parent_mask, ~bit);
-    atomicOr(s.vis + v, bit);
+    atomicOr(&s.vn[v].x, bit);
+    atomicOr(&s.lanes, bit);
+    s.pull = 0;                              // a new lane's first level: few entries, many vertices missing
     const unsigned long long old = atomicOr(s.f[s.cur] + v, bit);
     s.levels[(int64_t)r * s.n + v] = 0;
     if (s.parents) s.parents[(int64_t)r * s.n + v] = v;
@@ -415,7 +660,7 @@ int ms_sm_count() {
 
 // ---------------------------------------------------------- host side --
 struct MsContext {
-    DevBuf vis, f0, f1, nxt, act0, act1, pieces, state, roots;
+    DevBuf vn, f0, f1, act0, act1, pieces, state, roots;
     int64_t piece_cap = 0;
     cudaGraph_t graph[2] = {nullptr, nullptr};       // [without parents, with parents]
     cudaGraphExec_t exec[2] = {nullptr, nullptr};
@@ -452,10 +697,9 @@ bfs_status ms_ensure(bfs_graph* g) {
     const int64_t n = L.n;
     bfs_status rc = BFS_OK;
     c->piece_cap = L.nnz / kMsPiece + L.nnz / kMsHub + 16;
-    if (rc == BFS_OK) rc = c->vis.alloc(8 * n);
+    if (rc == BFS_OK) rc = c->vn.alloc(16 * n);
     if (rc == BFS_OK) rc = c->f0.alloc(8 * n);
     if (rc == BFS_OK) rc = c->f1.alloc(8 * n);
-    if (rc == BFS_OK) rc = c->nxt.alloc(8 * n);
     if (rc == BFS_OK) rc = c->act0.alloc(4 * n);
     if (rc == BFS_OK) rc = c->act1.alloc(4 * n);
     if (rc == BFS_OK) rc = c->pieces.alloc(sizeof(Item) * c->piece_cap);
@@ -475,10 +719,11 @@ bfs_status ms_ensure(bfs_graph* g) {
     h.nb = L.nb;
     h.n = n;
     h.nnz = L.nnz;
-    h.vis = c->vis.as<unsigned long long>();
+    h.vn = c->vn.as<ulonglong2>();
+    h.deg = L.deg.as<uint32_t>();
+    h.symmetric = g->symmetric;
     h.f[0] = c->f0.as<unsigned long long>();
     h.f[1] = c->f1.as<unsigned long long>();
-    h.nxt = c->nxt.as<unsigned long long>();
     h.act[0] = c->act0.as<int32_t>();
     h.act[1] = c->act1.as<int32_t>();
     h.pieces = c->pieces.as<Item>();
@@ -490,8 +735,22 @@ bfs_status ms_ensure(bfs_graph* g) {
     return BFS_OK;
 }
 
+// One level: from the active vertices or the destinations (the kernels of the
+// other side return at once), then the reduction.
+void launch_ms_level(bfs_graph* g, cudaGraphConditionalHandle handle, int use_handle, cudaStream_t st) {
+    MsContext* c = g->ms;
+    MsState* S = c->state.as<MsState>();
+    const int sms = ms_sm_count();
+    const int64_t ctas = (g->L.n + kMT - 1) / kMT;
+    const size_t scratch = sizeof(MsScratch) * (size_t)(c->expand_threads / 32);
+    ms_expand<<<sms * c->expand_ctas_per_sm, c->expand_threads, scratch, st>>>(S);
+    ms_pieces<<<sms * 4, kMT, 0, st>>>(S);
+    if (g->symmetric) ms_pull<<<(unsigned)std::min<int64_t>(ctas, (int64_t)sms * 8), kMT, 0, st>>>(S);
+    ms_reduce<<<(unsigned)std::min<int64_t>(ctas, (int64_t)sms * 8), kMT, 0, st>>>(S, handle, use_handle);
+}
+
 // Build the batch graph: reset, clear, roots, then WHILE(level) { expand,
-// pieces, reduce, finalize }.
+// pieces, pull, reduce }.
 bfs_status ms_build_graph(bfs_graph* g, int with_parents, cudaStream_t st) {
     MsContext* c = g->ms;
     if (c->exec[with_parents]) return BFS_OK;
@@ -535,10 +794,7 @@ bfs_status ms_build_graph(bfs_graph* g, int with_parents, cudaStream_t st) {
     BFS_CUDA_TRY(cudaGraphAddNode(&cond, graph, &last, nullptr, 1, &cp));
     cudaGraph_t body = cp.conditional.phGraph_out[0];
     BFS_CUDA_TRY(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
-    ms_expand<<<sms * c->expand_ctas_per_sm, c->expand_threads, 0, cs>>>(S);
-    ms_pieces<<<sms * 4, kMT, 0, cs>>>(S);
-    ms_reduce<<<sms * 8, kMT, 0, cs>>>(S);
-    ms_finalize<<<1, 1, 0, cs>>>(S, handle);
+    launch_ms_level(g, handle, 1, cs);
     ce = cudaStreamEndCapture(cs, &body);
     cudaStreamDestroy(cs);
     if (ce != cudaSuccess) {
@@ -755,14 +1011,8 @@ namespace {
 constexpr int64_t kMaxQueued = 1 << 20;      // default queue limit (bfs_server_set_queue_limit)
 
 bfs_status build_step_graph(ServeGraph* sg) {
-    MsContext* c = sg->g->ms;
-    MsState* S = c->state.as<MsState>();
-    const int sms = ms_sm_count();
     BFS_CUDA_TRY(cudaStreamBeginCapture(sg->stream, cudaStreamCaptureModeThreadLocal));
-    ms_expand<<<sms * c->expand_ctas_per_sm, c->expand_threads, 0, sg->stream>>>(S);
-    ms_pieces<<<sms * 4, kMT, 0, sg->stream>>>(S);
-    ms_reduce<<<sms * 8, kMT, 0, sg->stream>>>(S);
-    ms_step_end<<<1, 1, 0, sg->stream>>>(S);
+    launch_ms_level(sg->g, cudaGraphConditionalHandle{}, 0, sg->stream);
     cudaGraph_t graph = nullptr;
     BFS_CUDA_TRY(cudaStreamEndCapture(sg->stream, &graph));
     cudaGraphExec_t exec = nullptr;
