@@ -102,6 +102,7 @@ struct LevelArgs {
     const uint32_t* pi;
     uint32_t* t;
     const uint8_t* fsum;                // frontier summary: 1 per 1024 bits of f with a set bit
+    const uint32_t* fwords;             // the same per word: bit w of fwords says that word w of f is nonzero
     int32_t* parent;
     // exchange
     const void* xbuf;
@@ -1388,26 +1389,23 @@ __global__ void __launch_bounds__(kNT) decode_streams(LevelArgs a) {
 // one by the whole warp (kIlp x 32 entries per step); the warp's next bits
 // are one store (t is clear and no other kernel writes it this level).
 constexpr int64_t kBuLane = 32;
+constexpr int kBuIlp = 8;           // entries of a short row in flight
 
-__device__ __forceinline__ uint32_t warp_min(uint32_t x) {
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-        const uint32_t y = __shfl_xor_sync(0xffffffffu, x, d);
-        x = y < x ? y : x;
-    }
-    return x;
-}
-
+// The frontier test of an entry u.  A sparse frontier is tested word-wise
+// first: `words` has a bit per 32 vertices (64 KB at scale 24, in L1, where
+// the bitmap is 2 MB: 940 against 326 G scattered reads a second).
 struct BuFrontier {
     const uint32_t* g;        // the decoded streams, or the raw frontier (PLAIN)
-    uint32_t nb;
-    // the range of u and whether the frontier delivered to block (i, range) holds u
-    __device__ __forceinline__ uint32_t test(uint32_t u, uint32_t& j) const {
-        j = u / nb;
-        return (__ldg(g + (u >> 5)) >> (u & 31u)) & 1u;
+    const uint32_t* words;    // bit (u / 32): the frontier has a vertex in that word; nullptr: a dense frontier
+    __device__ __forceinline__ bool maybe(uint32_t u) const {
+        return !words || ((__ldg(words + (u >> 10)) >> ((u >> 5) & 31u)) & 1u);
     }
+    // whether the frontier delivered to block (i, range of u) holds u
+    __device__ __forceinline__ bool test(uint32_t u) const { return (__ldg(g + (u >> 5)) >> (u & 31u)) & 1u; }
 };
 
+// STATS: also count the columns and entries read (the stepwise loop asks for them).
+template <bool STATS>
 __global__ void __launch_bounds__(kNT) expand_bottom_up(LevelArgs a) {
     if (!a.ctl->bu) return;
     const int64_t words = (a.n + 31) >> 5;
@@ -1415,6 +1413,7 @@ __global__ void __launch_bounds__(kNT) expand_bottom_up(LevelArgs a) {
     const int64_t gstride = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const uint32_t nb = (uint32_t)a.nb;                                // n < 2^31
     const uint32_t NONE = 0xffffffffu;
+    const BuFrontier fr{a.mode != BFS_MODE_PLAIN ? a.gbits : a.f, a.ctl->frontier * 64 < a.n ? a.fwords : nullptr};
     unsigned long long edges = 0, cols = 0;
     for (int64_t w = gw0; w < words; w += gstride) {
         const uint32_t piw = __ldg(a.pi + w);
@@ -1426,30 +1425,43 @@ __global__ void __launch_bounds__(kNT) expand_bottom_up(LevelArgs a) {
             e0 = __ldg(a.bu_ptr + v);
             e1 = __ldg(a.bu_ptr + v + 1);
         }
-        const BuFrontier fr{a.mode != BFS_MODE_PLAIN ? a.gbits : a.f, nb};
         uint32_t best = NONE;
         if (mine && e1 - e0 <= kBuLane) {
-            uint32_t cur = NONE;                                        // range of the entries so far
-            for (int64_t e = e0; e < e1; e += kIlp) {
-                const int cnt = (e1 - e < kIlp) ? (int)(e1 - e) : kIlp;
-                uint32_t u[kIlp], j[kIlp], hit[kIlp];
+            uint32_t rend = 0;              // end of the range of the entries so far (STATS), of best's range (else)
+            bool stop = false;
+            for (int64_t e = e0; e < e1 && !stop; e += kBuIlp) {
+                uint32_t u[kBuIlp];
+                bool hit[kBuIlp];
+                bool some = false;
 #pragma unroll
-                for (int k = 0; k < kIlp; ++k) u[k] = (k < cnt) ? (uint32_t)__ldg(a.bu_adj + e + k) : 0u;
+                for (int k = 0; k < kBuIlp; ++k) u[k] = (e + k < e1) ? (uint32_t)__ldg(a.bu_adj + e + k) : NONE;
 #pragma unroll
-                for (int k = 0; k < kIlp; ++k) hit[k] = (k < cnt) ? fr.test(u[k], j[k]) : 0u;
-                bool stop = false;
+                for (int k = 0; k < kBuIlp; ++k) hit[k] = u[k] != NONE && fr.maybe(u[k]);
 #pragma unroll
-                for (int k = 0; k < kIlp; ++k) {
-                    if (k >= cnt || stop) continue;
-                    if (j[k] != cur) {                                  // a new range
-                        if (best != NONE) { stop = true; continue; }
-                        cur = j[k];
-                        ++cols;
-                    }
-                    ++edges;
-                    if (hit[k] && u[k] < best) best = u[k];
+                for (int k = 0; k < kBuIlp; ++k) {
+                    if (hit[k]) hit[k] = fr.test(u[k]);
+                    some |= hit[k];
                 }
-                if (stop) break;
+                if (!STATS && !some && best == NONE) continue;
+#pragma unroll
+                for (int k = 0; k < kBuIlp; ++k) {
+                    if (u[k] == NONE || stop) continue;
+                    if (STATS) {
+                        if (u[k] >= rend) {                             // a new range
+                            if (best != NONE) { stop = true; continue; }
+                            rend = (u[k] / nb + 1u) * nb;
+                            ++cols;
+                        }
+                        ++edges;
+                    } else if (best != NONE && u[k] >= rend) {
+                        stop = true;                                    // past the range of the first hit
+                        continue;
+                    }
+                    if (hit[k]) {
+                        if (!STATS && best == NONE) rend = (u[k] / nb + 1u) * nb;
+                        best = u[k] < best ? u[k] : best;
+                    }
+                }
             }
         }
         // long rows, one after the other, by the whole warp
@@ -1459,42 +1471,44 @@ __global__ void __launch_bounds__(kNT) expand_bottom_up(LevelArgs a) {
             lm &= lm - 1;
             const int64_t b0 = __shfl_sync(0xffffffffu, e0, o), b1 = __shfl_sync(0xffffffffu, e1, o);
             uint32_t wb = NONE, wend = NONE;                            // best so far and the end of its range
-            uint32_t jlast = NONE;                                      // range of the last entry scanned
+            uint32_t jlast = NONE;                                      // range of the last entry scanned (STATS)
             for (int64_t e = b0; e < b1; e += kIlp * 32) {
-                uint32_t u[kIlp], j[kIlp], hit[kIlp];
+                uint32_t u[kIlp];
+                bool hit[kIlp];
 #pragma unroll
                 for (int k = 0; k < kIlp; ++k) {
                     const int64_t x = e + k * 32 + lane_id();
                     u[k] = (x < b1) ? (uint32_t)__ldg(a.bu_adj + x) : NONE;
                 }
 #pragma unroll
-                for (int k = 0; k < kIlp; ++k) {
-                    hit[k] = 0u;
-                    j[k] = NONE;
-                    if (u[k] != NONE) hit[k] = fr.test(u[k], j[k]);
-                }
+                for (int k = 0; k < kIlp; ++k) hit[k] = u[k] != NONE && fr.maybe(u[k]);
                 uint32_t cand = NONE;
                 bool past = false;
 #pragma unroll
                 for (int k = 0; k < kIlp; ++k) {
-                    if (hit[k] && u[k] < cand) cand = u[k];
-                    // entries (in row order) that open a range
-                    uint32_t jp = __shfl_up_sync(0xffffffffu, j[k], 1);
-                    if (lane_id() == 0) jp = jlast;
-                    const uint32_t opens = __ballot_sync(0xffffffffu, u[k] != NONE && j[k] != jp);
-                    const uint32_t valid = __ballot_sync(0xffffffffu, u[k] != NONE);
-                    if (lane_id() == (uint32_t)o) { cols += __popc(opens); edges += __popc(valid); }
-                    const uint32_t jl = __shfl_sync(0xffffffffu, j[k], 31);
-                    if (jl != NONE) jlast = jl;
+                    if (hit[k] && u[k] < cand && fr.test(u[k])) cand = u[k];
+                    if (STATS) {            // entries (in row order) that open a range
+                        const uint32_t j = u[k] != NONE ? u[k] / nb : NONE;
+                        uint32_t jp = __shfl_up_sync(0xffffffffu, j, 1);
+                        if (lane_id() == 0) jp = jlast;
+                        const uint32_t opens = __ballot_sync(0xffffffffu, u[k] != NONE && j != jp);
+                        const uint32_t valid = __ballot_sync(0xffffffffu, u[k] != NONE);
+                        if (lane_id() == (uint32_t)o) { cols += __popc(opens); edges += __popc(valid); }
+                        const uint32_t jl = __shfl_sync(0xffffffffu, j, 31);
+                        if (jl != NONE) jlast = jl;
+                    }
                 }
-                cand = warp_min(cand);
-                if (cand < wb) {
-                    wb = cand;
-                    wend = (uint32_t)range_begin(a, cand / nb + 1);
+                if (__any_sync(0xffffffffu, cand != NONE)) {
+                    cand = __reduce_min_sync(0xffffffffu, cand);
+                    if (cand < wb) {
+                        wb = cand;
+                        wend = (uint32_t)range_begin(a, cand / nb + 1);
+                    }
                 }
+                if (wb == NONE) continue;
 #pragma unroll
                 for (int k = 0; k < kIlp; ++k) past |= u[k] != NONE && u[k] >= wend;
-                if (wb != NONE && __any_sync(0xffffffffu, past)) break;   // the best's range is complete
+                if (__any_sync(0xffffffffu, past)) break;               // the best's range is complete
             }
             if (lane_id() == (uint32_t)o) best = wb;
         }
@@ -1503,8 +1517,8 @@ __global__ void __launch_bounds__(kNT) expand_bottom_up(LevelArgs a) {
         const uint32_t m = __ballot_sync(0xffffffffu, found);
         if (lane_id() == 0 && m) a.t[w] = m;
     }
-    flush_counts(a, edges, cols);
-    if (blockIdx.x == 0 && threadIdx.x == 0) a.ctr[C_BOTTOM_UP] = 1ull;
+    if (STATS) flush_counts(a, edges, cols);
+    if (STATS && blockIdx.x == 0 && threadIdx.x == 0) a.ctr[C_BOTTOM_UP] = 1ull;
 }
 
 // ---------------------------------------------------------------- reduce --
@@ -1569,11 +1583,12 @@ constexpr int64_t kSmallReduce = 1 << 20;
 template <int WPW>
 __global__ void __launch_bounds__(kNT) reduce_level(uint32_t* __restrict__ t, uint32_t* __restrict__ pi,
                                                     uint32_t* __restrict__ f, uint8_t* __restrict__ fsum,
-                                                    int64_t words, int64_t n, int32_t* __restrict__ level,
-                                                    LevelCtl* ctl, unsigned long long* ctr,
+                                                    uint32_t* __restrict__ fwords, int64_t words, int64_t n,
+                                                    int32_t* __restrict__ level, LevelCtl* ctl, unsigned long long* ctr,
                                                     const uint32_t* __restrict__ deg, NextArgs nx) {
     constexpr int W = kNT / 32;                         // warps
     __shared__ unsigned long long s_sum[2][W];
+    __shared__ uint32_t s_any[W];
     __shared__ int s_last;
     const int32_t next_level = ctl->level + 1;
     const int lane = (int)lane_id(), warp = (int)(threadIdx.x >> 5);
@@ -1608,10 +1623,20 @@ __global__ void __launch_bounds__(kNT) reduce_level(uint32_t* __restrict__ t, ui
             dsum += (unsigned long long)d[0] + d[1] + d[2] + d[3];
         }
         if (WPW == 32) {
-            if (lane == 0) fsum[wb >> 5] = any ? 1 : 0;
+            if (lane == 0) {
+                fsum[wb >> 5] = any ? 1 : 0;
+                fwords[wb >> 5] = any;
+            }
         } else {                                        // the CTA's words are one byte of the summary
-            const int some = __syncthreads_or(any != 0u);
-            if (threadIdx.x == 0) fsum[w0 >> 5] = some ? 1 : 0;
+            __syncthreads();                            // the previous round's masks are read
+            if (lane == 0) s_any[warp] = any << (WPW * warp & 31);
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                uint32_t all = 0;
+                for (int k = 0; k < W; ++k) all |= s_any[k];
+                fsum[w0 >> 5] = all ? 1 : 0;
+                fwords[w0 >> 5] = all;
+            }
         }
     }
     static_assert(WPW == 32 || W * WPW == 32, "a warp or a CTA covers one byte of the frontier summary");
@@ -1667,7 +1692,7 @@ __global__ void level_first(LevelCtl* c, int64_t n, int win_ratio, int policy, i
 // the bottom-up scans skip them.
 __global__ void init_search(int32_t* __restrict__ level, int32_t* __restrict__ parent, int64_t n,
                             uint32_t* __restrict__ pi, uint32_t* __restrict__ fa, uint32_t* __restrict__ fb,
-                            int64_t words, uint8_t* __restrict__ fsum, int64_t fsum_len,
+                            int64_t words, uint8_t* __restrict__ fsum, uint32_t* __restrict__ fwords, int64_t fsum_len,
                             const uint32_t* __restrict__ iso) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += stride) {
@@ -1679,15 +1704,20 @@ __global__ void init_search(int32_t* __restrict__ level, int32_t* __restrict__ p
         fa[w] = 0u;
         fb[w] = 0u;
     }
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < fsum_len; q += stride) fsum[q] = 0;
+    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < fsum_len; q += stride) {
+        fsum[q] = 0;
+        fwords[q] = 0u;
+    }
 }
 
-__global__ void set_root(int32_t* level, int32_t* parent, uint32_t* pi, uint32_t* fa, uint8_t* fsum, int32_t root) {
+__global__ void set_root(int32_t* level, int32_t* parent, uint32_t* pi, uint32_t* fa, uint8_t* fsum, uint32_t* fwords,
+                         int32_t root) {
     level[root] = 0;
     parent[root] = root;
     pi[root >> 5] |= 1u << (root & 31);
     fa[root >> 5] |= 1u << (root & 31);
     fsum[root >> 10] = 1;
+    fwords[root >> 10] |= 1u << ((root >> 5) & 31);
 }
 
 // Pack the streams of this exchange into a trace (the receive buffer g'):
@@ -1863,6 +1893,7 @@ bfs_status ensure_workspace_once(bfs_graph* g) {
                                   {&W.fa, (size_t)(4 * W.bm_words)},
                                   {&W.fb, (size_t)(4 * W.bm_words)},
                                   {&W.fsum, (size_t)W.fsum_len},
+                                  {&W.fwords, sizeof(uint32_t) * (size_t)W.fsum_len},
                                   {&W.xbuf, (size_t)xbytes},
                                   {&W.xcount, sizeof(int64_t) * p2},
                                   {&W.chunk_base, sizeof(int64_t) * p2 * W.chunks_per_slot},
@@ -1900,7 +1931,7 @@ bfs_status ensure_workspace_once(bfs_graph* g) {
 
 void free_workspace(bfs_graph* g) {
     Workspace& W = g->W;
-    W.pi.release(); W.fa.release(); W.fb.release(); W.fsum.release(); W.xbuf.release();
+    W.pi.release(); W.fa.release(); W.fb.release(); W.fsum.release(); W.fwords.release(); W.xbuf.release();
     W.xcount.release(); W.chunk_base.release(); W.units.release(); W.counters.release(); W.pieces.release();
     W.level_scratch.release(); W.row_meta.release();
     W.tblk.release(); W.rowbuf.release(); W.rowcount.release(); W.rowfirst.release(); W.rowlive.release();
@@ -2030,10 +2061,12 @@ bfs_status run_search(bfs_graph* g, int32_t root, int32_t* parent, int32_t* leve
     if (stats) { stats->n_levels = 0; stats->trace_used = 0; stats->row_trace_used = 0; }
 
     init_search<<<sm_count() * 4, kNT, 0, st>>>(level, parent, L.n, W.pi.as<uint32_t>(), W.fa.as<uint32_t>(),
-                                                W.fb.as<uint32_t>(), W.bm_words, W.fsum.as<uint8_t>(), W.fsum_len,
+                                                W.fb.as<uint32_t>(), W.bm_words, W.fsum.as<uint8_t>(), W.fwords.as<uint32_t>(),
+                                                W.fsum_len,
                                                 bu_kernels ? L.iso.as<uint32_t>() : nullptr);
     BFS_CUDA_TRY(cudaGetLastError());
-    set_root<<<1, 1, 0, st>>>(level, parent, W.pi.as<uint32_t>(), W.fa.as<uint32_t>(), W.fsum.as<uint8_t>(), root);
+    set_root<<<1, 1, 0, st>>>(level, parent, W.pi.as<uint32_t>(), W.fa.as<uint32_t>(), W.fsum.as<uint8_t>(),
+                              W.fwords.as<uint32_t>(), root);
     BFS_CUDA_TRY(cudaGetLastError());
     BFS_CUDA_TRY(cudaMemsetAsync(ctr, 0, sizeof(unsigned long long) * C_NUM, st));
 
@@ -2140,6 +2173,7 @@ bfs_status run_search(bfs_graph* g, int32_t root, int32_t* parent, int32_t* leve
     a.f = f;
     a.t = t;
     a.fsum = W.fsum.as<uint8_t>();
+    a.fwords = W.fwords.as<uint32_t>();
     a.ctl = ctl;
     ea.frontier = f;
     ra.skip = &ctl->bu;                      // bottom-up levels have no row exchange
@@ -2210,7 +2244,8 @@ bfs_status run_search(bfs_graph* g, int32_t root, int32_t* parent, int32_t* leve
         }
         BFS_CUDA_TRY(cudaGetLastError());
         if (bu_kernels) {
-            expand_bottom_up<<<sm_count() * 8, kNT, 0, s>>>(a);
+            if (host) expand_bottom_up<true><<<sm_count() * 8, kNT, 0, s>>>(a);
+            else expand_bottom_up<false><<<sm_count() * 8, kNT, 0, s>>>(a);
             BFS_CUDA_TRY(cudaGetLastError());
         }
         if (host && timing) cudaEventRecord(W.ev[3], s);
@@ -2246,10 +2281,12 @@ bfs_status run_search(bfs_graph* g, int32_t root, int32_t* parent, int32_t* leve
         const NextArgs nx{L.n, max_levels, handle, host ? 0 : 1, lvl, 3 * p + 1};
         if (L.n < kSmallReduce)
             reduce_level<4><<<(unsigned)((W.bm_words + 31) / 32), kNT, 0, s>>>(
-                t, W.pi.as<uint32_t>(), f, W.fsum.as<uint8_t>(), W.bm_words, L.n, level, ctl, ctr, deg, nx);
+                t, W.pi.as<uint32_t>(), f, W.fsum.as<uint8_t>(), W.fwords.as<uint32_t>(), W.bm_words, L.n, level, ctl,
+                ctr, deg, nx);
         else
             reduce_level<32><<<std::min<int64_t>((W.bm_words + 255) / 256, sm_count() * 16), kNT, 0, s>>>(
-                t, W.pi.as<uint32_t>(), f, W.fsum.as<uint8_t>(), W.bm_words, L.n, level, ctl, ctr, deg, nx);
+                t, W.pi.as<uint32_t>(), f, W.fsum.as<uint8_t>(), W.fwords.as<uint32_t>(), W.bm_words, L.n, level, ctl,
+                ctr, deg, nx);
         BFS_CUDA_TRY(cudaGetLastError());
         if (host && timing) cudaEventRecord(W.ev[4], s);
         return BFS_OK;

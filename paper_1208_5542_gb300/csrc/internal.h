@@ -162,7 +162,7 @@ struct SearchGraph {
 // Per-search workspace (owned by the graph, reused by every search).
 struct Workspace {
     int64_t bm_words = 0;       // uint32 words of an n-bit bitmap (padded)
-    int64_t fsum_len = 0;       // bytes of the frontier summary (1 per 1024 bits)
+    int64_t fsum_len = 0;       // bytes of the frontier summary (1 per 1024 bits), words of its word-wise one
     int64_t slot_cap = 0;       // words (of the WAH width) per exchange slot
     int64_t chunk_words = 0;    // words per expansion chunk of a stream
     int64_t chunks_per_slot = 0;
@@ -170,7 +170,7 @@ struct Workspace {
     int wah_bits = 0;
     int mode = -1;
     DevBuf whole;               // the allocation that holds what every search needs
-    DevBuf pi, fa, fb, fsum, xbuf, xcount, chunk_base, units, counters, pieces;
+    DevBuf pi, fa, fb, fsum, fwords, xbuf, xcount, chunk_base, units, counters, pieces;
     DevBuf level_scratch;       // per-level work counters (3 per row)
     DevBuf row_meta;            // per-row piece bases and capacities
     int64_t piece_cap = 0;      // capacity of `pieces` (Item entries)
