@@ -83,9 +83,12 @@ struct MsState {
     // continuous batching (server): lane r's level of v is (iteration + 1) - lane_start[r]
     int32_t lane_start[64];
     unsigned long long alive;        // lanes that reached a new vertex in this iteration
-    int64_t nnz;                     // entries of the layout
+    unsigned long long steps;        // iterations of this launch
     unsigned long long err;          // first failed bounds check: code, then two values
     unsigned long long err_a, err_b;
+    unsigned long long running;      // lanes of this launch
+    const volatile int* call;        // mapped host word: nonzero asks the iterations to end
+    int64_t nnz;                     // entries of the layout
 };
 
 // A bounds check failed: keep the first one's code and values (the access is skipped).
@@ -516,9 +519,13 @@ __device__ void ms_advance(MsState& s, unsigned long long alive) {
 // new = nxt & ~vis; vis |= new; f' = new; level of every new lane, lane by lane
 // over the warp's vertices (coalesced stores); next active list, one hand-out
 // of places per CTA.  The last CTA to finish (a counter, no waiting) switches
-// to the next level; in the batch's loop (use_handle) it decides whether to
-// iterate again, in the server's step it leaves `alive` for the host.
-__global__ void __launch_bounds__(kMT) ms_reduce(MsState* S, cudaGraphConditionalHandle handle, int use_handle) {
+// to the next level and decides whether to iterate again: a batch while a lane
+// has a frontier vertex; a server's launch while every running lane has one,
+// the host does not call and fewer than kMsSteps levels ran (the host retires
+// and admits lanes between launches).
+constexpr unsigned long long kMsSteps = 1024;
+
+__global__ void __launch_bounds__(kMT) ms_reduce(MsState* S, cudaGraphConditionalHandle handle, int server) {
     constexpr int NW = kMT / 32;
     __shared__ uint32_t s_cnt[NW];
     __shared__ unsigned long long s_base, s_any[NW], s_deg[NW], s_miss[NW];
@@ -589,17 +596,23 @@ __global__ void __launch_bounds__(kMT) ms_reduce(MsState* S, cudaGraphConditiona
     if (atomicAdd(&s.done, 1u) != gridDim.x - 1) return;
     __threadfence();
     s.done = 0;
-    const unsigned long long cnt = __ldcg(&s.act_count[nxt_i]);
-    ms_advance(s, __ldcg(&s.alive));
-    if (use_handle) {
-        s.alive = 0;
-        cudaGraphSetConditional(handle, (cnt > 0 && s.level < s.max_levels) ? 1u : 0u);
+    const unsigned long long cnt = __ldcg(&s.act_count[nxt_i]), any = __ldcg(&s.alive);
+    ms_advance(s, any);
+    bool go;
+    if (server) {
+        s.steps += 1;
+        go = (s.running & ~any) == 0ull && s.steps < kMsSteps && s.err == 0ull && *s.call == 0;
+    } else {
+        go = cnt > 0 && s.level < s.max_levels;
     }
+    if (go || !server) s.alive = 0;                 // a server's host reads the last iteration's
+    cudaGraphSetConditional(handle, go ? 1u : 0u);
 }
 
 // Admission, phase A: lanes in `mask` start over -- clear their bits in every
 // lane word and their level rows.
-__global__ void ms_admit_clear(MsState* S, unsigned long long mask, const int32_t* lanes, int nlanes) {
+__global__ void ms_admit_clear(MsState* S, unsigned long long mask, const int32_t* lanes, int nlanes,
+                               unsigned long long running) {
     MsState& s = *S;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -617,7 +630,11 @@ __global__ void ms_admit_clear(MsState* S, unsigned long long mask, const int32_
         s.levels[(int64_t)r * s.n + (x - q * s.n)] = -1;
         if (s.parents) s.parents[(int64_t)r * s.n + (x - q * s.n)] = -1;
     }
-    if (tid == 0) s.alive = 0;
+    if (tid == 0) {
+        s.alive = 0;
+        s.steps = 0;
+        s.running = running;
+    }
 }
 
 // Admission, phase B: lane lanes[q] starts from roots[q] at this iteration,
@@ -647,7 +664,11 @@ __global__ void ms_admit_roots(MsState* S, const int32_t* lanes, const int32_t* 
     }
 }
 
-__global__ void ms_clear_alive(MsState* S) { S->alive = 0; }
+__global__ void ms_launch(MsState* S, unsigned long long running) {
+    S->alive = 0;
+    S->steps = 0;
+    S->running = running;
+}
 
 int ms_sm_count() {
     int dev = 0, v = 0;
@@ -737,7 +758,7 @@ bfs_status ms_ensure(bfs_graph* g) {
 
 // One level: from the active vertices or the destinations (the kernels of the
 // other side return at once), then the reduction.
-void launch_ms_level(bfs_graph* g, cudaGraphConditionalHandle handle, int use_handle, cudaStream_t st) {
+void launch_ms_level(bfs_graph* g, cudaGraphConditionalHandle handle, int server, cudaStream_t st) {
     MsContext* c = g->ms;
     MsState* S = c->state.as<MsState>();
     const int sms = ms_sm_count();
@@ -746,7 +767,7 @@ void launch_ms_level(bfs_graph* g, cudaGraphConditionalHandle handle, int use_ha
     ms_expand<<<sms * c->expand_ctas_per_sm, c->expand_threads, scratch, st>>>(S);
     ms_pieces<<<sms * 4, kMT, 0, st>>>(S);
     if (g->symmetric) ms_pull<<<(unsigned)std::min<int64_t>(ctas, (int64_t)sms * 8), kMT, 0, st>>>(S);
-    ms_reduce<<<(unsigned)std::min<int64_t>(ctas, (int64_t)sms * 8), kMT, 0, st>>>(S, handle, use_handle);
+    ms_reduce<<<(unsigned)std::min<int64_t>(ctas, (int64_t)sms * 8), kMT, 0, st>>>(S, handle, server);
 }
 
 // Build the batch graph: reset, clear, roots, then WHILE(level) { expand,
@@ -794,7 +815,7 @@ bfs_status ms_build_graph(bfs_graph* g, int with_parents, cudaStream_t st) {
     BFS_CUDA_TRY(cudaGraphAddNode(&cond, graph, &last, nullptr, 1, &cp));
     cudaGraph_t body = cp.conditional.phGraph_out[0];
     BFS_CUDA_TRY(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
-    launch_ms_level(g, handle, 1, cs);
+    launch_ms_level(g, handle, 0, cs);
     ce = cudaStreamEndCapture(cs, &body);
     cudaStreamDestroy(cs);
     if (ce != cudaSuccess) {
@@ -959,14 +980,15 @@ struct ServeGraph {
     bool lane_parents[64] = {};      // the query running in lane r asked for parents
     int32_t* h_admit = nullptr;      // pinned staging of `admit`
     unsigned long long* h_alive = nullptr;   // pinned copy of the alive mask
-    cudaGraphExec_t step = nullptr;  // expand, pieces, reduce, step end
+    int* h_call = nullptr;           // mapped: asks a launch's iterations to end (MsState::call)
+    cudaGraphExec_t step = nullptr;  // WHILE(level): iterations until a lane ends or the host calls
     cudaGraph_t step_graph = nullptr;
     int64_t lane_ticket[64];
     unsigned long long running = 0;
     std::deque<int64_t> pending;
     int64_t footprint = 0;
     int64_t iterations = 0;
-    bool inflight = false;           // an iteration is on the stream
+    std::atomic<bool> inflight{false};   // a launch is on the stream
     unsigned long long before = 0;   // lanes running in it
 };
 
@@ -983,6 +1005,7 @@ struct Request {
 }  // namespace bfsgb
 
 struct bfs_server {
+    cudaMemPool_t pool = nullptr;    // results; keeps up to kScratchKept bytes between them
     int64_t budget = 0;
     int64_t used = 0;                // resident graphs
     int64_t results_bytes = 0;       // results awaiting collection
@@ -1010,15 +1033,30 @@ namespace {
 
 constexpr int64_t kMaxQueued = 1 << 20;      // default queue limit (bfs_server_set_queue_limit)
 
+// A launch runs iterations on the device until a lane's frontier empties (its
+// result is to be handed out, its place given to a queued request) or the host
+// calls: no host round trip per level, as each used to cost (60-100 us with the
+// worker's polling, several times the level on small graphs).
 bfs_status build_step_graph(ServeGraph* sg) {
-    BFS_CUDA_TRY(cudaStreamBeginCapture(sg->stream, cudaStreamCaptureModeThreadLocal));
-    launch_ms_level(sg->g, cudaGraphConditionalHandle{}, 0, sg->stream);
     cudaGraph_t graph = nullptr;
-    BFS_CUDA_TRY(cudaStreamEndCapture(sg->stream, &graph));
+    BFS_CUDA_TRY(cudaGraphCreate(&graph, 0));
+    sg->step_graph = graph;                        // released with the server graph
+    cudaGraphConditionalHandle handle;
+    BFS_CUDA_TRY(cudaGraphConditionalHandleCreate(&handle, graph, 1, cudaGraphCondAssignDefault));
+    cudaGraphNodeParams cp = {};
+    cp.type = cudaGraphNodeTypeConditional;
+    cp.conditional.handle = handle;
+    cp.conditional.type = cudaGraphCondTypeWhile;
+    cp.conditional.size = 1;
+    cudaGraphNode_t cond = nullptr;
+    BFS_CUDA_TRY(cudaGraphAddNode(&cond, graph, nullptr, nullptr, 0, &cp));
+    cudaGraph_t body = cp.conditional.phGraph_out[0];
+    BFS_CUDA_TRY(cudaStreamBeginCaptureToGraph(sg->stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
+    launch_ms_level(sg->g, handle, 1, sg->stream);
+    BFS_CUDA_TRY(cudaStreamEndCapture(sg->stream, &body));
     cudaGraphExec_t exec = nullptr;
     cudaError_t e = cudaGraphInstantiate(&exec, graph, 0);
-    if (e != cudaSuccess) { cudaGraphDestroy(graph); return cuda_error(e, "cudaGraphInstantiate(step)", __FILE__, __LINE__); }
-    sg->step_graph = graph;
+    if (e != cudaSuccess) return cuda_error(e, "cudaGraphInstantiate(step)", __FILE__, __LINE__);
     sg->step = exec;
     return BFS_OK;
 }
@@ -1029,6 +1067,7 @@ void release_graph(ServeGraph* sg) {
     if (sg->step_graph) cudaGraphDestroy(sg->step_graph);
     if (sg->h_admit) cudaFreeHost(sg->h_admit);
     if (sg->h_alive) cudaFreeHost(sg->h_alive);
+    if (sg->h_call) cudaFreeHost(sg->h_call);
     if (sg->stream) cudaStreamDestroy(sg->stream);
     sg->levels.release();
     sg->parents.release();
@@ -1063,7 +1102,7 @@ bool finish_iteration(bfs_server* s, ServeGraph* sg) {
         if (!(done & (1ull << r))) continue;
         void* buf = nullptr;
         const int rows = sg->lane_parents[r] ? 2 : 1;
-        if (cudaMallocAsync(&buf, rows * sizeof(int32_t) * n, sg->stream) != cudaSuccess) { fail(s, "result allocation failed"); return false; }
+        if (cudaMallocFromPoolAsync(&buf, rows * sizeof(int32_t) * n, s->pool, sg->stream) != cudaSuccess) { fail(s, "result allocation failed"); return false; }
         cudaMemcpyAsync(buf, sg->levels.as<int32_t>() + (int64_t)r * n, sizeof(int32_t) * n,
                         cudaMemcpyDeviceToDevice, sg->stream);
         if (rows == 2)
@@ -1075,8 +1114,8 @@ bool finish_iteration(bfs_server* s, ServeGraph* sg) {
     if (!fin.empty() && cudaStreamSynchronize(sg->stream) != cudaSuccess) { fail(s, "result copy failed"); return false; }
     std::lock_guard<std::mutex> lk(s->mu);
     sg->running &= ~done;
-    ++sg->iterations;
-    ++s->iterations;
+    sg->iterations += (int64_t)sg->h_alive[1];
+    s->iterations += (int64_t)sg->h_alive[1];
     const auto now = std::chrono::steady_clock::now();
     for (auto& f : fin) {
         Request& q = s->req[f.first];
@@ -1089,6 +1128,13 @@ bool finish_iteration(bfs_server* s, ServeGraph* sg) {
     }
     if (!fin.empty()) s->cv_done.notify_all();
     return true;
+}
+
+// With the server's lock held: a launch in flight ends after its current level
+// if a queued request could take a free lane.
+void call(ServeGraph* sg) {
+    const unsigned long long all = sg->lanes < 64 ? (1ull << sg->lanes) - 1ull : ~0ull;
+    if (sg->inflight && !sg->pending.empty() && (sg->running & all) != all) *static_cast<volatile int*>(sg->h_call) = 1;
 }
 
 bool launch_iteration(bfs_server* s, ServeGraph* sg) {
@@ -1116,22 +1162,23 @@ bool launch_iteration(bfs_server* s, ServeGraph* sg) {
         ++nadm;
     }
     if (!sg->running) return false;
+    *static_cast<volatile int*>(sg->h_call) = 0;     // under the lock: a later call stands
     MsState* S = sg->g->ms->state.as<MsState>();
     if (nadm) {
         int32_t* d = sg->admit.as<int32_t>();
         if (cudaMemcpyAsync(d, sg->h_admit, sizeof(int32_t) * 192, cudaMemcpyHostToDevice, sg->stream) != cudaSuccess) {
             lk.unlock(); fail(s, "admission copy failed"); return false;
         }
-        ms_admit_clear<<<ms_sm_count() * 4, kMT, 0, sg->stream>>>(S, mask, d, nadm);
+        ms_admit_clear<<<ms_sm_count() * 4, kMT, 0, sg->stream>>>(S, mask, d, nadm, sg->running);
         ms_admit_roots<<<1, 64, 0, sg->stream>>>(S, d, d + 64, d + 128, nadm);
     } else {
-        ms_clear_alive<<<1, 1, 0, sg->stream>>>(S);
+        ms_launch<<<1, 1, 0, sg->stream>>>(S, sg->running);
     }
     if (cudaGraphLaunch(sg->step, sg->stream) != cudaSuccess) {
         lk.unlock(); fail(s, "iteration launch failed"); return false;
     }
     cudaMemcpyAsync(sg->h_alive, reinterpret_cast<char*>(S) + offsetof(MsState, alive),
-                    sizeof(unsigned long long) * 5, cudaMemcpyDeviceToHost, sg->stream);   // alive, nnz, err, a, b
+                    sizeof(unsigned long long) * 5, cudaMemcpyDeviceToHost, sg->stream);   // alive, steps, err, a, b
     sg->before = sg->running;
     sg->inflight = true;
     int lanes_now = 0;
@@ -1167,16 +1214,24 @@ bool serve_pass(bfs_server* s) {
 
 void serve_loop(bfs_server* s) {
     cudaSetDevice(s->device);
+    // a sleep takes some 70 us however short it is meant to be: the worker polls
+    // that long before it sleeps
+    constexpr int kSpins = 64;
+    int idle = 0;
     for (;;) {
         {
             std::unique_lock<std::mutex> lk(s->mu);
             if (s->stop || s->failed) break;
             bool work = false;
-            for (ServeGraph* sg : s->graphs) work |= sg->inflight || (sg->running != 0) || !sg->pending.empty();
+            for (ServeGraph* sg : s->graphs) work |= sg->inflight.load() || (sg->running != 0) || !sg->pending.empty();
             if (!work) s->cv_work.wait_for(lk, std::chrono::milliseconds(1));
             if (s->stop) break;
         }
-        if (!serve_pass(s)) {            // iterations in flight and nothing finished yet
+        if (serve_pass(s)) {
+            idle = 0;
+        } else if (++idle < kSpins) {    // iterations in flight and nothing finished yet
+            std::this_thread::yield();
+        } else {
             std::unique_lock<std::mutex> lk(s->mu);
             if (s->stop || s->failed) break;
             s->cv_work.wait_for(lk, std::chrono::microseconds(20));
@@ -1206,6 +1261,18 @@ bfs_status bfs_server_create(int64_t hbm_budget_bytes, int32_t max_lanes, bfs_se
     s->max_lanes = max_lanes;
     s->t0 = std::chrono::steady_clock::now();
     cudaGetDevice(&s->device);
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.handleTypes = cudaMemHandleTypeNone;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = s->device;
+    const cudaError_t pe = cudaMemPoolCreate(&s->pool, &props);
+    if (pe != cudaSuccess) {
+        delete s;
+        return cuda_error(pe, "cudaMemPoolCreate", __FILE__, __LINE__);
+    }
+    uint64_t keep = kScratchKept;
+    cudaMemPoolSetAttribute(s->pool, cudaMemPoolAttrReleaseThreshold, &keep);
     s->worker = std::thread(serve_loop, s);
     *out = s;
     return BFS_OK;
@@ -1243,6 +1310,9 @@ bfs_status bfs_server_add_graph(bfs_server_t s, bfs_graph_t g, int32_t* graph_id
         rc = set_error(BFS_ERR_OUT_OF_MEMORY, "pinned host allocation");
     if (rc == BFS_OK && cudaMallocHost(reinterpret_cast<void**>(&sg->h_alive), sizeof(unsigned long long) * 5) != cudaSuccess)
         rc = set_error(BFS_ERR_OUT_OF_MEMORY, "pinned host allocation");
+    if (rc == BFS_OK && cudaHostAlloc(reinterpret_cast<void**>(&sg->h_call), sizeof(int),
+                                      cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess)
+        rc = set_error(BFS_ERR_OUT_OF_MEMORY, "pinned host allocation");
     if (rc == BFS_OK && cudaStreamCreateWithFlags(&sg->stream, cudaStreamNonBlocking) != cudaSuccess)
         rc = set_error(BFS_ERR_CUDA, "stream creation failed");
     if (rc == BFS_OK) {
@@ -1253,8 +1323,12 @@ bfs_status bfs_server_add_graph(bfs_server_t s, bfs_graph_t g, int32_t* graph_id
                             cudaMemcpyHostToDevice, sg->stream) != cudaSuccess)
             rc = set_error(BFS_ERR_CUDA, "state copy failed");
         if (rc == BFS_OK) {
+            *sg->h_call = 0;
             ms_reset<<<1, 1, 0, sg->stream>>>(S);
             ms_clear<<<ms_sm_count() * 8, kMT, 0, sg->stream>>>(S);
+            const int* word = sg->h_call;            // unified addressing
+            cudaMemcpyAsync(reinterpret_cast<char*>(S) + offsetof(MsState, call), &word, sizeof(word),
+                            cudaMemcpyHostToDevice, sg->stream);
             if (cudaStreamSynchronize(sg->stream) != cudaSuccess) rc = set_error(BFS_ERR_CUDA, "lane state initialisation failed");
         }
     }
@@ -1292,6 +1366,7 @@ bfs_status bfs_server_submit_ex(bfs_server_t s, int32_t graph_id, int32_t root, 
     q.t_submit = std::chrono::steady_clock::now();
     s->req.emplace(t, q);
     sg->pending.push_back(t);
+    call(sg);
     ++s->queued;
     ++s->submitted;
     *ticket = t;
@@ -1334,6 +1409,11 @@ bfs_status bfs_server_wait(bfs_server_t s, int64_t ticket, int64_t timeout_us, i
     ServeGraph* sg = s->graphs[q.graph];
     const int64_t n = sg->g->L.n;
     s->results_bytes -= (q.parents ? 2 : 1) * sizeof(int32_t) * n;
+    bool queued = false;
+    for (ServeGraph* x : s->graphs) {
+        queued |= !x->pending.empty();
+        call(x);                                     // the budget may admit a queued request now
+    }
     lk.unlock();
     bfs_status rc = BFS_OK;
     // the result was allocated stream-ordered and completed before the request
@@ -1349,7 +1429,7 @@ bfs_status bfs_server_wait(bfs_server_t s, int64_t ticket, int64_t timeout_us, i
     cudaFreeAsync(q.result, 0);
     cudaError_t e = cudaStreamSynchronize(0);
     if (rc == BFS_OK && e != cudaSuccess) rc = cuda_error(e, "result copy", __FILE__, __LINE__);
-    s->cv_work.notify_one();
+    if (queued) s->cv_work.notify_one();             // else the worker has nothing to gain from waking
     return rc;
 }
 
@@ -1381,12 +1461,15 @@ bfs_status bfs_server_destroy(bfs_server_t s) {
     {
         std::lock_guard<std::mutex> lk(s->mu);
         s->stop = true;
+        for (ServeGraph* sg : s->graphs)
+            if (sg->h_call) *static_cast<volatile int*>(sg->h_call) = 1;
     }
     s->cv_work.notify_all();
     if (s->worker.joinable()) s->worker.join();
     for (auto& kv : s->req)
         if (kv.second.result) cudaFreeAsync(kv.second.result, 0);
     cudaStreamSynchronize(0);
+    cudaMemPoolDestroy(s->pool);
     for (ServeGraph* sg : s->graphs) {
         release_graph(sg);
         delete sg;
