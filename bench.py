@@ -707,13 +707,12 @@ def main():
     valid = invariant_ok == len(roots) and oracle_exact in (None, 1)
     # kernels of the timed steps, per level: the encoder's passes (not PLAIN; one launch for
     # short slots, else three), the expansion and the piece kernel, the row encoder's passes
-    # and the fold (row exchange), the reduction; per search the init, root and first-level
-    # kernels
+    # and the fold (row exchange), the reduction; per search the init kernel
     passes = 1 if -(-n // p) // (args.wah_bits - 1) <= 8 * CHUNK_GROUPS else 3
     launches_per_level = (0 if args.mode == 0 else passes) + 2 + 1 + (passes + 1 if value_rowx else 0)
     if args.direction != "top_down":     # bottom-up expansion (+ clear and decode of the streams)
         launches_per_level += 1 if args.mode == 0 else (4 if args.format == "adaptive" else 3)
-    gpu_launches = args.steps * sum(3 + launches_per_level * st.n_levels for st in main_arm["stats"])
+    gpu_launches = args.steps * sum(1 + launches_per_level * st.n_levels for st in main_arm["stats"])
 
     configs = None
     if not args.no_configs and args.workload == "s26" and world == 1:

@@ -1530,6 +1530,7 @@ struct NextArgs {
     int32_t max_levels;
     cudaGraphConditionalHandle handle;
     int use_handle;                 // the graph-launched loop: also clear the counters for the next level
+    volatile uint64_t* h_error;     // pinned host word: the graph-launched loop's error flag once it ends
     unsigned long long* lvl;        // row hand-out counters, nlvl of them
     int nlvl;
 };
@@ -1565,7 +1566,9 @@ __device__ void level_next(LevelCtl* c, unsigned long long* ctr, const NextArgs&
     c->dedup = (c->visited * 16 < n) ? 1 : 0;
     const int go = (f > 0 && __ldcg(ctr + C_ERROR) == 0 && c->level < nx.max_levels) ? 1 : 0;
     c->go = go;
-    if (nx.use_handle) cudaGraphSetConditional(nx.handle, go ? 1u : 0u);
+    if (!nx.use_handle) return;
+    cudaGraphSetConditional(nx.handle, go ? 1u : 0u);
+    if (!go) *nx.h_error = __ldcg(ctr + C_ERROR);
 }
 
 // x = t & ~pi; pi |= x; level of the new vertices; |x| and its degree sum; the
@@ -1669,55 +1672,69 @@ __global__ void __launch_bounds__(kNT) reduce_level(uint32_t* __restrict__ t, ui
     for (int k = threadIdx.x; k < nx.nlvl; k += kNT) nx.lvl[k] = 0ull;
 }
 
-__global__ void level_first(LevelCtl* c, int64_t n, int win_ratio, int policy, int alpha, int beta,
-                            const uint32_t* deg, int32_t root, int64_t entries) {
+struct InitArgs {
+    int32_t* level;
+    int32_t* parent;
+    int64_t n;
+    uint32_t* pi;
+    uint32_t* fa;
+    uint32_t* fb;
+    int64_t words;
+    uint8_t* fsum;
+    uint32_t* fwords;
+    int64_t fsum_len;
+    const uint32_t* iso;            // or nullptr
+    const uint32_t* deg;
+    int64_t entries;
+    int32_t root;
+    int32_t win_ratio, policy, alpha, beta;
+    LevelCtl* ctl;
+    unsigned long long* ctr;        // the counters, C_NUM of them
+    unsigned long long* lvl;        // row hand-out counters, nlvl of them
+    int nlvl;
+};
+
+// A search starts from nothing visited but the root -- or, with bottom-up
+// levels, from the vertices without entries marked visited (iso): no level
+// reaches them, and the bottom-up scans skip them.  One launch sets the
+// outputs, bitmaps, counters and the first level's values.
+__global__ void __launch_bounds__(kNT) init_search(InitArgs a) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t root = a.root;
+    for (int64_t v = tid; v < a.n; v += stride) {
+        a.level[v] = v == root ? 0 : -1;
+        a.parent[v] = v == root ? a.root : -1;
+    }
+    for (int64_t w = tid; w < a.words; w += stride) {
+        const uint32_t r = w == (root >> 5) ? 1u << (root & 31) : 0u;
+        a.pi[w] = (a.iso ? a.iso[w] : 0u) | r;
+        a.fa[w] = r;
+        a.fb[w] = 0u;
+    }
+    for (int64_t q = tid; q < a.fsum_len; q += stride) {
+        const bool r = q == (root >> 10);
+        a.fsum[q] = r ? 1 : 0;
+        a.fwords[q] = r ? 1u << ((root >> 5) & 31) : 0u;
+    }
+    for (int64_t q = tid; q < C_NUM; q += stride) a.ctr[q] = 0ull;
+    for (int64_t q = tid; q < a.nlvl; q += stride) a.lvl[q] = 0ull;
+    if (tid != 0) return;
+    LevelCtl* c = a.ctl;
     c->frontier = 1;
     c->visited = 1;
     c->level = 0;
     c->done = 0u;
     c->window = 0;
-    c->win_ratio = win_ratio;
-    c->dedup = (16 < n) ? 1 : 0;
+    c->win_ratio = a.win_ratio;
+    c->dedup = (16 < a.n) ? 1 : 0;
     c->go = 1;
-    c->policy = policy;
-    c->alpha = alpha;
-    c->beta = beta;
-    c->bu = (policy == BFS_DIRECTION_BOTTOM_UP) ? 1 : 0;
-    c->m_f = (int64_t)deg[root];
-    c->m_u = entries - c->m_f;
-}
-
-// A search starts from nothing visited -- or, with bottom-up levels, from the
-// vertices without entries marked visited (iso): no level reaches them, and
-// the bottom-up scans skip them.
-__global__ void init_search(int32_t* __restrict__ level, int32_t* __restrict__ parent, int64_t n,
-                            uint32_t* __restrict__ pi, uint32_t* __restrict__ fa, uint32_t* __restrict__ fb,
-                            int64_t words, uint8_t* __restrict__ fsum, uint32_t* __restrict__ fwords, int64_t fsum_len,
-                            const uint32_t* __restrict__ iso) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += stride) {
-        level[v] = -1;
-        parent[v] = -1;
-    }
-    for (int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; w < words; w += stride) {
-        pi[w] = iso ? iso[w] : 0u;
-        fa[w] = 0u;
-        fb[w] = 0u;
-    }
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < fsum_len; q += stride) {
-        fsum[q] = 0;
-        fwords[q] = 0u;
-    }
-}
-
-__global__ void set_root(int32_t* level, int32_t* parent, uint32_t* pi, uint32_t* fa, uint8_t* fsum, uint32_t* fwords,
-                         int32_t root) {
-    level[root] = 0;
-    parent[root] = root;
-    pi[root >> 5] |= 1u << (root & 31);
-    fa[root >> 5] |= 1u << (root & 31);
-    fsum[root >> 10] = 1;
-    fwords[root >> 10] |= 1u << ((root >> 5) & 31);
+    c->policy = a.policy;
+    c->alpha = a.alpha;
+    c->beta = a.beta;
+    c->bu = (a.policy == BFS_DIRECTION_BOTTOM_UP) ? 1 : 0;
+    c->m_f = (int64_t)a.deg[root];
+    c->m_u = a.entries - c->m_f;
 }
 
 // Pack the streams of this exchange into a trace (the receive buffer g'):
@@ -2060,15 +2077,15 @@ bfs_status run_search(bfs_graph* g, int32_t root, int32_t* parent, int32_t* leve
     if (tracing || row_tracing) BFS_TRY(slot_off.alloc(sizeof(int64_t) * (size_t)std::max<int64_t>(nslots, p2)));
     if (stats) { stats->n_levels = 0; stats->trace_used = 0; stats->row_trace_used = 0; }
 
-    init_search<<<sm_count() * 4, kNT, 0, st>>>(level, parent, L.n, W.pi.as<uint32_t>(), W.fa.as<uint32_t>(),
-                                                W.fb.as<uint32_t>(), W.bm_words, W.fsum.as<uint8_t>(), W.fwords.as<uint32_t>(),
-                                                W.fsum_len,
-                                                bu_kernels ? L.iso.as<uint32_t>() : nullptr);
+    LevelCtl* ctl = W.ctl.as<LevelCtl>();
+    const uint32_t* deg = L.deg.as<uint32_t>();
+    unsigned long long* lvl = W.level_scratch.as<unsigned long long>();
+    const InitArgs init{level, parent, L.n, W.pi.as<uint32_t>(), W.fa.as<uint32_t>(), W.fb.as<uint32_t>(), W.bm_words,
+                        W.fsum.as<uint8_t>(), W.fwords.as<uint32_t>(), W.fsum_len,
+                        bu_kernels ? L.iso.as<uint32_t>() : nullptr, deg, L.nnz, root, rowx ? 4 : 2, g->direction,
+                        g->alpha, g->beta, ctl, ctr, lvl, 3 * p + 1};
+    init_search<<<(unsigned)std::min<int64_t>((L.n + kNT - 1) / kNT, sm_count() * 4), kNT, 0, st>>>(init);
     BFS_CUDA_TRY(cudaGetLastError());
-    set_root<<<1, 1, 0, st>>>(level, parent, W.pi.as<uint32_t>(), W.fa.as<uint32_t>(), W.fsum.as<uint8_t>(),
-                              W.fwords.as<uint32_t>(), root);
-    BFS_CUDA_TRY(cudaGetLastError());
-    BFS_CUDA_TRY(cudaMemsetAsync(ctr, 0, sizeof(unsigned long long) * C_NUM, st));
 
     LevelArgs a;
     memset(&a, 0, sizeof(a));
@@ -2090,8 +2107,6 @@ bfs_status run_search(bfs_graph* g, int32_t root, int32_t* parent, int32_t* leve
     a.chunk_base = W.chunk_base.as<int64_t>();
     a.chunks_per_slot = W.chunks_per_slot;
     a.slot_unit_base = W.units.as<int64_t>();
-    unsigned long long* lvl = W.level_scratch.as<unsigned long long>();
-    BFS_CUDA_TRY(cudaMemsetAsync(lvl, 0, sizeof(unsigned long long) * (3 * p + 1), st));   // the first level's
     a.row_next = lvl;
     a.row_piece_count = lvl + p;
     a.row_piece_next = lvl + 2 * p;
@@ -2169,7 +2184,6 @@ bfs_status run_search(bfs_graph* g, int32_t root, int32_t* parent, int32_t* leve
 
     uint32_t* f = W.fa.as<uint32_t>();       // frontier of the level (reduce_level writes the next one here)
     uint32_t* t = W.fb.as<uint32_t>();       // next bits (cleared by reduce_level)
-    LevelCtl* ctl = W.ctl.as<LevelCtl>();
     a.f = f;
     a.t = t;
     a.fsum = W.fsum.as<uint8_t>();
@@ -2178,12 +2192,9 @@ bfs_status run_search(bfs_graph* g, int32_t root, int32_t* parent, int32_t* leve
     ea.frontier = f;
     ra.skip = &ctl->bu;                      // bottom-up levels have no row exchange
     const int32_t max_levels = (int32_t)std::min<int64_t>(L.n + 1, INT32_MAX);
-    const uint32_t* deg = L.deg.as<uint32_t>();
 
     if (dynamic)                     // the search's directories start as V
         BFS_CUDA_TRY(cudaMemcpyAsync(W.ddir.ptr, L.dir.ptr, W.ddir.bytes, cudaMemcpyDeviceToDevice, st));
-    level_first<<<1, 1, 0, st>>>(ctl, L.n, rowx ? 4 : 2, g->direction, g->alpha, g->beta, deg, root, L.nnz);
-    BFS_CUDA_TRY(cudaGetLastError());
 
     // One level: the same launch sequence every time.  `host` adds the
     // statistics, the trace and the phase events (and k is known on the host).
@@ -2278,7 +2289,7 @@ bfs_status run_search(bfs_graph* g, int32_t root, int32_t* parent, int32_t* leve
             cudaEventRecord(W.ev[5], s);
             cudaEventRecord(W.ev[6], s);
         }
-        const NextArgs nx{L.n, max_levels, handle, host ? 0 : 1, lvl, 3 * p + 1};
+        const NextArgs nx{L.n, max_levels, handle, host ? 0 : 1, W.h_counters + C_ERROR, lvl, 3 * p + 1};
         if (L.n < kSmallReduce)
             reduce_level<4><<<(unsigned)((W.bm_words + 31) / 32), kNT, 0, s>>>(
                 t, W.pi.as<uint32_t>(), f, W.fsum.as<uint8_t>(), W.fwords.as<uint32_t>(), W.bm_words, L.n, level, ctl,
@@ -2349,10 +2360,10 @@ bfs_status run_search(bfs_graph* g, int32_t root, int32_t* parent, int32_t* leve
             c.level = level;
             sg = &c;
         }
+        W.h_counters[C_ERROR] = 0;
         BFS_CUDA_TRY(cudaGraphLaunch(sg->exec, st));
-        BFS_CUDA_TRY(cudaMemcpyAsync(W.h_counters, ctr, sizeof(uint64_t) * C_NUM, cudaMemcpyDeviceToHost, st));
         BFS_CUDA_TRY(cudaStreamSynchronize(st));
-        const uint64_t* h = W.h_counters;
+        const volatile uint64_t* h = W.h_counters;
         if (h[C_ERROR] & 2ull) return set_error(BFS_ERR_INVALID_ARG, "trace capacity exceeded");
         if (h[C_ERROR])
             return set_error(BFS_ERR_CORRUPT, "device invariant check failed (code %llu)",

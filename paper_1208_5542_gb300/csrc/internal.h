@@ -187,7 +187,7 @@ struct Workspace {
     DevBuf colfirst;             // the column encoder's per-chunk first words (bottom-up decode)
     DevBuf xfmt;                 // per-slot format of the level-adaptive exchange
     DevBuf ddir;                 // dynamic cross directory: the search's copy D_{i,j} of the directories
-    SearchGraph sgraph[2];       // level loops as CUDA graphs, most recent configurations
+    SearchGraph sgraph[8];       // level loops as CUDA graphs, most recent configurations and output buffers
     int sgraph_next = 0;
     int64_t enc_cps = 0;         // encoder chunks per slot
     int64_t row_cap = 0;        // words (of the WAH width) per row buffer
