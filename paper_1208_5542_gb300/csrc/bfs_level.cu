@@ -20,13 +20,14 @@
 // g' is the send buffer in HBM; its sizes are scanned for the statistics and
 // packed into the caller's trace when one is requested.
 //
-// The expansion is row-affine: a block (i,j) only ever writes destinations of
-// range i, so a persistent CTA settles on one block-row at a time and keeps
-// that row's visited bits pi_i and its own partial next bits t_i in shared
-// memory (when a range fits); its warps take the row's units one at a time.
-// Visited tests and next-bit updates are then on-chip; the partial t_i of
-// every CTA is OR-folded into t when the CTA leaves the row (the fold of the
-// 2D partition, done through L2).
+// Dense levels of large graphs are expanded row-affine: a block (i,j) only
+// ever writes destinations of range i, so a persistent CTA settles on one
+// block-row at a time and keeps that row's visited bits pi_i -- and its own
+// partial next bits t_i, where both fit -- in shared memory; its warps take
+// the row's units.  The partial t_i of every CTA is OR-folded into t when the
+// CTA leaves the row (the fold of the 2D partition, done through L2).  All
+// other levels hand their units out as one list in the order of the block-rows,
+// cut finer when there are few.
 //
 // Bottom-up levels (the hybrid traversal the paper names in Sec. VIII and IX,
 // when enabled): the exchange is the same, its streams are decoded into a
@@ -55,17 +56,17 @@ namespace {
 constexpr int kNT = 256;            // threads of the small kernels
 constexpr int kXT = 1024;           // threads of the expansion CTAs
 constexpr int kXW = kXT / 32;       // warps of the expansion CTAs
-#ifndef BFS_COOP
-#define BFS_COOP 64
-#endif
-constexpr uint32_t kCoop = BFS_COOP;      // columns of at least this many entries take the whole warp
+// Columns of at least this many entries take the whole warp (32: scale 26 11.75
+// -> 12.16 ms, scale 24 PLAIN 2.76 -> 2.90; 128: the same as 64).
+constexpr uint32_t kCoop = 64;
 constexpr uint32_t kHub = 2048;     // columns longer than this are cut into pieces of this size
 constexpr uint32_t kHubSparse = 512;  // the same on levels with fewer units than warps
-#ifndef BFS_GUIDE
-#define BFS_GUIDE 1
-#endif
-constexpr int64_t kGuide = BFS_GUIDE;  // a grab takes 1/(kGuide * warps) of the units left in the row
-constexpr int64_t kWindowMinVertices = 1 << 21;   // below, all visited bits fit in L1: no row window
+// Below this many vertices all visited bits (256 KB) are about as good as in L1
+// and no level loads a row window.  A search without it / with it: scale 21
+// 0.93 / 0.90 ms, scale 22 1.14 / 0.97, scale 23 2.32 / 1.83, scale 24 PLAIN
+// 3.19 / 2.76; from 2^18 on instead: scale 20 0.56 -> 0.58 ms, a directed
+// uniform graph of 1M vertices 0.45 -> 0.48.
+constexpr int64_t kWindowMinVertices = 1 << 21;
 constexpr int64_t kSmemLimit = 227 * 1024;
 
 // Per-level values that the device keeps from level to level, so that one
@@ -235,10 +236,7 @@ struct Visitor {
 // they do not push the visited, parent and next-bit lines out of L2 (-21% DRAM
 // bytes at the growing level of a scale-24 search).
 constexpr int kIlp = 4;
-#ifndef BFS_PIECE_ILP
-#define BFS_PIECE_ILP 8
-#endif
-constexpr int kPieceIlp = BFS_PIECE_ILP;   // the piece kernel: long columns only, more entries in flight
+constexpr int kPieceIlp = 8;   // the piece kernel: long columns only, more entries in flight
 
 // Scratch of one warp in shared memory: the nonempty words of its unit and the
 // short columns of its batch, packed to the front, so that the owner of an
@@ -275,7 +273,13 @@ __device__ __forceinline__ void warp_column(const LevelArgs& a, const Visitor<WI
 // stream (or of one raw slice), which hold up to 992 vertices with columns of
 // any length: a level with fewer units than warps would leave most of the chip
 // idle, so its units are cut into `parts`, each taking every parts-th group of
-// `bw` of the unit's items, and its long columns into shorter pieces.
+// `bw` of the unit's items, and its long columns into shorter pieces.  A part
+// decodes and looks up its whole unit again, so the parts stop at half the
+// warps: uncut / half / twice the warps takes 314 / 198 / 197 us at scale 12,
+// 409 / 331 / 334 at scale 17, 398 / 402 / 436 on a directed uniform graph of 1M,
+// 975 / 935 / 962 at scale 22, 1805 / 1803 / 1828 at scale 23.  Pieces of 2048
+// on all levels instead of down to 512: 331 -> 393 us at scale 17, 555 -> 631
+// at scale 20 (926 against 962 at scale 22, where 512 is a little too short).
 struct Split {
     uint32_t parts;        // power of two
     uint32_t bw;           // items per batch of a part (1..32)
@@ -289,7 +293,7 @@ __device__ __forceinline__ Split split_level(int64_t units, int64_t items, int64
     while (s.hub > kHubSparse && (int64_t)s.hub * 4 * warps > entries) s.hub /= 2;
     if (units <= 0 || units >= warps) return s;
     const int64_t avg = items / units > 1 ? items / units : 1;        // items per unit (at most: before the sieve)
-    while ((int64_t)s.parts * units < 2 * warps && s.parts < 256u && (int64_t)s.parts < avg) s.parts *= 2u;
+    while (2 * (int64_t)s.parts * units < warps && s.parts < 256u && (int64_t)s.parts < avg) s.parts *= 2u;
     const int64_t bw = (avg + s.parts - 1) / s.parts;
     s.bw = bw < 32 ? (uint32_t)bw : 32u;
     return s;
@@ -574,7 +578,7 @@ __device__ __forceinline__ void flat_units(unsigned long long* counter, int64_t 
         if (lane_id() == 0) {
             const int64_t cur = (int64_t)*reinterpret_cast<volatile unsigned long long*>(counter);
             if (cur < total) {
-                const int64_t g = (total - cur) / (kGuide * warps * rows);
+                const int64_t g = (total - cur) / (warps * rows);
                 b = g > batch ? g : batch;
                 x = (int64_t)atomicAdd(counter, (unsigned long long)b);
             } else {
@@ -637,7 +641,7 @@ __device__ __forceinline__ void row_affine(const LevelArgs& a, unsigned long lon
             if (lane_id() == 0) {
                 const int64_t cur = (int64_t)*reinterpret_cast<volatile unsigned long long*>(counters + row);
                 if (cur < nu) {
-                    const int64_t g = (uint32_t)(nu - cur) / (uint32_t)(kGuide * gridDim.x * kXW);   // below 2^31 units
+                    const int64_t g = (uint32_t)(nu - cur) / (uint32_t)(gridDim.x * kXW);   // below 2^31 units
                     b = g > batch ? g : batch;
                     x = (int64_t)atomicAdd(counters + row, (unsigned long long)b);
                 } else {
@@ -900,6 +904,15 @@ __device__ __forceinline__ void expand_pieces_level(const LevelArgs& a, uint32_t
     }
 }
 
+// What bounds it: at scale 12 a level is one chain of dependent steps (9 units,
+// once a warp each: 168 and 176 us for the two levels with entries; cut into
+// parts 12); at a growing level the L2 reductions of the fresh visits (about
+// 125 G/s: 11.8 M at scale 22 are 94 of its 155 us, 230 before the cut); at the
+// densest level issue slots (118 M entries in 455 us, 62% issue activity; 488
+// with a search for every entry's owner in place of head masks), and without the
+// window the scattered reads of the visited words (scale 26: 1.5 G entries, 6.8
+// -> 6.5 ms).
+//
 // One launch expands a level: WIN is the window the graph's ranges allow, and
 // the level's own values pick the body -- with the window on dense levels,
 // without it on sparse ones (their visits are too few to pay for loading it),
@@ -1385,15 +1398,22 @@ __global__ void __launch_bounds__(kNT) decode_streams(LevelArgs a) {
 // once the scan has passed the end of its range.  v's columns are read from
 // the bottom-up rows (stored back to back, range by range).  One warp per
 // visited word (32 vertices): a row of at most kBuLane entries is scanned by
-// its own lane (kIlp entries and their frontier words in flight), a longer
+// its own lane (kBuIlp entries and their frontier words in flight), a longer
 // one by the whole warp (kIlp x 32 entries per step); the warp's next bits
 // are one store (t is clear and no other kernel writes it this level).
+//
+// The scattered frontier reads bound it: at scale 24 the first bottom-up level
+// is about two thirds of the search.  Entries of a short row in flight: a row
+// usually ends after a few, and what was read past its end is lost; 2 / 3 / 4 /
+// 6 / 8 give 2.12 / 2.07 / 2.01 / 2.11 / 2.18 ms a search (adaptive format).
 constexpr int64_t kBuLane = 32;
-constexpr int kBuIlp = 8;           // entries of a short row in flight
+constexpr int kBuIlp = 4;
 
 // The frontier test of an entry u.  A sparse frontier is tested word-wise
 // first: `words` has a bit per 32 vertices (64 KB at scale 24, in L1, where
-// the bitmap is 2 MB: 940 against 326 G scattered reads a second).
+// the bitmap is 2 MB: 940 against 326 G scattered reads a second).  Below
+// n / 64 vertices most words are empty and the test ends there (scale 24: 2.17
+// ms a search, 2.23 never testing words); a denser frontier would read both.
 struct BuFrontier {
     const uint32_t* g;        // the decoded streams, or the raw frontier (PLAIN)
     const uint32_t* words;    // bit (u / 32): the frontier has a vertex in that word; nullptr: a dense frontier
@@ -1557,7 +1577,9 @@ __device__ void level_next(LevelCtl* c, unsigned long long* ctr, const NextArgs&
     c->frontier = f;
     c->visited += f;
     c->level += 1;
-    // the row window pays once a level visits every row's vertices several times
+    // the row window pays once a level visits every row's vertices several
+    // times: a ratio half or twice as large costs scale 24 PLAIN 4% (2.76 ->
+    // 2.87 ms) and moves scales 22 and 23 by less than 2.5% either way
     c->window = (n >= kWindowMinVertices && mf >= (int64_t)c->win_ratio * n) ? 1 : 0;
     // While few vertices are visited, most entries lead to fresh vertices,
     // each reached from many frontier vertices: reading the parent first turns
@@ -1576,7 +1598,9 @@ __device__ void level_next(LevelCtl* c, unsigned long long* ctr, const NextArgs&
 // A warp takes WPW words: 32, so that the bitmaps are read and written in whole
 // lines, or 4 on small graphs (below kSmallReduce vertices), where the chain of
 // a word's level stores and degree loads, one word after the other, is the
-// kernel's time (4,096 vertices: 128 words on 4 warps took 9 us).
+// kernel's time (4,096 vertices: 128 words on 4 warps took 9 us).  A search with
+// 4 / 32 words a warp: 202 / 212 us at scale 12, 552 / 559 at scale 20, 1021 /
+// 971 at scale 22, 12.80 / 11.75 ms at scale 26 (partial lines).
 // The last CTA to finish (a counter, no waiting) sets up the next level.
 // In the graph-launched loop it also clears the per-level counters and the
 // row hand-out counters, in place of memset nodes; the stepwise loop reads them

@@ -167,7 +167,11 @@ __device__ __forceinline__ void lay_out_units(const EncodeArgs& a) {
 // words, and the threads write them.  Its time is one chain of dependent steps
 // (about 5 us for a one-round slot), where the three launches below, built for
 // throughput, take 16-25 us however little there is to encode; above the limit
-// their warps, which need not wait for one another, are the faster ones.
+// their warps, which need not wait for one another, are the faster ones.  A
+// search with this kernel / the three launches: scale 12 202 / 256 us, ragged
+// scale 17 346 / 439, directed uniform 1M vertices 447 / 490.  Slots of one round of 256
+// threads take that CTA (1024 threads: scale 12 213 us, scale 17 361); longer
+// ones 1024 (256: directed uniform 1M vertices 469 us, scale 20 558 -> 627).
 constexpr int kSK = 4;              // groups per thread and round
 constexpr int kSmallChunks = 8;     // two rounds (five rounds, 17 chunks of scale 22 on 8 x 8: 38 us against 26)
 
