@@ -416,10 +416,11 @@ BFS_API bfs_status bfs_batch_autotune(bfs_graph_t g, const int32_t *roots, int32
 /*
  * Query server with continuous batching (no counterpart in the paper, which
  * runs one search at a time): graphs stay resident with up to 64 lanes of the
- * batched search each; a server thread runs one level of every running lane
- * per iteration, each graph on its own stream (their work overlaps on the
- * GPU), admits queued queries into free lanes at every iteration boundary and
- * retires lanes whose frontier emptied.  Every result is the level and
+ * batched search each; an iteration runs one level of every running lane of a
+ * graph, each graph on its own stream (their work overlaps on the GPU).
+ * Iterations repeat on the device until a lane's frontier empties or a query
+ * comes in that a free lane can take; the server thread then retires the
+ * lanes that ended and admits queued queries into free ones.  Every result is the level and
  * parent vectors of a single search from the query's root, the same as
  * bfs_run alone.
  * Graphs are admitted against `hbm_budget_bytes` by footprint (layout + lane
