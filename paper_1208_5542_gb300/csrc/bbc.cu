@@ -584,7 +584,7 @@ bfs_status bfs_bbc_decode(const uint8_t* bytes, int64_t nbytes_in, int64_t nbits
     Scratch tmp;
     BFS_TRY(tmp.alloc(parts.bytes, st));
     HostFlag bad;
-    BFS_TRY(bad.take());
+    BFS_TRY(bad.take(st));
     char* t = tmp.as<char>();
     uint32_t* outb = reinterpret_cast<uint32_t*>(t + p_outb);
     uint8_t* exits = reinterpret_cast<uint8_t*>(t + p_exits);
@@ -606,7 +606,7 @@ bfs_status bfs_bbc_decode(const uint8_t* bytes, int64_t nbytes_in, int64_t nbits
     bbc_expand<<<xgrid, kBT, 0, st>>>(bytes, nbytes_in, nbytes, entry, obase, held, reinterpret_cast<uint8_t*>(bits), err);
     bbc_outcome<<<1, 1, 0, st>>>(reinterpret_cast<const uint8_t*>(bits), nbits, held, err, bad.device());
     BFS_CUDA_TRY(cudaGetLastError());
-    BFS_CUDA_TRY(cudaStreamSynchronize(st));
+    BFS_TRY(bad.wait());
     if (bad.value()) return set_error(BFS_ERR_CORRUPT, "malformed BBC stream");
     return BFS_OK;
 }

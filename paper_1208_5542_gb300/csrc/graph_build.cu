@@ -140,7 +140,8 @@ bfs_status Scratch::alloc(size_t nbytes, cudaStream_t st) {
     return BFS_OK;
 }
 
-bfs_status HostFlag::take() {
+bfs_status HostFlag::take(cudaStream_t st) {
+    stream = st;
     std::unique_lock<std::mutex> lk(t_flag_mu);
     if (!t_flags) {
         void* p = nullptr;
@@ -161,8 +162,15 @@ bfs_status HostFlag::take() {
     }
 }
 
+bfs_status HostFlag::wait() {
+    BFS_CUDA_TRY(cudaStreamSynchronize(stream));
+    waited = true;
+    return BFS_OK;
+}
+
 HostFlag::~HostFlag() {
     if (slot < 0) return;
+    if (!waited) cudaStreamSynchronize(stream);
     std::lock_guard<std::mutex> lk(t_flag_mu);
     t_flag_used[slot / 64] &= ~(1ull << (slot % 64));
     t_flag_free.notify_one();

@@ -83,16 +83,23 @@ struct Scratch {
 // Two 8-byte words of mapped pinned memory for a call's kernels to report in
 // (an error, a count): read by the host after the stream has been
 // synchronised, with no copy.  kHostFlags pairs live in one page for the life
-// of the process; a call (which takes one) that finds none free waits for one.
+// of the process; a call that finds none free waits for one, so a call never
+// takes a second pair while it holds one (kHostFlags threads, each holding a
+// pair and waiting for another, would wait for ever).  A pair goes back only
+// when no kernel can write it any more: wait() synchronises the stream, and a
+// call that leaves before that (an error) synchronises on its way out.
 constexpr int kHostFlags = 256;
 
 struct HostFlag {
     int slot = -1;
+    cudaStream_t stream = nullptr;
+    bool waited = false;
     HostFlag() = default;
     HostFlag(const HostFlag&) = delete;
     HostFlag& operator=(const HostFlag&) = delete;
     ~HostFlag();
-    bfs_status take();                              // cleared
+    bfs_status take(cudaStream_t st);               // cleared; for kernels launched on st
+    bfs_status wait();
     volatile unsigned long long* device(int word = 0) const;
     unsigned long long value(int word = 0) const;
 };

@@ -161,15 +161,16 @@ bfs_status bfs_plwah_decode(const uint32_t* words, int64_t nwords, int64_t nbits
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     Scratch wah;
     BFS_TRY(wah.alloc(sizeof(uint32_t) * (size_t)(2 * nwords + 1), st));
-    HostFlag said;                                    // error, count
-    BFS_TRY(said.take());
+    int64_t h_cnt = 0;
     if (nwords > 0) {
+        HostFlag said;                                // error, count; given back before the WAH decode takes its own
+        BFS_TRY(said.take(st));
         BFS_CUDA_TRY(launch_cluster(wah_from_plwah, st, words, nwords, nbits, wah.as<uint32_t>(),
                                     said.device(1), said.device(0)));
-        BFS_CUDA_TRY(cudaStreamSynchronize(st));
+        BFS_TRY(said.wait());
+        h_cnt = (int64_t)said.value(1);
+        if (said.value(0)) return set_error(BFS_ERR_CORRUPT, "malformed PLWAH stream (a fill of length 0)");
     }
-    const int64_t h_cnt = (int64_t)said.value(1);
-    if (said.value(0)) return set_error(BFS_ERR_CORRUPT, "malformed PLWAH stream (a fill of length 0)");
     const bfs_status rc = bfs_wah_decode(wah.ptr, h_cnt, nbits, 32, bits, stream);
     if (rc == BFS_ERR_CORRUPT) return set_error(BFS_ERR_CORRUPT, "malformed PLWAH stream");
     return rc;

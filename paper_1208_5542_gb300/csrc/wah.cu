@@ -1381,7 +1381,7 @@ bfs_status bfs_wah_decode(const void* words, int64_t nwords, int64_t nbits, int3
         return set_error(BFS_ERR_INVALID_ARG, "bad decode arguments");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     HostFlag err;
-    BFS_TRY(err.take());
+    BFS_TRY(err.take(st));
     // a stream inside the output would be overwritten while it is read: decoded aside
     const size_t out_bytes = sizeof(uint32_t) * (size_t)((nbits + 31) / 32);
     const char *w0 = static_cast<const char*>(words), *b0 = reinterpret_cast<const char*>(bits);
@@ -1393,7 +1393,7 @@ bfs_status bfs_wah_decode(const void* words, int64_t nwords, int64_t nbits, int3
     }
     BFS_TRY(launch_wah_decode_bitmap(words, nwords, nbits, word_bits, dst, err.device(), st));
     if (dst != bits) BFS_CUDA_TRY(cudaMemcpyAsync(bits, dst, out_bytes, cudaMemcpyDeviceToDevice, st));
-    BFS_CUDA_TRY(cudaStreamSynchronize(st));
+    BFS_TRY(err.wait());
     if (err.value()) return set_error(BFS_ERR_CORRUPT, "malformed WAH stream");
     return BFS_OK;
 }
