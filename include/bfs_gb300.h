@@ -483,6 +483,13 @@ BFS_API bfs_status bfs_server_destroy(bfs_server_t s);
 BFS_API bfs_status bfs_debug_fail_allocation(int64_t k);
 
 /*
+ * For tests of the codecs: the calling thread's encodes and decodes run on at
+ * most `ctas` CTAs (1, 2, 4, 8 or 16; 0 lifts the cap), as they do on a device
+ * or partition that cannot place a larger cluster.  The streams are the same.
+ */
+BFS_API bfs_status bfs_debug_codec_ctas(int32_t ctas);
+
+/*
  * WAH-encode one bitmap (Sec. IV, Table 3) on the device.
  *   bits: device, bit b of the bitmap = bit b%32 of bits[b/32], nbits >= 0
  *         bits in ceil(nbits/32) words.

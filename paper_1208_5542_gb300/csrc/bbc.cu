@@ -147,7 +147,8 @@ __global__ void __launch_bounds__(kCT) scan_cluster(const uint32_t* in, const ui
     if (n_dev) n = *n_dev;
     uint32_t carry = 0;
     int turn = 0;
-    for (int64_t b = 0; b < n; b += kClusterRound, ++turn) {
+    const int64_t round = cluster_round();
+    for (int64_t b = 0; b < n; b += round, ++turn) {
         const int64_t i0 = b + cluster_thread() * kCK;
         uint32_t x[kCK], sum = 0, all;
 #pragma unroll
@@ -551,10 +552,10 @@ bfs_status bfs_bbc_encode(const uint32_t* bits, int64_t nbits, uint8_t* bytes, i
     const int egrid = (int)std::min<int64_t>((nbytes + kBT - 1) / kBT, (int64_t)sms * 16);
     BFS_CUDA_TRY(cudaMemsetAsync(mpos, 0xFF, 4 * (size_t)nbytes, st));
     bbc_flags<<<grid, kBT, 0, st>>>(bits, nbits, nbytes, flags, tiles);
-    BFS_CUDA_TRY(launch_cluster(scan_cluster, st, tiles, nullptr, ntiles, tiles, nunits, nullptr));
+    BFS_CUDA_TRY(launch_cluster<scan_cluster>(st, tiles, nullptr, ntiles, tiles, nunits, nullptr));
     bbc_number<<<grid, kBT, 0, st>>>(flags, nbytes, tiles, upos, mpos);
     bbc_sizes<<<egrid, kBT, 0, st>>>(bits, nbits, nbytes, upos, mpos, nunits, sizes);
-    BFS_CUDA_TRY(launch_cluster(scan_cluster, st, sizes, nunits, int64_t(0), offs, nullptr, nbytes_out));
+    BFS_CUDA_TRY(launch_cluster<scan_cluster>(st, sizes, nunits, int64_t(0), offs, nullptr, nbytes_out));
     bbc_heads<<<egrid, kBT, 0, st>>>(bits, nbits, nbytes, upos, mpos, nunits, offs, bytes);
     bbc_tails<<<egrid, kBT, 0, st>>>(bits, nbits, nbytes, upos, mpos, nunits, offs, bytes);
     BFS_CUDA_TRY(cudaGetLastError());
@@ -601,7 +602,7 @@ bfs_status bfs_bbc_decode(const uint8_t* bytes, int64_t nbytes_in, int64_t nbits
     bbc_groups<<<ggrid, kBT, 0, st>>>(exits, nch, gexits);
     bbc_chain<<<1, 1024, 0, st>>>(gexits, ng, gentry, err);
     bbc_fill<<<ggrid, kBT, 0, st>>>(exits, outb, nch, gentry, entry, obase);
-    BFS_CUDA_TRY(launch_cluster(scan_cluster, st, obase, nullptr, nch, obase, held, nullptr));
+    BFS_CUDA_TRY(launch_cluster<scan_cluster>(st, obase, nullptr, nch, obase, held, nullptr));
     const int xgrid = (int)std::min<int64_t>((nch * 32 + kBT - 1) / kBT, (int64_t)sms * 16);
     bbc_expand<<<xgrid, kBT, 0, st>>>(bytes, nbytes_in, nbytes, entry, obase, held, reinterpret_cast<uint8_t*>(bits), err);
     bbc_outcome<<<1, 1, 0, st>>>(reinterpret_cast<const uint8_t*>(bits), nbits, held, err, bad.device());

@@ -8,9 +8,13 @@
 // shared memory with one hardware barrier, needs no scratch in device memory
 // (a call can be captured, and calls on several streams share nothing), and
 // is scheduled as a whole.  An encode and a decode of such a slice through the
-// API, host work and synchronisation included: 1.02 -> 0.13 ms.
+// API, host work and synchronisation included: 1.02 -> 0.13 ms.  16 CTAs are
+// more than the portable 8, and a partition of the device may not have their
+// SMs side by side: a kernel takes the largest size that the device can place,
+// down to one CTA, which runs anywhere (the round shrinks with it).
 #pragma once
 
+#include <atomic>
 #include <cooperative_groups.h>
 #include <cstdint>
 
@@ -18,10 +22,15 @@
 
 namespace bfsgb {
 
-constexpr int kCC = 16;             // CTAs of a codec cluster (non-portable size: see launch_cluster)
+constexpr int kCC = 16;             // the most CTAs of a codec cluster (non-portable size: see launch_cluster)
 constexpr int kCT = 1024;           // threads per CTA
 constexpr int kCK = 8;              // elements per thread and round
-constexpr int64_t kClusterRound = (int64_t)kCC * kCT * kCK;
+constexpr int kCDevices = 64;       // devices whose cluster size is remembered
+
+// Elements per round of the running cluster.
+__device__ __forceinline__ int64_t cluster_round() {
+    return (int64_t)cooperative_groups::this_cluster().num_blocks() * kCT * kCK;
+}
 
 // Shared memory of a cluster scan; the two slots of `part` alternate, so that
 // one cluster barrier per scan is enough (a slot is written again only after
@@ -47,7 +56,7 @@ __device__ __forceinline__ T cluster_excl_scan(T x, T identity, Op op, ClusterSc
     cl.sync();
     if (threadIdx.x < 32) {
         const int l = (int)threadIdx.x;
-        const T v = l < kCC ? *cl.map_shared_rank(&s.part[turn & 1], l) : identity;
+        const T v = l < (int)cl.num_blocks() ? *cl.map_shared_rank(&s.part[turn & 1], l) : identity;
         T incl = v;
 #pragma unroll
         for (int d = 1; d < kCC; d <<= 1) {
@@ -72,24 +81,62 @@ __device__ __forceinline__ int64_t cluster_thread() {
     return (int64_t)cooperative_groups::this_cluster().block_rank() * kCT + threadIdx.x;
 }
 
-// Launch one cluster of kCC CTAs.  16 CTAs need the kernel's consent to a
-// cluster larger than the portable 8.
-template <typename... P, typename... A>
-cudaError_t launch_cluster(void (*kernel)(P...), cudaStream_t st, A... args) {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
+// The calling thread's cap on the CTAs of a codec cluster (bfs_debug_codec_ctas;
+// kCC unless a test lowered it).
+int codec_ctas_cap();
+
+struct ClusterConfig {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(kCC);
-    cfg.blockDim = dim3(kCT);
-    cfg.stream = st;
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = kCC;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+    ClusterConfig(int ctas, cudaStream_t st) {
+        cfg.gridDim = dim3(ctas);
+        cfg.blockDim = dim3(kCT);
+        cfg.stream = st;
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = ctas;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+    }
+};
+
+// The largest power of two of CTAs, at most kCC, of which the current device
+// can place a cluster of this kernel (asked once per kernel and device).
+// More than 8 need the kernel's consent.
+template <typename... P>
+cudaError_t cluster_ctas(void (*kernel)(P...), std::atomic<int>* known, int* ctas) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < kCDevices && (*ctas = known[dev].load()) > 0) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) cudaGetLastError();            // the portable sizes are left
+    for (*ctas = kCC; *ctas > 1; *ctas /= 2) {
+        int fit = 0;
+        ClusterConfig c(*ctas, nullptr);
+        if (cudaOccupancyMaxActiveClusters(&fit, kernel, &c.cfg) == cudaSuccess && fit > 0) break;
+        cudaGetLastError();
+    }
+    if (dev < kCDevices) known[dev].store(*ctas);
+    return cudaSuccess;
+}
+
+template <typename... P, typename... A>
+cudaError_t launch_sized(void (*kernel)(P...), int ctas, cudaStream_t st, A... args) {
+    ClusterConfig c(ctas, st);
+    return cudaLaunchKernelEx(&c.cfg, kernel, static_cast<P>(args)...);
+}
+
+// Launch one cluster.
+template <auto Kernel, typename... A>
+cudaError_t launch_cluster(cudaStream_t st, A... args) {
+    static std::atomic<int> known[kCDevices];
+    int ctas = 1;
+    const cudaError_t e = cluster_ctas(Kernel, known, &ctas);
+    if (e != cudaSuccess) return e;
+    const int cap = codec_ctas_cap();
+    return launch_sized(Kernel, ctas < cap ? ctas : cap, st, args...);
 }
 
 }  // namespace bfsgb

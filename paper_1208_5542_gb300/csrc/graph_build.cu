@@ -15,6 +15,7 @@
 #include <new>
 #include <utility>
 
+#include "cluster.cuh"
 #include "common.cuh"
 #include "internal.h"
 
@@ -105,7 +106,11 @@ std::mutex t_flag_mu;
 std::condition_variable t_flag_free;
 unsigned long long* t_flags = nullptr;             // kHostFlags pairs, mapped and portable
 uint64_t t_flag_used[kHostFlags / 64] = {};
+
+thread_local int t_codec_ctas = kCC;
 }
+
+int codec_ctas_cap() { return t_codec_ctas; }
 
 bfs_status Scratch::alloc(size_t nbytes, cudaStream_t st) {
     int64_t k = g_fail_countdown.load();
@@ -974,6 +979,13 @@ const char* bfs_status_string(bfs_status s) {
         case BFS_ERR_NOT_FOUND: return "BFS_ERR_NOT_FOUND";
     }
     return "BFS_ERR_UNKNOWN";
+}
+
+bfs_status bfs_debug_codec_ctas(int32_t ctas) {
+    if (ctas < 0 || ctas > kCC || (ctas & (ctas - 1)))
+        return set_error(BFS_ERR_INVALID_ARG, "codec CTAs %d not 0 or a power of two up to %d", ctas, kCC);
+    t_codec_ctas = ctas ? ctas : kCC;
+    return BFS_OK;
 }
 
 bfs_status bfs_debug_fail_allocation(int64_t k) {

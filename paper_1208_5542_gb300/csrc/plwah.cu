@@ -42,7 +42,8 @@ __global__ void __launch_bounds__(kCT) plwah_from_wah(const uint32_t* __restrict
     auto is_fill = [&](uint32_t w) { return (w & kTop) != 0u; };
     int64_t carry = 0;
     int turn = 0;
-    for (int64_t base = 0; base < nw; base += kClusterRound, ++turn) {
+    const int64_t round = cluster_round();
+    for (int64_t base = 0; base < nw; base += round, ++turn) {
         const int64_t k0 = base + cluster_thread() * kCK;
         uint32_t word[kCK], emit = 0;
         uint32_t before = (k0 > 0 && k0 <= body) ? wah[k0 - 1] : 0u;   // no fill before the first word
@@ -87,7 +88,8 @@ __global__ void __launch_bounds__(kCT) wah_from_plwah(const uint32_t* __restrict
     int64_t carry = 0;
     bool bad = false;
     int turn = 0;
-    for (int64_t base = 0; base < nw; base += kClusterRound, ++turn) {
+    const int64_t round = cluster_round();
+    for (int64_t base = 0; base < nw; base += round, ++turn) {
         const int64_t k0 = base + cluster_thread() * kCK;
         uint32_t w[kCK], c = 0;
 #pragma unroll
@@ -148,7 +150,7 @@ bfs_status bfs_plwah_encode(const uint32_t* bits, int64_t nbits, uint32_t* words
     int64_t* cnt = tmp.as<int64_t>();
     uint32_t* wah = reinterpret_cast<uint32_t*>(cnt + 1);
     BFS_TRY(launch_wah_encode(bits, nbits, 32, wah, cnt, st));
-    BFS_CUDA_TRY(launch_cluster(plwah_from_wah, st, wah, cnt, nbits, words, nwords));
+    BFS_CUDA_TRY(launch_cluster<plwah_from_wah>(st, wah, cnt, nbits, words, nwords));
     BFS_CUDA_TRY(cudaStreamSynchronize(st));
     return BFS_OK;
 }
@@ -165,7 +167,7 @@ bfs_status bfs_plwah_decode(const uint32_t* words, int64_t nwords, int64_t nbits
     if (nwords > 0) {
         HostFlag said;                                // error, count; given back before the WAH decode takes its own
         BFS_TRY(said.take(st));
-        BFS_CUDA_TRY(launch_cluster(wah_from_plwah, st, words, nwords, nbits, wah.as<uint32_t>(),
+        BFS_CUDA_TRY(launch_cluster<wah_from_plwah>(st, words, nwords, nbits, wah.as<uint32_t>(),
                                     said.device(1), said.device(0)));
         BFS_TRY(said.wait());
         h_cnt = (int64_t)said.value(1);

@@ -73,7 +73,8 @@ __global__ void __launch_bounds__(kCT) wah_encode_bitmap(const uint32_t* bits, i
     int64_t run_start = 0;     // start group of the run holding the group before the round
     auto group = [&](int64_t g) { return bitmap_bits<W>(bits, words, g * GB) & T::ONES; };
     int turn = 0;
-    for (int64_t tb = 0; tb < G; tb += kClusterRound, ++turn) {
+    const int64_t round = cluster_round();
+    for (int64_t tb = 0; tb < G; tb += round, ++turn) {
         const int64_t g0 = tb + cluster_thread() * kCK;
         W x[kCK];
         int ty[kCK + 1];
@@ -1202,7 +1203,8 @@ __global__ void __launch_bounds__(kCT) wah_decode_bitmap(const W* in, int64_t nw
             atomicOr(bits + w + 2, (uint32_t)(v >> (sizeof(W) * 8 - sh)));
     };
     int turn = 0;
-    for (int64_t wb = 0; wb < nwords; wb += kClusterRound, ++turn) {
+    const int64_t round = cluster_round();
+    for (int64_t wb = 0; wb < nwords; wb += round, ++turn) {
         const int64_t x0 = wb + cluster_thread() * kCK;
         W y[kCK];
         long long len[kCK], sum = 0, tot;
@@ -1259,9 +1261,9 @@ __global__ void __launch_bounds__(kCT) wah_decode_bitmap(const W* in, int64_t nw
 bfs_status launch_wah_encode(const uint32_t* bits, int64_t nbits, int wah_bits, void* words, int64_t* count,
                              cudaStream_t st) {
     if (wah_bits == 32)
-        BFS_CUDA_TRY(launch_cluster(wah_encode_bitmap<uint32_t>, st, bits, nbits, static_cast<uint32_t*>(words), count));
+        BFS_CUDA_TRY(launch_cluster<wah_encode_bitmap<uint32_t>>(st, bits, nbits, static_cast<uint32_t*>(words), count));
     else
-        BFS_CUDA_TRY(launch_cluster(wah_encode_bitmap<unsigned long long>, st, bits, nbits,
+        BFS_CUDA_TRY(launch_cluster<wah_encode_bitmap<unsigned long long>>(st, bits, nbits,
                                     static_cast<unsigned long long*>(words), count));
     return BFS_OK;
 }
@@ -1314,10 +1316,10 @@ bfs_status launch_wah_decode_bitmap(const void* words, int64_t nwords, int64_t n
     const int64_t out_words = (nbits + 31) / 32;
     if (out_words > 0) BFS_CUDA_TRY(cudaMemsetAsync(bits, 0, sizeof(uint32_t) * (size_t)out_words, st));
     if (wah_bits == 32)
-        BFS_CUDA_TRY(launch_cluster(wah_decode_bitmap<uint32_t>, st, static_cast<const uint32_t*>(words), nwords, nbits,
+        BFS_CUDA_TRY(launch_cluster<wah_decode_bitmap<uint32_t>>(st, static_cast<const uint32_t*>(words), nwords, nbits,
                                     bits, err));
     else
-        BFS_CUDA_TRY(launch_cluster(wah_decode_bitmap<unsigned long long>, st,
+        BFS_CUDA_TRY(launch_cluster<wah_decode_bitmap<unsigned long long>>(st,
                                     static_cast<const unsigned long long*>(words), nwords, nbits, bits, err));
     return BFS_OK;
 }

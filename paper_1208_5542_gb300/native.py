@@ -86,6 +86,7 @@ _SIGS = {
     "bfs_run": (ctypes.c_int, [vp, i32, vp, vp, P(RunStats), vp]),
     "bfs_check_search": (ctypes.c_int, [vp, i32, vp, vp, vp]),
     "bfs_debug_fail_allocation": (ctypes.c_int, [i64]),
+    "bfs_debug_codec_ctas": (ctypes.c_int, [i32]),
     "bfs_server_set_queue_limit": (ctypes.c_int, [vp, i64]),
     "bfs_run_batch": (ctypes.c_int, [vp, vp, i32, vp, vp, P(BatchStats), vp]),
     "bfs_batch_autotune": (ctypes.c_int, [vp, vp, i32, vp, P(i32), P(i32), vp]),
