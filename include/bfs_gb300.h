@@ -309,7 +309,10 @@ typedef struct {
     float ms_directory_update;   /* dynamic cross directory: the frontier's bits evaluated before
                                     the exchange (bfs_graph_set_dynamic_directory; 0 without it) */
     int64_t compress_chunks;     /* chunks of 1024 groups the column sieve + compress read (each:
-                                    the chunk's frontier and directory bits) */
+                                    the chunk's frontier and directory bits).  Counted in the
+                                    recorded search, which reads no slot without frontier bits;
+                                    without statistics the one-launch encoder of short slots
+                                    reads those of one round (at most 4096 groups) as well */
     int64_t row_compress_chunks; /* chunks the row sieve + compress read (partial and visited bits) */
 } bfs_level_stats;
 

@@ -173,6 +173,16 @@ __device__ __forceinline__ void lay_out_units(const EncodeArgs& a) {
 // scale 17 346 / 439, directed uniform 1M vertices 447 / 490.  Slots of one round of 256
 // threads take that CTA (1024 threads: scale 12 213 us, scale 17 361); longer
 // ones 1024 (256: directed uniform 1M vertices 469 us, scale 20 558 -> 627).
+// All of its CTAs run, whether their slots hold anything or not, so it takes at
+// most two CTAs of 1024 threads per SM (or as many threads in small ones); with more
+// slots (p x p of them) the persistent passes, which handle live chunks only, are
+// the faster ones.  A search with this kernel / the three launches: scale 20 on 16 x
+// 16 (256 CTAs of 1024) 483 / 481 us, on 24 x 24 (576) 597 / 535, with the row
+// exchange 833 / 726; scale 18 on 32 x 32 (1024 CTAs of 256) 360 / 366, on 64 x 64
+// (4096) 693 / 634; scale 22 on 128 x 128 (16384 of 1024) 6677 / 3564.
+// The adaptive format adds the raw writer, with CTAs for every slot, to the
+// passes, and its one-round slots are always encoded here (scale 18 on 64 x 64 687
+// / 749, on 256 x 256 6605 / 6731; two-round slots, scale 22 on 64 x 64: 2646 / 1927).
 constexpr int kSK = 4;              // groups per thread and round
 constexpr int kSmallChunks = 8;     // two rounds (five rounds, 17 chunks of scale 22 on 8 x 8: 38 us against 26)
 
@@ -1281,12 +1291,15 @@ bfs_status launch_wah_encode_parallel(const EncodeArgs& a, int wah_bits, void* s
     uint8_t* fl = static_cast<uint8_t*>(flags);
     if (a.adaptive && (wah_bits != 32 || !a.fmt)) return set_error(BFS_ERR_INVALID_ARG, "adaptive format needs 32-bit words");
     const int64_t groups = a.nb / (wah_bits - 1);
-    if (groups <= (int64_t)kSmallChunks * kTile) {
+    const int small_nt = groups <= 256 * kSK ? 256 : 1024;
+    const int64_t room = (int64_t)(grid / kEWBlocks) * 2 * 1024;    // threads: two large CTAs per SM
+    const bool few = (int64_t)a.nslots * small_nt <= room || (a.adaptive && small_nt == 256);
+    if (groups <= (int64_t)kSmallChunks * kTile && few) {
         if (wah_bits == 32) {
-            if (groups <= 256 * kSK) enc_small<uint32_t, 256><<<a.nslots, 256, 0, st>>>(a, cps, setbits);
+            if (small_nt == 256) enc_small<uint32_t, 256><<<a.nslots, 256, 0, st>>>(a, cps, setbits);
             else enc_small<uint32_t, 1024><<<a.nslots, 1024, 0, st>>>(a, cps, setbits);
         } else {
-            if (groups <= 256 * kSK) enc_small<unsigned long long, 256><<<a.nslots, 256, 0, st>>>(a, cps, setbits);
+            if (small_nt == 256) enc_small<unsigned long long, 256><<<a.nslots, 256, 0, st>>>(a, cps, setbits);
             else enc_small<unsigned long long, 1024><<<a.nslots, 1024, 0, st>>>(a, cps, setbits);
         }
     } else if (wah_bits == 32) {
