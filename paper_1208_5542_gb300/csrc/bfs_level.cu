@@ -1406,8 +1406,18 @@ __global__ void __launch_bounds__(kNT) decode_streams(LevelArgs a) {
 // is about two thirds of the search.  Entries of a short row in flight: a row
 // usually ends after a few, and what was read past its end is lost; 2 / 3 / 4 /
 // 6 / 8 give 2.12 / 2.07 / 2.01 / 2.11 / 2.18 ms a search (adaptive format).
+//
+// A step over a short row tests its entries' ranges whether one hit or not: with
+// a shortcut past that (32 registers, 64 warps per SM) the long rows' one-warp
+// chains of a sparse level wait on all the others, and a bottom-up search at
+// scale 22 takes 4.10 ms instead of 3.31 (40 registers, 48 warps), at scale 24
+// 9.36 instead of 7.65.  The words are dealt out to twice the CTAs that fit at once,
+// so that an SM that is done early takes another one: 8 / 12 / 16 / 24 CTAs per SM
+// give 1.86 / 1.68 / 1.66 / 1.65 ms for a hybrid search at scale 24, 3.31 / 3.15 /
+// 3.13 / 3.07 bottom-up at scale 22, 235.9 / 238.5 / 240.2 / 243.3 us hybrid at scale 17.
 constexpr int64_t kBuLane = 32;
 constexpr int kBuIlp = 4;
+constexpr int kBuCtas = 12;         // CTAs per SM (6 are resident)
 
 // The frontier test of an entry u.  A sparse frontier is tested word-wise
 // first: `words` has a bit per 32 vertices (64 KB at scale 24, in L1, where
@@ -1452,17 +1462,13 @@ __global__ void __launch_bounds__(kNT) expand_bottom_up(LevelArgs a) {
             for (int64_t e = e0; e < e1 && !stop; e += kBuIlp) {
                 uint32_t u[kBuIlp];
                 bool hit[kBuIlp];
-                bool some = false;
 #pragma unroll
                 for (int k = 0; k < kBuIlp; ++k) u[k] = (e + k < e1) ? (uint32_t)__ldg(a.bu_adj + e + k) : NONE;
 #pragma unroll
                 for (int k = 0; k < kBuIlp; ++k) hit[k] = u[k] != NONE && fr.maybe(u[k]);
 #pragma unroll
-                for (int k = 0; k < kBuIlp; ++k) {
+                for (int k = 0; k < kBuIlp; ++k)
                     if (hit[k]) hit[k] = fr.test(u[k]);
-                    some |= hit[k];
-                }
-                if (!STATS && !some && best == NONE) continue;
 #pragma unroll
                 for (int k = 0; k < kBuIlp; ++k) {
                     if (u[k] == NONE || stop) continue;
@@ -2279,8 +2285,10 @@ bfs_status run_search(bfs_graph* g, int32_t root, int32_t* parent, int32_t* leve
         }
         BFS_CUDA_TRY(cudaGetLastError());
         if (bu_kernels) {
-            if (host) expand_bottom_up<true><<<sm_count() * 8, kNT, 0, s>>>(a);
-            else expand_bottom_up<false><<<sm_count() * 8, kNT, 0, s>>>(a);
+            const int64_t ctas = ((L.n + 31) / 32 + kNT / 32 - 1) / (kNT / 32);      // a warp per visited word
+            const unsigned bgrid = (unsigned)std::min<int64_t>(ctas, (int64_t)sm_count() * kBuCtas);
+            if (host) expand_bottom_up<true><<<bgrid, kNT, 0, s>>>(a);
+            else expand_bottom_up<false><<<bgrid, kNT, 0, s>>>(a);
             BFS_CUDA_TRY(cudaGetLastError());
         }
         if (host && timing) cudaEventRecord(W.ev[3], s);
