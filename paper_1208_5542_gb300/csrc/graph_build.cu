@@ -363,6 +363,8 @@ constexpr int kAllBuckets = 16384;                              // buckets of al
 constexpr int kColThreads = 1024;
 constexpr int kColWindow = 32768;                               // columns counted together in shared memory
 constexpr int kMaxPartGrid = 32;                                // grids up to 32 x 32 (1024 blocks) are partitioned
+constexpr int kColCtas = 152;
+constexpr int64_t kMinShare = 32768;                            // entries of a part of a split bucket, at least
 
 struct PartArgs {
     const int32_t* src;
@@ -472,49 +474,96 @@ constexpr size_t kPartSmem = sizeof(uint2) * 2 * kPartTile + (sizeof(uint32_t) +
                              sizeof(uint16_t) * 2 * kPartTile;
 static_assert(kGroupBuckets == 2 * kPartThreads, "a thread scans two buckets");
 
-// One CTA per bucket of a group, kColWindow of its columns at a time (a bucket
-// with more columns reads its entries again, from L2).
+// Work of a CTA: a bucket of a group, or a share of a large one's entries.
+struct ColUnit {
+    int64_t e0, e1;         // entries
+    int32_t bucket;
+    int32_t share;          // -1: the whole bucket; else its row of `before`
+};
+
+// One CTA per unit, taken in turn from *next, kColWindow of its bucket's columns
+// at a time (a bucket with more columns reads its entries again, from L2).
 //   COUNT: the entries of every column, written to cnt (the group's counts).
+//          The shares of a split bucket add theirs to cnt (zero before) and
+//          keep what was there: the place of their entries in the column.
 //   else:  every entry into its column (order inside a column is arbitrary);
 //          off holds the columns' offsets in their blocks, ir_base the blocks'.
+// A bucket with many times the entries of the others would leave the chip to
+// one CTA (a Kronecker graph whose labels are not scrambled: 6% of scale 22's
+// entries on 8 x 8 in one of 1024 buckets: COUNT and fill took 1.6 + 5.9 ms, the
+// build 11.4; with the shares of split_buckets 5.7).
 template <bool COUNT>
 __global__ void __launch_bounds__(kColThreads) bucket_columns(PartArgs a, const uint2* __restrict__ pairs,
-                                                              const int64_t* __restrict__ starts, int buckets,
+                                                              const ColUnit* __restrict__ units, int nunits, int* next,
                                                               uint32_t* __restrict__ cnt,
+                                                              uint32_t* __restrict__ before, int64_t before_cols,
                                                               const int64_t* __restrict__ ir_base,
                                                               int32_t* __restrict__ ir) {
     extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ int s_unit;
     uint32_t* s_col = reinterpret_cast<uint32_t*>(smem);
     constexpr int K = 4;
-    for (int bkt = blockIdx.x; bkt < buckets; bkt += gridDim.x) {
-        const uint32_t block = (uint32_t)bkt / (uint32_t)a.parts, part = (uint32_t)bkt % (uint32_t)a.parts;
+    for (;;) {
+        if (threadIdx.x == 0) s_unit = atomicAdd(next, 1);
+        __syncthreads();
+        const int x0 = s_unit;
+        __syncthreads();
+        if (x0 >= nunits) return;
+        const ColUnit un = units[x0];
+        const uint32_t block = (uint32_t)un.bucket / (uint32_t)a.parts, part = (uint32_t)un.bucket % (uint32_t)a.parts;
         const uint32_t first = part << a.shift;
         const uint32_t cols = first < a.nb ? min(1u << a.shift, a.nb - first) : 0u;
-        const int64_t e0 = starts[bkt], e1 = starts[bkt + 1];
         for (uint32_t w0 = 0; w0 < cols; w0 += kColWindow) {
             const uint32_t wn = min((uint32_t)kColWindow, cols - w0);
             const uint32_t c0 = block * a.nb + first + w0;         // count index of the window's first column
             uint32_t* g = cnt + c0;
-            for (uint32_t c = threadIdx.x; c < wn; c += kColThreads) s_col[c] = COUNT ? 0u : g[c];
+            uint32_t* bf = un.share >= 0 ? before + un.share * before_cols + w0 : nullptr;
+            for (uint32_t c = threadIdx.x; c < wn; c += kColThreads) s_col[c] = COUNT ? 0u : g[c] + (bf ? bf[c] : 0u);
             __syncthreads();
             int32_t* out = COUNT ? nullptr : ir + ir_base[block];
-            for (int64_t e = e0 + threadIdx.x; e < e1; e += K * kColThreads) {
+            for (int64_t e = un.e0 + threadIdx.x; e < un.e1; e += K * kColThreads) {
                 uint2 x[K];
 #pragma unroll
-                for (int k = 0; k < K; ++k) x[k] = e + k * kColThreads < e1 ? pairs[e + k * kColThreads] : make_uint2(~0u, 0u);
+                for (int k = 0; k < K; ++k) x[k] = e + k * kColThreads < un.e1 ? pairs[e + k * kColThreads] : make_uint2(~0u, 0u);
 #pragma unroll
                 for (int k = 0; k < K; ++k) {
-                    if (e + k * kColThreads >= e1 || x[k].x - c0 >= wn) continue;
+                    if (e + k * kColThreads >= un.e1 || x[k].x - c0 >= wn) continue;
                     const uint32_t pos = atomicAdd(s_col + (x[k].x - c0), 1u);
                     if (!COUNT) out[pos] = (int32_t)x[k].y;
                 }
             }
             __syncthreads();
             if (COUNT)
-                for (uint32_t c = threadIdx.x; c < wn; c += kColThreads) g[c] = s_col[c];
+                for (uint32_t c = threadIdx.x; c < wn; c += kColThreads) {
+                    if (!bf) g[c] = s_col[c];
+                    else bf[c] = s_col[c] ? atomicAdd(g + c, s_col[c]) : 0u;
+                }
             __syncthreads();
         }
     }
+}
+
+// The units of buckets with `held` entries each, laid out from entry 0 on.  A
+// bucket of more than a CTA's mean is cut into shares of half of it (the largest
+// units first, then).  Returns the number of shares.
+int split_buckets(const uint64_t* held, int buckets, std::vector<ColUnit>& units) {
+    int64_t total = 0;
+    for (int b = 0; b < buckets; ++b) total += (int64_t)held[b];
+    const int64_t share = std::max(kMinShare, total / (2 * kColCtas));
+    int shares = 0;
+    int64_t at = 0;
+    units.clear();
+    for (int b = 0; b < buckets; ++b) {
+        const int64_t end = at + (int64_t)held[b];
+        if (end - at <= 2 * share) units.push_back({at, end, b, -1});
+        else
+            for (int64_t e = at; e < end; e += share) units.push_back({e, std::min(e + share, end), b, shares++});
+        at = end;
+    }
+    if (shares)
+        std::stable_sort(units.begin(), units.end(),
+                         [](const ColUnit& x, const ColUnit& y) { return x.e1 - x.e0 > y.e1 - y.e0; });
+    return shares;
 }
 
 // The parts of a block's source range: as many as give kColWindow columns
@@ -688,11 +737,19 @@ bfs_status build_layout(bfs_graph* g, int64_t n, int64_t m, const int32_t* d_src
     PartArgs pa{d_src, d_dst, m, symmetrize, p, 1, 31, (uint32_t)n, (uint32_t)nb};
     if (partitioned) choose_parts(pa);
     const int buckets = (int)nblocks * pa.parts, per_row = p * pa.parts;
-    DevBuf cnt, pairs;
-    Scratch err, cursor, starts;
+    DevBuf cnt;
+    Scratch said, cursor;
     BFS_TRY(cnt.alloc(sizeof(uint32_t) * nblocks * nb));
-    BFS_TRY(err.alloc(sizeof(unsigned long long), st));
-    BFS_CUDA_TRY(cudaMemsetAsync(err.ptr, 0, sizeof(unsigned long long), st));
+    BFS_TRY(said.alloc(sizeof(unsigned long long), st));
+    BFS_CUDA_TRY(cudaMemsetAsync(said.ptr, 0, sizeof(unsigned long long), st));
+    unsigned long long h_said = 0;                                     // bad ids
+    auto hear = [&]() -> bfs_status {
+        BFS_CUDA_TRY(cudaGetLastError());
+        BFS_CUDA_TRY(cudaMemcpyAsync(&h_said, said.ptr, sizeof(h_said), cudaMemcpyDeviceToHost, st));
+        BFS_CUDA_TRY(cudaStreamSynchronize(st));
+        if (h_said) return set_error(BFS_ERR_INVALID_ARG, "an edge names a vertex outside [0, %lld)", (long long)n);
+        return BFS_OK;
+    };
     std::vector<uint64_t> held(partitioned ? buckets : 0);             // entries per bucket
     if (partitioned) {
         const size_t cursor_bytes = sizeof(unsigned long long) * std::max(buckets, kGroupBuckets);
@@ -702,19 +759,10 @@ bfs_status build_layout(bfs_graph* g, int64_t n, int64_t m, const int32_t* d_src
         BFS_CUDA_TRY(cudaFuncSetAttribute(bucket_counts, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)(sizeof(uint32_t) * kAllBuckets)));
         bucket_counts<<<152 * 3, kPartThreads, smem, st>>>(pa, buckets, cursor.as<unsigned long long>(),
-                                                           err.as<unsigned long long>());
-    } else {
-        BFS_CUDA_TRY(cudaMemsetAsync(cnt.ptr, 0, cnt.bytes, st));
-        count_entries<<<grid_for(m, 256), 256, 0, st>>>(d_src, d_dst, m, symmetrize, n, nb, row_stride,
-                                                        cnt.as<uint32_t>(), err.as<unsigned long long>());
-    }
-    BFS_CUDA_TRY(cudaGetLastError());
-    unsigned long long h_err = 0;
-    BFS_CUDA_TRY(cudaMemcpyAsync(&h_err, err.ptr, sizeof(h_err), cudaMemcpyDeviceToHost, st));
-    if (partitioned)
+                                                           said.as<unsigned long long>());
         BFS_CUDA_TRY(cudaMemcpyAsync(held.data(), cursor.ptr, sizeof(uint64_t) * buckets, cudaMemcpyDeviceToHost, st));
-    BFS_CUDA_TRY(cudaStreamSynchronize(st));
-    if (h_err) return set_error(BFS_ERR_INVALID_ARG, "an edge names a vertex outside [0, %lld)", (long long)n);
+        BFS_TRY(hear());
+    }
 
     BFS_TRY(alloc_parts(L.small, {{&L.dir, sizeof(uint32_t) * nblocks * L.dir_stride},
                                   {&L.rank, sizeof(uint32_t) * nblocks * L.dir_stride},
@@ -743,12 +791,11 @@ bfs_status build_layout(bfs_graph* g, int64_t n, int64_t m, const int32_t* d_src
         return BFS_OK;
     };
 
-    if (!partitioned) {
-        BFS_TRY(counted(0, p));
-    } else {
-        // groups of block-rows: at most kGroupBuckets buckets, and entries that fit the
-        // partition buffer (an eighth of all entries, at least 1 GiB); every group
-        // reads all tuples once
+    auto partitioned_columns = [&]() -> bfs_status {
+        // groups of block-rows: at most kGroupBuckets buckets, and an eighth of all
+        // entries, at least 1 GiB of them (a block-row that holds more is a group of
+        // its own: with p = 1 the buffer takes twice the entries' own memory); every
+        // group reads all tuples once
         struct Group { int r0, r1; int64_t entries; };
         std::vector<Group> groups;
         const int64_t room = std::max<int64_t>(L.nnz / 8, (1ll << 30) / (int64_t)sizeof(uint2));
@@ -764,37 +811,63 @@ bfs_status build_layout(bfs_graph* g, int64_t n, int64_t m, const int32_t* d_src
                 groups.back() = {groups.back().r0, r + 1, groups.back().entries + row};
             most = std::max(most, groups.back().entries);
         }
+        DevBuf pairs;                                                   // released on return: the column offsets come next
+        Scratch d_base, d_units, d_next;
+        constexpr size_t kMaxUnits = kGroupBuckets + 3 * kColCtas;      // 2 kColCtas shares and one more per split bucket
         BFS_TRY(pairs.alloc(sizeof(uint2) * (size_t)most));
-        BFS_TRY(starts.alloc(sizeof(int64_t) * (kGroupBuckets + 1 + (size_t)nblocks), st));
+        BFS_TRY(d_base.alloc(sizeof(int64_t) * (size_t)nblocks, st));
+        BFS_TRY(d_units.alloc(sizeof(ColUnit) * kMaxUnits, st));
+        BFS_TRY(d_next.alloc(2 * sizeof(int), st));
         std::vector<int64_t> base((size_t)nblocks, 0);                  // first entry of every block
         for (int64_t b = 0, at = 0; b < nblocks; ++b) {
             base[b] = at;
             for (int k = 0; k < pa.parts; ++k) at += (int64_t)held[(size_t)b * pa.parts + k];
         }
-        int64_t* d_base = starts.as<int64_t>() + kGroupBuckets + 1;
-        BFS_CUDA_TRY(cudaMemcpyAsync(d_base, base.data(), sizeof(int64_t) * nblocks, cudaMemcpyHostToDevice, st));
+        BFS_CUDA_TRY(cudaMemcpyAsync(d_base.ptr, base.data(), sizeof(int64_t) * nblocks, cudaMemcpyHostToDevice, st));
         const int col_smem = (int)sizeof(uint32_t) * (int)std::min<int64_t>(kColWindow, nb);
+        const int64_t bucket_cols = std::min<int64_t>(1ll << pa.shift, nb);
         BFS_CUDA_TRY(cudaFuncSetAttribute(partition_entries, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPartSmem));
         for (auto k : {bucket_columns<true>, bucket_columns<false>})
             BFS_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)sizeof(uint32_t) * kColWindow));
+        std::vector<ColUnit> units;
         for (const Group& g : groups) {
             const int b0 = g.r0 * per_row, nbk = (g.r1 - g.r0) * per_row;
-            std::vector<int64_t> at((size_t)nbk + 1, 0);
-            for (int k = 0; k < nbk; ++k) at[k + 1] = at[k] + (int64_t)held[(size_t)b0 + k];
-            BFS_CUDA_TRY(cudaMemcpyAsync(starts.ptr, at.data(), sizeof(int64_t) * (nbk + 1), cudaMemcpyHostToDevice, st));
-            BFS_CUDA_TRY(cudaMemcpyAsync(cursor.ptr, starts.ptr, sizeof(int64_t) * nbk, cudaMemcpyDeviceToDevice, st));
+            std::vector<int64_t> at((size_t)nbk, 0);
+            for (int k = 0; k + 1 < nbk; ++k) at[k + 1] = at[k] + (int64_t)held[(size_t)b0 + k];
+            const int shares = split_buckets(held.data() + b0, nbk, units);
+            if (units.size() > kMaxUnits) return set_error(BFS_ERR_CUDA, "layout build: %zu units", units.size());
+            uint32_t* c = cnt.as<uint32_t>() + g.r0 * row_stride;
+            Scratch before;                                             // per share and column: the entries of the shares before
+            if (shares) {
+                BFS_TRY(before.alloc(sizeof(uint32_t) * (size_t)(shares * bucket_cols), st));
+                BFS_CUDA_TRY(cudaMemsetAsync(c, 0, sizeof(uint32_t) * (size_t)((g.r1 - g.r0) * row_stride), st));
+            }
+            BFS_CUDA_TRY(cudaMemcpyAsync(cursor.ptr, at.data(), sizeof(int64_t) * nbk, cudaMemcpyHostToDevice, st));
+            BFS_CUDA_TRY(cudaMemcpyAsync(d_units.ptr, units.data(), sizeof(ColUnit) * units.size(), cudaMemcpyHostToDevice, st));
+            BFS_CUDA_TRY(cudaMemsetAsync(d_next.ptr, 0, 2 * sizeof(int), st));
             partition_entries<<<152 * 2, kPartThreads, kPartSmem, st>>>(pa, g.r0, g.r1, (uint32_t)b0,
                                                                         cursor.as<unsigned long long>(), pairs.as<uint2>());
-            uint32_t* c = cnt.as<uint32_t>() + g.r0 * row_stride;
-            bucket_columns<true><<<152, kColThreads, col_smem, st>>>(pa, pairs.as<uint2>(), starts.as<int64_t>(), nbk, c,
-                                                                     nullptr, nullptr);
+            bucket_columns<true><<<kColCtas, kColThreads, col_smem, st>>>(
+                pa, pairs.as<uint2>(), d_units.as<ColUnit>(), (int)units.size(), d_next.as<int>(), c,
+                before.as<uint32_t>(), bucket_cols, nullptr, nullptr);
             BFS_CUDA_TRY(cudaGetLastError());
-            BFS_TRY(counted(g.r0, g.r1));                                // synchronises: `at` is free to go
-            bucket_columns<false><<<152, kColThreads, col_smem, st>>>(pa, pairs.as<uint2>(), starts.as<int64_t>(), nbk, c,
-                                                                      d_base + (int64_t)g.r0 * p, L.ir.as<int32_t>());
+            BFS_TRY(counted(g.r0, g.r1));                                // synchronises: the host arrays are free to go
+            bucket_columns<false><<<kColCtas, kColThreads, col_smem, st>>>(
+                pa, pairs.as<uint2>(), d_units.as<ColUnit>(), (int)units.size(), d_next.as<int>() + 1, c,
+                before.as<uint32_t>(), bucket_cols, d_base.as<int64_t>() + (int64_t)g.r0 * p, L.ir.as<int32_t>());
             BFS_CUDA_TRY(cudaGetLastError());
         }
+        return BFS_OK;
+    };
+    if (partitioned) {
+        BFS_TRY(partitioned_columns());
+    } else {
+        BFS_CUDA_TRY(cudaMemsetAsync(cnt.ptr, 0, cnt.bytes, st));
+        count_entries<<<grid_for(m, 256), 256, 0, st>>>(d_src, d_dst, m, symmetrize, n, nb, row_stride,
+                                                        cnt.as<uint32_t>(), said.as<unsigned long long>());
+        BFS_TRY(hear());
+        BFS_TRY(counted(0, p));
     }
 
     // rank = exclusive scan of popcounts per block; nnzc_b = totals

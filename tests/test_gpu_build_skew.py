@@ -1,0 +1,58 @@
+"""The partitioned graph build on skewed graphs (buckets cut into shares) on a GB300 against the oracle."""
+import numpy as np
+import pytest
+
+import graphgen
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+def kronecker(n, m, seed=5):
+    """Kronecker tuples without scrambled labels: block (0, 0) holds most entries."""
+    rng = np.random.default_rng(seed)
+    src, dst = np.zeros(m, np.int64), np.zeros(m, np.int64)
+    k = (n - 1).bit_length()
+    for _ in range(k):
+        r = rng.random(m, dtype=np.float32)
+        row = r >= 0.76
+        src, dst = 2 * src + row, 2 * dst + ((r >= 0.95) | ((r >= 0.57) & ~row))
+    return (src * n >> k).astype(np.int32), (dst * n >> k).astype(np.int32)
+
+
+def tuples(kind, n, m):
+    if kind == "kronecker":
+        return kronecker(n, m)
+    src, dst = graphgen.random_edges(n, m, seed=n)
+    if kind == "star":                      # one column with half of the entries
+        src[:] = n // 3
+    if kind == "narrow":                    # all columns in one bucket, its last window ragged
+        src[:] = n - 1 - src % 40_000
+    return src, dst
+
+
+@pytest.mark.parametrize("kind,n,m,p,symmetrize", [
+    ("kronecker", 1 << 21, 3_000_000, 8, True), ("kronecker", 1_600_001, 6_000_000, 8, False),
+    ("kronecker", 13_000_003, 3_000_000, 1, True), ("star", 1_800_001, 3_000_000, 7, True),
+    ("star", 6_300_673, 4_000_000, 2, False), ("narrow", 6_300_673, 4_000_000, 2, False),
+    ("narrow", 13_000_003, 4_000_000, 1, False),
+    ("kronecker", 17_000_003, 35_000_000, 32, True),      # several shared-memory windows per bucket, some of them split
+    ])
+def test_skewed_build(kind, n, m, p, symmetrize):
+    import torch
+    from paper_1208_5542_gb300 import bfs
+    src, dst = tuples(kind, n, m)
+    go = oracle.csr(n, src, dst, symmetrize=symmetrize)
+    g = bfs.Graph.from_edges(n, src, dst, symmetrize=symmetrize, p=p)
+    assert g.n_entries == len(go.col)
+    pairs = [(i, j) for i in range(p) for j in range(p)]
+    for i, j in pairs if p <= 4 else pairs[:: p + 3]:
+        want = oracle.pack_bits(oracle.directory(go, p, i, j))
+        assert (g.directory(i, j).cpu().numpy().view(np.uint32) == want).all(), (i, j)
+    deg = np.diff(go.row_ptr)
+    root = int(src[0])
+    lv, pa = oracle.bfs(go, root)
+    parent, level, st = g.run(root, stats=True, max_levels=1024)
+    torch.cuda.synchronize()
+    assert (level.cpu().numpy() == lv).all() and (parent.cpu().numpy() == pa).all()
+    assert sum(v["edges_scanned"] for v in st.levels) == int(deg[lv >= 0].sum())
