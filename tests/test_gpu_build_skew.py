@@ -1,4 +1,5 @@
-"""The partitioned graph build on skewed graphs (buckets cut into shares) on a GB300 against the oracle."""
+"""The partitioned graph build on skewed graphs (buckets cut into shares), and the graphs that are built in tuple
+order after all, on a GB300 against the oracle."""
 import numpy as np
 import pytest
 
@@ -28,6 +29,9 @@ def tuples(kind, n, m):
         src[:] = n // 3
     if kind == "narrow":                    # all columns in one bucket, its last window ragged
         src[:] = n - 1 - src % 40_000
+    if kind == "mesh":                      # neighbours in order, a shortcut now and then
+        src = (np.arange(m, dtype=np.int64) * n // m).astype(np.int32)
+        dst[np.arange(m) % 16 != 0] = np.minimum(src + 1, n - 1)[np.arange(m) % 16 != 0]
     return src, dst
 
 
@@ -37,7 +41,7 @@ def tuples(kind, n, m):
     ("star", 6_300_673, 4_000_000, 2, False), ("narrow", 6_300_673, 4_000_000, 2, False),
     ("narrow", 13_000_003, 4_000_000, 1, False),
     ("kronecker", 17_000_003, 35_000_000, 32, True),      # several shared-memory windows per bucket, some of them split
-    ])
+    ("mesh", 6_300_673, 6_400_000, 2, True), ("uniform", 6_300_673, 500_000, 4, True)])      # in tuple order after all
 def test_skewed_build(kind, n, m, p, symmetrize):
     import torch
     from paper_1208_5542_gb300 import bfs
