@@ -112,6 +112,10 @@ BFS_API bfs_status bfs_last_error(char *buf, int64_t len);
  * each block stored column-compressed over its nonempty source columns with
  * the directory vector V_{i,j} of Eq. 4 as the column index.  The graph owns
  * all of its device memory.  Synchronises `cuda_stream`.
+ * While it runs, the build holds the copied tuples (8 bytes each), 4 bytes per
+ * block-row and vertex and, on large graphs, a partition buffer of 8 bytes per
+ * entry of one group of block-rows (about an eighth of all entries, one
+ * block-row at least); when the buffer cannot be had, it builds without it.
  * Errors: BFS_ERR_INVALID_ARG for n outside [1, 2^31-1], n_edges < 0, an id
  * outside [0, n), a bad option; BFS_ERR_OUT_OF_MEMORY; BFS_ERR_CUDA.
  */
@@ -480,7 +484,8 @@ BFS_API bfs_status bfs_server_destroy(bfs_server_t s);
  * paper): the k-th device allocation the library makes from now on (k >= 1;
  * allocations of graphs, search workspaces, batches, server lanes and codec
  * scratch) fails as if the device were out of memory, and the call that made
- * it returns BFS_ERR_OUT_OF_MEMORY after releasing what it had allocated.
+ * it returns BFS_ERR_OUT_OF_MEMORY after releasing what it had allocated (a
+ * graph build goes on without a partition buffer that it cannot have).
  * k = 0 disarms.  Process-wide; not for production use.
  */
 BFS_API bfs_status bfs_debug_fail_allocation(int64_t k);

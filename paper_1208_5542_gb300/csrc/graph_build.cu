@@ -356,7 +356,7 @@ __global__ void scatter_entries(const int32_t* __restrict__ src, const int32_t* 
 // partitioned entry is its column's count index, relative to the first
 // block-row of its group, and its destination.
 //
-// Two kinds of graph are built in tuple order whatever their size:
+// Three kinds of graph are built in tuple order whatever their size:
 //   - with few entries per count: the partitioned build reads and writes every
 //     count where the direct one touches the entries' own.  Uniform 2^25 vertices
 //     on 8 x 8, entries per count 1/16: 6.87 ms against 7.48, 1/8: 9.15 against
@@ -364,7 +364,9 @@ __global__ void scatter_entries(const int32_t* __restrict__ src, const int32_t* 
 //   - whose tuples come in an order in which neighbours share their columns'
 //     sectors (a mesh in its natural order, a sorted directed graph): the counts
 //     they touch are on chip anyway.  A 3000 x 3000 grid on 8 x 8 2.30 ms against
-//     3.46, a sorted directed scale-24 graph on 16 x 16 10.1 against 15.7.
+//     3.46, a sorted directed scale-24 graph on 16 x 16 10.1 against 15.7;
+//   - whose partition buffer does not fit in memory beside the counts and the
+//     entries.
 constexpr int kPartThreads = 512;
 constexpr int kPartTuples = 8;                                  // per thread and tile
 constexpr int kPartTile = kPartThreads * kPartTuples;           // tuples per tile: up to twice the entries
@@ -904,8 +906,16 @@ bfs_status build_layout(bfs_graph* g, int64_t n, int64_t m, const int32_t* d_src
         return BFS_OK;
     };
     if (partitioned) {
-        BFS_TRY(partitioned_columns());
-    } else {
+        const bfs_status rc = partitioned_columns();
+        if (rc == BFS_ERR_OUT_OF_MEMORY) {                               // the direct build needs none of it
+            partitioned = false;
+            nnz_b.clear();
+            BFS_CUDA_TRY(cudaMemsetAsync(L.deg.ptr, 0, L.deg.bytes, st));
+        } else if (rc != BFS_OK) {
+            return rc;
+        }
+    }
+    if (!partitioned) {
         BFS_CUDA_TRY(cudaMemsetAsync(cnt.ptr, 0, cnt.bytes, st));
         count_entries<<<grid_for(m, 256), 256, 0, st>>>(d_src, d_dst, m, symmetrize, n, nb, row_stride,
                                                         cnt.as<uint32_t>(), said.as<unsigned long long>());

@@ -1,5 +1,5 @@
 """The partitioned graph build on skewed graphs (buckets cut into shares), and the graphs that are built in tuple
-order after all, on a GB300 against the oracle."""
+order after all, on a GB300 against the oracle; a build whose partition buffer does not fit."""
 import numpy as np
 import pytest
 
@@ -60,3 +60,30 @@ def test_skewed_build(kind, n, m, p, symmetrize):
     torch.cuda.synchronize()
     assert (level.cpu().numpy() == lv).all() and (parent.cpu().numpy() == pa).all()
     assert sum(v["edges_scanned"] for v in st.levels) == int(deg[lv >= 0].sum())
+
+
+def test_build_without_room_for_the_partition():
+    """Every allocation of a partitioned build fails once: those that the direct build does not need cost nothing."""
+    from paper_1208_5542_gb300 import bfs
+    from paper_1208_5542_gb300.native import BfsError
+    n, p = 1 << 21, 7
+    src, dst = tuples("uniform", n, 3_000_000)
+    go = oracle.csr(n, src, dst)
+    root = int(src[0])
+    lv, pa = oracle.bfs(go, root)
+    built = []
+    for k in range(1, 30):
+        bfs.debug_fail_allocation(k)
+        try:
+            g = bfs.Graph.from_edges(n, src, dst, p=p)
+        except BfsError as e:
+            assert "OUT_OF_MEMORY" in str(e)
+            built.append(False)
+            continue
+        finally:
+            bfs.debug_fail_allocation(0)
+        built.append(True)
+        parent, level, _ = g.run(root)
+        assert (level.cpu().numpy() == lv).all() and (parent.cpu().numpy() == pa).all(), k
+    # some failure was absorbed: a build that succeeded, and a later allocation whose failure was not
+    assert not built[0] and built[-1] and any(a and not b for a, b in zip(built, built[1:])), built
