@@ -557,17 +557,34 @@ __device__ void window_enter(const LevelArgs& a, uint32_t* s_pi, uint32_t* s_t, 
 }
 
 // Hand out the units [0, total) of a level without a row window: a warp takes
-// `batch` consecutive units at a time.  Few units are dealt out in turn (no
-// counter to wait for), many by a counter: a guided hand-out of a share of
-// what is left (at least `batch`), so that early grabs are large and the last
-// ones small.  The units come in the order of the block-rows; the share is one
+// `batch` consecutive units at a time.  Few units (up to `deal` per warp) are dealt
+// out in turn (no counter to wait for), many by a counter: a guided hand-out of a
+// share of what is left (at least `batch`), so that early grabs are large and the
+// last ones small.  The units come in the order of the block-rows; the share is one
 // of a row's units, so that all warps work on about one row at a time (its
 // visited, next and parent lines stay on chip).
+// A heavy level (four entries per vertex of the graph) ends on two units at a time:
+// with eight, or dealt out up to there, the warps with the last units keep the chip
+// waiting (ms a search, scale 24 on 4 x 4 3.35 against 2.88, with the row exchange 3.99 /
+// 3.44, PLAIN 2.98 / 2.73, unscrambled 18.5 / 9.7, uniform 20M 4.95 / 4.01; one at a
+// time 2.84, 3.39, 2.65 and 3.95, but uniform 25M on 16 x 16 8.36 against 8.00).  The units
+// of the others hold too little for that (PLAIN, uniform 2^25 of edge factor 2:
+// 4.29 with eight, 4.67 with two).
+struct HandOut {
+    int64_t batch, deal;
+};
+
+__device__ __forceinline__ HandOut hand_out(const LevelArgs& a, int64_t total, int64_t light) {
+    if (a.ctl->m_f < 4 * a.n) return HandOut{light, 4 * light};
+    return HandOut{total > 4 * (int64_t)gridDim.x * kXW ? 2 : 1, 4};
+}
+
 template <typename Work>
-__device__ __forceinline__ void flat_units(unsigned long long* counter, int64_t total, int64_t batch, int rows,
+__device__ __forceinline__ void flat_units(unsigned long long* counter, int64_t total, HandOut h, int rows,
                                            Work do_units) {
+    const int64_t batch = h.batch;
     const int64_t warps = (int64_t)gridDim.x * kXW;
-    if (total <= 4 * warps * batch) {
+    if (total <= h.deal * warps) {
         const int64_t stride = warps * batch;
         for (int64_t x = ((int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * batch; x < total; x += stride)
             do_units(x, (x + batch < total) ? x + batch : total);
@@ -778,7 +795,8 @@ __device__ __forceinline__ void expand_wah_level(const LevelArgs& a, uint32_t* s
     };
     if (WIN == kWinNone) {
         const int64_t each = (units << shift) / (2 * (int64_t)gridDim.x * kXW);   // few hand-outs per warp
-        flat_units(a.row_next, units << shift, each < 1 ? 1 : (each < 8 ? each : 8), p, do_units);
+        flat_units(a.row_next, units << shift, hand_out(a, units << shift, each < 1 ? 1 : (each < 8 ? each : 8)), p,
+                   do_units);
     } else {
         auto row_begin = [&](int r) -> int64_t { return a.slot_unit_base[(int64_t)r * p] << shift; };
         auto units_in_row = [&](int r) -> int64_t {
@@ -843,7 +861,7 @@ __device__ __forceinline__ void expand_plain_level(const LevelArgs& a, uint32_t*
     const bool dense = a.ctl->frontier * 64 >= a.n;
     const int64_t batch = dense ? (sp.parts > 1 ? 1 : 2) : (each < 32 ? each : 32);
     if (WIN == kWinNone) {
-        flat_units(a.row_next, total, dense ? (each < 8 ? each : 8) : batch, p, do_units);
+        flat_units(a.row_next, total, hand_out(a, total, dense ? (each < 8 ? each : 8) : batch), p, do_units);
     } else {
         auto row_begin = [&](int r) -> int64_t { return (per_row << shift) * r; };
         auto units_in_row = [&](int) -> int64_t { return per_row << shift; };
@@ -884,7 +902,7 @@ __device__ __forceinline__ void expand_pieces_level(const LevelArgs& a, uint32_t
                 if (n <= 4 * warps) {
                     for (; next < begin + n; next += warps) piece(base + next - begin);
                 } else {
-                    flat_units(a.row_piece_next + row, n, 1, 1, [&](int64_t x, int64_t xe) {
+                    flat_units(a.row_piece_next + row, n, HandOut{1, 4}, 1, [&](int64_t x, int64_t xe) {
                         for (; x < xe; ++x) piece(base + x);
                     });
                     next += n;
