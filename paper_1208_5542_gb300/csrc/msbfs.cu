@@ -1142,6 +1142,7 @@ void call(ServeGraph* sg) {
 
 bool launch_iteration(bfs_server* s, ServeGraph* sg) {
     std::unique_lock<std::mutex> lk(s->mu);
+    if (s->stop) return false;                       // the call that ends the last launch is not taken back
     // admission into free lanes, while the results would fit in the budget
     int nadm = 0;
     unsigned long long mask = 0;
