@@ -112,7 +112,7 @@ BFS_API bfs_status bfs_last_error(char *buf, int64_t len);
  * each block stored column-compressed over its nonempty source columns with
  * the directory vector V_{i,j} of Eq. 4 as the column index.  The graph owns
  * all of its device memory.  Synchronises `cuda_stream`.
- * While it runs, the build holds the copied tuples (8 bytes each), 4 bytes per
+ * While it runs, the build holds the tuples (8 bytes each), 4 bytes per
  * block-row and vertex and, on large graphs, a partition buffer of 8 bytes per
  * entry of one group of block-rows (about an eighth of all entries, one
  * block-row at least); when the buffer cannot be had, it builds without it.

@@ -127,7 +127,6 @@ struct LevelArgs {
     // compressed row exchange (the fold of the 2D partition): per block (i,j)
     // the destinations it reached, t_{i,j}, as a bitmap of range i; the
     // encoder turns t_{i,j} & ~pi_i into the row buffer of slot i*p + j
-    int row_exchange;
     uint32_t* tblk;                     // p*p partial bitmaps, dir_stride words each
     const void* rowbuf;                 // row buffers: p*p slots of row_cap words
     int64_t row_cap;
@@ -1039,7 +1038,7 @@ constexpr int kFoldIlp = 4;         // word tiles whose loads a fold warp issues
 //   ROWS = false: the column slots of a bottom-up level decoded into the one
 //     bitmap the bottom-up scan reads -- the OR over the block-rows i of slots
 //     (i, j) (COMPRESS_SIEVE) or slot j (COMPRESS); a raw slot of the adaptive
-//     format is ORed word by word, vector slots are left to decode_streams.
+//     format is ORed word by word, vector slots are left to decode_vectors.
 // Malformed streams set C_ERROR (16).
 template <typename W, bool ROWS>
 __global__ void __launch_bounds__(kFT) fold_slots(LevelArgs a) {
@@ -1083,7 +1082,7 @@ __global__ void __launch_bounds__(kFT) fold_slots(LevelArgs a) {
             const int64_t count = counts[s];
             if (!ROWS && a.fmt) {
                 const int fm = (int)a.fmt[s];
-                if (fm == FMT_LIST) continue;                   // decode_streams ORs the offsets
+                if (fm == FMT_LIST) continue;                   // decode_vectors ORs the offsets
                 if (fm == FMT_RAW) {                            // the slice's raw words of this chunk
                     const uint32_t* in = static_cast<const uint32_t*>(a.xbuf) + s * a.slot_cap;
                     const int64_t w0 = b0 >> 5, w1 = (b1 + 31) >> 5;
@@ -1293,29 +1292,6 @@ __global__ void __launch_bounds__(kNT) dyn_sieve(LevelArgs a, uint32_t* __restri
 }
 
 // ------------------------------------------------------------- bottom-up --
-// OR the group bits `bits` (bit q = bitmap bit bit0 + q) into a bitmap.
-template <typename W>
-__device__ __forceinline__ void or_bits(uint32_t* dst, int64_t bit0, W bits) {
-    if (!bits) return;
-    const int64_t w = bit0 >> 5;
-    const uint32_t sh = (uint32_t)(bit0 & 31);
-    if constexpr (sizeof(W) == 4) {
-        atomicOr(dst + w, bits << sh);
-        if (sh) {
-            const uint32_t hi = bits >> (32 - sh);
-            if (hi) atomicOr(dst + w + 1, hi);
-        }
-    } else {
-        const unsigned long long x = bits;
-        const uint32_t w0 = (uint32_t)(x << sh);
-        const uint32_t w1 = sh ? (uint32_t)(x >> (32 - sh)) : (uint32_t)(x >> 32);
-        const uint32_t w2 = sh ? (uint32_t)(x >> (64 - sh)) : 0u;
-        if (w0) atomicOr(dst + w, w0);
-        if (w1) atomicOr(dst + w + 1, w1);
-        if (w2) atomicOr(dst + w + 2, w2);
-    }
-}
-
 // Zero the decoded bitmap (bottom-up levels only).
 __global__ void __launch_bounds__(kNT) clear_gbits(LevelArgs a) {
     if (!a.ctl->bu) return;
@@ -1325,20 +1301,16 @@ __global__ void __launch_bounds__(kNT) clear_gbits(LevelArgs a) {
         q[x] = make_uint4(0u, 0u, 0u, 0u);
 }
 
-// The exchanged streams decoded into one n-bit bitmap (bottom-up levels only):
-// bit q of the stream of slot (i, j) lands on vertex begin(j) + q, ORed over
-// the block-rows i.  A block (i, j) only ever tests vertices u of range j with
-// a neighbour in range i, whose bit its own stream carries (V_{i,j}(u) = 1):
-// the OR holds exactly that bit, and one bitmap serves every block-row.  One
-// warp per 32-word unit of the decoder's plan (COMPRESS: the plan of row 0,
-// whose blocks hold the p streams once), each word placed by a scan of run
-// lengths from its chunk's group base; literal groups and the active word are
-// ORed in, 1-fill runs set by the whole warp, 0-fills left as cleared.
-template <typename W>
-__global__ void __launch_bounds__(kNT) decode_streams(LevelArgs a) {
+// The exchanged slots that went as vectors of offsets, ORed into the bitmap
+// that fold_slots decodes the others to (bottom-up levels of the level-adaptive
+// format): offset q of slot (i, j) is bit begin(j) + q, ORed over the block-rows i.
+// A block (i, j) only ever tests vertices u of range j with a neighbour in range
+// i, whose bit its own slot carries (V_{i,j}(u) = 1): the OR holds exactly that
+// bit, and one bitmap serves every block-row.  One warp per 32-element unit of
+// the decoder's plan (COMPRESS: the plan of row 0, whose blocks hold the p slots
+// once).
+__global__ void __launch_bounds__(kNT) decode_vectors(LevelArgs a) {
     if (!a.ctl->bu) return;
-    using T = Wah<W>;
-    constexpr int GB = T::GB;
     const int p = a.p;
     const bool sieve = a.mode == BFS_MODE_COMPRESS_SIEVE;
     const int nblk = sieve ? p * p : p;
@@ -1360,49 +1332,12 @@ __global__ void __launch_bounds__(kNT) decode_streams(LevelArgs a) {
         } else {
             while (sl + 1 < nblk && a.slot_unit_base[sl + 1] <= g) ++sl;
         }
-        const int64_t s = sl, k = g - a.slot_unit_base[sl];
-        const int64_t j = sieve ? s % p : s;
-        const int64_t jb = range_begin(a, j), jl = range_begin(a, j + 1) - jb;
-        const int64_t G = (uint32_t)jl / (uint32_t)GB;
-        const int r = (int)((uint32_t)jl - (uint32_t)G * (uint32_t)GB);
-        const W* in = static_cast<const W*>(a.xbuf) + s * a.slot_cap;
-        const int64_t count = a.xcount[s];
-        const int64_t xw = k * 32 + lane_id();
-        const W y = (xw < count) ? in[xw] : W(0);
-        uint32_t* dst = a.gbits;
-        const int fm = a.fmt ? (int)a.fmt[s] : FMT_WAH;
-        if (fm != FMT_LIST) continue;            // fold_slots decodes the WAH and raw slots
-        if (xw < count) or_bits<uint32_t>(dst, jb + (int64_t)(uint32_t)y, 1u);   // a vertex offset
-        continue;
-        const uint32_t glen = (xw < count) ? (uint32_t)word_groups<W>(y) : 0u;
-        const uint32_t gincl = warp_incl_sum(glen);
-        const int64_t gs = a.chunk_base[s * a.chunks_per_slot + k] + (int64_t)(gincl - glen);
-        bool one = false;
-        if (xw < count) {
-            if (gs < G) {
-                if (!is_fill<W>(y)) or_bits<W>(dst, jb + gs * GB, T::from_payload(y));
-                else one = (y & T::VAL) != W(0);
-            } else if (r > 0) {
-                or_bits<W>(dst, jb + G * GB, T::from_active(y, r));
-            }
-        }
-        uint32_t m = __ballot_sync(0xffffffffu, one);
-        while (m) {
-            const int o = __ffs(m) - 1;
-            m &= m - 1;
-            const int64_t g0 = __shfl_sync(0xffffffffu, gs, o);
-            int64_t g1 = g0 + __shfl_sync(0xffffffffu, (int64_t)glen, o);
-            if (g1 > G) g1 = G;
-            const int64_t b0 = jb + g0 * GB, b1 = jb + g1 * GB;   // bits [b0, b1)
-            if (b1 <= b0) continue;
-            const int64_t w0 = b0 >> 5, w1 = (b1 - 1) >> 5;
-            for (int64_t w = w0 + lane_id(); w <= w1; w += 32) {
-                uint32_t mask = 0xffffffffu;
-                if (w == w0) mask &= 0xffffffffu << (b0 & 31);
-                if (w == w1) mask &= 0xffffffffu >> (31 - ((b1 - 1) & 31));
-                atomicOr(dst + w, mask);
-            }
-        }
+        if (a.fmt[sl] != FMT_LIST) continue;
+        const int64_t x = (g - a.slot_unit_base[sl]) * 32 + lane_id();
+        if (x >= a.xcount[sl]) continue;
+        const uint32_t* in = static_cast<const uint32_t*>(a.xbuf) + (int64_t)sl * a.slot_cap;
+        const uint32_t v = (uint32_t)range_begin(a, sieve ? sl % p : sl) + in[x];
+        atomicOr(a.gbits + (v >> 5), 1u << (v & 31u));
     }
 }
 
@@ -1937,7 +1872,6 @@ bfs_status ensure_workspace_once(bfs_graph* g) {
     W.fsum_len = ((W.bm_words + 31) / 32 + 64 + 3) / 4 * 4;   // whole 32-bit words
     const int64_t cap32 = L.nb / 31 + 2, cap64 = L.nb / 63 + 2;
     W.slot_cap = cap32;
-    W.chunk_words = 32;
     W.chunks_per_slot = (cap32 + 31) / 32;
     const int64_t xbytes = p2 * std::max<int64_t>(4 * cap32, 8 * cap64);
     W.enc_cps = parallel_encode_chunks(L.nb, 32);                       // 31-bit groups: the most chunks
@@ -2165,7 +2099,6 @@ bfs_status run_search(bfs_graph* g, int32_t root, int32_t* parent, int32_t* leve
     a.mode = mode;
     a.plain_upb = (L.nb + 1023) / 1024;               // 32 raw words per PLAIN unit
     a.win_words = W.win_words;
-    a.row_exchange = rowx ? 1 : 0;
     a.tblk = W.tblk.as<uint32_t>();
     a.rowbuf = W.rowbuf.ptr;
     a.row_cap = row_cap;
@@ -2248,7 +2181,7 @@ bfs_status run_search(bfs_graph* g, int32_t root, int32_t* parent, int32_t* leve
     // statistics, the trace and the phase events (and k is known on the host).
     auto level_body = [&](cudaStream_t s, bool host, int32_t k, cudaGraphConditionalHandle handle) -> bfs_status {
         // per-level counters (the error flag and the trace cursor persist): the
-        // stepwise loop clears them here, the graph-launched loop's level_next
+        // stepwise loop clears them here, the graph-launched loop's reduce_level
         // at the end of the level before (and the search's setup for the first)
         if (host) {
             BFS_CUDA_TRY(cudaMemsetAsync(ctr, 0, sizeof(unsigned long long) * C_ERROR, s));
@@ -2275,7 +2208,7 @@ bfs_status run_search(bfs_graph* g, int32_t root, int32_t* parent, int32_t* leve
                 const int fgrid = (int)std::min<int64_t>(std::max<int64_t>(fitems, 1), (int64_t)sm_count() * 4);
                 if (wbits == 32) fold_slots<uint32_t, false><<<fgrid, kFT, 0, s>>>(a);
                 else fold_slots<unsigned long long, false><<<fgrid, kFT, 0, s>>>(a);
-                if (adaptive) decode_streams<uint32_t><<<sm_count() * 8, kNT, 0, s>>>(a);   // vector slots
+                if (adaptive) decode_vectors<<<sm_count() * 8, kNT, 0, s>>>(a);
                 BFS_CUDA_TRY(cudaGetLastError());
             }
             if (host && timing) cudaEventRecord(W.ev[1], s);

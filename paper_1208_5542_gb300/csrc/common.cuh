@@ -51,16 +51,6 @@ __device__ __forceinline__ T warp_incl_sum(T x) {
 }
 
 template <typename T>
-__device__ __forceinline__ T warp_incl_max(T x) {
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        T y = __shfl_up_sync(0xffffffffu, x, d);
-        if (static_cast<int>(lane_id()) >= d) x = y > x ? y : x;
-    }
-    return x;
-}
-
-template <typename T>
 __device__ __forceinline__ T warp_sum(T x) {
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) x += __shfl_xor_sync(0xffffffffu, x, d);
@@ -87,27 +77,6 @@ __device__ __forceinline__ T block_incl_sum(T x, T* smem, T* total) {
     *total = smem[NW - 1];
     __syncthreads();
     return pre + incl;
-}
-
-// Block-wide inclusive max (same contract as block_incl_sum).
-template <int NT, typename T>
-__device__ __forceinline__ T block_incl_max(T x, T* smem, T* total) {
-    constexpr int NW = NT / 32;
-    const int w = threadIdx.x >> 5;
-    T incl = warp_incl_max(x);
-    if (lane_id() == 31) smem[w] = incl;
-    __syncthreads();
-    if (w == 0) {
-        T s = (lane_id() < NW) ? smem[lane_id()] : smem[0];
-        s = warp_incl_max(s);
-        if (lane_id() < NW) smem[lane_id()] = s;
-    }
-    __syncthreads();
-    T r = incl;
-    if (w > 0) { T p = smem[w - 1]; r = p > r ? p : r; }
-    *total = smem[NW - 1];
-    __syncthreads();
-    return r;
 }
 
 struct OpSum {

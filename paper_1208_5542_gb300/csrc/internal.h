@@ -139,7 +139,6 @@ struct __align__(16) Item {
 enum Counter : int {
     C_NEXT_COUNT = 0,    // vertices in the next frontier
     C_UNITS,             // work units of the expansion (WAH chunks)
-    C_ITEMS,             // decoded (vertex, block) items
     C_HITS,              // items with a nonempty column
     C_EDGES,             // adjacency entries scanned
     C_ERROR,             // nonzero: an invariant failed (code)
@@ -147,7 +146,6 @@ enum Counter : int {
     C_ROW_TRACE_USED,    // uint32 elements of the row-buffer trace written so far
     C_WAH_WORDS,         // words of all streams of this level
     C_EXCHANGED,         // set bits carried by the exchange
-    C_PIECES,            // pieces of long columns queued for the piece kernel
     C_ROW_WORDS,         // WAH words of the compressed row exchange
     C_NEXT_DEGREE,       // degree sum of the next frontier (direction choice)
     C_BOTTOM_UP,         // 1: this level ran bottom-up
@@ -171,11 +169,7 @@ struct Workspace {
     int64_t bm_words = 0;       // uint32 words of an n-bit bitmap (padded)
     int64_t fsum_len = 0;       // bytes of the frontier summary (1 per 1024 bits), words of its word-wise one
     int64_t slot_cap = 0;       // words (of the WAH width) per exchange slot
-    int64_t chunk_words = 0;    // words per expansion chunk of a stream
     int64_t chunks_per_slot = 0;
-    int slots = 0;              // exchange slots of the current mode
-    int wah_bits = 0;
-    int mode = -1;
     DevBuf whole;               // the allocation that holds what every search needs
     DevBuf pi, fa, fb, fsum, fwords, xbuf, xcount, chunk_base, units, counters, pieces;
     DevBuf level_scratch;       // per-level work counters (3 per row)

@@ -18,9 +18,9 @@
 // with an entry u -> v, by a (select, min) reduction per new lane bit.
 //
 // The whole batch is one CUDA-graph launch: the initialisation, then a
-// conditional WHILE node whose body is one level (expand, long-column pieces,
-// reduce, and a one-thread kernel that decides whether to iterate again from
-// the active count).  No host round trip per level.  Kernels read their
+// conditional WHILE node whose body is one level (expand, long-column pieces, or
+// the destinations' side; the reduction, whose last CTA decides from the active
+// count whether to iterate again).  No host round trip per level.  Kernels read their
 // arguments from a device-resident state block, so the graph is built once per
 // graph handle and reused by every call.
 #include <algorithm>
@@ -956,12 +956,14 @@ extern "C" bfs_status bfs_batch_autotune(bfs_graph_t g, const int32_t* roots, in
 
 // ===================================================================== server
 // Continuous batching over resident graphs.  Every graph keeps up to 64 lanes
-// of the bit-parallel search resident on the device; a server thread runs
-// iterations (one BFS level of every running lane) on each graph's own stream,
-// so the graphs' work overlaps on the GPU.  At every iteration boundary queued
-// requests are admitted into free lanes (a lane admitted at iteration s reports
-// level = iteration + 1 - s), and lanes whose frontier emptied are retired:
-// their level row is copied to a result buffer and the request completes.
+// of the bit-parallel search resident on the device; a server thread launches
+// iterations (one BFS level of every running lane each) on each graph's own
+// stream, so the graphs' work overlaps on the GPU.  A launch repeats iterations on
+// the device until a lane's frontier empties, a queued request could take a free
+// lane (the host calls) or kMsSteps of them ran.  Then the lanes that ended are
+// retired (their level row is copied to a result buffer and the request
+// completes) and queued requests are admitted into free lanes (a lane admitted at
+// iteration s reports level = iteration + 1 - s).
 // Graphs are admitted against an HBM budget by their footprint (layout, lane
 // state and level rows); results awaiting collection count against it too, and
 // admission of new requests pauses while they would not fit.
@@ -1085,10 +1087,7 @@ void fail(bfs_server* s, const char* what) {
     s->cv_done.notify_all();
 }
 
-// Every graph advances on its own: when its iteration has finished (a stream
-// query, no waiting on the other graphs) its lanes whose frontier emptied are
-// retired, queued requests are admitted into free lanes, and the next
-// iteration is launched.  Returns whether any graph made progress.
+// Retire the lanes whose frontier emptied in the launch that has finished.
 bool finish_iteration(bfs_server* s, ServeGraph* sg) {
     if (sg->h_alive[2]) {
         char msg[160];
@@ -1191,6 +1190,10 @@ bool launch_iteration(bfs_server* s, ServeGraph* sg) {
     return true;
 }
 
+// Every graph advances on its own: when its launch has finished (a stream
+// query, no waiting on the other graphs) its lanes whose frontier emptied are
+// retired, queued requests are admitted into free lanes, and the next launch
+// is made.  Returns whether any graph made progress.
 bool serve_pass(bfs_server* s) {
     std::vector<ServeGraph*> gs;
     {

@@ -2,9 +2,10 @@
 // fused with the cross-directory sieve (Alg. 3, Sec. V-A), and the standalone
 // codec entry points of the C ABI.
 //
-// The search's encoder works on all slots of an exchange at once in three
-// data-parallel passes (enc_chunk_*); the codec entry points encode or decode
-// one bitmap with one cluster of CTAs (wah_encode_bitmap, wah_decode_bitmap).
+// The search's encoder works on all slots of an exchange at once, in three
+// data-parallel passes (enc_chunk_*) or, where the slots are short and few, in one
+// launch (enc_small); the codec entry points encode or decode one bitmap with one
+// cluster of CTAs (wah_encode_bitmap, wah_decode_bitmap).
 #include <algorithm>
 #include <cstring>
 #include <mutex>

@@ -46,9 +46,6 @@ template <> struct Wah<uint32_t> {
     static constexpr uint32_t CNT = 0x3fffffffu;
     static constexpr uint32_t ONES = 0x7fffffffu;
     // group bits (bit q = bitmap bit pos+q) of a bitmap
-    __device__ static __forceinline__ uint32_t group(const uint32_t* bm, uint64_t pos) {
-        return bits32_at(bm, pos) & ONES;
-    }
     __device__ static __forceinline__ uint32_t group_cg(const uint32_t* bm, uint64_t pos) {
         return bits32_at_cg(bm, pos) & ONES;
     }
@@ -73,9 +70,6 @@ template <> struct Wah<unsigned long long> {
     static constexpr unsigned long long VAL = 0x4000000000000000ull;
     static constexpr unsigned long long CNT = 0x3fffffffffffffffull;
     static constexpr unsigned long long ONES = 0x7fffffffffffffffull;
-    __device__ static __forceinline__ unsigned long long group(const uint32_t* bm, uint64_t pos) {
-        return bits64_at(bm, pos) & ONES;
-    }
     __device__ static __forceinline__ unsigned long long group_cg(const uint32_t* bm, uint64_t pos) {
         return bits64_at(bm, pos) & ONES;
     }
