@@ -706,12 +706,19 @@ def main():
 
     valid = invariant_ok == len(roots) and oracle_exact in (None, 1)
     # kernels of the timed steps, per level: the encoder's passes (not PLAIN; one launch for
-    # short slots, else three), the expansion and the piece kernel, the row encoder's passes
+    # few short slots, else three), the expansion and the piece kernel, the row encoder's passes
     # and the fold (row exchange), the reduction; per search the init kernel
-    passes = 1 if -(-n // p) // (args.wah_bits - 1) <= 8 * CHUNK_GROUPS else 3
-    launches_per_level = (0 if args.mode == 0 else passes) + 2 + 1 + (passes + 1 if value_rowx else 0)
-    if args.direction != "top_down":     # bottom-up expansion (+ clear and decode of the streams)
-        launches_per_level += 1 if args.mode == 0 else (4 if args.format == "adaptive" else 3)
+    groups = -(-n // p) // (args.wah_bits - 1)
+    cta = 256 if groups <= CHUNK_GROUPS else 1024
+    sms = torch.cuda.get_device_properties(dev).multi_processor_count
+
+    def passes(slots, adaptive=False):   # the library's rule for the one-launch encoder
+        few = slots * cta <= sms * 2048 or (adaptive and cta == 256)
+        return 1 if groups <= 8 * CHUNK_GROUPS and few else 3 + int(adaptive)
+    enc = 0 if args.mode == 0 else passes(p * p if args.mode == 2 else p, args.format == "adaptive")
+    launches_per_level = enc + 2 + 1 + (passes(p * p) + 1 if value_rowx else 0)
+    if args.direction != "top_down":     # bottom-up expansion (+ decode of the streams, cleared first if ranges share words)
+        launches_per_level += 1 + (args.mode != 0) * (1 + int(-(-n // p) % 32 != 0) + int(args.format == "adaptive"))
     gpu_launches = args.steps * sum(1 + launches_per_level * st.n_levels for st in main_arm["stats"])
 
     configs = None
@@ -928,7 +935,8 @@ def bench_batch(args, bfs, graphgen, torch, dev):
                 for k in range(0, 64, 16))
     return {"metric": "aggregate GTEPS of one 64-root bit-parallel batch", "value": round(sum(m) / t_batch / 1e9, 3),
             "unit": "GTEPS", "n_gpus": 1, "steps": args.steps, "warmup": args.warmup,
-            "ms_per_step": round(1e3 * t_batch, 3), "higher_is_better": True, "dtype": "int32", "data": "synthetic",
+            "ms_per_step": round(1e3 * t_batch, 3), "ms_steps": [round(1e3 * t, 3) for t in times],
+            "higher_is_better": True, "dtype": "int32", "data": "synthetic",
             "config": {"workload": "kronecker-s20-ef16-grid8x8-batch64", "launch": "one CUDA graph per batch",
                        "autotuned_shape": {"threads": shape[0], "ctas_per_sm": shape[1]},
                        "l2": "flushed (256 MiB write) before every batch"},
