@@ -261,6 +261,13 @@ def _bitmap_words(bits, words_in: int) -> torch.Tensor:
     return src
 
 
+def _after_current(stream) -> int:
+    """Order ``stream`` after the current one, whose tensors the call reads and writes; its handle."""
+    if stream is not None and stream.cuda_stream != torch.cuda.current_stream().cuda_stream:
+        stream.wait_stream(torch.cuda.current_stream())
+    return _stream_ptr(stream)
+
+
 def wah_encode(bits: torch.Tensor, nbits: int, word_bits: int = 32, stream=None) -> torch.Tensor:
     """Encode the first ``nbits`` bits of ``bits`` (int32 CUDA words, bit b = bit b%32 of word b//32).
 
@@ -271,7 +278,9 @@ def wah_encode(bits: torch.Tensor, nbits: int, word_bits: int = 32, stream=None)
     out = torch.empty(max(1, cap), dtype=torch.int32 if word_bits == 32 else torch.int64, device="cuda")
     cnt = torch.empty(1, dtype=torch.int64, device="cuda")
     check(native.lib().bfs_wah_encode(_ptr(src), int(nbits), int(word_bits), _ptr(out), int(cap), _ptr(cnt),
-                                      _stream_ptr(stream)))
+                                      _after_current(stream)))
+    if stream is not None:
+        stream.synchronize()                # the call is only ordered on it; the count is read on the current stream
     return out[: int(cnt.item())]
 
 
@@ -279,7 +288,7 @@ def wah_decode(words: torch.Tensor, nbits: int, word_bits: int = 32, stream=None
     """Decode a stream (int32 / int64 CUDA tensor) into int32 bitmap words; raises on a malformed stream."""
     out = torch.empty(max(1, (nbits + 31) // 32), dtype=torch.int32, device="cuda")
     check(native.lib().bfs_wah_decode(_ptr(words) if words.numel() else None, int(words.numel()), int(nbits),
-                                      int(word_bits), _ptr(out), _stream_ptr(stream)))
+                                      int(word_bits), _ptr(out), _after_current(stream)))
     return out[: (nbits + 31) // 32]
 
 
@@ -289,7 +298,7 @@ def plwah_encode(bits: torch.Tensor, nbits: int, stream=None) -> torch.Tensor:
     cap = nbits // 31 + 1
     out = torch.empty(max(1, cap), dtype=torch.int32, device="cuda")
     cnt = torch.empty(1, dtype=torch.int64, device="cuda")
-    check(native.lib().bfs_plwah_encode(_ptr(src), int(nbits), _ptr(out), int(cap), _ptr(cnt), _stream_ptr(stream)))
+    check(native.lib().bfs_plwah_encode(_ptr(src), int(nbits), _ptr(out), int(cap), _ptr(cnt), _after_current(stream)))
     return out[: int(cnt.item())]
 
 
@@ -297,7 +306,7 @@ def plwah_decode(words: torch.Tensor, nbits: int, stream=None) -> torch.Tensor:
     """Decode a PLWAH stream (int32 CUDA tensor) into int32 bitmap words; raises on a malformed stream."""
     out = torch.empty(max(1, (nbits + 31) // 32), dtype=torch.int32, device="cuda")
     check(native.lib().bfs_plwah_decode(_ptr(words) if words.numel() else None, int(words.numel()), int(nbits),
-                                        _ptr(out), _stream_ptr(stream)))
+                                        _ptr(out), _after_current(stream)))
     return out[: (nbits + 31) // 32]
 
 
@@ -308,7 +317,7 @@ def bbc_encode(bits: torch.Tensor, nbits: int, stream=None) -> torch.Tensor:
     cap = n + n // 15 + 11
     out = torch.empty(cap, dtype=torch.uint8, device="cuda")
     cnt = torch.empty(1, dtype=torch.int64, device="cuda")
-    check(native.lib().bfs_bbc_encode(_ptr(src), int(nbits), _ptr(out), int(cap), _ptr(cnt), _stream_ptr(stream)))
+    check(native.lib().bfs_bbc_encode(_ptr(src), int(nbits), _ptr(out), int(cap), _ptr(cnt), _after_current(stream)))
     return out[: int(cnt.item())]
 
 
@@ -316,7 +325,7 @@ def bbc_decode(data: torch.Tensor, nbits: int, stream=None) -> torch.Tensor:
     """Decode a BBC stream (uint8 CUDA tensor) into int32 bitmap words; raises on a malformed stream."""
     out = torch.empty(max(1, (nbits + 31) // 32), dtype=torch.int32, device="cuda")
     check(native.lib().bfs_bbc_decode(_ptr(data) if data.numel() else None, int(data.numel()), int(nbits),
-                                      _ptr(out), _stream_ptr(stream)))
+                                      _ptr(out), _after_current(stream)))
     return out[: (nbits + 31) // 32]
 
 
