@@ -394,7 +394,12 @@ __global__ void __launch_bounds__(kMT) ms_pieces(MsState* S) {
 // bit of the first block-row that has one (a column is in any order: it is
 // read to its end for such a lane).  A lane of the warp scans its column kMsIlp
 // entries at a time; the rest of a column beyond kMsPullLane entries is read
-// by the whole warp.
+// by the whole warp, which takes the smallest parent of every search lane over
+// its entries and keeps it in a register to the column's end (an atomic per entry
+// and search lane instead: 17 lanes with parents at scale 20 on 4 x 4 2.26 ms against
+// 1.88, 64 lanes 5.25 against 4.47).  Four CTAs per SM, 62 registers; left to itself
+// the compiler takes 48 and spills (uniform scale 20 on 8 x 8, 64 lanes: 2.42 ms
+// against 2.29).
 constexpr uint32_t kMsPullLane = 32;
 
 // Lower the parents of v in the lanes `bits` to u; v belongs to one thread.
@@ -405,7 +410,7 @@ __device__ __forceinline__ void ms_parents(const MsState& s, int64_t v, int32_t 
     }
 }
 
-__global__ void __launch_bounds__(kMT) ms_pull(MsState* S) {
+__global__ void __launch_bounds__(kMT, 4) ms_pull(MsState* S) {
     MsState& s = *S;
     if (!s.pull) return;
     const unsigned long long* f = s.f[s.cur];
@@ -455,28 +460,46 @@ __global__ void __launch_bounds__(kMT) ms_pull(MsState* S) {
                 const uint32_t cl = __shfl_sync(0xffffffffu, len, src);
                 const unsigned long long c0 = __shfl_sync(0xffffffffu, need0, src);
                 unsigned long long cn = __shfl_sync(0xffffffffu, need, src);
-                __syncwarp();               // the parents lowered by lane src are seen below
+                uint32_t best[2] = {~0u, ~0u};          // smallest parents of search lanes lane_id(), lane_id() + 32
                 for (uint32_t e0 = kMsPullLane; e0 < cl && (cn | (c0 & pmask)); e0 += 32 * kMsIlp) {
-                    unsigned long long w = 0;
+                    int32_t u[kMsIlp];
+                    unsigned long long h[kMsIlp], w = 0;
 #pragma unroll
                     for (int k = 0; k < kMsIlp; ++k) {
                         const uint32_t x = e0 + 32 * k + lane_id();
-                        if (x >= cl) continue;
-                        const int32_t u = __ldg(s.ir + cb + x);
-                        if ((uint64_t)(uint32_t)u >= (uint64_t)s.n) {
-                            ms_fault(S, 2, (uint32_t)u, (uint64_t)cv);
-                            continue;
-                        }
-                        const unsigned long long h = __ldg(f + u) & c0;
-                        w |= h;
-                        for (unsigned long long m = h & pmask; m; m &= m - 1ull)
-                            atomicMin(reinterpret_cast<unsigned int*>(s.parents) +
-                                          (int64_t)(__ffsll((long long)m) - 1) * s.n + cv, (unsigned int)u);
+                        u[k] = x < cl ? __ldg(s.ir + cb + x) : -1;
+                    }
+#pragma unroll
+                    for (int k = 0; k < kMsIlp; ++k) {
+                        h[k] = 0ull;
+                        if (u[k] < 0) continue;
+                        if ((uint64_t)(uint32_t)u[k] < (uint64_t)s.n) h[k] = __ldg(f + u[k]) & c0;
+                        else ms_fault(S, 2, (uint32_t)u[k], (uint64_t)cv);
+                        w |= h[k];
                     }
                     const uint32_t lo = __reduce_or_sync(0xffffffffu, (uint32_t)w);
                     const uint32_t hi = __reduce_or_sync(0xffffffffu, (uint32_t)(w >> 32));
-                    cn &= ~(((unsigned long long)hi << 32) | lo);
+                    const unsigned long long hit = ((unsigned long long)hi << 32) | lo;
+                    cn &= ~hit;
+                    for (unsigned long long m = hit & pmask; m; m &= m - 1ull) {
+                        const int b = __ffsll((long long)m) - 1;
+                        uint32_t c = ~0u;
+#pragma unroll
+                        for (int k = 0; k < kMsIlp; ++k)
+                            if ((h[k] >> b) & 1ull) c = min(c, (uint32_t)u[k]);
+                        c = __reduce_min_sync(0xffffffffu, c);
+                        if ((int)lane_id() == b) best[0] = min(best[0], c);
+                        if ((int)lane_id() + 32 == b) best[1] = min(best[1], c);
+                    }
                 }
+                __syncwarp();               // the parents lowered by lane src are seen below
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    if (best[k] == ~0u) continue;
+                    unsigned int* q = reinterpret_cast<unsigned int*>(s.parents) + (int64_t)(lane_id() + 32 * k) * s.n + cv;
+                    if (best[k] < *q) *q = best[k];
+                }
+                __syncwarp();
                 if ((int)lane_id() == src) need = cn;
             }
             got |= need0 & ~need;
@@ -491,12 +514,15 @@ __global__ void __launch_bounds__(kMT) ms_pull(MsState* S) {
 // The next level runs from the destinations' side when the vertices that miss
 // a lane hold no more entries than the active ones -- a visit there is a read,
 // from the sources' side a read and often an atomic, and a miss in any of 64
-// lanes means that the whole column is read -- or, when a lane wants parents
-// (an atomic per entry and lane on the sources' side), up to kMsPullParents
-// times as many.  A level with few entries stays on the sources' side.
-// Scale 20, 64 lanes: 1.28 ms (never: 1.82; always on dense levels: 1.85), with
-// parents 4.7 (never: 7.2).
-constexpr unsigned long long kMsPullParents = 8;
+// lanes means that the whole column is read -- or, when lanes want parents (an
+// atomic per entry and lane on the sources' side), up to kMsPullParents times as
+// many.  With one block-row a column is read to its end for such a lane, and the
+// factor only pays for more than 32 of them.  A level with few entries stays on
+// the sources' side.  Scale 20, 64 lanes: 1.28 ms (never: 1.82; always on dense
+// levels: 1.85).  With parents, on one block: 17 lanes 3.07 ms with the factor, 1.66
+// without, uniform with 64 lanes 4.00 and 5.04; on 8 x 8 with 5 lanes, uniform, a
+// factor of 8 gives 0.74 ms, 4 gives 0.59.
+constexpr unsigned long long kMsPullParents = 4;
 constexpr unsigned long long kMsPullShare = 64;
 
 // One level ends: switch to the next one's buffers (one thread, the level's
@@ -515,7 +541,8 @@ __device__ void ms_advance(MsState& s, unsigned long long alive) {
     s.act_edges = 0;
     s.miss_edges = 0;
     s.lanes = alive;
-    const unsigned long long worth = s.parents && (s.parent_mask & alive) ? kMsPullParents : 1ull;
+    const int parents = s.parents ? __popcll(s.parent_mask & alive) : 0;
+    const unsigned long long worth = parents > (s.p == 1 ? 32 : 0) ? kMsPullParents : 1ull;
     s.pull = (s.symmetric && worth * e * kMsPullShare > (unsigned long long)s.nnz && miss <= worth * e) ? 1 : 0;
 }
 
