@@ -325,8 +325,8 @@ def level_rooflines(stats, n, wbits, peak, peak_src, workload):
                 acc["compress_sieve"][0] += 2 * chunk_bytes * ls["compress_chunks"] + ls["wah_bytes"]
                 acc["compress_sieve"][1] += ls["ms_compress_sieve"]
                 acc["compress_sieve"][2] += 1
-            # reduce: t, pi read; pi, f, t written (20 B per 32-bit word); a level per discovered vertex
-            acc["reduce"][0] += 20 * ((n + 31) // 32) + 4 * discovered + n // 1024
+            # reduce: t, pi read; pi, f, t written (20 B per 32-bit word); a level and a degree per discovered vertex
+            acc["reduce"][0] += 20 * ((n + 31) // 32) + 8 * discovered + n // 1024
             acc["reduce"][1] += ls["ms_reducing"]
             acc["reduce"][2] += 1
             if ls["row_compress_chunks"] or ls["row_wah_bytes"]:
