@@ -923,12 +923,12 @@ __device__ __forceinline__ void expand_pieces_level(const LevelArgs& a, uint32_t
 
 // What bounds it: at scale 12 a level is one chain of dependent steps (9 units,
 // once a warp each: 168 and 176 us for the two levels with entries; cut into
-// parts 12); at a growing level the L2 reductions of the fresh visits (about
-// 125 G/s: 11.8 M at scale 22 are 94 of its 155 us, 230 before the cut); at the
-// densest level issue slots (118 M entries in 455 us, 62% issue activity; 488
-// with a search for every entry's owner in place of head masks), and without the
-// window the scattered reads of the visited words (scale 26: 1.5 G entries, 6.8
-// -> 6.5 ms).
+// parts 12); at a growing level the latency of scattered parent reads and L2
+// reductions (scale 22: 12 M entries in 58 us and 42 of pieces, 22% issue activity,
+// L2 at 18%; scale 24: 286 M in 1.1 ms, L2 at 50%); at the densest level issue slots
+// (scale 22: 118 M entries in 435 us, 63% issue activity; 488 with a search for
+// every entry's owner in place of head masks), and without the window the
+// scattered reads of the visited words (scale 26: 1.5 G entries, 6.8 -> 6.5 ms).
 //
 // One launch expands a level: WIN is the window the graph's ranges allow, and
 // the level's own values pick the body -- with the window on dense levels,
